@@ -330,6 +330,14 @@ int gptq2d_internal_test_hook(int key, long value);
 int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alpha,
                          const double *A, long lda, const double *B, long ldb,
                          double beta, double *C, long ldc, void *stream);
+/* The same product on the int8 tensor cores by error-free splitting, as the set-up and the objective use it for their
+ * large products: both operands are written as seven base-256 digit planes in the caller's workspace (256-byte aligned,
+ * K <= 16384).  Exposed for tests. */
+size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K);
+int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha,
+                               const double *A, long lda, const double *B, long ldb,
+                               double beta, double *C, long ldc,
+                               void *workspace, size_t workspace_bytes, int *info, void *stream);
 
 #ifdef __cplusplus
 }

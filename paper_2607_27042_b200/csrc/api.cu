@@ -4,6 +4,7 @@
 #include "round_internal.cuh"
 #include "factor.cuh"
 #include "gemm.cuh"
+#include "i8_gemm.cuh"
 #include <algorithm>
 #include <atomic>
 #include <mutex>
@@ -12,7 +13,7 @@
 namespace gptq2d {
 size_t objective_workspace_bytes(int m, int n);
 int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long ldz, const double *A, long lda,
-                     const double *B, long ldb, double *obj, void *ws, cudaStream_t stream);
+                     const double *B, long ldb, double *obj, void *ws, int *info, cudaStream_t stream);
 
 __global__ void margin_kernel(const double *max_abs_e, double *min_margin) { *min_margin = 0.5 - *max_abs_e; }
 
@@ -542,7 +543,7 @@ int gptq2d_objective(int m, int n, const double *X, long ldx, const int32_t *Z, 
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
-    return launch_objective(m, n, X, ldx, Z, ldz, A, lda, B, ldb, obj, workspace, stream);
+    return launch_objective(m, n, X, ldx, Z, ldz, A, lda, B, ldb, obj, workspace, info, stream);
 }
 
 int gptq2d_internal_test_hook(int key, long value) {
@@ -575,6 +576,32 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
     g.M = M; g.N = N; g.K = K; g.alpha = alpha; g.beta = beta;
     g.A = A; g.lda = lda; g.B = B; g.ldb = ldb; g.C = C; g.ldc = ldc; g.batch = 1;
     return launch_gemm(g, static_cast<cudaStream_t>(stream_)) == cudaSuccess ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
+}
+
+size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K) {
+    if (M < 1 || N < 1 || K < 1) return 0;
+    return i8_planes_bytes(M, K, 1) + i8_planes_bytes(N, K, 1);
+}
+
+int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha, const double *A, long lda,
+                               const double *B, long ldb, double beta, double *C, long ldc, void *workspace,
+                               size_t workspace_bytes, int *info, void *stream_) {
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    if (M < 1 || N < 1 || K < 1 || K > I8_MAX_K || !A || !B || !C) return GPTQ2D_ERR_INVALID_ARG;
+    if (lda < (transa ? M : K) || ldb < (transb ? K : N) || ldc < N) return GPTQ2D_ERR_INVALID_ARG;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_internal_gemm_split_workspace_bytes(M, N, K))
+        return GPTQ2D_ERR_WORKSPACE;
+    int st = check_device();
+    if (st != GPTQ2D_OK) return st;
+    if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    GemmArgs g{};
+    g.M = M; g.N = N; g.K = K; g.alpha = alpha; g.beta = beta; g.C = C; g.ldc = ldc; g.batch = 1;
+    const I8Planes pa = i8_planes_at(workspace, M, K, 1);
+    const I8Planes pb = i8_planes_at(static_cast<char *>(workspace) + i8_planes_bytes(M, K, 1), N, K, 1);
+    cudaError_t e = i8_split(pa, A, lda, 0, !transa, stream);
+    if (e == cudaSuccess) e = i8_split(pb, B, ldb, 0, transb != 0, stream);
+    if (e != cudaSuccess || !launch_gemm_i8(g, pa, pb, info, stream, &e) || e != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    return GPTQ2D_OK;
 }
 
 }  // extern "C"

@@ -17,6 +17,7 @@
 #include "dmma_gemm.cuh"
 #include "gemm.cuh"
 #include "factor.cuh"
+#include "i8_gemm.cuh"
 
 namespace gptq2d {
 
@@ -339,12 +340,17 @@ int launch_factor_small(int nsides, const FactorSmallSide *dev_sides, int *info,
 
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
 
+// Digit planes of the operands of one large product at a time (i8_gemm.cuh).  The largest is the Gram's one k x k operand;
+// the two of a product of the inverse have at most k^2 entries together, plus padding.
+constexpr int FACTOR_I8_MIN = 1024;      // orders below keep the fp64 product: their products have few tiles
+static size_t factor_i8_bytes(int k) { return k < FACTOR_I8_MIN ? 0 : i8_planes_bytes(k + 512, k + 512, 1); }
+
 // one side: three k x k matrices (Gram / Cholesky factor, its inverse, a product buffer) and the pivots
 size_t factor_side_workspace_bytes(int k) {
     long ld = round_up(k, 16);
     size_t mat = (size_t)ld * (size_t)round_up(k, 16) * sizeof(double);
     size_t b = 3 * mat + (size_t)round_up(k, 32) * sizeof(double) + 256;
-    return (b + 255) / 256 * 256;
+    return (b + 255) / 256 * 256 + factor_i8_bytes(k);
 }
 // the two sides are factorised at the same time (two streams), each in its own part of the workspace
 size_t factor_workspace_bytes(int m, int n) { return factor_side_workspace_bytes(m) + factor_side_workspace_bytes(n); }
@@ -370,6 +376,22 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     double *T = X + mat;
     double *p = T + mat;
     const int nblk = (k + FB - 1) / FB;
+    char *i8_at = static_cast<char *>(ws) + (factor_side_workspace_bytes(k) - factor_i8_bytes(k));
+    // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream`, so one set of planes
+    // serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
+    auto product = [&](const GemmArgs &g, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
+        const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
+        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > factor_i8_bytes(k)) return launch_gemm(g, stream);
+        const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);
+        const I8Planes pb = same ? pa : i8_planes_at(i8_at + bytesA, g.N, g.K, g.batch);
+        I8Inner undo = inner;
+        undo.inverse = !inner.inverse;
+        cudaError_t e = i8_split(pa, g.A, g.lda, g.strideA, g.opA == OP_N, stream, undo, diag_a);
+        if (e == cudaSuccess && !same) e = i8_split(pb, g.B, g.ldb, g.strideB, g.opB == OP_T, stream, inner, diag_b);
+        if (e != cudaSuccess) return e;
+        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b)) return launch_gemm(g, stream);
+        return e;
+    };
 
     CK(cudaMemsetAsync(X, 0, mat * sizeof(double), stream));
     {   // Gram, lower tiles: S = M^T M or M M^T
@@ -380,7 +402,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         g.alpha = 1.0; g.beta = 0.0;
         g.A = M; g.lda = ldm; g.B = M; g.ldb = ldm;
         g.C = G; g.ldc = ld; g.batch = 1; g.lower_tiles_only = 1;
-        CK(launch_gemm(g, stream));
+        CK(product(g, true, true, true));      // a Cholesky basis has a dominant diagonal
     }
     const size_t diag_smem = (128 * 129 + 128 * 129 / 2) * sizeof(double);
     CK(cudaFuncSetAttribute(factor_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem));
@@ -397,6 +419,10 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     auto panel = [&](int K, cudaStream_t s) -> int {       // in place: P_K,0:k0 = W^T G_K,0:k0
         const long k0 = (long)K * FB;
         const int bs = (int)((k - k0) < FB ? (k - k0) : FB);
+        if (bs == FB) {
+            CK(launch_gemm_rank128(FB, (int)k0, 1.0, X + k0 * ld + k0, ld, G + k0 * ld, ld, 0.0, G + k0 * ld, ld, s));
+            return GPTQ2D_OK;
+        }
         GemmArgs g{};
         g.opA = OP_T; g.opB = OP_N;
         g.M = bs; g.N = (int)k0; g.K = bs;
@@ -408,21 +434,38 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     };
     // trailing update with the panel of block row K: rows [r0, r1) of the leading part,
     // G[r0:r1, 0:r1] -= P_K,r0:r1^T P_K,0:r1 (lower tiles only when the rows start at 0)
+    auto update = [&](const GemmArgs &t, cudaStream_t s) -> cudaError_t {
+        return (s == stream && t.lower_tiles_only) ? product(t, true) : launch_gemm(t, s);      // rows from 0 on: A and B are the same panel
+    };
     auto trailing = [&](int K, long r0, long r1, cudaStream_t s) -> int {
         const long k0 = (long)K * FB;
         const int bs = (int)((k - k0) < FB ? (k - k0) : FB);
         if (r1 <= r0) return GPTQ2D_OK;
+        // a few block rows: narrow tiles
+        if (bs == FB && r0 > 0 && r1 - r0 < 4 * FB) {
+            CK(launch_gemm_rank128((int)(r1 - r0), (int)r1, -1.0, G + k0 * ld + r0, ld, G + k0 * ld, ld, 1.0, G + r0 * ld, ld, s));
+            return GPTQ2D_OK;
+        }
         GemmArgs t{};
         t.opA = OP_T; t.opB = OP_N;
         t.M = (int)(r1 - r0); t.N = (int)r1; t.K = bs;
         t.alpha = -1.0; t.beta = 1.0;
         t.A = G + k0 * ld + r0; t.lda = ld; t.B = G + k0 * ld; t.ldb = ld;
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
-        CK(launch_gemm(t, s));
+        CK(update(t, s));
         return GPTQ2D_OK;
     };
-    // the same update with the panels of block rows [K0, K1) at once (contraction over all their rows): a rank-128
-    // update runs at 23.5 TFLOP/s, rank 256 at 28, rank 512 at 31.5 (measured, 8192^2 target, C read and rewritten)
+    // the same update with the panels of block rows [K0, K1) at once (contraction over all their rows), on the int8 tensor
+    // cores: a rank-512 update of an 8192 x 8192 target runs at 63 TFLOP/s there, at 31.7 on the fp64 tensor path (rank 128:
+    // 29 against 24).  The panels are split once, by split_panels; both updates of an outer block read the same planes.
+    auto panel_planes = [&](int K0, int K1) -> I8Planes {
+        const long k0 = (long)K0 * FB, k1 = (long)K1 * FB < k ? (long)K1 * FB : k;
+        return i8_planes_at(i8_at, (int)k0, (int)(k1 - k0), 1);
+    };
+    auto split_panels = [&](int K0, int K1, cudaStream_t s) -> int {
+        CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));
+        return GPTQ2D_OK;
+    };
     auto trailing_multi = [&](int K0, int K1, long r0, long r1, cudaStream_t s) -> int {
         const long k0 = (long)K0 * FB;
         const long k1 = (long)K1 * FB < k ? (long)K1 * FB : k;
@@ -433,12 +476,15 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.alpha = -1.0; t.beta = 1.0;
         t.A = G + k0 * ld + r0; t.lda = ld; t.B = G + k0 * ld; t.ldb = ld;
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
-        CK(launch_gemm(t, s));
+        const I8Planes pl = panel_planes(K0, K1);
+        cudaError_t e = cudaSuccess;
+        if (!launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
+        CK(e);
         return GPTQ2D_OK;
     };
-    constexpr int OUTER = 4;                 // block rows per outer block (512 rows; 2, 6 and 8 measured slower at order 8192)
-    // (orders below about 5 500 are faster with the one-level loop further down: 11.9 against 12.2 ms at 4096, 28.9
-    // against 29.2 at 6144, but 62.0 against 60.2 at 8192)
+    constexpr int OUTER = 4;                 // block rows per outer block (512 rows)
+    // (orders below about 5 500 are a little faster with the one-level loop further down: 6.56 against 6.66 ms at 4096, two
+    // sides; from 6144 on the rank-512 updates win)
     if (look && nblk >= 44) {
         // Two-level right-looking factorisation.  The block rows are grouped four by four into outer blocks of 512
         // rows.  Inside an outer block S the 128-row steps run as before (diag, panel, update of the outer block's
@@ -464,11 +510,12 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
                     if ((st = trailing(K, (long)Kb * FB, (long)K * FB, sp)) != GPTQ2D_OK) return st;
                 }
                 if (S == 0) break;
-                CK(cudaEventRecord(look->panel, sp));
                 if (S + 1 <= nS - 1 && S + 1 >= 2) CK(cudaStreamWaitEvent(sp, look->t2[(S + 1) & 1], 0));
-                int st = trailing_multi(Kb, Ke, (long)(S - 1) * OUTER * FB, (long)Kb * FB, sp);
-                if (st != GPTQ2D_OK) return st;
+                // (the large update of S+1, just waited for, was also the last reader of the planes)
+                int st = split_panels(Kb, Ke, sp);
+                if (st != GPTQ2D_OK || (st = trailing_multi(Kb, Ke, (long)(S - 1) * OUTER * FB, (long)Kb * FB, sp)) != GPTQ2D_OK) return st;
                 if (S >= 2) {
+                    CK(cudaEventRecord(look->panel, sp));
                     CK(cudaStreamWaitEvent(stream, look->panel, 0));
                     if ((st = trailing_multi(Kb, Ke, 0, (long)(S - 1) * OUTER * FB, stream)) != GPTQ2D_OK) return st;
                     CK(cudaEventRecord(look->t2[S & 1], stream));
@@ -485,7 +532,10 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
             int st = diag(K, stream);
             if (st != GPTQ2D_OK) return st;
             if (K == 0) break;
-            if ((st = panel(K, stream)) != GPTQ2D_OK || (st = trailing(K, 0, (long)K * FB, stream)) != GPTQ2D_OK) return st;
+            if ((st = panel(K, stream)) != GPTQ2D_OK) return st;
+            // block row K - 1 by itself, as with look-ahead: a tile's update goes through the same kernel on one stream or two
+            const long r0 = nblk < 4 ? 0 : (long)(K - 1) * FB;
+            if ((st = trailing(K, r0, (long)K * FB, stream)) != GPTQ2D_OK || (st = trailing(K, 0, r0, stream)) != GPTQ2D_OK) return st;
         }
     } else {
         // Spine (diag K, panel K, then the update of block row K-1, which the next diagonal block needs) on
@@ -521,38 +571,51 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         if (st_spine != GPTQ2D_OK) return st_spine;
         if (!joined) return GPTQ2D_ERR_CUDA;
     }
-    // X = P^{-1}: diagonal blocks are in place; double the block size level by level
-    for (long b = FB; b < k; b *= 2) {
-        const long npair_full = k / (2 * b);            // pairs with two full halves
-        const long rem = k - npair_full * 2 * b;        // what is left after them
-        for (int pass = 0; pass < 2; ++pass) {
-            long s0, b2, cnt;
-            if (pass == 0) { s0 = 0; b2 = b; cnt = npair_full; }
-            else { s0 = npair_full * 2 * b; b2 = rem - b; cnt = 1; }
-            if (cnt <= 0 || b2 <= 0) continue;
-            const long off11 = s0 * ld + s0, off21 = (s0 + b) * ld + s0, off22 = (s0 + b) * ld + (s0 + b);
-            const long stride = 2 * b * (ld + 1);
-            GemmArgs g1{};   // T21 = P21 X11
-            g1.opA = OP_N; g1.opB = OP_N;
-            g1.M = (int)b2; g1.N = (int)b; g1.K = (int)b;
-            g1.alpha = 1.0; g1.beta = 0.0;
-            g1.A = G + off21; g1.lda = ld; g1.strideA = stride;
-            g1.B = X + off11; g1.ldb = ld; g1.strideB = stride;
-            g1.C = T + off21; g1.ldc = ld; g1.strideC = stride;
-            g1.batch = (int)cnt;
-            g1.b_lower = 1;  // X11 is lower triangular
-            CK(launch_gemm(g1, stream));
-            GemmArgs g2{};   // X21 = -X22 T21
-            g2.opA = OP_N; g2.opB = OP_N;
-            g2.M = (int)b2; g2.N = (int)b; g2.K = (int)b2;
-            g2.alpha = -1.0; g2.beta = 0.0;
-            g2.A = X + off22; g2.lda = ld; g2.strideA = stride;
-            g2.B = T + off21; g2.ldb = ld; g2.strideB = stride;
-            g2.C = X + off21; g2.ldc = ld; g2.strideC = stride;
-            g2.batch = (int)cnt;
-            g2.a_lower = 1;  // X22 is lower triangular
-            CK(launch_gemm(g2, stream));
-        }
+    // X = P^{-1}: diagonal blocks are in place; double the block size level by level.  A pair (s0, b), (s0 + b, b2) becomes one
+    // block: X21 = -X22 (P21 X11).  The last block of a level may be longer or shorter than b; where a level has an odd number
+    // of blocks, the last one joins the pair before it at once (carried up alone, the 4 rows left over at order 4100 met a
+    // block of 4096 columns: two products of one tile row and the longest contraction, 0.56 ms of 7.3).
+    auto join = [&](long s0, long b1, long b2, long cnt, long step) -> int {     // cnt pairs, `step` rows apart
+        const long off11 = s0 * ld + s0, off21 = (s0 + b1) * ld + s0, off22 = (s0 + b1) * ld + (s0 + b1);
+        const long stride = step * (ld + 1);
+        GemmArgs g1{};   // T21 = P21 X11
+        g1.opA = OP_N; g1.opB = OP_N;
+        g1.M = (int)b2; g1.N = (int)b1; g1.K = (int)b1;
+        g1.alpha = 1.0; g1.beta = 0.0;
+        g1.A = G + off21; g1.lda = ld; g1.strideA = stride;
+        g1.B = X + off11; g1.ldb = ld; g1.strideB = stride;
+        g1.C = T + off21; g1.ldc = ld; g1.strideC = stride;
+        g1.batch = (int)cnt;
+        g1.b_lower = 1;  // X11 is lower triangular
+        // column j of P carries the scale of P[j][j], row j of X its inverse
+        I8Inner inner;
+        inner.p = p + s0; inner.stride = step;
+        CK(product(g1, false, false, true, inner));
+        GemmArgs g2{};   // X21 = -X22 T21
+        g2.opA = OP_N; g2.opB = OP_N;
+        g2.M = (int)b2; g2.N = (int)b1; g2.K = (int)b2;
+        g2.alpha = -1.0; g2.beta = 0.0;
+        g2.A = X + off22; g2.lda = ld; g2.strideA = stride;
+        g2.B = T + off21; g2.ldb = ld; g2.strideB = stride;
+        g2.C = X + off21; g2.ldc = ld; g2.strideC = stride;
+        g2.batch = (int)cnt;
+        g2.a_lower = 1;  // X22 is lower triangular
+        CK(product(g2, false, true, false));
+        return GPTQ2D_OK;
+    };
+    long nb = nblk, last = k - (long)(nblk - 1) * FB;           // blocks of this level: nb - 1 of b rows and one of `last`
+    for (long b = FB; nb > 1; b *= 2) {
+        const bool odd = (nb & 1) != 0;
+        const long pairs = nb / 2;
+        // the second block of the last pair is the odd-sized one unless a single block follows
+        const long uniform = (odd || last == b) ? pairs : pairs - 1;
+        int st = GPTQ2D_OK;
+        if (uniform > 0) st = join(0, b, b, uniform, 2 * b);
+        if (st == GPTQ2D_OK && uniform < pairs) st = join((pairs - 1) * 2 * b, b, last, 1, 0);
+        if (st == GPTQ2D_OK && odd) st = join((pairs - 1) * 2 * b, 2 * b, last, 1, 0);
+        if (st != GPTQ2D_OK) return st;
+        last = odd ? 2 * b + last : b + last;
+        nb = pairs;
     }
     dim3 grid((k + 31) / 32, (k + 31) / 32);
     factor_finish_kernel<<<grid, 256, 0, stream>>>(X, ld, p, k, out, ldo, side, dinv);

@@ -329,4 +329,93 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t stream) {
     return launch_t<false, false>(g, stream);
 }
 
+// ---------------------------------------------------------------------------------------------
+// One block row of the blocked Cholesky at a time: contraction of 128, output 128 x NT per CTA.  A 128 x 128 tile takes a CTA
+// 17 us of DMMA time whatever the number of tiles, and a block row has k0 / 128 of them (32 at order 4096, for 148 SMs);
+// tiles of 32 columns take 4.3 us, of 16 columns 2.2.  All of K is staged at once, in four groups of copies.
+constexpr int R128_LDA = 132;            // row pitches (doubles) == 4 mod 16: fragment loads touch 16 different 8-byte banks
+template <int NT>
+__global__ void __launch_bounds__(256, 1) gemm_rank128_kernel(double alpha, const double *A, long lda, const double *B, long ldb,
+                                                              double beta, double *C, long ldc) {
+    constexpr int LDB = NT + 4, NF = NT / 16;                  // fragments of 8 columns per warp
+    extern __shared__ __align__(16) double smem[];
+    double *As = smem, *Bs = smem + 128 * R128_LDA;            // [k][m], [k][n]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int wm = warp >> 1, wn = warp & 1;                   // 4 x 2 warps, each 32 rows x NT / 2 columns
+    A += (long)blockIdx.y * 128;
+    B += (long)blockIdx.x * NT;
+    C += (long)blockIdx.y * 128 * ldc + (long)blockIdx.x * NT;
+#pragma unroll
+    for (int grp = 0; grp < 4; ++grp) {
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {                       // 32 rows of k x 128: 2048 copies of 16 bytes
+            const int c = tid + it * 256, k = grp * 32 + (c >> 6), m = (c & 63) * 2;
+            cp_async16(As + k * R128_LDA + m, A + (long)k * lda + m, 16);
+        }
+#pragma unroll
+        for (int it = 0; it < NT / 16; ++it) {
+            const int c = tid + it * 256, k = grp * 32 + c / (NT / 2), n = (c % (NT / 2)) * 2;
+            cp_async16(Bs + k * LDB + n, B + (long)k * ldb + n, 16);
+        }
+        cp_async_commit();
+    }
+    double acc[4][NF][2];
+    double *c00 = C + (long)(wm * 32 + g) * ldc + wn * (NT / 2) + t * 2;
+    double2 old[4][NF];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < NF; ++b) {
+            acc[a][b][0] = acc[a][b][1] = 0.0;
+            old[a][b] = beta != 0.0 ? *reinterpret_cast<const double2 *>(c00 + (long)(a * 8) * ldc + b * 8) : double2{0.0, 0.0};
+        }
+#pragma unroll
+    for (int grp = 0; grp < 4; ++grp) {
+        if (grp == 0) cp_async_wait<3>(); else if (grp == 1) cp_async_wait<2>(); else if (grp == 2) cp_async_wait<1>(); else cp_async_wait<0>();
+        __syncthreads();
+#pragma unroll
+        for (int kk = grp * 32; kk < grp * 32 + 32; kk += 4) {
+            double af[4], bf[NF];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) af[a] = As[(kk + t) * R128_LDA + wm * 32 + a * 8 + g];
+#pragma unroll
+            for (int b = 0; b < NF; ++b) bf[b] = Bs[(kk + t) * LDB + wn * (NT / 2) + b * 8 + g];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < NF; ++b) dmma_m8n8k4(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
+        }
+    }
+    // (in place: every copy of this CTA's columns of B has landed before the barrier of the last group)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < NF; ++b) {
+            double2 o;
+            o.x = fma(beta, old[a][b].x, alpha * acc[a][b][0]);
+            o.y = fma(beta, old[a][b].y, alpha * acc[a][b][1]);
+            *reinterpret_cast<double2 *>(c00 + (long)(a * 8) * ldc + b * 8) = o;
+        }
+}
+
+template <int NT>
+static cudaError_t launch_rank128_t(int M, int N, double alpha, const double *A, long lda, const double *B, long ldb, double beta,
+                                    double *C, long ldc, cudaStream_t stream) {
+    const size_t smem = (size_t)128 * (R128_LDA + NT + 4) * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(gemm_rank128_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(gemm_rank128_kernel<NT>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    gemm_rank128_kernel<NT><<<dim3(N / NT, M / 128), 256, smem, stream>>>(alpha, A, lda, B, ldb, beta, C, ldc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_rank128(int M, int N, double alpha, const double *A, long lda, const double *B, long ldb, double beta,
+                                double *C, long ldc, cudaStream_t stream) {
+    if (M <= 0 || N <= 0) return cudaSuccess;
+    // tiles of 16 columns while they fit the SMs in one wave, of 32 beyond
+    if ((long)(M / 128) * (N / 16) <= 148) return launch_rank128_t<16>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
+    return launch_rank128_t<32>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
+}
+
 }  // namespace gptq2d

@@ -29,6 +29,11 @@ struct GemmArgs {
 
 // Enqueues the GEMM on `stream`.  Returns cudaSuccess or the launch error.
 cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t stream);
+// C = alpha * A^T B + beta * C for a contraction of exactly 128 (A: 128 x M, B: 128 x N, row-major), M a multiple of 128,
+// N of 32, everything 16-byte aligned with even leading dimensions.  With M = 128, C may be B (in place).
+// For the serial spine of the set-up: narrow tiles, so that one block row occupies all SMs for a short time.
+cudaError_t launch_gemm_rank128(int M, int N, double alpha, const double *A, long lda, const double *B, long ldb, double beta,
+                                double *C, long ldc, cudaStream_t stream);
 // 1 (default): products with a ragged tile edge whose operands are 16-byte aligned with even leading dimensions
 // go through the TMA-fed kernel, full tiles through the cp.async kernel; 3: TMA-fed kernel whenever the operands
 // allow it; 2: the same with a CTA barrier per slab; 0: everything through the cp.async kernel.

@@ -1,0 +1,66 @@
+// fp64 products on the int8 tensor cores (tcgen05), by error-free splitting (Ozaki, Ogita, Oishi, Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix multiplication", 2012): host interface.
+//
+// Every row of op(A) and every column of op(B) is scaled by a power of two and written as I8_DIGITS signed base-256
+// digits; products of digit planes are exact in int32, and the planes whose weights stay within I8_DIGITS + 1 digits
+// are summed.  See i8_gemm.cu.
+#pragma once
+#include <cuda_runtime.h>
+#include <stddef.h>
+#include <stdint.h>
+#include "gemm.cuh"
+
+namespace gptq2d {
+
+constexpr int I8_DIGITS = 7;            // 56 bits below the largest entry of a row
+constexpr int I8_KCHUNK = 64;           // k-depth of a pipeline stage; planes are padded to a multiple of it
+constexpr int I8_MAX_K = 16384;         // 7 products of |digits| <= 128 per k: 7 * 2^14 * K < 2^31
+
+// The digit planes of `batch` matrices (rows x K each, K contiguous):
+// planes[d][b * rows_pad + r][k], d = 0 the most significant digit; scale[b * rows_pad + r] = 2^(e - 36), 2^e the power
+// of two that the row's digits (as 0.d1 d2 .. in base 256) are to be multiplied by, NaN for a row with a non-finite entry.
+struct I8Planes {
+    int8_t *planes;
+    double *scale;
+    unsigned *maxbits;                  // scratch of the splitting pass: high word of a row's largest magnitude
+    int *range;                         // per 128 rows: {number of k-chunks - first chunk with an entry, last such chunk + 1}, 0 0 if none
+    int rows, K, batch;
+    long rows_pad, k_pad;
+    long plane_rows;                    // rows from one plane to the next
+    // the planes of rows [r0, r0 + count) of a single matrix; r0 a multiple of 128
+    I8Planes part(int r0, int count) const {
+        I8Planes v = *this;
+        v.planes += (long)r0 * k_pad; v.scale += r0; v.maxbits += r0; v.range += r0 / 128 * 2;
+        v.rows = count; v.rows_pad = (count + 127L) / 128 * 128;
+        return v;
+    }
+};
+size_t i8_planes_bytes(int rows, int K, int batch);
+// lays an I8Planes out at `at` (256-byte aligned)
+I8Planes i8_planes_at(void *at, int rows, int K, int batch);
+// Splits: element (r, k) of matrix b is src[b * stride + r * ld + k] (k_contig) or src[b * stride + k * ld + r].
+// With `inner`, entry k of every row is first multiplied by the power of two nearest below p[k] (or by its inverse):
+// where the rows of one operand grow along k as those of the other shrink, the two factors cancel in the product and
+// neither operand's digits are spent on the range.
+struct I8Inner {
+    const double *p = nullptr;          // positive; matrix b starts at p + b * stride
+    long stride = 0;
+    bool inverse = false;
+};
+// `skip_diagonal`: entries with k == r are left out (launch_gemm_i8 adds what they contribute).
+cudaError_t i8_split(const I8Planes &pl, const double *src, long ld, long stride, bool k_contig, cudaStream_t stream,
+                     const I8Inner &inner = I8Inner(), bool skip_diagonal = false);
+// Whether a product of this size is worth splitting: see i8_gemm.cu.
+bool gemm_i8_pays(long M, long N, long K, long batch);
+// C[b] = alpha * op(A[b]) op(B[b]) + beta * C[b] from the planes of op(A) (rows = M) and of op(B)^T (rows = N).
+// Takes M, N, K, alpha, beta, C, ldc, strideC, batch, lower_tiles_only, sumsq_partials from `g` (triangular operands
+// need no flag: the chunks of k in which an operand's 128 rows hold zeros only are skipped).  `diag_a`, `diag_b`: the
+// planes of that operand lack its diagonal, whose products are added in fp64 on the way out, from the operands in `g`.
+// A unit or dominant diagonal (triangular factors, their inverses, Cholesky bases) would otherwise set the scale of its
+// row, and the digits of all other entries with it.
+// `info`: the call's status words (a bounded wait that runs out is reported there), may be NULL.
+// False: no tensor map can be had (no driver entry point); nothing was launched.
+bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
+                    bool diag_a = false, bool diag_b = false);
+
+}  // namespace gptq2d

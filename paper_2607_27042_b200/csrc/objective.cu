@@ -1,6 +1,8 @@
 // Objective of Eq. 7: || A (Z - X) B ||_F^2, as two GEMMs and a deterministic reduction.
 #include "common.cuh"
+#include <algorithm>
 #include "gemm.cuh"
+#include "i8_gemm.cuh"
 
 namespace gptq2d {
 
@@ -28,12 +30,21 @@ __global__ void __launch_bounds__(1024) sum_partials_kernel(const double *part, 
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
 void launch_sumsq_plain(const double *M, int m, int n, long ld, double *part, int *count, cudaStream_t s);
 
-size_t objective_workspace_bytes(int m, int n) {
+// Digit planes of both operands of one of the two products at a time (i8_gemm.cuh), 0 if neither is worth splitting.
+static size_t objective_i8_bytes(int m, int n) {
+    size_t b = 0;
+    if (gemm_i8_pays(m, n, m, 1)) b = i8_planes_bytes(m, m, 1) + i8_planes_bytes(n, m, 1);
+    if (gemm_i8_pays(m, n, n, 1)) b = std::max(b, i8_planes_bytes(m, n, 1) + i8_planes_bytes(n, n, 1));
+    return b;
+}
+
+static size_t objective_f64_bytes(int m, int n) {
     long ld = round_up(n, 16);
     size_t mat = (size_t)m * ld * sizeof(double);
     size_t tiles = (size_t)((m + 127) / 128) * ((n + 127) / 128);
-    return 2 * mat + round_up((long)(tiles * sizeof(double)), 256) + 256;
+    return round_up((long)(2 * mat + round_up((long)(tiles * sizeof(double)), 256) + 256), 256);
 }
+size_t objective_workspace_bytes(int m, int n) { return objective_f64_bytes(m, n) + objective_i8_bytes(m, n); }
 
 #define CK(x)                                          \
     do {                                               \
@@ -41,7 +52,7 @@ size_t objective_workspace_bytes(int m, int n) {
     } while (0)
 
 int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long ldz, const double *A, long lda,
-                     const double *B, long ldb, double *obj, void *ws, cudaStream_t stream) {
+                     const double *B, long ldb, double *obj, void *ws, int *info, cudaStream_t stream) {
     const long ld = round_up(n, 16);
     const size_t mat = (size_t)m * ld;
     double *R = static_cast<double *>(ws);
@@ -51,6 +62,17 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
     long tot = (long)m * n;
     residual_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(m, n, X, ldx, Z, ldz, R, ld);
     CK(cudaGetLastError());
+    auto product = [&](const GemmArgs &g) -> cudaError_t {
+        if (!gemm_i8_pays(g.M, g.N, g.K, 1)) return launch_gemm(g, stream);
+        char *at = static_cast<char *>(ws) + objective_f64_bytes(m, n);
+        const I8Planes pa = i8_planes_at(at, g.M, g.K, 1);
+        const I8Planes pb = i8_planes_at(at + i8_planes_bytes(g.M, g.K, 1), g.N, g.K, 1);
+        cudaError_t e = i8_split(pa, g.A, g.lda, 0, true, stream);
+        if (e == cudaSuccess) e = i8_split(pb, g.B, g.ldb, 0, false, stream);
+        if (e != cudaSuccess) return e;
+        if (!launch_gemm_i8(g, pa, pb, info, stream, &e)) return launch_gemm(g, stream);
+        return e;
+    };
     const double *left = R;
     if (A) {   // T1 = A R
         GemmArgs g{};
@@ -58,7 +80,7 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
         g.M = m; g.N = n; g.K = m;
         g.alpha = 1.0; g.beta = 0.0;
         g.A = A; g.lda = lda; g.B = R; g.ldb = ld; g.C = T1; g.ldc = ld; g.batch = 1;
-        CK(launch_gemm(g, stream));
+        CK(product(g));
         left = T1;
     }
     GemmArgs g{};   // sum of squares of left * B, or of left itself when B is the identity
@@ -68,7 +90,7 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
         g.alpha = 1.0; g.beta = 0.0;
         g.A = left; g.lda = ld; g.B = B; g.ldb = ldb; g.C = nullptr; g.ldc = ld; g.batch = 1;
         g.sumsq_partials = part;
-        CK(launch_gemm(g, stream));
+        CK(product(g));
         sum_partials_kernel<<<1, 1024, 0, stream>>>(part, tiles, obj);
     } else {
         // || left ||_F^2 directly

@@ -39,6 +39,7 @@ EXPORTS = (
     "gptq2d_round_blocked_workspace_bytes", "gptq2d_round_blocked",
     "gptq2d_factor_batched_workspace_bytes", "gptq2d_factor_batched",
     "gptq2d_internal_test_hook", "gptq2d_internal_gemm",
+    "gptq2d_internal_gemm_split_workspace_bytes", "gptq2d_internal_gemm_split",
 )
 FACTOR_SMALL_MAX = 128
 
@@ -103,6 +104,11 @@ def _load():
     lib.gptq2d_round_static.argtypes = [i32, i32, vp, lng, vp, lng, vp, lng, vp, lng, vp, lng, vp, vp, vp]
     lib.gptq2d_internal_gemm.restype = i32
     lib.gptq2d_internal_gemm.argtypes = [i32, i32, i32, i32, i32, c.c_double, vp, lng, vp, lng, c.c_double, vp, lng, vp]
+    lib.gptq2d_internal_gemm_split_workspace_bytes.restype = sz
+    lib.gptq2d_internal_gemm_split_workspace_bytes.argtypes = [i32, i32, i32]
+    lib.gptq2d_internal_gemm_split.restype = i32
+    lib.gptq2d_internal_gemm_split.argtypes = [i32, i32, i32, i32, i32, c.c_double, vp, lng, vp, lng, c.c_double, vp, lng,
+                                               vp, sz, vp, vp]
     lib.gptq2d_internal_test_hook.restype = i32
     lib.gptq2d_internal_test_hook.argtypes = [i32, lng]
     lib.gptq2d_round_static_max_dim.restype = sz
@@ -428,6 +434,27 @@ def gptq2d_internal_gemm(A, B, C, transa=False, transb=False, alpha=1.0, beta=0.
     pC, ldc = _mat(C, torch.float64, "C")
     st = _lib.gptq2d_internal_gemm(int(transa), int(transb), M, N, K, float(alpha), pA, lda, pB, ldb, float(beta),
                                    pC, ldc, _stream_ptr(stream))
+    if st != OK:
+        raise Gptq2dError(st)
+    return C
+
+
+def gptq2d_internal_gemm_split_workspace_bytes(M, N, K):
+    return int(_lib.gptq2d_internal_gemm_split_workspace_bytes(M, N, K))
+
+
+def gptq2d_internal_gemm_split(A, B, C, transa=False, transb=False, alpha=1.0, beta=0.0, workspace=None, info=None,
+                               stream=None):
+    """C = alpha op(A) op(B) + beta C on the int8 tensor cores by error-free splitting (as gptq2d_internal_gemm)."""
+    M, N = C.shape
+    K = A.shape[0] if transa else A.shape[1]
+    pA, lda = _mat(A, torch.float64, "A")
+    pB, ldb = _mat(B, torch.float64, "B")
+    pC, ldc = _mat(C, torch.float64, "C")
+    nbytes = gptq2d_internal_gemm_split_workspace_bytes(M, N, K)
+    workspace = _workspace(nbytes, C.device) if workspace is None else workspace
+    st = _lib.gptq2d_internal_gemm_split(int(transa), int(transb), M, N, K, float(alpha), pA, lda, pB, ldb, float(beta),
+                                         pC, ldc, _ptr(workspace), workspace.numel(), _ptr(info), _stream_ptr(stream))
     if st != OK:
         raise Gptq2dError(st)
     return C
