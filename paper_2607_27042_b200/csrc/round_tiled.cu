@@ -332,15 +332,6 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
         cp_async_commit();
         cp_async_wait<0>();
     };
-    if (tid == 7 * 32) {
-        // this quadrant is about to sweep: the one below it and the one to its right may start getting ready
-        const int qi = sm.q >> 1, qj = sm.q & 1;
-        if (qi == 0) quadrant_arrive(p, sm.I, sm.J, sm.q + 2);
-        else if (sm.I + 1 < p.ntm) quadrant_arrive(p, sm.I + 1, sm.J, sm.q - 2);
-        if (qj == 0) quadrant_arrive(p, sm.I, sm.J, sm.q + 1);
-        else if (sm.J + 1 < p.ntn) quadrant_arrive(p, sm.I, sm.J + 1, sm.q - 1);
-    }
-    __syncwarp();
     if (fresh && warp == 7) fetch_block(0);
 
     TS_MARK(2);                                          // tables, first fetch
@@ -400,18 +391,23 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
             leaf_pull(Ys, Cs, Ls, Us, a, b, g, t);
             __syncwarp();
             TS_MARK(lw <= 7 ? 6 : 10);                       // leaf_pull
-            // Phase A.  Lane l owns entries (i0, j) and (i0 + 4, j) of the 8 x 8 leaf, i0 = l & 3,
-            // j = l >> 2.  At step s the lane whose entry lies on anti-diagonal s rounds it and posts
-            // the error (by column) and the final C value (by row) to a 16-double per-warp exchange
-            // buffer; after a warp barrier EVERY lane applies one downward and one rightward push
-            // to both of its entries (Algorithm 3 lines 8-16 restricted to the leaf).  The pushes
-            // are branch-free: the coefficients come from tables that hold zeros wherever no push
-            // is due (source not on this anti-diagonal, or entry already rounded), so stale
-            // exchange slots are multiplied by zero.
+            // Phase A.  Lane l owns entries (i0, j) and (i0 + 4, j) of the 8 x 8 leaf, i0 = l & 3, j = l >> 2.  At step s the
+            // entry on anti-diagonal s is rounded and its error (by column) and final C value (by row) go to a 16-double
+            // per-warp exchange buffer; after a warp barrier EVERY lane applies one downward and one rightward push to both
+            // of its entries (Algorithm 3 lines 8-16 restricted to the leaf).  Y and C receive the same downward pushes, so
+            // W = Y - C is kept, which receives the rightward ones only, and Y = W + C is formed to round.
+            // Nothing branches.  The push coefficients come from tables that hold zeros wherever no push is due (source
+            // not on this anti-diagonal, or entry already rounded), so stale exchange slots are multiplied by zero; and
+            // every lane rounds both entries at every step, of which only the values at the entry's own step are posted:
+            // before it W and C are incomplete, after it they do not change any more, so the last step leaves every lane's
+            // final values.  A step is a chain of latencies (add 8, round 16, subtract 8, add 8, store to load 35, fma 8);
+            // the branch around the rounding, with the range check in it, cost another 60 of 180 cycles (one warp
+            // alone, 8 x 8 leaf: 2696 -> 1808 cycles; eight warps 3087 -> 2762, where the shared-memory pipe is the bound).
             const int i0 = lane & 3, j = lane >> 2;
             double *yp = Ys + CI((a * 8 + i0) * QLD + b * 8 + j, QMAT - 4 * QLD, 114);
             double *cp = Cs + CI((a * 8 + i0) * QLD + b * 8 + j, QMAT - 4 * QLD, 115);
-            double y0 = yp[0], y1 = yp[4 * QLD], c0 = cp[0], c1 = cp[4 * QLD];
+            double c0 = cp[0], c1 = cp[4 * QLD], w0 = yp[0] - c0, w1 = yp[4 * QLD] - c1;
+            double y0, y1, g0, g1;
             // tabL[row][7 + is] = L(row, is) for 0 <= is < row else 0; at step s, is = s - j
             const double *tl0 = tabL + CI((a * 8 + i0) * TAB_LD + 7 - j, (Q - 4) * TAB_LD - 14, 116);
             const double *tl1 = tl0 + 4 * TAB_LD;
@@ -421,31 +417,42 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
             double *exw = xch + warp * 32;
             int z0 = 0, z1 = 0;
             const int t0 = i0 + j, t1 = t0 + 4;
+            // round half to even: adding and subtracting 1.5 * 2^52 leaves the integer, whose low word is the sum's; values that
+            // do not fit 32 bits are looked for after the leaf, by the high word that each had at its own step (a NaN reaches
+            // entries rounded before it through the zero coefficients)
+            constexpr double MAGIC = 6755399441055744.0;
+            int h0 = 0, h1 = 0;
 #pragma unroll
             for (int s = 0; s < 15; ++s) {
+                const double v0 = w0 + c0, v1 = w1 + c1, r0 = v0 + MAGIC, r1 = v1 + MAGIC;
+                z0 = t0 == s ? __double2loint(r0) : z0; z1 = t1 == s ? __double2loint(r1) : z1;
+                h0 = t0 == s ? __double2hiint(v0) : h0; h1 = t1 == s ? __double2hiint(v1) : h1;
+                y0 = (r0 - MAGIC) - v0; y1 = (r1 - MAGIC) - v1;         // line 5: E = Z - Y
+                g0 = c0 + y0; g1 = c1 + y1;                             // fold, L_ii = 1
+                if (s == 14) break;
                 double *ex = exw + (s & 1) * 16;                        // [0..7] e by column, [8..15] C by row
-                const bool r0 = (t0 == s), r1 = (t1 == s);
-                if (r0 || r1) {
-                    const double yv = r0 ? y0 : y1;
-                    const double zv = rint(yv);
-                    const double e = zv - yv;                           // line 5: E = Z - Y
-                    const double cf = (r0 ? c0 : c1) + e;               // fold, L_ii = 1
-                    ex[j] = e;
-                    ex[8 + i0 + (r0 ? 0 : 4)] = cf;
-                    if (r0) { y0 = e; c0 = cf; z0 = (int)zv; }
-                    else { y1 = e; c1 = cf; z1 = (int)zv; }
-                    if (!(fabs(yv) < 2147483648.0)) {                   // not representable: remember the first
-                        const unsigned long long gr = row0 + a * 8 + i0 + (r0 ? 0 : 4), gc = col0 + b * 8 + j;
-                        const unsigned long long key = ((gr + gc) << 42) | ((isfinite(yv) ? 1ull : 0ull) << 41) |
-                                                       (gr << 20) | gc;
-                        if (gr < (unsigned long long)p.m && gc < (unsigned long long)p.n && key < badkey) badkey = key;
-                    }
+                const double l0 = tl0[s], l1 = tl1[s], u0 = tu0[s], u1 = tu1[s];
+                if (t0 == s || t1 == s) {
+                    ex[j] = t0 == s ? y0 : y1;
+                    ex[8 + i0 + (t0 == s ? 0 : 4)] = t0 == s ? g0 : g1;
                 }
                 __syncwarp();
                 const double ed = ex[j], cr0 = ex[8 + i0], cr1 = ex[12 + i0];
-                const double l0 = tl0[s], l1 = tl1[s], u0 = tu0[s], u1 = tu1[s];
-                y0 = fma(l0, ed, y0); c0 = fma(l0, ed, c0); y0 = fma(cr0, u0, y0);   // fold, push down, push right
-                y1 = fma(l1, ed, y1); c1 = fma(l1, ed, c1); y1 = fma(cr1, u1, y1);
+                c0 = fma(l0, ed, c0); w0 = fma(cr0, u0, w0);            // push down, push right
+                c1 = fma(l1, ed, c1); w1 = fma(cr1, u1, w1);
+            }
+            c0 = g0; c1 = g1;
+            {   // values that do not fit 32 bits (high word at or above that of 2^31; infinities and NaNs are): remember the first
+                if (max(h0 & 0x7fffffff, h1 & 0x7fffffff) >= 0x41e00000) {
+                    auto look = [&](int h, int row, int &z) {
+                        if ((h & 0x7fffffff) < 0x41e00000) return;
+                        z = (int)__hiloint2double(h, 0);                // saturates
+                        const unsigned long long gr = row0 + a * 8 + row, gc = col0 + b * 8 + j;
+                        const unsigned long long key = ((gr + gc) << 42) | (((h & 0x7fffffff) < 0x7ff00000 ? 1ull : 0ull) << 41) | (gr << 20) | gc;
+                        if (gr < (unsigned long long)p.m && gc < (unsigned long long)p.n && key < badkey) badkey = key;
+                    };
+                    look(h0, i0, z0); look(h1, i0 + 4, z1);
+                }
             }
             yp[0] = y0; yp[4 * QLD] = y1; cp[0] = c0; cp[4 * QLD] = c1;
             TS_MARK(lw <= 7 ? 7 : 11);                       // the 15 anti-diagonal steps
@@ -592,6 +599,15 @@ __device__ __forceinline__ void sweep_quadrant(int I, int J, int q, double *smem
     }
 
     TS_MARK(0);                                          // pulls from the two nearest tiles
+    if (tid == 7 * 32) {
+        // This quadrant is about to sweep: the one below it and the one to its right may start getting ready.  Told here, before
+        // this quadrant's own operand loads: what they do first (their pulls and loads, 60 thousand cycles) takes longer than the
+        // nine leaf-waves that they run behind this one (1024 x 4096: 2.76 -> 2.49 ms against telling them at the first leaf-wave).
+        if (qi == 0) quadrant_arrive(p, I, J, q + 2);
+        else if (I + 1 < p.ntm) quadrant_arrive(p, I + 1, J, q - 2);
+        if (qj == 0) quadrant_arrive(p, I, J, q + 1);
+        else if (J + 1 < p.ntn) quadrant_arrive(p, I, J + 1, q - 1);
+    }
     // ---- 2. operands of the sweep
     Stream sm;
     sm.I = I; sm.J = J; sm.q = q;
