@@ -241,13 +241,17 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
         small.push_back(FactorSmallSide{q.m, 0, b, q.A, q.lda, q.L, q.ldl, q.dL});
         small.push_back(FactorSmallSide{q.n, 1, b, q.B, q.ldb, q.U, q.ldu, q.dU});
     }
+    std::stable_sort(small.begin(), small.end(),
+                     [](const FactorSmallSide &x, const FactorSmallSide &y) { return factor_small_class(x.k) < factor_small_class(y.k); });
+    int small_counts[3] = {0, 0, 0};
+    for (const FactorSmallSide &q : small) ++small_counts[factor_small_class(q.k)];
     char *w = static_cast<char *>(workspace);
     if (!small.empty()) {
         // pageable source: the copy is staged before the call returns, so the vector may go out of scope
         if (cudaMemcpyAsync(w, small.data(), small.size() * sizeof(FactorSmallSide), cudaMemcpyHostToDevice, stream) !=
             cudaSuccess)
             return GPTQ2D_ERR_CUDA;
-        st = launch_factor_small((int)small.size(), reinterpret_cast<const FactorSmallSide *>(w), info, stream);
+        st = launch_factor_small(small_counts, reinterpret_cast<const FactorSmallSide *>(w), info, stream);
         if (st != GPTQ2D_OK) return st;
     }
     char *wl = w + factor_batched_table_bytes(count);

@@ -23,171 +23,215 @@ namespace gptq2d {
 
 constexpr int FB = 128;
 
-// One CTA.  S: bs x bs Schur complement (lower triangle read).  Writes P (lower, in place),
-// W = P^{-1} (full block, zeros above the diagonal) and diag(P).
-// The block is padded to 128 x 128 with the identity in shared memory.  Cholesky runs from the last
-// index to the first, blocked sixteen rows at a time (row scaling + rank-one update of the block's own rows
-// per step, one rank-16 DMMA update of the rows above per block); the inverse is built from 32 x 32 diagonal blocks by doubling,
-// W21 = -W22 (P21 W11), both products as m8n8k4 DMMA fragments, with the temporary product kept in
-// the unused upper triangle of the P array.
-__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }   // packed lower triangle
+// Cholesky factor and inverse of one block, in shared memory, by one CTA of 256 threads.  Orders up to NP (64, 96 or 128: the
+// block is padded to NP x NP with the identity).  a[NP][NP + 4]: row pitch == 4 mod 16 doubles, so that the 8 x 4 fragments of
+// the fp64 tensor path touch sixteen different 8-byte banks.  w: packed lower triangle.
+__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
+template <int NP>
+struct CholBlock {
+    static constexpr int LD = NP + 4;
+    static constexpr size_t SMEM = (size_t)(NP * LD + NP * (NP + 1) / 2) * sizeof(double);
+};
 
-// In place, in shared memory, by one CTA of 256 threads: a [128][129] holds the lower triangle of a Schur
-// complement padded to 128 x 128 with the identity (bs rows are real); on return its lower triangle is P
-// (S = P^T P, Cholesky from the last index to the first) and w is the packed lower triangle of W = P^{-1}.
-// Ends with a barrier.  err_c: what a non-positive pivot reports in info[3], beside its index and the side.
-__device__ __forceinline__ void chol_inverse_128(double *a, double *w, int bs, int *info, int side, int k0, int err_c) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    // Blocked, sixteen rows R = [r_lo, r_hi) at a time from the last block to the first, three barriers a block:
-    //  (1) warp 0 factors the block's own 16 x 16 part in place (the unblocked steps -- scale row k, rank-one update of
-    //      the rows of R above k -- between warp barriers only) and leaves 1 / P[k][k] in s_rk;
-    //  (2) every column j < r_lo of the block's rows is a triangular solve of its own, one thread per column, sixteen
-    //      values in registers:  P[k][j] = (A[k][j] - sum_{k' in R, k' > k} P[k'][k] P[k'][j]) / P[k][k],  k descending;
-    //  (3) the rows above the block receive the block's sixteen rank-one updates at once, as 8 x 8 fragments of the
-    //      lower triangle on the fp64 tensor path (four m8n8k4 products each).
-    // (The unblocked loop rewrote up to 128 x 128 entries of shared memory per step behind two CTA barriers: 57 of the
-    // kernel's 102 us.)  Rows from bs on are identity padding: they factor to the identity and contribute nothing.
-    __shared__ double s_rk[16];
-    // warp 0's share of the 16 x 16 lower triangle in (1): entries e = lane + 32 u -> (ii, jj), jj <= ii, row by row
-    int tri_i[4], tri_j[4];
+// X21 = -W22 (P21 W11) for PAIRS pairs of blocks (b1 and b2 rows, `step` rows apart, the first at 0), on the fp64 tensor path.  A warp
+// takes a row of 8 x 8 fragments of a pair (a 1 / CP part of its columns), all of them at once: one fragment of the left
+// operand is loaded for FU products in flight.  The temporary product lies, transposed, above the diagonal of a.
+template <int NP, int PAIRS, int B1, int B2, int CP>
+__device__ __forceinline__ void inverse_join(double *a, double *w, int step) {
+    constexpr int LD = CholBlock<NP>::LD, FU = B1 / 8 / CP, ROWS = PAIRS * (B2 / 8);
+    static_assert(ROWS * CP <= 8, "one unit per warp");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int row = warp / CP, pr = row / (B2 / 8), fr = row - pr * (B2 / 8), s0 = pr * step, f0 = (warp - row * CP) * FU;
+    const bool on = row < ROWS;
+    double c[FU][2];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        int ii = 0, r = (tid & 31) + 32 * u;
-        while (r > ii) { r -= ii + 1; ++ii; }
-        tri_i[u] = ii; tri_j[u] = r;
-    }
-    for (int kb = (bs - 1) >> 4; kb >= 0; --kb) {
-        const int r_lo = 16 * kb;
-        if (tid < 32) {
-            for (int kk = 15; kk >= 0; --kk) {
-                const int k = r_lo + kk;
-                double d = a[k * 129 + k];
-                if (!(d > 0.0) || !isfinite(d)) {
-                    if (tid == 0) report(info, GPTQ2D_ERR_NOT_SPD, k0 + k, side, err_c);
-                    d = 1.0;
-                }
-                double rk = rsqrt(d);
-                rk = rk * fma(-0.5 * d, rk * rk, 1.5);         // one Newton step: 1 / sqrt(d) to the last bit or two
-                // entries (i, j) of the rows of R above k, r_lo <= j <= i < k: at most 120, four per lane
-                double v[4], pi[4], pj[4];
-                int at[4];
+    for (int f = 0; f < FU; ++f) c[f][0] = c[f][1] = 0.0;
+    if (on) {                                                  // T = P21 W11
+        for (int kk = 8 * f0; kk < B1; kk += 4) {              // W11[k][c] = 0 for k < c
+            const int k = kk + t;
+            const double af = a[(s0 + B1 + 8 * fr + g) * LD + s0 + k];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool on = tri_i[u] < kk;
-                    at[u] = on ? (r_lo + tri_i[u]) * 129 + r_lo + tri_j[u] : -1;
-                    v[u] = on ? a[at[u]] : 0.0;
-                    pi[u] = on ? a[k * 129 + r_lo + tri_i[u]] * rk : 0.0;
-                    pj[u] = on ? a[k * 129 + r_lo + tri_j[u]] * rk : 0.0;
-                }
-                __syncwarp();
-                if (tid < kk) a[k * 129 + r_lo + tid] *= rk;   // P[k][r_lo + tid]
-                if (tid == 0) { a[k * 129 + k] = d * rk; s_rk[kk] = rk; }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (at[u] >= 0) a[at[u]] = fma(-pi[u], pj[u], v[u]);
-                __syncwarp();
+            for (int f = 0; f < FU; ++f) {
+                const int cc = 8 * (f0 + f) + g;
+                const double bf = k >= cc ? w[tri(s0 + k, s0 + min(cc, k))] : 0.0;         // index clamped: stays inside the array
+                dmma_m8n8k4(c[f][0], c[f][1], af, bf);
             }
         }
-        __syncthreads();
-        if (kb > 0 && tid < r_lo) {
-            double x[16];
 #pragma unroll
-            for (int kk = 0; kk < 16; ++kk) x[kk] = a[(r_lo + kk) * 129 + tid];
-#pragma unroll
-            for (int kk = 15; kk >= 0; --kk) {
-                double sum = x[kk];
-#pragma unroll
-                for (int k2 = 15; k2 > kk; --k2) sum = fma(-a[(r_lo + k2) * 129 + r_lo + kk], x[k2], sum);
-                x[kk] = sum * s_rk[kk];
-            }
-#pragma unroll
-            for (int kk = 0; kk < 16; ++kk) a[(r_lo + kk) * 129 + tid] = x[kk];
-        }
-        __syncthreads();
-        if (kb > 0) {
-            // leading (16 kb) x (16 kb) lower triangle -= P[R, :]^T P[R, :]
-            const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-            const int nb = 2 * kb, nfrag = nb * (nb + 1) / 2;
-            for (int f = warp; f < nfrag; f += 8) {
-                int bi = 0, r = f;
-                while (r > bi) { r -= bi + 1; ++bi; }
-                const int bj = r;
-                double c0 = 0.0, c1 = 0.0;
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const double *row = a + (r_lo + 4 * kk + t) * 129;
-                    dmma_m8n8k4(c0, c1, row[8 * bi + g], row[8 * bj + g]);
-                }
-                const int ri = 8 * bi + g, cj = 8 * bj + 2 * t;
-                if (cj <= ri) a[ri * 129 + cj] -= c0;
-                if (cj + 1 <= ri) a[ri * 129 + cj + 1] -= c1;
-            }
-            __syncthreads();
-        }
-    }
-    // ---- W = P^{-1}.  Level 0: the four 32 x 32 diagonal blocks, one column per thread.
-    if (tid < 128) {
-        const int r0 = tid & ~31, j = tid & 31;
-        w[tri(r0 + j, r0 + j)] = 1.0 / a[(r0 + j) * 129 + r0 + j];
-        for (int i = j + 1; i < 32; ++i) {
-            double s0 = 0.0, s1 = 0.0;
-            int k = j;
-            for (; k + 1 < i; k += 2) {
-                s0 = fma(a[(r0 + i) * 129 + r0 + k], w[tri(r0 + k, r0 + j)], s0);
-                s1 = fma(a[(r0 + i) * 129 + r0 + k + 1], w[tri(r0 + k + 1, r0 + j)], s1);
-            }
-            if (k < i) s0 = fma(a[(r0 + i) * 129 + r0 + k], w[tri(r0 + k, r0 + j)], s0);
-            w[tri(r0 + i, r0 + j)] = -(s0 + s1) / a[(r0 + i) * 129 + r0 + i];
+        for (int f = 0; f < FU; ++f) {
+            double *dst = a + (s0 + 8 * (f0 + f) + 2 * t) * LD + s0 + B1 + 8 * fr + g;
+            dst[0] = c[f][0];
+            dst[LD] = c[f][1];
+            c[f][0] = c[f][1] = 0.0;
         }
     }
     __syncthreads();
-    // ---- doubling: blocks of b = 32, then 64, on the fp64 tensor path.  The 128 / (2 b) pairs have b / 8
-    // rows of 8 x 8 fragments each, eight rows in all: one per warp, which takes every fragment of its row.
-    // The triangular operands come from the packed array, zeros where the packed array has no entry.
-    {
-        const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-        for (int b = 32; b < 128; b *= 2) {
-            const int nf = b >> 3, pr = warp / nf, fr = warp - pr * nf, s0 = pr * 2 * b;
-            // T = P21 W11, stored above the diagonal at rows s0 .., columns s0 + b ..
-            for (int fc = 0; fc < nf; ++fc) {
-                double c0 = 0.0, c1 = 0.0;
-                const int cc = 8 * fc + g;
-                for (int kk = 8 * fc; kk < b; kk += 4) {       // W11[k][c] = 0 for k < c
-                    const int k = kk + t;
-                    const double af = a[(s0 + b + 8 * fr + g) * 129 + s0 + k];
-                    const double bf = k >= cc ? w[tri(s0 + k, s0 + min(cc, k))] : 0.0;     // index clamped: stays inside the array
-                    dmma_m8n8k4(c0, c1, af, bf);
+    if (on) {                                                  // W21 = -W22 T
+        const int rr = 8 * fr + g;
+        for (int kk = 0; kk < 8 * fr + 8; kk += 4) {           // W22[r][k] = 0 for k > r
+            const int k = kk + t;
+            const double af = k <= rr ? w[tri(s0 + B1 + rr, s0 + B1 + min(k, rr))] : 0.0;
+#pragma unroll
+            for (int f = 0; f < FU; ++f) dmma_m8n8k4(c[f][0], c[f][1], af, a[(s0 + 8 * (f0 + f) + g) * LD + s0 + B1 + k]);
+        }
+#pragma unroll
+        for (int f = 0; f < FU; ++f) {
+            double *dst = w + tri(s0 + B1 + rr, s0 + 8 * (f0 + f) + 2 * t);
+            dst[0] = -c[f][0];
+            dst[1] = -c[f][1];
+        }
+    }
+    __syncthreads();
+}
+
+// 1 / sqrt(d) to the last bit or two, d > 0 and finite: the hardware's approximation (relative error below 2^-20) and two
+// Newton steps r += r/2 (1 - d r r), which leave 2^-41 and then rounding.  In line and without the library function's range
+// handling it is 60 cycles shorter, 128 times on the serial chain of a block; the approximation flushes denormals, so the
+// smallest pivots take the function.
+__device__ __forceinline__ double pivot_rsqrt(double d) {
+    if (d < 0x1p-1000) return rsqrt(d);
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
+    r = fma(0.5 * r, fma(-d * r, r, 1.0), r);
+    return fma(0.5 * r, fma(-d * r, r, 1.0), r);
+}
+
+// a holds the lower triangle of a Schur complement (bs rows are real); on return its lower triangle is P (S = P^T P, Cholesky from
+// the last index to the first) and w is the packed lower triangle of W = P^{-1}.  Ends with a barrier.
+// err_c: what a non-positive pivot reports in info[3], beside its index and the side.
+template <int NP>
+__device__ __forceinline__ void chol_inverse(double *a, double *w, int bs, int *info, int side, int k0, int err_c) {
+    constexpr int LD = CholBlock<NP>::LD;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    // Blocked, sixteen rows R = [r_lo, r_hi) at a time from the last block to the first, three barriers a block:
+    //  (1) warp 0 factors the block's own 16 x 16 part, a column per lane in registers (lanes 16 - 31 repeat lanes 0 - 15);
+    //  (2) every column j < r_lo of the block's rows is a triangular solve of its own, one thread per column, sixteen
+    //      values in registers:  P[k][j] = (A[k][j] - sum_{k' in R, k' > k} P[k'][k] P[k'][j]) / P[k][k],  k descending;
+    //  (3) the rows above the block receive the block's sixteen rank-one updates at once, as 8 x 8 fragments of the
+    //      lower triangle on the fp64 tensor path (four m8n8k4 products each), two rows of fragments per warp.
+    // Rows from bs on are identity padding: they factor to the identity and contribute nothing.
+    // The whole is a chain of latencies.  In (1) a step's chain is: reciprocal square root of the pivot, scaling of the lane's entry
+    // of row k, update of the next pivot by the lane that owns it, one shuffle to all; the other updates of the step fill
+    // the time of the next square root.  Order 128, thousands of cycles (with the loads and stores around it 84 -> 45 us): (1) 62 -> 34,
+    // (3) 30 -> 13 (fragments were decoded one by one), inverse 49 -> 16 (one chain per column of 32, one fragment at a time).
+    __shared__ double s_rk[16];
+    for (int kb = (bs - 1) >> 4; kb >= 0; --kb) {
+        const int r_lo = 16 * kb;
+        if (warp == 0) {
+            const int j = lane & 15;
+            double x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = a[(r_lo + i) * LD + r_lo + j];              // rows i < j: never used
+            double d = __shfl_sync(0xffffffffu, x[15], 15), rmine = 0.0;
+            int bad = -1;
+#pragma unroll
+            for (int kk = 15; kk >= 0; --kk) {
+                if (!(d > 0.0) || !isfinite(d)) { bad = max(bad, kk); d = 1.0; }
+                const double rk = pivot_rsqrt(d);
+                const double pk = x[kk] * rk;                  // P[k][j], j < k
+                if (kk > 0) {
+                    x[kk - 1] = fma(-__shfl_sync(0xffffffffu, pk, kk - 1), pk, x[kk - 1]);
+                    const double dn = __shfl_sync(0xffffffffu, x[kk - 1], kk - 1);
+#pragma unroll
+                    for (int i = kk - 2; i >= 0; --i) x[i] = fma(-__shfl_sync(0xffffffffu, pk, i), pk, x[i]);
+                    x[kk] = j == kk ? d * rk : pk;
+                    if (j == kk) rmine = rk;
+                    d = dn;
+                } else {
+                    x[0] = j == 0 ? d * rk : pk;
+                    if (j == 0) rmine = rk;
                 }
-                double *dst = a + (s0 + 8 * fr + g) * 129 + s0 + b + 8 * fc + 2 * t;
-                dst[0] = c0;
-                dst[1] = c1;
+            }
+            if (bad >= 0 && lane == 0) report(info, GPTQ2D_ERR_NOT_SPD, k0 + r_lo + bad, side, err_c);
+            if (lane < 16) {
+                s_rk[j] = rmine;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (i >= j) a[(r_lo + i) * LD + r_lo + j] = x[i];
+            }
+        }
+        __syncthreads();
+        if (kb > 0) {
+            if (tid < r_lo) {
+                double x[16];
+#pragma unroll
+                for (int kk = 0; kk < 16; ++kk) x[kk] = a[(r_lo + kk) * LD + tid];
+#pragma unroll
+                for (int kk = 15; kk >= 0; --kk) {
+                    double sum = x[kk];
+#pragma unroll
+                    for (int k2 = 15; k2 > kk; --k2) sum = fma(-a[(r_lo + k2) * LD + r_lo + kk], x[k2], sum);
+                    x[kk] = sum * s_rk[kk];
+                }
+#pragma unroll
+                for (int kk = 0; kk < 16; ++kk) a[(r_lo + kk) * LD + tid] = x[kk];
             }
             __syncthreads();
-            // W21 = -W22 T
-            for (int fc = 0; fc < nf; ++fc) {
-                double c0 = 0.0, c1 = 0.0;
-                const int rr = 8 * fr + g;
-                for (int kk = 0; kk < 8 * fr + 8; kk += 4) {   // W22[r][k] = 0 for k > r
-                    const int k = kk + t;
-                    const double af = k <= rr ? w[tri(s0 + b + rr, s0 + b + min(k, rr))] : 0.0;
-                    const double bf = a[(s0 + k) * 129 + s0 + b + 8 * fc + g];
-                    dmma_m8n8k4(c0, c1, af, bf);
+            // leading (16 kb) x (16 kb) lower triangle -= P[R, :]^T P[R, :]
+            const int nb = 2 * kb;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int bi = nb - 1 - (h ? 15 - warp : warp);                // a long row of fragments and a short one
+                if (bi < 0) continue;
+                double af[4];
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) af[kk] = a[(r_lo + 4 * kk + t) * LD + 8 * bi + g];
+                const int ri = 8 * bi + g;
+#pragma unroll 2
+                for (int bj = 0; bj <= bi; ++bj) {
+                    const int cj = 8 * bj + 2 * t;
+                    double c0 = 0.0, c1 = 0.0;
+                    const double o0 = a[ri * LD + cj], o1 = a[ri * LD + cj + 1];
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) dmma_m8n8k4(c0, c1, af[kk], a[(r_lo + 4 * kk + t) * LD + 8 * bj + g]);
+                    if (cj <= ri) a[ri * LD + cj] = o0 - c0;
+                    if (cj + 1 <= ri) a[ri * LD + cj + 1] = o1 - c1;
                 }
-                double *dst = w + tri(s0 + b + rr, s0 + 8 * fc + 2 * t);
-                dst[0] = -c0;
-                dst[1] = -c1;
             }
             __syncthreads();
         }
+    }
+    // ---- W = P^{-1}.  Level 0: the 16 x 16 diagonal blocks, one column per thread, in registers.
+    if (tid < NP) {
+        const int r0 = tid & ~15, j = tid & 15;
+        const double inv = 1.0 / a[(r0 + j) * LD + r0 + j];
+        double y[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+            for (int k = 0; k < i; ++k) {
+                if (k & 1) s1 = fma(a[(r0 + i) * LD + r0 + k], y[k], s1);
+                else s0 = fma(a[(r0 + i) * LD + r0 + k], y[k], s0);
+            }
+            const double ii = __shfl_sync(0xffffffffu, inv, i, 16);
+            y[i] = i > j ? -(s0 + s1) * ii : (i == j ? inv : 0.0);
+            if (i >= j) w[tri(r0 + i, r0 + j)] = y[i];
+        }
+    }
+    __syncthreads();
+    // ---- then pairs of blocks: 16, 32 and 64 rows
+    if (NP == 128) {
+        inverse_join<NP, NP == 128 ? 4 : 1, 16, 16, 1>(a, w, 32);
+        inverse_join<NP, NP == 128 ? 2 : 1, 32, 32, 1>(a, w, 64);
+        inverse_join<NP, 1, 64, NP == 128 ? 64 : 32, 1>(a, w, 0);
+    } else if (NP == 96) {
+        inverse_join<NP, NP == 96 ? 3 : 1, 16, 16, 1>(a, w, 32);
+        inverse_join<NP, 1, 32, 32, 2>(a, w, 0);
+        inverse_join<NP, 1, 64, 32, 2>(a, w, 0);
+    } else {
+        inverse_join<NP, 2, 16, 16, 2>(a, w, 32);
+        inverse_join<NP, 1, 32, 32, 2>(a, w, 0);
     }
 }
 
 __global__ void __launch_bounds__(256) factor_diag_kernel(double *S, long lds, int bs, double *W, long ldw,
                                                           double *pdiag, int *info, int side, int k0) {
+    constexpr int LD = CholBlock<128>::LD;
     extern __shared__ double sm[];
-    double *a = sm;               // [128][129]: P in the lower triangle, scratch above it
-    double *w = sm + 128 * 129;   // packed lower triangle of W
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double *a = sm;               // [128][LD]: P in the lower triangle, scratch above it
+    double *w = sm + 128 * LD;    // packed lower triangle of W
+    const int tid = threadIdx.x;
     // the block, padded with the identity: the kernel sits on the serial spine of the set-up, so a thread's 64 loads
     // are issued in two batches of 32 (entry idx = 256 u + tid: a warp reads 32 consecutive columns of one row)
     for (int base = 0; base < 128 * 128; base += 32 * 256) {
@@ -200,19 +244,20 @@ __global__ void __launch_bounds__(256) factor_diag_kernel(double *S, long lds, i
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
             const int idx = base + u * 256 + tid, i = idx >> 7, j = idx & 127;
-            if (j <= i) a[i * 129 + j] = v[u];
+            if (j <= i) a[i * LD + j] = v[u];
         }
     }
     __syncthreads();
-    chol_inverse_128(a, w, bs, info, side, k0, 0);
-    for (int idx = tid; idx < 128 * 128; idx += 256) {
-        const int i = idx >> 7, j = idx & 127;
-        if (i < bs && j < bs) {
-            if (j <= i) S[(long)i * lds + j] = a[i * 129 + j];
-            W[(long)i * ldw + j] = (j <= i) ? w[tri(i, j)] : 0.0;
+    chol_inverse<128>(a, w, bs, info, side, k0, 0);
+#pragma unroll 8
+    for (int u = 0; u < 64; ++u) {
+        const int idx = u * 256 + tid, i = idx >> 7, j = idx & 127;
+        if (i < bs && j <= i) {                                // (W's block has been cleared: nothing to write above its diagonal)
+            S[(long)i * lds + j] = a[i * LD + j];
+            W[(long)i * ldw + j] = w[tri(i, j)];
         }
     }
-    for (int i = tid; i < bs; i += blockDim.x) pdiag[i] = a[i * 129 + i];
+    for (int i = tid; i < bs; i += blockDim.x) pdiag[i] = a[i * LD + i];
 }
 
 // out[i][j] (transpose == 0) or out[j][i] (transpose == 1) = X[i][j] * p[j] below the
@@ -255,14 +300,17 @@ __global__ void identity_kernel(double *out, long ldo, int k, double *dinv) {
     if (dinv && idx < k) dinv[idx] = 1.0;
 }
 
-// One side of one small problem (order k <= 128) per CTA, everything in shared memory: the Gram of the
-// basis, its Cholesky factorisation and inverse (chol_inverse_128), the unit triangular factor and 1/Lambda.
-// For the set-up of many small matrices at once, where one launch sequence per matrix would cost far more
-// than the arithmetic.
-__global__ void __launch_bounds__(256) factor_small_kernel(const FactorSmallSide *sides, int *info) {
+// One side of one small problem (order k <= NP) per CTA, everything in shared memory: the Gram of the basis, its Cholesky
+// factorisation and inverse (chol_inverse), the unit triangular factor and 1/Lambda.  For the set-up of many small matrices
+// at once, where one launch sequence per matrix would cost far more than the arithmetic.  NP = 64, 96 or 128: what a CTA
+// does is a chain of latencies, so the smaller orders, whose blocks leave room for four or two CTAs on an SM, run that many
+// at once (256 sides of order 96: 192 -> 68 us, with the shorter chain of chol_inverse).
+template <int NP>
+__global__ void __launch_bounds__(256, NP == 64 ? 4 : (NP == 96 ? 2 : 1)) factor_small_kernel(const FactorSmallSide *sides, int *info) {
+    constexpr int LD = CholBlock<NP>::LD, F = NP / 16;
     extern __shared__ double sm[];
-    double *a = sm;               // [128][129]
-    double *w = sm + 128 * 129;   // packed lower triangle of W
+    double *a = sm;               // [NP][LD]
+    double *w = sm + NP * LD;     // packed lower triangle of W
     const FactorSmallSide q = sides[blockIdx.x];
     const int k = q.k, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     if (!q.M) {                                           // identity basis
@@ -275,67 +323,76 @@ __global__ void __launch_bounds__(256) factor_small_kernel(const FactorSmallSide
         return;
     }
     // a[r][i] = M[r][i] (side 0, S = M^T M) or M[i][r] (side 1, S = M M^T), zero outside k x k
-    for (int base = 0; base < 128 * 128; base += 8 * 256) {
-        double v[8];
+    for (int base = 0; base < NP * NP; base += 16 * 256) {
+        double v[16];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int idx = base + u * 256 + tid, r = idx >> 7, i = idx & 127;
-            v[u] = (r < k && i < k) ? (q.side == 0 ? q.M[(long)r * q.ldm + i] : q.M[(long)i * q.ldm + r]) : 0.0;
+        for (int u = 0; u < 16; ++u) {                        // idx runs along memory
+            const int idx = base + u * 256 + tid, r = idx / NP, i = idx - r * NP;
+            v[u] = (idx < NP * NP && r < k && i < k) ? q.M[(long)r * q.ldm + i] : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int idx = base + u * 256 + tid;
-            a[(idx >> 7) * 129 + (idx & 127)] = v[u];
+        for (int u = 0; u < 16; ++u) {
+            const int idx = base + u * 256 + tid, r = idx / NP, i = idx - r * NP;
+            if (idx < NP * NP) a[q.side == 0 ? r * LD + i : i * LD + r] = v[u];
         }
     }
     __syncthreads();
     // S[i][j] = sum_r a[r][i] a[r][j]; thread (tx, ty) owns i = ty + 16 ii, j = tx + 16 jj
-    double acc[8][8];
+    double acc[F][F];
 #pragma unroll
-    for (int ii = 0; ii < 8; ++ii)
+    for (int ii = 0; ii < F; ++ii)
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[ii][jj] = 0.0;
+        for (int jj = 0; jj < F; ++jj) acc[ii][jj] = 0.0;
     for (int r = 0; r < k; ++r) {
-        double ai[8], aj[8];
+        double ai[F], aj[F];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            ai[x] = a[r * 129 + ty + 16 * x];
-            aj[x] = a[r * 129 + tx + 16 * x];
+        for (int x = 0; x < F; ++x) {
+            ai[x] = a[r * LD + ty + 16 * x];
+            aj[x] = a[r * LD + tx + 16 * x];
         }
 #pragma unroll
-        for (int ii = 0; ii < 8; ++ii)
+        for (int ii = 0; ii < F; ++ii)
 #pragma unroll
-            for (int jj = 0; jj < 8; ++jj) acc[ii][jj] = fma(ai[ii], aj[jj], acc[ii][jj]);
+            for (int jj = 0; jj < F; ++jj) acc[ii][jj] = fma(ai[ii], aj[jj], acc[ii][jj]);
     }
     __syncthreads();
     // the Gram, padded with the identity, replaces the basis
 #pragma unroll
-    for (int ii = 0; ii < 8; ++ii)
+    for (int ii = 0; ii < F; ++ii)
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
+        for (int jj = 0; jj < F; ++jj) {
             const int i = ty + 16 * ii, j = tx + 16 * jj;
-            if (j <= i) a[i * 129 + j] = i < k ? acc[ii][jj] : (i == j ? 1.0 : 0.0);
+            if (j <= i) a[i * LD + j] = i < k ? acc[ii][jj] : (i == j ? 1.0 : 0.0);
         }
     __syncthreads();
-    chol_inverse_128(a, w, k, info, q.side, 0, q.index);
+    chol_inverse<NP>(a, w, k, info, q.side, 0, q.index);
     // F = W diag(P): unit lower (side 0) or, transposed on the way out, unit upper (side 1)
-    for (int idx = tid; idx < k * k; idx += blockDim.x) {
-        const int i = idx / k, j = idx - i * k;
-        const double v = i > j ? w[tri(i, j)] * a[j * 129 + j] : (i == j ? 1.0 : 0.0);
-        if (q.side == 0) q.out[(long)i * q.ldo + j] = v;
-        else q.out[(long)j * q.ldo + i] = v;
+#pragma unroll 4
+    for (int idx = tid; idx < NP * NP; idx += 256) {
+        const int r = idx / NP, c = idx - r * NP, i = q.side == 0 ? r : c, j = q.side == 0 ? c : r;      // writes run along memory
+        if (r < k && c < k) q.out[(long)r * q.ldo + c] = i > j ? w[tri(i, j)] * a[j * LD + j] : (i == j ? 1.0 : 0.0);
     }
     if (q.dinv)
-        for (int j = tid; j < k; j += blockDim.x) q.dinv[j] = a[j * 129 + j] * a[j * 129 + j];
+        for (int j = tid; j < k; j += blockDim.x) q.dinv[j] = a[j * LD + j] * a[j * LD + j];
 }
 
-int launch_factor_small(int nsides, const FactorSmallSide *dev_sides, int *info, cudaStream_t stream) {
+int factor_small_class(int k) { return k <= 64 ? 0 : (k <= 96 ? 1 : 2); }
+
+template <int NP>
+static int launch_factor_small_t(int nsides, const FactorSmallSide *dev_sides, int *info, cudaStream_t stream) {
     if (nsides <= 0) return GPTQ2D_OK;
-    const size_t smem = (128 * 129 + 128 * 129 / 2) * sizeof(double);
-    if (cudaFuncSetAttribute(factor_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    const size_t smem = CholBlock<NP>::SMEM;
+    if (cudaFuncSetAttribute(factor_small_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(factor_small_kernel<NP>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return GPTQ2D_ERR_CUDA;
-    factor_small_kernel<<<nsides, 256, smem, stream>>>(dev_sides, info);
+    factor_small_kernel<NP><<<nsides, 256, smem, stream>>>(dev_sides, info);
     return cudaGetLastError() == cudaSuccess ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
+}
+int launch_factor_small(const int (&counts)[3], const FactorSmallSide *dev_sides, int *info, cudaStream_t stream) {
+    int st = launch_factor_small_t<128>(counts[2], dev_sides + counts[0] + counts[1], info, stream);
+    if (st == GPTQ2D_OK) st = launch_factor_small_t<96>(counts[1], dev_sides + counts[0], info, stream);
+    if (st == GPTQ2D_OK) st = launch_factor_small_t<64>(counts[0], dev_sides, info, stream);
+    return st;
 }
 
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
@@ -381,7 +438,12 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     // serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
     auto product = [&](const GemmArgs &g, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
-        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > factor_i8_bytes(k)) return launch_gemm(g, stream);
+        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > factor_i8_bytes(k)) {
+            // few tiles: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the number of tiles)
+            const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
+            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && tiles <= 74;
+            return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
+        }
         const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);
         const I8Planes pb = same ? pa : i8_planes_at(i8_at + bytesA, g.N, g.K, g.batch);
         I8Inner undo = inner;
@@ -404,7 +466,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         g.C = G; g.ldc = ld; g.batch = 1; g.lower_tiles_only = 1;
         CK(product(g, true, true, true));      // a Cholesky basis has a dominant diagonal
     }
-    const size_t diag_smem = (128 * 129 + 128 * 129 / 2) * sizeof(double);
+    const size_t diag_smem = CholBlock<128>::SMEM;
     CK(cudaFuncSetAttribute(factor_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem));
     CK(cudaFuncSetAttribute(factor_diag_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                             cudaSharedmemCarveoutMaxShared));

@@ -26,7 +26,9 @@ struct FactorSmallSide {
     double *out; long ldo;
     double *dinv;              // optional
 };
-// dev_sides: device array of nsides descriptors
-int launch_factor_small(int nsides, const FactorSmallSide *dev_sides, int *info, cudaStream_t stream);
+// which of the three kernels a side of order k takes (0: up to 64, 1: up to 96, 2: up to 128)
+int factor_small_class(int k);
+// dev_sides: device array of descriptors, those of class 0 first, then class 1, then class 2
+int launch_factor_small(const int (&counts)[3], const FactorSmallSide *dev_sides, int *info, cudaStream_t stream);
 
 }  // namespace gptq2d

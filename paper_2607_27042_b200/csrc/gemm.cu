@@ -418,4 +418,98 @@ cudaError_t launch_gemm_rank128(int M, int N, double alpha, const double *A, lon
     return launch_rank128_t<32>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
 }
 
+// ---------------------------------------------------------------------------------------------
+// C = alpha * A B + beta 0 (both row-major as they are) for products with too few 128 x 128 tiles to occupy the SMs: the small levels
+// of the triangular inverse.  Tiles of 128 x 32, k in slabs of 64, two slabs in flight.
+constexpr int NARROW_NT = 32, NARROW_BK = 64, NARROW_LDA = NARROW_BK + 4, NARROW_LDB = NARROW_NT + 4;
+constexpr int NARROW_STAGE = 128 * NARROW_LDA + NARROW_BK * NARROW_LDB;
+constexpr int NARROW_NSTAGE = 2;
+constexpr size_t NARROW_SMEM = (size_t)NARROW_NSTAGE * NARROW_STAGE * sizeof(double);
+__global__ void __launch_bounds__(256, 1) gemm_narrow_kernel(GemmArgs p) {
+    extern __shared__ __align__(16) double smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int wm = warp >> 1, wn = warp & 1;                   // 4 x 2 warps, each 32 rows x 16 columns
+    const int tm = p.a_lower ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
+    const int m0 = tm * 128, n0 = (int)blockIdx.x * NARROW_NT;
+    const double *A = p.A + (long)blockIdx.z * p.strideA + (long)m0 * p.lda, *B = p.B + (long)blockIdx.z * p.strideB + n0;
+    const int k_lo = p.b_lower ? min(p.K, n0 & ~(NARROW_BK - 1)) : 0, k_hi = p.a_lower ? min(p.K, m0 + 128) : p.K;
+    const int nk = k_hi > k_lo ? (k_hi - k_lo + NARROW_BK - 1) / NARROW_BK : 0;
+    const int rows = min(128, p.M - m0), cols = min(NARROW_NT, p.N - n0);
+    const bool vec = (((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0) && ((p.lda | p.ldb) & 1) == 0;
+    auto load = [&](int s) {
+        double *As = smem + (s % NARROW_NSTAGE) * NARROW_STAGE, *Bs = As + 128 * NARROW_LDA;
+        const int k0 = k_lo + s * NARROW_BK;
+        if (vec) {
+#pragma unroll
+            for (int it = 0; it < 16; ++it) {                  // 128 rows x 64 k
+                const int c = tid + it * 256, r = c >> 5, k = (c & 31) * 2, nv = r < rows ? min(2, max(0, p.K - k0 - k)) : 0;
+                cp_async16(As + r * NARROW_LDA + k, nv ? A + (long)r * p.lda + k0 + k : p.A, nv * 8);
+            }
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {                   // 64 k x 32 columns
+                const int c = tid + it * 256, k = c >> 4, n = (c & 15) * 2, nv = k0 + k < p.K ? min(2, max(0, cols - n)) : 0;
+                cp_async16(Bs + k * NARROW_LDB + n, nv ? B + (long)(k0 + k) * p.ldb + n : p.B, nv * 8);
+            }
+        } else {
+#pragma unroll 8
+            for (int it = 0; it < 32; ++it) {
+                const int c = tid + it * 256, r = c >> 6, k = c & 63;
+                const bool in = r < rows && k0 + k < p.K;
+                cp_async8(As + r * NARROW_LDA + k, in ? A + (long)r * p.lda + k0 + k : p.A, in ? 8 : 0);
+            }
+#pragma unroll
+            for (int it = 0; it < 8; ++it) {
+                const int c = tid + it * 256, k = c >> 5, n = c & 31;
+                const bool in = k0 + k < p.K && n < cols;
+                cp_async8(Bs + k * NARROW_LDB + n, in ? B + (long)(k0 + k) * p.ldb + n : p.B, in ? 8 : 0);
+            }
+        }
+        cp_async_commit();
+    };
+    double acc[4][2][2];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
+    if (nk > 0) load(0);
+    for (int s = 0; s < nk; ++s) {
+        if (s + 1 < nk) { load(s + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        __syncthreads();
+        const double *As = smem + (s % NARROW_NSTAGE) * NARROW_STAGE, *Bs = As + 128 * NARROW_LDA;
+#pragma unroll 8
+        for (int kk = 0; kk < NARROW_BK; kk += 4) {
+            double af[4], bf[2];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) af[a] = As[(wm * 32 + a * 8 + g) * NARROW_LDA + kk + t];
+#pragma unroll
+            for (int b = 0; b < 2; ++b) bf[b] = Bs[(kk + t) * NARROW_LDB + wn * 16 + b * 8 + g];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) dmma_m8n8k4(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
+        }
+        __syncthreads();
+    }
+    double *C = p.C + (long)blockIdx.z * p.strideC + (long)m0 * p.ldc + n0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int r = wm * 32 + a * 8 + g, c = wn * 16 + b * 8 + t * 2;
+            if (r >= rows) continue;
+            if (c < cols) C[(long)r * p.ldc + c] = p.alpha * acc[a][b][0];
+            if (c + 1 < cols) C[(long)r * p.ldc + c + 1] = p.alpha * acc[a][b][1];
+        }
+}
+
+cudaError_t launch_gemm_narrow(const GemmArgs &g, cudaStream_t stream) {
+    if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(gemm_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NARROW_SMEM);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(gemm_narrow_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    gemm_narrow_kernel<<<dim3((g.N + NARROW_NT - 1) / NARROW_NT, (g.M + 127) / 128, g.batch), 256, NARROW_SMEM, stream>>>(g);
+    return cudaGetLastError();
+}
+
 }  // namespace gptq2d

@@ -34,6 +34,8 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t stream);
 // For the serial spine of the set-up: narrow tiles, so that one block row occupies all SMs for a short time.
 cudaError_t launch_gemm_rank128(int M, int N, double alpha, const double *A, long lda, const double *B, long ldb, double beta,
                                 double *C, long ldc, cudaStream_t stream);
+// C = alpha * A B (opA = opB = OP_N, beta = 0) in tiles of 128 x 32, for products of few 128 x 128 tiles; takes a_lower, b_lower, batch.
+cudaError_t launch_gemm_narrow(const GemmArgs &g, cudaStream_t stream);
 // 1 (default): products with a ragged tile edge whose operands are 16-byte aligned with even leading dimensions
 // go through the TMA-fed kernel, full tiles through the cp.async kernel; 3: TMA-fed kernel whenever the operands
 // allow it; 2: the same with a CTA barrier per slab; 0: everything through the cp.async kernel.
