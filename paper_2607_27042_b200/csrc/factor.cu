@@ -84,18 +84,6 @@ __device__ __forceinline__ void inverse_join(double *a, double *w, int step) {
     __syncthreads();
 }
 
-// 1 / sqrt(d) to the last bit or two, d > 0 and finite: the hardware's approximation (relative error below 2^-20) and two
-// Newton steps r += r/2 (1 - d r r), which leave 2^-41 and then rounding.  In line and without the library function's range
-// handling it is 60 cycles shorter, 128 times on the serial chain of a block; the approximation flushes denormals, so the
-// smallest pivots take the function.
-__device__ __forceinline__ double pivot_rsqrt(double d) {
-    if (d < 0x1p-1000) return rsqrt(d);
-    double r;
-    asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
-    r = fma(0.5 * r, fma(-d * r, r, 1.0), r);
-    return fma(0.5 * r, fma(-d * r, r, 1.0), r);
-}
-
 // a holds the lower triangle of a Schur complement (bs rows are real); on return its lower triangle is P (S = P^T P, Cholesky from
 // the last index to the first) and w is the packed lower triangle of W = P^{-1}.  Ends with a barrier.
 // err_c: what a non-positive pivot reports in info[3], beside its index and the side.
@@ -127,7 +115,8 @@ __device__ __forceinline__ void chol_inverse(double *a, double *w, int bs, int *
 #pragma unroll
             for (int kk = 15; kk >= 0; --kk) {
                 if (!(d > 0.0) || !isfinite(d)) { bad = max(bad, kk); d = 1.0; }
-                const double rk = pivot_rsqrt(d);
+                double rk = rsqrt(d);
+                rk = rk * fma(-0.5 * d, rk * rk, 1.5);         // one Newton step: 1 / sqrt(d) to the last bit or two
                 const double pk = x[kk] * rk;                  // P[k][j], j < k
                 if (kk > 0) {
                     x[kk - 1] = fma(-__shfl_sync(0xffffffffu, pk, kk - 1), pk, x[kk - 1]);
