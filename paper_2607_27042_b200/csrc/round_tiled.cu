@@ -182,21 +182,6 @@ __device__ __forceinline__ void quad_mma(QAcc &acc, const double *As, const doub
             for (int b = 0; b < 4; ++b) dmma_m8n8k4(acc.v[a][b][0], acc.v[a][b][1], af[a], bf[b]);
     }
 }
-// D (64 x 64 with row stride ld, global or shared) += acc
-__device__ __forceinline__ void quad_add_to(double *D, long ld, const QAcc &acc, bool global_cg) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int wr = warp >> 1, wc = warp & 1;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            double2 *ptr = reinterpret_cast<double2 *>(D + (long)(wr * 16 + a * 8 + g) * ld + wc * 32 + b * 8 + t * 2);
-            double2 v = global_cg ? __ldcg(ptr) : *ptr;
-            v.x += acc.v[a][b][0];
-            v.y += acc.v[a][b][1];
-            *ptr = v;
-        }
-}
 // Leaf (a, b) of the quadrant collects, right before it is swept, all the feedback it is due from
 // the leaves already swept (left-looking): the downward pushes of the leaves above it through L,
 //     P = sum_{a' < a} L[a, a'] E[a', b]       (folded into C and pushed into Y)
@@ -498,6 +483,21 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
 // 64 x 64 diagonal blocks of both factors into one shared-memory matrix: below the diagonal
 // L[r0 + i][r0 + k], above it U[c0 + k][c0 + j], zeros on it and outside the matrices.
 __device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKernelParams &p, int r0, int c0) {
+    const bool vec = p.l_al16 && p.u_al16 && r0 + Q <= p.m && c0 + Q <= p.n;      // whole blocks in 16-byte pieces
+    if (vec) {
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+            const int c = threadIdx.x + it * TILED_THREADS;
+            const int i = c >> 5, j = (c & 31) * 2;
+            // the piece that holds the diagonal: its off-diagonal entry only (from L if i is odd, from U if it is even)
+            const bool lower = j < i, diag = (i & ~1) == j;
+            const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
+            if (!diag) cp_async16(dst + CI(i * QLD + j, QMAT - 1, 121), src, 16);
+            else cp_async8(dst + i * QLD + j + ((i & 1) ^ 1), (i & 1) ? src : src + 1, 8);
+        }
+        if (threadIdx.x < Q) dst[threadIdx.x * (QLD + 1)] = 0.0;
+        return;
+    }
 #pragma unroll
     for (int it = 0; it < 16; ++it) {
         const int c = threadIdx.x + it * TILED_THREADS;
@@ -630,24 +630,33 @@ __device__ __forceinline__ void sweep_quadrant(int I, int J, int q, double *smem
     load_quadrant_async(Cs, cQ, p.np);
     load_quadrant_async(Ys, eQ, p.np);
     cp_async_commit();
-    double xv[16];
+    // X of the quadrant, zero outside the matrix, in the layout of the accumulators (quad_mma)
+    const int xr = row0 + ((tid >> 6) * 16 + ((tid & 31) >> 2)), xc = col0 + ((tid >> 5) & 1) * 32 + (tid & 3) * 2;
+    double xv[2][4][2];
 #pragma unroll
-    for (int it = 0; it < 16; ++it) {                     // X of the quadrant, zero outside the matrix
-        int c = tid + it * TILED_THREADS;
-        int gr = row0 + (c >> 6), gc = col0 + (c & 63);
-        xv[it] = (gr < p.m && gc < p.n) ? __ldg(p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122)) : 0.0;
-    }
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int gr = xr + a * 8, gc = xc + b * 8 + h;
+                xv[a][b][h] = (gr < p.m && gc < p.n) ? __ldg(p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122)) : 0.0;
+            }
     cp_async_wait<0>();
     __syncthreads();
-    quad_add_to(Cs, QLD, accC, false);                    // Cd = far part + pulls from complete quadrants
-    quad_add_to(Ys, QLD, accR, false);                    // Rt likewise
-    __syncthreads();
+    // Cd = far part + pulls from complete quadrants; Rt likewise; Y = X + Rt + Cd
 #pragma unroll
-    for (int it = 0; it < 16; ++it) {                     // Y = X + Rt + Cd
-        int c = tid + it * TILED_THREADS;
-        int r = c >> 6, cc = c & 63;
-        Ys[CI(r * QLD + cc, QMAT, 123)] += xv[it] + Cs[r * QLD + cc];
-    }
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int at = CI((xr - row0 + a * 8) * QLD + xc - col0 + b * 8, QMAT - 1, 123);
+            double2 *cq = reinterpret_cast<double2 *>(Cs + at), *yq = reinterpret_cast<double2 *>(Ys + at);
+            double2 cv = *cq, yv = *yq;
+            cv.x += accC.v[a][b][0]; cv.y += accC.v[a][b][1];
+            yv.x += accR.v[a][b][0]; yv.y += accR.v[a][b][1];
+            yv.x += xv[a][b][0] + cv.x; yv.y += xv[a][b][1] + cv.y;
+            *cq = cv; *yq = yv;
+        }
     TS_MARK(1);                                          // operand loads, Y = X + Rt + Cd
     quadrant_sweep(Ys, Cs, LU, Lfa, Ufl, stg, tabL, tabU, row0, col0, sm, p, max_abs_e);
     __syncthreads();
