@@ -103,6 +103,8 @@ int gptq2d_factor(int m, int n,
  *   is implied).  They must stay fixed during the call (Section 6, first caveat).
  * Initialisation (Y <- X, C <- 0; Algorithm 3 lines 4-5) is part of this call.
  * Device errors: NONFINITE, INT_OVERFLOW (Z is int32), DEVICE_TIMEOUT.
+ * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 5632 run as four blocks in three kernels, with the
+ * products between the blocks on the int8 tensor cores (error-free splitting, at least as exact), all on `stream`.
  * Calls on different streams must use different workspaces.
  */
 size_t gptq2d_round_workspace_bytes(int m, int n, int precision);
@@ -317,6 +319,7 @@ int gptq2d_objective(int m, int n,
  *          site 999) is checked; [0..3] receive {GPTQ2D_ERR_CHECK, 999, 7, 3}, [4] the redirected index 0.
  *   key 6: how the fp32 mode's contraction gets its operand slabs.  0 (default): bulk tensor copies (TMA) where
  *          the driver offers tensor maps, cp.async otherwise; 1: cp.async always.  Comparison runs and tests.
+ *   key 7: smaller order from which on resident fp64 sweeps run in 2 x 2 blocks (0: the default).  Workspace queries follow it.
  * Returns GPTQ2D_OK, or GPTQ2D_ERR_INVALID_ARG for an unknown key.
  */
 int gptq2d_internal_test_hook(int key, long value);

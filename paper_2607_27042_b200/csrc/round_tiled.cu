@@ -41,6 +41,10 @@
 #include "common.cuh"
 #include "dmma_gemm.cuh"
 #include "round_internal.cuh"
+#include "i8_gemm.cuh"
+#include "tma_host.cuh"
+#include <algorithm>
+#include <atomic>
 #include <vector>
 
 namespace gptq2d {
@@ -96,6 +100,10 @@ struct TiledKernelParams {
     double *max_abs_e;
     int *info;
     int l_al16, u_al16;
+    // a block of a larger matrix (launch_round_split): where it begins there (status words), and which far sums its regions of
+    // Cbuf (bit 0) and Ebuf (bit 1) hold already when the launch begins: those of the blocks above and to the left
+    int row_off, col_off, preloaded;
+    int report_index;            // matrix index in the status words
     // batched launches only (one descriptor per matrix in device memory; the kernel argument then
     // carries the shared scheduler words, the totals in ntasks / ntiles_total, and these tables)
     int batch_index;             // -1: single-matrix launch
@@ -476,7 +484,7 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
     if (tid == 0 && s_badkey != ~0ull) {
         const unsigned long long k = s_badkey;
         report(p.info, ((k >> 41) & 1ull) ? GPTQ2D_ERR_INT_OVERFLOW : GPTQ2D_ERR_NONFINITE,
-               (int)((k >> 20) & 0x1fffffull), (int)(k & 0xfffffull), max(p.batch_index, 0));
+               (int)((k >> 20) & 0x1fffffull) + p.row_off, (int)(k & 0xfffffull) + p.col_off, p.report_index);
     }
 }
 
@@ -995,7 +1003,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
         if (k != cur) {
             if (cur >= 0 && s_ctx[cur][3] > 0) store_acc(acc, tile_region(cur), VIEW(s_ctx[cur][6]).np, wm, wn, g, t);
-            if (s_ctx[k][3] > 0) load_acc(acc, tile_region(k), pk.np, wm, wn, g, t);
+            if (s_ctx[k][3] > 0 || ((pk.preloaded >> s_ctx[k][0]) & 1)) load_acc(acc, tile_region(k), pk.np, wm, wn, g, t);
             else acc.zero();
             cur = k;
         }
@@ -1098,7 +1106,39 @@ static TiledLayout tiled_layout(int m, int n) {
     return l;
 }
 
-size_t round_tiled_workspace_bytes(int m, int n) { return tiled_layout(m, n).total; }
+// ---- large matrices in 2 x 2 blocks (launch_round_split below): its own bookkeeping, behind the E and C buffers.  One header and ring
+// for each of the three launches and flags for each of the four blocks (cleared per call), then two descriptors and a table
+// of far parts for the launch that sweeps two blocks at once (written per call, on the device).
+constexpr int SPLIT_MIN = 5632;          // smaller of the two orders from which on (5120 x 5120: 11.1 ms whole, 11.6 in blocks; 6144 x 6144: 17.5 and 16.3)
+static std::atomic<long> g_split_min{SPLIT_MIN};
+void round_split_set_min(long order) { g_split_min.store(order > 0 ? order : SPLIT_MIN); }
+struct SplitLayout {
+    int m0, n0;                          // rows / columns of the first block (multiples of T); 0: not split
+    size_t hdr_off[3], flags_off[4], desc_off, table_off, zero_off, total;
+};
+static size_t split_flag_bytes(int m, int n) {
+    const size_t tm = (m + T - 1) / T, tiles = tm * ((n + T - 1) / T);
+    return 2 * pad256(tiles * sizeof(unsigned)) + 2 * pad256(4 * tiles * sizeof(unsigned)) + pad256(tm * sizeof(unsigned));
+}
+static SplitLayout split_layout(int m, int n) {
+    SplitLayout l{};
+    const TiledLayout t = tiled_layout(m, n);
+    l.total = t.total;
+    if (std::min(m, n) < g_split_min.load() || t.ntm < 2 || t.ntn < 2) return l;
+    l.m0 = (t.ntm + 1) / 2 * T; l.n0 = (t.ntn + 1) / 2 * T;
+    size_t off = l.zero_off = pad256(t.total);
+    for (int k = 0; k < 3; ++k) { l.hdr_off[k] = off; off += 256 + 4096 * sizeof(unsigned); }
+    const int ms[2] = {l.m0, m - l.m0}, ns[2] = {l.n0, n - l.n0};
+    for (int k = 0; k < 4; ++k) { l.flags_off[k] = off; off += split_flag_bytes(ms[k >> 1], ns[k & 1]); }
+    l.desc_off = off; off += pad256(2 * sizeof(TiledKernelParams));
+    l.table_off = off;
+    const size_t tm0 = l.m0 / T, tn0 = l.n0 / T;
+    off += pad256(2 * (tm0 * (t.ntn - tn0) + (t.ntm - tm0) * tn0) * sizeof(unsigned));
+    l.total = off;
+    return l;
+}
+
+size_t round_tiled_workspace_bytes(int m, int n) { return split_layout(m, n).total; }
 
 // the same layout for the sixteen-warp kernel (round_fused.cu), which shares the workspace format
 struct TiledLayoutView {
@@ -1115,12 +1155,18 @@ unsigned *round_tiled_rowdone(void *ws, int m, int n) {
     return reinterpret_cast<unsigned *>(static_cast<char *>(ws) + tiled_layout(m, n).rowdone_off);
 }
 
+static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, cudaStream_t stream);
+
 int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStream_t stream) {
     TiledLayout l = tiled_layout(in.m, in.n);
-    if (ws_bytes < l.total) return GPTQ2D_ERR_WORKSPACE;
+    if (ws_bytes < round_tiled_workspace_bytes(in.m, in.n)) return GPTQ2D_ERR_WORKSPACE;
     {
         // large resident problems: far contractions and quadrant tasks side by side on every SM
         const int st = launch_round_fused(in, ws, ws_bytes, stream, false);
+        if (st != -1) return st;
+    }
+    {
+        const int st = launch_round_split(in, ws, ws_bytes, stream);
         if (st != -1) return st;
     }
     char *w = static_cast<char *>(ws);
@@ -1258,6 +1304,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         d.l_al16 = ((reinterpret_cast<uintptr_t>(in.L) & 15) == 0) && ((in.ldl & 1) == 0);
         d.u_al16 = ((reinterpret_cast<uintptr_t>(in.U) & 15) == 0) && ((in.ldu & 1) == 0);
         d.batch_index = b;
+        d.report_index = b;
         d.spin_limit = d.panel_spin_limit = SPIN_LIMIT;
         d.ntiles_total = (int)tiles;
         desc[b] = d;
@@ -1308,6 +1355,176 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     if (min_margin) {
         batched_margin_kernel<<<(count + 255) / 256, 256, 0, stream>>>(
             reinterpret_cast<const double *>(w + l.maxe_off), min_margin, count);
+        if (cudaGetLastError() != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    }
+    return GPTQ2D_OK;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Large matrices in 2 x 2 blocks.  With the matrix cut behind row m0 and column n0 (tile boundaries), the restatement on tiles at
+// the head of this file holds for the four blocks, too: block (0, 0) is a sweep of its own; (0, 1) starts from Rt = C00 U01 and
+// (1, 0) from Cd = L10 E00; (1, 1) from Cd = L10 E01 and Rt = C10 U01.  Half of all flops are in these four products,
+// and they are plain matrix products of finished operands, so they run on the int8 tensor cores (i8_gemm.cu) at 80 TFLOP/s
+// where the far parts of the sweep run at 35.  Three sweeps (the middle one takes two blocks in one launch) replace one; each has
+// its own ramp, which is why small matrices are not cut.
+// 8192 x 8192: 38.0 -> 31.7 ms, 7168 x 7168 26.4 -> 23.4, 6144 x 6144 17.5 -> 16.3, 4096 x 4096 6.6 -> 8.0 (not cut).
+// Nothing but the workspace is used: a product's digit planes lie in rows of Ebuf whose blocks have not been swept yet, or in
+// rows of Cbuf that nobody reads any more; where they do not fit at once k is cut.
+
+// descriptors and claim order of a launch that sweeps two matrices (what the host builds for batched launches)
+__global__ void __launch_bounds__(256) split_pair_kernel(TiledKernelParams a, TiledKernelParams b, TiledKernelParams *desc, unsigned *table) {
+    if (threadIdx.x == 0) { desc[0] = a; desc[1] = b; }
+    auto count = [](int ntm, int ntn, int w) { return w < ntm + ntn - 1 ? min(ntm - 1, w) - max(0, w - ntn + 1) + 1 : 0; };
+    const int waves = max(a.ntm + a.ntn, b.ntm + b.ntn) - 1;
+    for (int w = threadIdx.x; w < waves; w += blockDim.x) {
+        int at = 0;
+        for (int v = 0; v < w; ++v) at += 2 * (count(a.ntm, a.ntn, v) + count(b.ntm, b.ntn, v));
+        for (int m = 0; m < 2; ++m) {
+            const int ntm = m ? b.ntm : a.ntm, ntn = m ? b.ntn : a.ntn, lo = max(0, w - ntn + 1), hi = min(ntm - 1, w);
+            for (int k = 0; k < count(ntm, ntn, w); ++k)
+                for (int type = 0; type < 2; ++type) {
+                    const int I = type == 0 ? hi - k : lo + k;
+                    table[at++] = ((unsigned)m << 17) | ((unsigned)type << 16) | ((unsigned)I << 8) | (unsigned)(w - I);
+                }
+        }
+    }
+}
+
+// The status words of the three launches -> the call's: data errors (a non-finite or too large value) in the order of the sweep,
+// that is by anti-diagonal over the whole matrix; anything else in the order of the launches.
+__global__ void split_status_kernel(const int *a, const int *b, const int *c, int *info) {
+    if (info[0] != 0) return;                                  // a product gave up
+    const int *s[3] = {a, b, c}, *best = nullptr;
+    for (int k = 0; k < 3 && !best; ++k)
+        if (s[k][0] != 0 && s[k][0] != GPTQ2D_ERR_NONFINITE && s[k][0] != GPTQ2D_ERR_INT_OVERFLOW) best = s[k];
+    if (!best)
+        for (int k = 0; k < 3; ++k)
+            if (s[k][0] != 0 && (!best || s[k][1] + s[k][2] < best[1] + best[2])) best = s[k];
+    if (best)
+        for (int k = 0; k < 4; ++k) info[k] = best[k];
+}
+
+// C (M x N, padded to whole tiles, row pitch ldc) = A B on the int8 tensor cores; A: M x K row-major, B: K x N row-major.  The digit planes
+// of kparts pieces of k in turn lie at `at`.
+static int split_product(int M, int N, int K, int kparts, const double *A, long lda, const double *B, long ldb, double *C, long ldc, void *at,
+                         int *info, cudaStream_t stream) {
+    const int step = ((K + kparts - 1) / kparts + T - 1) / T * T;
+    for (int k0 = 0; k0 < K; k0 += step) {
+        const int kk = std::min(step, K - k0);
+        const I8Planes pa = i8_planes_at(at, M, kk, 1), pb = i8_planes_at(static_cast<char *>(at) + i8_planes_bytes(M, kk, 1), N, kk, 1);
+        GemmArgs g{};
+        g.opA = OP_N; g.opB = OP_N;
+        g.M = (M + T - 1) / T * T; g.N = (N + T - 1) / T * T; g.K = kk;       // padding included: the planes hold zeros there
+        g.alpha = 1.0; g.beta = k0 ? 1.0 : 0.0;
+        g.A = A + k0; g.lda = lda; g.B = B + (long)k0 * ldb; g.ldb = ldb; g.C = C; g.ldc = ldc; g.batch = 1;
+        cudaError_t e = i8_split(pa, g.A, lda, 0, true, stream);
+        if (e == cudaSuccess) e = i8_split(pb, g.B, ldb, 0, false, stream);
+        if (e == cudaSuccess && !launch_gemm_i8(g, pa, pb, info, stream, &e)) return GPTQ2D_ERR_CUDA;
+        if (e != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    }
+    return GPTQ2D_OK;
+}
+// pieces of k for which the planes of an M x K and a K x N operand fit in `room` bytes; 0: none of up to eight
+static int split_kparts(int M, int N, int K, size_t room) {
+    for (int p = 1; p <= 8; ++p) {
+        const int step = ((K + p - 1) / p + T - 1) / T * T;
+        if (step <= I8_MAX_K && i8_planes_bytes(M, step, 1) + i8_planes_bytes(N, step, 1) <= room) return p;
+    }
+    return 0;
+}
+
+// -1: this matrix is not swept in blocks
+static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, cudaStream_t stream) {
+    const SplitLayout sl = split_layout(in.m, in.n);
+    if (sl.m0 == 0 || in.panels_ready || ws_bytes < sl.total || !tensor_map_encoder()) return -1;
+    const TiledLayout l = tiled_layout(in.m, in.n);
+    char *w = static_cast<char *>(ws);
+    const long np = (long)l.ntn * T;
+    double *E = reinterpret_cast<double *>(w + l.e_off), *C = reinterpret_cast<double *>(w + l.c_off);
+    const int m0 = sl.m0, n0 = sl.n0, m1 = in.m - m0, n1 = in.n - n0;
+    // room for digit planes: first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
+    const size_t room0 = (size_t)(l.ntm * T - m0) * np * sizeof(double), room1 = (size_t)m0 * np * sizeof(double);
+    const int k10 = split_kparts(m1, n0, m0, room0), k01 = split_kparts(m0, n1, n0, room0);
+    const int k11 = split_kparts(m1, n1, m0, room1), k11r = split_kparts(m1, n1, n0, room1);
+    if (!k10 || !k01 || !k11 || !k11r) return -1;
+
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    if (cudaMemsetAsync(w, 0, 256, stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;                     // max |E|
+    if (cudaMemsetAsync(w + sl.zero_off, 0, sl.desc_off - sl.zero_off, stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+    auto block = [&](int bi, int bj, int launch, int preloaded) {
+        const long r = bi ? m0 : 0, c = bj ? n0 : 0;
+        TiledKernelParams d{};
+        d.m = bi ? m1 : m0; d.n = bj ? n1 : n0;
+        d.ntm = (d.m + T - 1) / T; d.ntn = (d.n + T - 1) / T;
+        const size_t tiles = (size_t)d.ntm * d.ntn;
+        d.ntasks = (int)(2 * tiles); d.ntiles_total = (int)tiles;
+        d.np = np;
+        d.X = in.X + r * in.ldx + c; d.ldx = in.ldx;
+        d.L = in.L + r * in.ldl + r; d.ldl = in.ldl;
+        d.U = in.U + c * in.ldu + c; d.ldu = in.ldu;
+        d.Z = in.Z + r * in.ldz + c; d.ldz = in.ldz;
+        d.Euser = in.E ? in.E + r * in.lde + c : nullptr; d.lde = in.lde;
+        d.Ebuf = E + r * np + c; d.Cbuf = C + r * np + c;
+        unsigned *hdr = reinterpret_cast<unsigned *>(w + sl.hdr_off[launch]);
+        d.counter = hdr; d.abort = hdr + 1; d.q_head = hdr + 2; d.q_tail = hdr + 3; d.tiles_done = hdr + 4;
+        d.q_slots = hdr + 64; d.qmask = QCAP - 1;
+        char *f = w + sl.flags_off[bi * 2 + bj];
+        d.flagS = reinterpret_cast<unsigned *>(f); f += pad256(tiles * sizeof(unsigned));
+        d.quad_done = reinterpret_cast<unsigned *>(f); f += pad256(tiles * sizeof(unsigned));
+        d.qdep = reinterpret_cast<unsigned *>(f); f += pad256(4 * tiles * sizeof(unsigned));
+        d.qprog = reinterpret_cast<unsigned *>(f); f += pad256(4 * tiles * sizeof(unsigned));
+        d.rowdone = reinterpret_cast<unsigned *>(f);
+        d.max_abs_e = workspace_max_abs_e(ws);
+        d.info = reinterpret_cast<int *>(hdr + 8);
+        d.l_al16 = ((reinterpret_cast<uintptr_t>(d.L) & 15) == 0) && ((in.ldl & 1) == 0);
+        d.u_al16 = ((reinterpret_cast<uintptr_t>(d.U) & 15) == 0) && ((in.ldu & 1) == 0);
+        d.row_off = (int)r; d.col_off = (int)c; d.preloaded = preloaded;
+        d.batch_index = -1;
+        d.spin_limit = d.panel_spin_limit = SPIN_LIMIT;
+        return d;
+    };
+    auto sweep_one = [&](TiledKernelParams p) -> int {
+        const void *kernel = (const void *)round_tiled_kernel<false, false>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+        void *args[] = {&p};
+        return cudaLaunchCooperativeKernel(kernel, dim3(std::min(sms, p.ntasks)), dim3(TILED_THREADS), args, TILED_SMEM, stream) == cudaSuccess
+                   ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
+    };
+    int st = sweep_one(block(0, 0, 0, 0));
+    void *at = E + (long)m0 * np;
+    if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, k10, in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, k01, C, np, in.U + n0, in.ldu, E + n0, np, at, in.info, stream);
+    if (st != GPTQ2D_OK) return st;
+    {
+        TiledKernelParams a = block(0, 1, 1, 2), b = block(1, 0, 1, 1), p{};
+        a.batch_index = 0; b.batch_index = 1;
+        TiledKernelParams *desc = reinterpret_cast<TiledKernelParams *>(w + sl.desc_off);
+        unsigned *table = reinterpret_cast<unsigned *>(w + sl.table_off);
+        split_pair_kernel<<<1, 256, 0, stream>>>(a, b, desc, table);
+        if (cudaGetLastError() != cudaSuccess) return GPTQ2D_ERR_CUDA;
+        p.ntasks = a.ntasks + b.ntasks; p.ntiles_total = a.ntiles_total + b.ntiles_total;
+        p.batch_index = -1;
+        p.counter = a.counter; p.abort = a.abort; p.q_head = a.q_head; p.q_tail = a.q_tail; p.tiles_done = a.tiles_done;
+        p.q_slots = a.q_slots; p.qmask = a.qmask;
+        p.info = a.info;
+        p.probs = desc; p.far_tasks = table;
+        p.spin_limit = p.panel_spin_limit = SPIN_LIMIT;
+        const void *kernel = (const void *)round_tiled_kernel<true, false>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess) return GPTQ2D_ERR_CUDA;
+        void *args[] = {&p};
+        if (cudaLaunchCooperativeKernel(kernel, dim3(std::min(sms, p.ntasks)), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
+            return GPTQ2D_ERR_CUDA;
+    }
+    at = C;
+    st = split_product(m1, n1, m0, k11, in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, k11r, C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, in.info, stream);
+    if (st == GPTQ2D_OK) st = sweep_one(block(1, 1, 2, 3));
+    if (st != GPTQ2D_OK) return st;
+    if (in.info) {
+        auto words = [&](int k) { return reinterpret_cast<const int *>(w + sl.hdr_off[k]) + 8; };
+        split_status_kernel<<<1, 1, 0, stream>>>(words(0), words(1), words(2), in.info);
         if (cudaGetLastError() != cudaSuccess) return GPTQ2D_ERR_CUDA;
     }
     return GPTQ2D_OK;

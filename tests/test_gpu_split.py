@@ -1,0 +1,60 @@
+"""Resident sweeps in 2 x 2 blocks (the route of large matrices) at small sizes: blocks of one tile and of several, ragged last tiles, odd
+leading dimensions, products whose digit planes fit only piece by piece."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from oracle import cref
+from certify import certified_case
+from paper_2607_27042_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture()
+def g():
+    from paper_2607_27042_b200 import gptq2d
+    gptq2d.gptq2d_internal_test_hook(7, 129)
+    yield gptq2d
+    gptq2d.gptq2d_internal_test_hook(7, 0)
+
+
+def padded(a, extra):
+    r, c = a.shape
+    buf = torch.full((r, c + extra), float("nan"), dtype=torch.float64, device="cuda")
+    buf[:, :c] = torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    return buf[:, :c]
+
+
+@pytest.mark.parametrize("m,n,extra", [(129, 130, 0), (256, 256, 0), (300, 330, 1), (200, 1000, 2), (1000, 140, 3), (770, 645, 0)])
+def test_blocks_equal_the_oracle_and_the_single_sweep(g, m, n, extra):
+    def draw(seed):
+        X, A, B = W.gaussian_like(m, n, seed)
+        L, U, _, _ = O.feedback_factors(A, B)
+        return X, L, U
+    (X, L, U), ref, _ = certified_case(draw, cref.nested, m + n)
+    dX, dL, dU = padded(X, extra), padded(L, extra), padded(U, extra)
+    ws = torch.full((g.gptq2d_round_workspace_bytes(m, n),), 0xff, dtype=torch.uint8, device="cuda")
+    Z, E, mm, info = g.gptq2d_round(dX, dL, dU, workspace=ws, want_E=True, want_margin=True)
+    g.check_info(info)
+    assert np.array_equal(Z.cpu().numpy().astype(np.int64), ref["Z"])
+    g.gptq2d_internal_test_hook(7, 0)
+    Z1, E1, mm1, info = g.gptq2d_round(dX, dL, dU, want_E=True, want_margin=True)
+    g.check_info(info)
+    assert torch.equal(Z, Z1)
+    # both sum the same terms in fp64: the bar of all error comparisons in these tests
+    assert float((E - E1).abs().max()) < 1e-9 and abs(float(mm[0]) - float(mm1[0])) < 1e-9
+
+
+@pytest.mark.parametrize("where", [[(7, 20)], [(400, 30)], [(20, 500)], [(380, 470)], [(250, 250), (2, 400)]])
+def test_status_words_name_the_first_anti_diagonal(g, where):
+    X, A, B = W.gaussian_like(410, 520, 3)
+    L, U, _, _ = O.feedback_factors(A, B)
+    for i, j in where:
+        X[i, j] = np.nan
+    Z, E, mm, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0))
+    vals = info.cpu().tolist()
+    i, j = min(where, key=lambda p: p[0] + p[1])
+    # inside an 8 x 8 leaf a NaN reaches entries that exact arithmetic would spare: the anti-diagonal is known to a leaf's 15
+    assert vals[0] == 6 and abs(vals[1] + vals[2] - i - j) < 15 and vals[3] == 0
