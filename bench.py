@@ -34,6 +34,7 @@ GRADED_SEED = {0: 0, 1: 0, 2: 0, 3: 0, 4: 1000}
 
 METRIC = "rounded entries/s (m*n / sweep time)"
 UNIT = "entries/s"
+SPLIT_MIN = 5632            # smaller order from which on a resident fp64 sweep runs in 2 x 2 blocks
 FP64_NOMINAL_TFLOPS = 37.2     # 148 SMs x 64 fp64 FMA/clk x 2 x 1.965 GHz; the run also measures the library's own 8192^3 product
 BF16_NOMINAL_TFLOPS = 2250.0
 FP32_NOMINAL_TFLOPS = 74.4     # 148 SMs x 128 fp32 FMA/clk x 2 x 1.965 GHz
@@ -254,6 +255,10 @@ def run_cuda(args):
     scaled_bf16 = peaks["bf16_tflops"] * FP64_NOMINAL_TFLOPS / BF16_NOMINAL_TFLOPS if peaks["bf16_tflops"] else None
     kernel_name = ("round_tiled_f32_kernel" if args.fp32 else "round_pull_kernel" if args.pull else
                    "round_fused_kernel" if args.fused else "round_tiled_kernel")
+    launches = 1
+    if kernel_name == "round_tiled_kernel" and min(m, n) >= SPLIT_MIN:
+        # four blocks: three sweeps, descriptors, status; four products of two operands each (two splitting kernels an operand)
+        kernel_name, launches = "round_tiled_kernel in 2x2 blocks + i8_gemm_kernel", 3 + 2 + 4 * (2 * 2 + 1)
     traffic = None
     tp = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(tp):
@@ -300,7 +305,7 @@ def run_cuda(args):
         "config": {"workload": name, "m": m, "n": n, "seed": args.seed, "replicas": world,
                    "l2": "inputs (X, L, U: %.0f MB) exceed the 126 MB L2" % (8e-6 * (m * n + m * m + n * n)),
                    "timed": "gptq2d_round (init + sweep); factorisation timed separately"},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps,
+        "clocks": clocks, "e2e": e2e, "gpu_launches": launches * args.steps,
         "roofline": roofline, "factor_ms": factor_ms,
         # set-up flops per side of order k: Gram (lower tiles) k^3, reverse Cholesky k^3 / 3, triangular inverse k^3 / 3
         "factor_tflops": ((m ** 3 + n ** 3) * (1.0 + 1.0 / 3 + 1.0 / 3)) / (factor_ms * 1e-3) / 1e12,
