@@ -1125,7 +1125,11 @@ static SplitLayout split_layout(int m, int n) {
     const TiledLayout t = tiled_layout(m, n);
     l.total = t.total;
     if (std::min(m, n) < g_split_min.load() || t.ntm < 2 || t.ntn < 2) return l;
-    l.m0 = (t.ntm + 1) / 2 * T; l.n0 = (t.ntn + 1) / 2 * T;
+    // The middle launch goes through the batched kernel, whose claim table and ready ring hold tile indices in 8 bits, so the
+    // first block (the largest) must stay within its limit.  Longer matrices are swept whole, with 14 and 15 bits.
+    const int m0 = (t.ntm + 1) / 2 * T, n0 = (t.ntn + 1) / 2 * T;
+    if (std::max(m0, n0) > BATCH_MAX_DIM) return l;
+    l.m0 = m0; l.n0 = n0;
     size_t off = l.zero_off = pad256(t.total);
     for (int k = 0; k < 3; ++k) { l.hdr_off[k] = off; off += 256 + 4096 * sizeof(unsigned); }
     const int ms[2] = {l.m0, m - l.m0}, ns[2] = {l.n0, n - l.n0};

@@ -113,3 +113,23 @@ def test_batched_setup_argument_checks_need_no_gpu():
     bad[0].ldl = 10                                             # leading dimension below m
     assert lib.gptq2d_factor_batched(1, c.cast(bad, c.c_void_p), None, 0, None, None) == 1
     assert lib.gptq2d_factor_batched(3, c.cast(small, c.c_void_p), None, 0, None, None) == 2      # WORKSPACE
+
+
+def test_long_matrices_are_not_swept_in_blocks():
+    """A block's tile indices have 8 bits (32 768 rows or columns); a matrix with a longer block is swept whole.  The workspace
+    query shows which: the bookkeeping of a sweep in blocks comes on top of that of the whole sweep."""
+    from paper_2607_27042_b200 import gptq2d as g
+
+    def in_blocks(m, n):
+        got = g.gptq2d_round_workspace_bytes(m, n)
+        g.gptq2d_internal_test_hook(7, 1 << 30)
+        try:
+            return got > g.gptq2d_round_workspace_bytes(m, n)
+        finally:
+            g.gptq2d_internal_test_hook(7, 0)
+
+    assert in_blocks(5632, 5632) and not in_blocks(5631, 70000)
+    for m, n in ((5632, 65536), (65536, 5632), (65409, 65409)):
+        assert in_blocks(m, n), (m, n)
+    for m, n in ((5632, 65537), (65537, 5632), (5632, 65664), (65664, 65664), (6000, 130000)):
+        assert not in_blocks(m, n), (m, n)
