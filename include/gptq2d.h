@@ -46,7 +46,8 @@ typedef enum {
                                           entry on the first anti-diagonal where one was met (inside an 8 x 8
                                           block of the sweep a NaN also reaches neighbours that exact arithmetic
                                           would spare, so this may be a neighbour of the offending input)    */
-    GPTQ2D_ERR_INT_OVERFLOW = 7,       /* device: |corrected value| >= 2^31; info[1] = row, info[2] = col  */
+    GPTQ2D_ERR_INT_OVERFLOW = 7,       /* device: |corrected value| >= 2^31, or it rounds to 2^31; info[1] = row,
+                                          info[2] = col (Z is saturated there) */
     GPTQ2D_ERR_DEVICE_TIMEOUT = 8,     /* device: a bounded wait gave up; info[1] = where it waited     */
     GPTQ2D_ERR_TOO_LARGE = 9,          /* gptq2d_round_static: m or n beyond GPTQ2D_STATIC_MAX_DIM;
                                           gptq2d_round_batched: beyond its count / dimension limits     */

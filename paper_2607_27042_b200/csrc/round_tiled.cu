@@ -411,7 +411,7 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
             int z0 = 0, z1 = 0;
             const int t0 = i0 + j, t1 = t0 + 4;
             // round half to even: adding and subtracting 1.5 * 2^52 leaves the integer, whose low word is the sum's; values that
-            // do not fit 32 bits are looked for after the leaf, by the high word that each had at its own step (a NaN reaches
+            // do not fit 32 bits are looked for after the leaf, by the words that each had at its own step (a NaN reaches
             // entries rounded before it through the zero coefficients)
             constexpr double MAGIC = 6755399441055744.0;
             int h0 = 0, h1 = 0;
@@ -435,11 +435,14 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
                 c1 = fma(l1, ed, c1); w1 = fma(cr1, u1, w1);
             }
             c0 = g0; c1 = g1;
-            {   // values that do not fit 32 bits (high word at or above that of 2^31; infinities and NaNs are): remember the first
-                if (max(h0 & 0x7fffffff, h1 & 0x7fffffff) >= 0x41e00000) {
+            {   // values that do not fit 32 bits: remember the first.  Either the high word is at or above that of 2^31 (infinities and NaNs
+                // are), or the value is within half of 2^31 and rounds to it: the low word of the sum is then that of -2^31
+                constexpr int TOP = (int)0x80000000;
+                if (max(h0 & 0x7fffffff, h1 & 0x7fffffff) >= 0x41e00000 || (z0 == TOP && h0 >= 0) || (z1 == TOP && h1 >= 0)) {
                     auto look = [&](int h, int row, int &z) {
-                        if ((h & 0x7fffffff) < 0x41e00000) return;
-                        z = (int)__hiloint2double(h, 0);                // saturates
+                        if ((h & 0x7fffffff) >= 0x41e00000) z = (int)__hiloint2double(h, 0);        // saturates
+                        else if (z == TOP && h >= 0) z = 0x7fffffff;
+                        else return;
                         const unsigned long long gr = row0 + a * 8 + row, gc = col0 + b * 8 + j;
                         const unsigned long long key = ((gr + gc) << 42) | (((h & 0x7fffffff) < 0x7ff00000 ? 1ull : 0ull) << 41) | (gr << 20) | gc;
                         if (gr < (unsigned long long)p.m && gc < (unsigned long long)p.n && key < badkey) badkey = key;
