@@ -12,6 +12,12 @@
  *     be 8-byte aligned; 16-byte alignment with even leading dimensions is faster.
  *   - Nothing is allocated: scratch comes from a caller-provided device workspace
  *     whose size the matching *_workspace_bytes query returns (256-byte aligned).
+ *     Part of that size may only serve speed, and a workspace without that part is accepted too; the results are the same
+ *     to rounding.  The set-up needs three square matrices of order k rounded up to 16, k rounded up to 32 values and 256
+ *     bytes a side, the objective two m x n matrices (rows rounded up to 16) and a value per 128 x 128 tile; what the
+ *     query returns on top holds the digit planes of large products (7 (k + 512) min(k + 512, 16384) bytes a side from
+ *     order 1024 on), without which all products run on the fp64 tensor path.  A sweep needs two m x n matrices
+ *     (both sizes rounded up to 128) and its bookkeeping; less than 1 MB more lets a large one run in blocks.
  *   - `stream` is a cudaStream_t passed as void* (NULL = default stream).  Calls
  *     enqueue work and return; they do not synchronise.
  *   - The return value reports argument / launch errors found on the host
@@ -37,7 +43,7 @@ extern "C" {
 typedef enum {
     GPTQ2D_OK = 0,
     GPTQ2D_ERR_INVALID_ARG = 1,        /* null pointer, m or n < 1, ld too small, misaligned pointer   */
-    GPTQ2D_ERR_WORKSPACE = 2,          /* workspace missing, misaligned or smaller than the query says  */
+    GPTQ2D_ERR_WORKSPACE = 2,          /* workspace missing, misaligned or too small (below what the call needs)  */
     GPTQ2D_ERR_UNSUPPORTED_DEVICE = 3, /* current device is not compute capability 10.x                 */
     GPTQ2D_ERR_CUDA = 4,               /* a CUDA runtime call failed (launch, attribute query, copy)    */
     GPTQ2D_ERR_NOT_SPD = 5,            /* device: Gram pivot <= 0 or non-finite; info[1] = pivot index,

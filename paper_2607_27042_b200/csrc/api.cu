@@ -11,9 +11,9 @@
 #include <vector>
 
 namespace gptq2d {
-size_t objective_workspace_bytes(int m, int n);
+size_t objective_workspace_bytes(int m, int n, bool planes);
 int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long ldz, const double *A, long lda,
-                     const double *B, long ldb, double *obj, void *ws, int *info, cudaStream_t stream);
+                     const double *B, long ldb, double *obj, void *ws, bool planes, int *info, cudaStream_t stream);
 
 __global__ void margin_kernel(const double *max_abs_e, double *min_margin) { *min_margin = 0.5 - *max_abs_e; }
 
@@ -148,28 +148,28 @@ const char *gptq2d_status_string(int status) {
 
 size_t gptq2d_factor_workspace_bytes(int m, int n) {
     if (m < 1 || n < 1) return 0;
-    return factor_workspace_bytes(m, n);
+    return factor_workspace_bytes(m, n, true);
 }
 
 // Both sides of one problem, arguments already checked, `info` already cleared.
 static int factor_pair(int m, int n, const double *A, long lda, const double *B, long ldb, double *L, long ldl, double *U,
-                       long ldu, double *dL, double *dU, void *workspace, int *info, cudaStream_t stream) {
+                       long ldu, double *dL, double *dU, void *workspace, bool planes, int *info, cudaStream_t stream) {
     // The two sides are independent.  Each has a serial spine (one small diagonal-block kernel per 128
     // rows, between the panel and trailing updates) that leaves most SMs idle, so the B side runs on a
     // second stream and its GEMMs fill the gaps of the A side and vice versa.
-    char *wsB = static_cast<char *>(workspace) + factor_side_workspace_bytes(m);
+    char *wsB = static_cast<char *>(workspace) + factor_side_workspace_bytes(m, planes);
     HostPipe *hp = (A && B) ? host_pipe() : nullptr;
     if (!hp) {
-        int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, info, stream, nullptr);
+        int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, nullptr);
         if (st != GPTQ2D_OK) return st;
-        return factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, info, stream, nullptr);
+        return factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, stream, nullptr);
     }
     std::unique_lock<std::mutex> lock(hp->enqueue);
     if (cudaEventRecord(hp->inputs_free, stream) != cudaSuccess ||
         cudaStreamWaitEvent(hp->copy, hp->inputs_free, 0) != cudaSuccess)
         return GPTQ2D_ERR_CUDA;
-    int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, info, stream, hp->look[0].spine ? &hp->look[0] : nullptr);
-    int st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, info, hp->copy, hp->look[1].spine ? &hp->look[1] : nullptr);
+    int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, hp->look[0].spine ? &hp->look[0] : nullptr);
+    int st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, hp->copy, hp->look[1].spine ? &hp->look[1] : nullptr);
     // join even if an enqueue failed, so that nothing of this call is left running behind the caller's stream
     if (cudaEventRecord(hp->copies_done, hp->copy) != cudaSuccess ||
         cudaStreamWaitEvent(stream, hp->copies_done, 0) != cudaSuccess)
@@ -184,12 +184,13 @@ int gptq2d_factor(int m, int n, const double *A, long lda, const double *B, long
     if (m < 1 || n < 1 || !L || !U || ldl < m || ldu < n) return GPTQ2D_ERR_INVALID_ARG;
     if ((A && lda < m) || (B && ldb < n)) return GPTQ2D_ERR_INVALID_ARG;
     if (!aligned(A, 8) || !aligned(B, 8) || !aligned(L, 8) || !aligned(U, 8)) return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_factor_workspace_bytes(m, n))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < factor_workspace_bytes(m, n, false))
         return GPTQ2D_ERR_WORKSPACE;
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
-    return factor_pair(m, n, A, lda, B, ldb, L, ldl, U, ldu, dL, dU, workspace, info, stream);
+    return factor_pair(m, n, A, lda, B, ldb, L, ldl, U, ldu, dL, dU, workspace,
+                       workspace_bytes >= factor_workspace_bytes(m, n, true), info, stream);
 }
 
 static size_t factor_batched_table_bytes(int count) { return pad256((size_t)2 * count * sizeof(FactorSmallSide)); }
@@ -199,20 +200,23 @@ static bool factor_problem_is_large(const gptq2d_factor_problem_t &q) {
     return q.m > FACTOR_SMALL_MAX || q.n > FACTOR_SMALL_MAX;
 }
 
-size_t gptq2d_factor_batched_workspace_bytes(int count, const gptq2d_factor_problem_t *pr) {
+static size_t factor_batched_bytes(int count, const gptq2d_factor_problem_t *pr, bool planes) {
     if (count < 1 || !pr) return 0;
     size_t large = 0;
     int nlarge = 0;
     for (int b = 0; b < count; ++b) {
         if (pr[b].m < 1 || pr[b].n < 1) return 0;
         if (factor_problem_is_large(pr[b])) {
-            large = std::max(large, factor_workspace_bytes(pr[b].m, pr[b].n));
+            large = std::max(large, factor_workspace_bytes(pr[b].m, pr[b].n, planes));
             ++nlarge;
         }
     }
     // several problems of the blocked route run side by side, each in a slot of its own
     large *= (size_t)std::min(nlarge, (int)HostPipe::POOL);
     return factor_batched_table_bytes(count) + large;
+}
+size_t gptq2d_factor_batched_workspace_bytes(int count, const gptq2d_factor_problem_t *pr) {
+    return factor_batched_bytes(count, pr, true);
 }
 
 int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *workspace, size_t workspace_bytes,
@@ -227,8 +231,9 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
             !aligned(q.dU, 8))
             return GPTQ2D_ERR_INVALID_ARG;
     }
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_factor_batched_workspace_bytes(count, pr))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < factor_batched_bytes(count, pr, false))
         return GPTQ2D_ERR_WORKSPACE;
+    const bool planes = workspace_bytes >= factor_batched_bytes(count, pr, true);
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
@@ -259,7 +264,7 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
     int nlarge = 0;
     for (int b = 0; b < count; ++b)
         if (factor_problem_is_large(pr[b])) {
-            slot_bytes = std::max(slot_bytes, factor_workspace_bytes(pr[b].m, pr[b].n));
+            slot_bytes = std::max(slot_bytes, factor_workspace_bytes(pr[b].m, pr[b].n, planes));
             ++nlarge;
         }
     HostPipe *hp = nlarge > 1 ? host_pipe() : nullptr;
@@ -268,7 +273,7 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
         for (int b = 0; b < count; ++b) {
             const gptq2d_factor_problem_t &q = pr[b];
             if (!factor_problem_is_large(q)) continue;
-            st = factor_pair(q.m, q.n, q.A, q.lda, q.B, q.ldb, q.L, q.ldl, q.U, q.ldu, q.dL, q.dU, wl, info, stream);
+            st = factor_pair(q.m, q.n, q.A, q.lda, q.B, q.ldb, q.L, q.ldl, q.U, q.ldu, q.dL, q.dU, wl, planes, info, stream);
             if (st != GPTQ2D_OK) return st;
         }
         return GPTQ2D_OK;
@@ -286,8 +291,8 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
         if (!factor_problem_is_large(q)) continue;
         const int k = idx++ % nslots;
         char *wk = wl + (size_t)k * slot_bytes;
-        int s1 = factor_one_side(q.m, q.A, q.lda, 0, q.L, q.ldl, q.dL, wk, info, hp->pool[k], nullptr);
-        int s2 = factor_one_side(q.n, q.B, q.ldb, 1, q.U, q.ldu, q.dU, wk + factor_side_workspace_bytes(q.m), info,
+        int s1 = factor_one_side(q.m, q.A, q.lda, 0, q.L, q.ldl, q.dL, wk, planes, info, hp->pool[k], nullptr);
+        int s2 = factor_one_side(q.n, q.B, q.ldb, 1, q.U, q.ldu, q.dU, wk + factor_side_workspace_bytes(q.m, planes), planes, info,
                                  hp->pool[k], nullptr);
         if (first_err == GPTQ2D_OK) first_err = s1 != GPTQ2D_OK ? s1 : s2;
     }
@@ -309,6 +314,9 @@ size_t gptq2d_round_workspace_bytes(int m, int n, int precision) {
     if (precision == GPTQ2D_FP64_PULL) return round_pull_workspace_bytes(m, n);
     return 0;
 }
+static size_t round_min_workspace_bytes(int m, int n, int precision) {
+    return precision == GPTQ2D_FP64 ? round_tiled_min_workspace_bytes(m, n) : gptq2d_round_workspace_bytes(m, n, precision);
+}
 
 int gptq2d_round(int m, int n, const double *X, long ldx, const double *L, long ldl, const double *U, long ldu,
                  int32_t *Z, long ldz, double *E, long lde, double *min_margin, int precision, void *workspace,
@@ -322,7 +330,7 @@ int gptq2d_round(int m, int n, const double *X, long ldx, const double *L, long 
     if (precision != GPTQ2D_FP64 && precision != GPTQ2D_FP32 && precision != GPTQ2D_FP64_UNTILED &&
         precision != GPTQ2D_FP64_PULL && precision != GPTQ2D_FP32_UNTILED)
         return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_round_workspace_bytes(m, n, precision))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < round_min_workspace_bytes(m, n, precision))
         return GPTQ2D_ERR_WORKSPACE;
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
@@ -399,8 +407,13 @@ int gptq2d_round_host(int m, int n, const double *hX, const double *hL, const do
     if (m < 1 || n < 1 || !hX || !hL || !hU || !hZ) return GPTQ2D_ERR_INVALID_ARG;
     size_t need = gptq2d_round_host_workspace_bytes(m, n, precision);
     if (need == 0) return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return GPTQ2D_ERR_WORKSPACE;
     size_t inner = gptq2d_round_workspace_bytes(m, n, precision);
+    if (workspace_bytes < need) {
+        need -= inner;
+        inner = round_min_workspace_bytes(m, n, precision);
+        need += inner;
+    }
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return GPTQ2D_ERR_WORKSPACE;
     char *w = static_cast<char *>(workspace);
     char *p = w + pad256(inner);
     double *dX = reinterpret_cast<double *>(p); p += pad256((size_t)m * n * 8);
@@ -531,7 +544,7 @@ int gptq2d_round_host(int m, int n, const double *hX, const double *hL, const do
 
 size_t gptq2d_objective_workspace_bytes(int m, int n) {
     if (m < 1 || n < 1) return 0;
-    return objective_workspace_bytes(m, n);
+    return objective_workspace_bytes(m, n, true);
 }
 
 int gptq2d_objective(int m, int n, const double *X, long ldx, const int32_t *Z, long ldz, const double *A, long lda,
@@ -542,12 +555,13 @@ int gptq2d_objective(int m, int n, const double *X, long ldx, const int32_t *Z, 
     if ((A && lda < m) || (B && ldb < n)) return GPTQ2D_ERR_INVALID_ARG;
     if (!aligned(X, 8) || !aligned(Z, 4) || !aligned(A, 8) || !aligned(B, 8) || !aligned(obj, 8))
         return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_objective_workspace_bytes(m, n))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < objective_workspace_bytes(m, n, false))
         return GPTQ2D_ERR_WORKSPACE;
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
-    return launch_objective(m, n, X, ldx, Z, ldz, A, lda, B, ldb, obj, workspace, info, stream);
+    return launch_objective(m, n, X, ldx, Z, ldz, A, lda, B, ldb, obj, workspace,
+                            workspace_bytes >= objective_workspace_bytes(m, n, true), info, stream);
 }
 
 int gptq2d_internal_test_hook(int key, long value) {

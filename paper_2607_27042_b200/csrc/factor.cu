@@ -18,6 +18,7 @@
 #include "gemm.cuh"
 #include "factor.cuh"
 #include "i8_gemm.cuh"
+#include <algorithm>
 
 namespace gptq2d {
 
@@ -387,19 +388,21 @@ int launch_factor_small(const int (&counts)[3], const FactorSmallSide *dev_sides
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
 
 // Digit planes of the operands of one large product at a time (i8_gemm.cuh).  The largest is the Gram's one k x k operand;
-// the two of a product of the inverse have at most k^2 entries together, plus padding.
+// the two of a product of the inverse have at most k rows together, plus padding.  Contractions end at I8_MAX_K.
 constexpr int FACTOR_I8_MIN = 1024;      // orders below keep the fp64 product: their products have few tiles
-static size_t factor_i8_bytes(int k) { return k < FACTOR_I8_MIN ? 0 : i8_planes_bytes(k + 512, k + 512, 1); }
+static size_t factor_i8_bytes(int k) { return k < FACTOR_I8_MIN ? 0 : i8_planes_bytes(k + 512, std::min(k + 512, I8_MAX_K), 1); }
 
 // one side: three k x k matrices (Gram / Cholesky factor, its inverse, a product buffer) and the pivots
-size_t factor_side_workspace_bytes(int k) {
+size_t factor_side_workspace_bytes(int k, bool planes) {
     long ld = round_up(k, 16);
     size_t mat = (size_t)ld * (size_t)round_up(k, 16) * sizeof(double);
     size_t b = 3 * mat + (size_t)round_up(k, 32) * sizeof(double) + 256;
-    return (b + 255) / 256 * 256 + factor_i8_bytes(k);
+    return (b + 255) / 256 * 256 + (planes ? factor_i8_bytes(k) : 0);
 }
 // the two sides are factorised at the same time (two streams), each in its own part of the workspace
-size_t factor_workspace_bytes(int m, int n) { return factor_side_workspace_bytes(m) + factor_side_workspace_bytes(n); }
+size_t factor_workspace_bytes(int m, int n, bool planes) {
+    return factor_side_workspace_bytes(m, planes) + factor_side_workspace_bytes(n, planes);
+}
 
 #define CK(x)                                          \
     do {                                               \
@@ -407,7 +410,7 @@ size_t factor_workspace_bytes(int m, int n) { return factor_side_workspace_bytes
     } while (0)
 
 // side 0: S = M^T M -> out = F (unit lower).  side 1: S = M M^T -> out = F^T (unit upper).
-int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws,
+int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws, bool planes,
                     int *info, cudaStream_t stream, const FactorLookahead *look) {
     if (!M) {
         long tot = (long)k * k;
@@ -422,12 +425,13 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     double *T = X + mat;
     double *p = T + mat;
     const int nblk = (k + FB - 1) / FB;
-    char *i8_at = static_cast<char *>(ws) + (factor_side_workspace_bytes(k) - factor_i8_bytes(k));
+    char *i8_at = static_cast<char *>(ws) + factor_side_workspace_bytes(k, false);
+    const size_t i8_room = planes ? factor_i8_bytes(k) : 0;
     // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream`, so one set of planes
     // serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
     auto product = [&](const GemmArgs &g, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
-        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > factor_i8_bytes(k)) {
+        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
             // few tiles: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the number of tiles)
             const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
             const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && tiles <= 74;
@@ -514,7 +518,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         return i8_planes_at(i8_at, (int)k0, (int)(k1 - k0), 1);
     };
     auto split_panels = [&](int K0, int K1, cudaStream_t s) -> int {
-        CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));
+        if (i8_room) CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));
         return GPTQ2D_OK;
     };
     auto trailing_multi = [&](int K0, int K1, long r0, long r1, cudaStream_t s) -> int {
@@ -529,7 +533,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
         const I8Planes pl = panel_planes(K0, K1);
         cudaError_t e = cudaSuccess;
-        if (!launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
+        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
         CK(e);
         return GPTQ2D_OK;
     };

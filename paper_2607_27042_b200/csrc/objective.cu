@@ -44,7 +44,8 @@ static size_t objective_f64_bytes(int m, int n) {
     size_t tiles = (size_t)((m + 127) / 128) * ((n + 127) / 128);
     return round_up((long)(2 * mat + round_up((long)(tiles * sizeof(double)), 256) + 256), 256);
 }
-size_t objective_workspace_bytes(int m, int n) { return objective_f64_bytes(m, n) + objective_i8_bytes(m, n); }
+// without room for planes both products are fp64 ones
+size_t objective_workspace_bytes(int m, int n, bool planes) { return objective_f64_bytes(m, n) + (planes ? objective_i8_bytes(m, n) : 0); }
 
 #define CK(x)                                          \
     do {                                               \
@@ -52,7 +53,7 @@ size_t objective_workspace_bytes(int m, int n) { return objective_f64_bytes(m, n
     } while (0)
 
 int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long ldz, const double *A, long lda,
-                     const double *B, long ldb, double *obj, void *ws, int *info, cudaStream_t stream) {
+                     const double *B, long ldb, double *obj, void *ws, bool planes, int *info, cudaStream_t stream) {
     const long ld = round_up(n, 16);
     const size_t mat = (size_t)m * ld;
     double *R = static_cast<double *>(ws);
@@ -63,7 +64,7 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
     residual_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(m, n, X, ldx, Z, ldz, R, ld);
     CK(cudaGetLastError());
     auto product = [&](const GemmArgs &g) -> cudaError_t {
-        if (!gemm_i8_pays(g.M, g.N, g.K, 1)) return launch_gemm(g, stream);
+        if (!planes || !gemm_i8_pays(g.M, g.N, g.K, 1)) return launch_gemm(g, stream);
         char *at = static_cast<char *>(ws) + objective_f64_bytes(m, n);
         const I8Planes pa = i8_planes_at(at, g.M, g.K, 1);
         const I8Planes pb = i8_planes_at(at + i8_planes_bytes(g.M, g.K, 1), g.N, g.K, 1);

@@ -12,6 +12,8 @@
 // O(m n (m + n)) flops of the sweep.
 #include <cuda_runtime.h>
 #include "../../include/gptq2d.h"
+#include "factor.cuh"
+#include "round_internal.cuh"
 
 namespace gptq2d {
 
@@ -74,7 +76,8 @@ int gptq2d_factor_reverse(int m, int n, const double *A, long lda, const double 
     if ((A && lda < m) || (B && ldb < n)) return GPTQ2D_ERR_INVALID_ARG;
     if (!aligned(A, 8) || !aligned(B, 8) || !aligned(Lr, 8) || !aligned(Ur, 8) || !aligned(dL, 8) || !aligned(dU, 8))
         return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_factor_reverse_workspace_bytes(m, n))
+    const size_t own = gptq2d_factor_reverse_workspace_bytes(m, n) - gptq2d_factor_workspace_bytes(m, n);
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < own + factor_workspace_bytes(m, n, false))
         return GPTQ2D_ERR_WORKSPACE;
     const size_t mm = pad256((size_t)m * m * 8), nn = pad256((size_t)n * n * 8);
     char *w = static_cast<char *>(workspace);
@@ -88,7 +91,7 @@ int gptq2d_factor_reverse(int m, int n, const double *A, long lda, const double 
     if (A && !flip(Ap, (long)m, A, lda, m, m, 0, 1, stream)) return GPTQ2D_ERR_CUDA;
     if (B && !flip(Bp, (long)n, B, ldb, n, n, 1, 0, stream)) return GPTQ2D_ERR_CUDA;
     int st = gptq2d_factor(m, n, A ? Ap : nullptr, m, B ? Bp : nullptr, n, Lp, m, Up, n, dLp, dUp, w,
-                           gptq2d_factor_workspace_bytes(m, n), info, stream_);
+                           workspace_bytes - own, info, stream_);
     if (st != GPTQ2D_OK) return st;
     if (!flip(Lr, ldl, Lp, (long)m, m, m, 1, 1, stream) || !flip(Ur, ldu, Up, (long)n, n, n, 1, 1, stream))
         return GPTQ2D_ERR_CUDA;
@@ -112,7 +115,8 @@ int gptq2d_round_reverse(int m, int n, const double *X, long ldx, const double *
     if (!aligned(X, 8) || !aligned(Lr, 8) || !aligned(Ur, 8) || !aligned(Z, 4) || !aligned(E, 8) ||
         !aligned(min_margin, 8))
         return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_round_reverse_workspace_bytes(m, n))
+    const size_t own = gptq2d_round_reverse_workspace_bytes(m, n) - gptq2d_round_workspace_bytes(m, n, GPTQ2D_FP64);
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < own + round_tiled_min_workspace_bytes(m, n))
         return GPTQ2D_ERR_WORKSPACE;
     char *w = static_cast<char *>(workspace);
     double *Xp = reinterpret_cast<double *>(w); w += pad256((size_t)m * n * 8);
@@ -124,7 +128,7 @@ int gptq2d_round_reverse(int m, int n, const double *X, long ldx, const double *
         !flip(Up, (long)n, Ur, ldu, n, n, 1, 1, stream))
         return GPTQ2D_ERR_CUDA;
     int st = gptq2d_round(m, n, Xp, n, Lp, m, Up, n, Zp, n, E ? Ep : nullptr, n, min_margin, GPTQ2D_FP64, w,
-                          gptq2d_round_workspace_bytes(m, n, GPTQ2D_FP64), info, stream_);
+                          workspace_bytes - own, info, stream_);
     if (st != GPTQ2D_OK) return st;
     if (!flip(Z, ldz, Zp, (long)n, m, n, 1, 1, stream)) return GPTQ2D_ERR_CUDA;
     if (E && !flip(E, lde, Ep, (long)n, m, n, 1, 1, stream)) return GPTQ2D_ERR_CUDA;
@@ -146,7 +150,8 @@ int gptq2d_round_f32in(int m, int n, const float *X, long ldx, const float *L, l
     if (!aligned(X, 4) || !aligned(L, 4) || !aligned(U, 4) || !aligned(Z, 4) || !aligned(E, 8) ||
         !aligned(min_margin, 8))
         return GPTQ2D_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gptq2d_round_f32in_workspace_bytes(m, n))
+    const size_t own = gptq2d_round_f32in_workspace_bytes(m, n) - gptq2d_round_workspace_bytes(m, n, GPTQ2D_FP64);
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < own + round_tiled_min_workspace_bytes(m, n))
         return GPTQ2D_ERR_WORKSPACE;
     char *w = static_cast<char *>(workspace);
     double *Xd = reinterpret_cast<double *>(w); w += pad256((size_t)m * n * 8);
@@ -156,7 +161,7 @@ int gptq2d_round_f32in(int m, int n, const float *X, long ldx, const float *L, l
         !widen(Ud, (long)n, U, ldu, n, n, stream))
         return GPTQ2D_ERR_CUDA;
     return gptq2d_round(m, n, Xd, n, Ld, m, Ud, n, Z, ldz, E, lde, min_margin, GPTQ2D_FP64, w,
-                        gptq2d_round_workspace_bytes(m, n, GPTQ2D_FP64), info, stream_);
+                        workspace_bytes - own, info, stream_);
 }
 
 }  // extern "C"

@@ -56,6 +56,8 @@ struct TiledParams {
 constexpr int COPY_BLOCK_TILES_LOG2 = 2;
 constexpr int COPY_BLOCK = 128 << COPY_BLOCK_TILES_LOG2;
 size_t round_tiled_workspace_bytes(int m, int n);
+// the least that will do: without the bookkeeping of a sweep in blocks, a large matrix is swept whole
+size_t round_tiled_min_workspace_bytes(int m, int n);
 // device array inside the workspace: for each row of 128 x 128 tiles, how many of its tiles are swept
 unsigned *round_tiled_rowdone(void *ws, int m, int n);
 int launch_round_tiled(const TiledParams &p, void *ws, size_t ws_bytes, cudaStream_t stream);

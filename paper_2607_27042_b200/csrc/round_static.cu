@@ -57,7 +57,7 @@ extern "C" int gptq2d_round_static(int m, int n, const double *X, long ldx, cons
     if (ldx < n || ldl < m || ldu < n || ldz < n || (E && lde < n)) return GPTQ2D_ERR_INVALID_ARG;
     auto al = [](const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; };
     if (!al(X, 8) || !al(L, 8) || !al(U, 8) || !al(Z, 4) || !al(E, 8) || !al(min_margin, 8)) return GPTQ2D_ERR_INVALID_ARG;
-    if (round_tiled_workspace_bytes(m, n) > STATIC_BYTES) return GPTQ2D_ERR_TOO_LARGE;
+    if (round_tiled_min_workspace_bytes(m, n) > STATIC_BYTES) return GPTQ2D_ERR_TOO_LARGE;
     int dev = 0, major = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;

@@ -1146,6 +1146,7 @@ static SplitLayout split_layout(int m, int n) {
 }
 
 size_t round_tiled_workspace_bytes(int m, int n) { return split_layout(m, n).total; }
+size_t round_tiled_min_workspace_bytes(int m, int n) { return tiled_layout(m, n).total; }
 
 // the same layout for the sixteen-warp kernel (round_fused.cu), which shares the workspace format
 struct TiledLayoutView {
@@ -1166,7 +1167,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
 
 int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStream_t stream) {
     TiledLayout l = tiled_layout(in.m, in.n);
-    if (ws_bytes < round_tiled_workspace_bytes(in.m, in.n)) return GPTQ2D_ERR_WORKSPACE;
+    if (ws_bytes < l.total) return GPTQ2D_ERR_WORKSPACE;
     {
         // large resident problems: far contractions and quadrant tasks side by side on every SM
         const int st = launch_round_fused(in, ws, ws_bytes, stream, false);
