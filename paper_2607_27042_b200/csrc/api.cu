@@ -614,7 +614,9 @@ int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, doub
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
     GemmArgs g{};
-    g.M = M; g.N = N; g.K = K; g.alpha = alpha; g.beta = beta; g.C = C; g.ldc = ldc; g.batch = 1;
+    g.opA = transa ? OP_T : OP_N; g.opB = transb ? OP_T : OP_N;
+    g.M = M; g.N = N; g.K = K; g.alpha = alpha; g.beta = beta; g.A = A; g.lda = lda; g.B = B; g.ldb = ldb;
+    g.C = C; g.ldc = ldc; g.batch = 1;
     const I8Planes pa = i8_planes_at(workspace, M, K, 1);
     const I8Planes pb = i8_planes_at(static_cast<char *>(workspace) + i8_planes_bytes(M, K, 1), N, K, 1);
     cudaError_t e = i8_split(pa, A, lda, 0, !transa, stream);

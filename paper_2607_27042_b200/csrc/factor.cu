@@ -444,7 +444,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         cudaError_t e = i8_split(pa, g.A, g.lda, g.strideA, g.opA == OP_N, stream, undo, diag_a);
         if (e == cudaSuccess && !same) e = i8_split(pb, g.B, g.ldb, g.strideB, g.opB == OP_T, stream, inner, diag_b);
         if (e != cudaSuccess) return e;
-        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b)) return launch_gemm(g, stream);
+        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b, I8_LEAST_SETUP)) return launch_gemm(g, stream);
         return e;
     };
 
@@ -533,7 +533,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
         const I8Planes pl = panel_planes(K0, K1);
         cudaError_t e = cudaSuccess;
-        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
+        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e, false, false, I8_LEAST_SETUP)) e = launch_gemm(t, s);
         CK(e);
         return GPTQ2D_OK;
     };

@@ -7,7 +7,8 @@
 // set-up at order 8192 was 9e-14 off instead of 1e-15.)  What the last digit rounds off is of the order
 // 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
 // entries: 4e-16 against 3e-15 of the fp64 tensor path).  The eight int32 sums (one per p + q) are put together in int64
-// and fp64.
+// and fp64.  An entry far below the largest of its row keeps fewer than its 53 bits, which matters where the largest one meets
+// a zero; a tile in which it does is recognised by its result and computed in fp64 instead (end of the kernel).
 //
 // Kernel.  One CTA per 128 x 128 tile of C; tcgen05.mma kind::i8 (M 128, N 128, K 32), accumulators in tensor memory.
 // Four accumulators of 128 columns fill it, so a tile takes two passes over k: p + q = 6 .. 9 (24 products), then
@@ -212,7 +213,7 @@ constexpr int I8_STAGE2_BYTES = 2 * I8_TOP * I8_TILE_BYTES;    // 64 KB
 constexpr int I8_STAGES2 = 3;
 static_assert(I8_STAGES2 * I8_STAGE2_BYTES <= I8_STAGES * I8_STAGE_BYTES, "pass 2 reuses the memory of pass 1");
 constexpr int I8_OUT_LD = 130;                                 // row pitch (doubles) of the tile on its way out: rows start on 16 bytes
-constexpr size_t I8_SMEM = (size_t)I8_STAGES * I8_STAGE_BYTES + 1024;
+constexpr size_t I8_SMEM = (size_t)I8_STAGES * I8_STAGE_BYTES + 1024;       // (leaves 2 KB of a CTA's 227 for what is declared in the kernel)
 static_assert(128 * I8_OUT_LD * 8 <= I8_STAGES * I8_STAGE_BYTES, "the output tile reuses the stages");
 constexpr int I8_THREADS = 320;                                // warps 0-7 epilogue, 8 TMA, 9 MMA and tensor memory
 
@@ -236,9 +237,9 @@ __device__ __forceinline__ void i8_mma(unsigned d_tmem, unsigned long long a, un
 __device__ __forceinline__ void i8_commit(unsigned long long *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void i8_tmem_ld8(int (&v)[8], unsigned addr) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+__device__ __forceinline__ void i8_tmem_ld4(int (&v)[4], unsigned addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                  : "r"(addr));
 }
 __device__ __forceinline__ void i8_tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
@@ -264,18 +265,52 @@ struct I8Params {
     int diag_a, diag_b;
     const double *A; long ai, aj, strideA;
     const double *B; long bi, bj, strideB;
+    const unsigned *topA, *topB;                               // high words of the largest magnitude of every row of either operand's planes
+    int rowsA, rowsB;                                          // rows that exist there
+    double least;
     int *info;
 };
 
+// The tile once more in fp64, for operands that its digits do not suit (see below): alpha * op(A) op(B) over [k_lo, k_hi) into the output
+// tile in shared memory, or the sum of its squares.  Warps 0 - 7, the others have left.  The loop is gemm.cu's, at its speed.
+template <bool A_KCONTIG, bool B_KCONTIG>
+__device__ __noinline__ double i8_tile_in_fp64(const I8Params &p, int bz, int m0, int n0, int k_lo, int k_hi, double *smem, bool sumsq) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wm = warp >> 2, wn = warp & 3, g = lane >> 2, t = lane & 3;
+    Operand A, B;
+    A.ptr = p.A + (long)bz * p.strideA + (long)m0 * p.ai + (long)k_lo * p.aj;
+    A.ld = A_KCONTIG ? p.ai : p.aj;
+    A.mn_valid = min(128, p.rowsA - m0);
+    A.aligned16 = ((reinterpret_cast<uintptr_t>(A.ptr) & 15) == 0) && ((A.ld & 1) == 0);
+    B.ptr = p.B + (long)bz * p.strideB + (long)n0 * p.bj + (long)k_lo * p.bi;
+    B.ld = B_KCONTIG ? p.bj : p.bi;
+    B.mn_valid = min(128, p.rowsB - n0);
+    B.aligned16 = ((reinterpret_cast<uintptr_t>(B.ptr) & 15) == 0) && ((B.ld & 1) == 0);
+    Acc acc;
+    acc.zero();
+    gemm_tile<A_KCONTIG, B_KCONTIG, 3>(acc, smem, A, B, k_hi - k_lo);
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const double x0 = p.alpha * acc.v[a][b][0], x1 = p.alpha * acc.v[a][b][1];
+            if (sumsq) s = fma(x1, x1, fma(x0, x0, s));        // (rows and columns that do not exist are zeros)
+            else *reinterpret_cast<double2 *>(smem + (wm * 64 + a * 8 + g) * I8_OUT_LD + wn * 32 + b * 8 + 2 * t) = double2{x0, x1};
+        }
+    return s;
+}
+
 __global__ void __launch_bounds__(I8_THREADS, 1)
-i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __grid_constant__ CUtensorMap mapB7,
+i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUtensorMap mapA7, const __grid_constant__ CUtensorMap mapB7,
                const __grid_constant__ CUtensorMap mapA4, const __grid_constant__ CUtensorMap mapB4) {
     extern __shared__ __align__(16) unsigned char i8_raw[];
     __shared__ __align__(8) unsigned long long bar_full[I8_STAGES], bar_empty[I8_STAGES], bar_full2[I8_STAGES2], bar_empty2[I8_STAGES2], bar_acc, bar_drained;
     __shared__ unsigned s_tmem, s_abort;
     __shared__ double s_sum[8];
-    __shared__ double s_scale[128];                            // of the tile's columns
+    __shared__ int s_scale[128];                               // of the tile's columns: high words (the low ones are zero)
+    __shared__ unsigned s_seen[8];                             // bit per row (words 0 - 3) and column (4 - 7): it has an entry that is large enough, see below
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    CHECKED_SET_INFO(p.info);
     // Tiles in groups of sixteen tile rows, column by column inside a group, so that the CTAs that run at one time share
     // operand tiles in L2; the last rows first, which have the longest contractions where there are lower triangles.
     int tm, tn;
@@ -305,7 +340,8 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
         mbar_init_fence();
         s_abort = 0u;
     }
-    if (tid < 128) s_scale[tid] = __ldg(p.scaleB + (long)bz * p.rowsB_pad + n0 + tid);
+    if (tid < 8) s_seen[tid] = 0u;
+    if (tid < 128) s_scale[tid] = __double2hiint(__ldg(p.scaleB + (long)bz * p.rowsB_pad + n0 + tid));
     // Rows that start on 16 bytes leave as bulk copies, or bulk additions where beta = 1: the tile's old values then never
     // come to this SM, and the next CTA starts while L2 is still adding (rank-512 update of an 8192 x 8192 matrix: the
     // load-add-store loop took 21.6 of a tile's 76 thousand cycles).
@@ -325,6 +361,7 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
         atomicExch(&s_abort, 1u);
     };
 
+    bool looked_at = false;                                    // row tid or column tid - 128 of the tile has an entry at all
     if (warp == 8) {
         if (lane == 0) {
             const int ra = (int)(bz * p.rowsA_pad) + m0, rb = (int)(bz * p.rowsB_pad) + n0;
@@ -415,6 +452,10 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
         const unsigned lane_base = tmem + ((unsigned)((warp & 3) * 32) << 16) + (unsigned)c0;
         double part[64];
         bool ok = true;
+        // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
+        const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = (tall || !wide) && !p.sumsq_partials;
+        looked_at = (tid < 128 ? by_rows : by_cols) &&
+                    __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128) != 0u;
         if (!p.sumsq_partials && p.beta != 0.0 && !bulk_out) {  // the old values are needed at the end: ask for them now
             const int rows = out_rows, cols = out_cols;
             const double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
@@ -432,15 +473,15 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
             if (ok) {
                 i8_fence_after();
 #pragma unroll
-                for (int c = 0; c < 64; c += 8) {              // exact: |sums| < 2^31
-                    int g6[8], g7[8], g8[8], g9[8];
-                    i8_tmem_ld8(g6, lane_base + c);
-                    i8_tmem_ld8(g7, lane_base + 128 + c);
-                    i8_tmem_ld8(g8, lane_base + 256 + c);
-                    i8_tmem_ld8(g9, lane_base + 384 + c);
+                for (int c = 0; c < 64; c += 4) {              // exact: |sums| < 2^31
+                    int g6[4], g7[4], g8[4], g9[4];
+                    i8_tmem_ld4(g6, lane_base + c);
+                    i8_tmem_ld4(g7, lane_base + 128 + c);
+                    i8_tmem_ld4(g8, lane_base + 256 + c);
+                    i8_tmem_ld4(g9, lane_base + 384 + c);
                     i8_tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
+                    for (int j = 0; j < 4; ++j)
                         part[c + j] = fma(i8_to_double(g6[j]), 16777216.0, i8_to_double(g9[j] + g8[j] * 256ll + g7[j] * 65536ll));
                 }
                 i8_fence_before();
@@ -456,15 +497,15 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
             if (ok) {
                 i8_fence_after();
 #pragma unroll
-                for (int c = 0; c < 64; c += 8) {
-                    int g2[8], g3[8], g4[8], g5[8];
-                    i8_tmem_ld8(g2, lane_base + c);
-                    i8_tmem_ld8(g3, lane_base + 128 + c);
-                    i8_tmem_ld8(g4, lane_base + 256 + c);
-                    i8_tmem_ld8(g5, lane_base + 384 + c);
+                for (int c = 0; c < 64; c += 4) {
+                    int g2[4], g3[4], g4[4], g5[4];
+                    i8_tmem_ld4(g2, lane_base + c);
+                    i8_tmem_ld4(g3, lane_base + 128 + c);
+                    i8_tmem_ld4(g4, lane_base + 256 + c);
+                    i8_tmem_ld4(g5, lane_base + 384 + c);
                     i8_tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
+                    for (int j = 0; j < 4; ++j) {
                         const double hi = fma(i8_to_double(g2[j]), 16777216.0, i8_to_double(g5[j] + g4[j] * 256ll + g3[j] * 65536ll));
                         part[c + j] = fma(hi, 4294967296.0, part[c + j]);
                     }
@@ -475,14 +516,33 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
             for (int c = 0; c < 64; ++c) part[c] = 0.0;
         }
         if (ok) {
-            // the scales of both sides are powers of two and are multiplied first: no overflow that the product itself lacks
+            // Which rows and columns have a digit sum of at least `least`, for the check below.  (High words compared as fp32 numbers: one
+            // instruction with the absolute value.  The diagonal of a Gram, the same rows on both sides, says nothing about its
+            // other entries and is left out.)
+            const float least = __int_as_float(__double2hiint(nchunk * I8_KCHUNK > 128 ? p.least * 0x1p72 : p.least * 0x1p71));     // (digit sums count 2^-72)
+            const int at_diagonal = tall && p.topA + bz * p.rowsA_pad + m0 == p.topB + bz * p.rowsB_pad + n0 ? row - c0 : -1;
+            bool row_seen = false;
+            unsigned cols_seen[2] = {0u, 0u};
+#pragma unroll
+            for (int c = 0; c < 64; ++c) {
+                const bool seen = fabsf(__int_as_float(__double2hiint(part[c]))) >= least && c != at_diagonal;
+                row_seen |= seen;
+                if (__any_sync(0xffffffffu, seen)) cols_seen[c >> 5] |= 1u << (c & 31);
+            }
+            const unsigned rows_seen = __ballot_sync(0xffffffffu, row_seen);
+            if (lane == 0) {
+                atomicOr(&s_seen[warp & 3], rows_seen);
+                atomicOr(&s_seen[4 + (c0 >> 5)], cols_seen[0]);
+                atomicOr(&s_seen[5 + (c0 >> 5)], cols_seen[1]);
+            }
+            // (the scales are powers of two; that their product is one too is part of the check below)
             const double sa = __ldg(p.scaleA + (long)bz * p.rowsA_pad + m0 + row);
-            const double *sb = s_scale + c0;
+            const auto sb = [&](int c) { return __hiloint2double(s_scale[c0 + c], 0); };
             if (p.sumsq_partials) {
                 double s = 0.0;
 #pragma unroll
                 for (int c = 0; c < 64; ++c) {
-                    const double x = p.alpha * (part[c] * (sa * sb[c]));
+                    const double x = p.alpha * (part[c] * (sa * sb(c)));
                     s = fma(x, x, s);
                 }
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -490,7 +550,7 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
             } else {
                 double *out = reinterpret_cast<double *>(stages) + row * I8_OUT_LD + c0;
 #pragma unroll
-                for (int c = 0; c < 64; ++c) out[c] = p.alpha * (part[c] * (sa * sb[c]));
+                for (int c = 0; c < 64; ++c) out[c] = p.alpha * (part[c] * (sa * sb(c)));
                 if (bulk_out) fence_proxy_async();             // the copy engine reads what was just written
             }
         }
@@ -500,6 +560,33 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
     i8_fence_after();
     if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
     if (*(volatile unsigned *)&s_abort) return;                // the tile is not written
+    // Do the digits suit the operands?  They cut every entry at the same distance below the largest of its row (of op(A) and of
+    // op(B)^T), so where the large entries of a row meet zeros or small ones only, the result has lost digits that a product in fp64
+    // keeps: an outlier channel whose residuals happen to be zero.  The loss shows in the result.  With every row scaled to a largest
+    // entry of 1/4 to 1/2, the cut moves an entry by 2^-57.8 (|a| + |b|), norms of its two rows, below 2^-59 sqrt(K) for normal or
+    // uniform entries.  So a tile is kept if the largest entry of each of its rows and columns is at least p.least, and computed in
+    // fp64 otherwise.  1/32 (I8_LEAST) is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the
+    // largest entry of a row; contractions of 128 and fewer, the corners of triangles, are kept from half of it on.  For a sum of
+    // squares the rows alone are looked at.
+    const bool in_fp64 = __syncthreads_or((looked_at && nchunk > 0 && !((s_seen[tid >> 5] >> lane) & 1u)));
+    if (warp >= 8) return;                                     // (barriers below are met by the other eight)
+    double sumsq = 0.0;
+    if (in_fp64) {
+        int k_first = k_lo, k_hi = max(k_lo, min(p.K, k_lo + nchunk * I8_KCHUNK));
+        if (p.diag_a) { k_first = min(k_first, m0); k_hi = max(k_hi, min(p.K, m0 + 128)); }     // the chunks count without the diagonals
+        if (p.diag_b) { k_first = min(k_first, n0); k_hi = max(k_hi, min(p.K, n0 + 128)); }
+        double *tile = reinterpret_cast<double *>(stages);
+        const bool a_kcontig = p.aj == 1, b_kcontig = p.bi == 1, sq = p.sumsq_partials != nullptr;
+        if (a_kcontig) sumsq = b_kcontig ? i8_tile_in_fp64<true, true>(p, bz, m0, n0, k_first, k_hi, tile, sq) : i8_tile_in_fp64<true, false>(p, bz, m0, n0, k_first, k_hi, tile, sq);
+        else sumsq = b_kcontig ? i8_tile_in_fp64<false, true>(p, bz, m0, n0, k_first, k_hi, tile, sq) : i8_tile_in_fp64<false, false>(p, bz, m0, n0, k_first, k_hi, tile, sq);
+        if (sq) {
+            for (int o = 16; o > 0; o >>= 1) sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
+            if (lane == 0) s_sum[warp] = sumsq;
+        } else if (bulk_out) {
+            fence_proxy_async();
+        }
+        __syncthreads();
+    }
     if (p.sumsq_partials) {
         if (tid == 0) {
             double tot = 0.0;
@@ -521,11 +608,12 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
         }
         return;
     }
-    if (warp < 8) {
+    {
         const double *in = reinterpret_cast<const double *>(stages);
         double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
         const int rows = out_rows, cols = out_cols;
         const double *Ab = p.A + (long)bz * p.strideA, *Bb = p.B + (long)bz * p.strideB;
+        const bool diag_a = p.diag_a && !in_fp64, diag_b = p.diag_b && !in_fp64;
         for (int r4 = warp * 4; r4 < rows; r4 += 32) {         // four rows of the tile per warp: sixteen loads in flight
             double old[4][4];
             if (p.beta != 0.0) {
@@ -542,8 +630,8 @@ i8_gemm_kernel(I8Params p, const __grid_constant__ CUtensorMap mapA7, const __gr
                     if (r4 + i < rows && lane + 32 * j < cols) {
                         double x = in[(r4 + i) * I8_OUT_LD + lane + 32 * j];
                         const long gi = m0 + r4 + i, gj = n0 + lane + 32 * j;
-                        if (p.diag_a && gi < p.K) x = fma(p.alpha * Ab[gi * (p.ai + p.aj)], Bb[gi * p.bi + gj * p.bj], x);
-                        if (p.diag_b && gj < p.K && !(p.diag_a && gi == gj))
+                        if (diag_a && gi < p.K) x = fma(p.alpha * Ab[gi * (p.ai + p.aj)], Bb[gi * p.bi + gj * p.bj], x);
+                        if (diag_b && gj < p.K && !(diag_a && gi == gj))
                             x = fma(p.alpha * Ab[gi * p.ai + gj * p.aj], Bb[gj * (p.bi + p.bj)], x);
                         Cb[(long)(r4 + i) * p.ldc + lane + 32 * j] = p.beta != 0.0 ? fma(p.beta, old[i][j], x) : x;
                     }
@@ -572,7 +660,7 @@ static bool encode_planes_map(CUtensorMap *map, const I8Planes &pl, int planes) 
 }
 
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
-                    bool diag_a, bool diag_b) {
+                    bool diag_a, bool diag_b, double least) {
     *err = cudaSuccess;
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return true;
     if (g.K > I8_MAX_K) return false;
@@ -586,11 +674,12 @@ bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int
     p.scaleA = A.scale; p.scaleB = B.scale; p.rowsA_pad = A.rows_pad; p.rowsB_pad = B.rows_pad;
     p.lower_tiles_only = g.lower_tiles_only;
     p.rangeA = A.range; p.rangeB = B.range;
+    p.topA = A.maxbits; p.topB = B.maxbits; p.rowsA = A.rows; p.rowsB = B.rows;
     p.diag_a = diag_a; p.diag_b = diag_b;
     p.A = g.A; p.strideA = g.strideA; p.ai = g.opA == OP_N ? g.lda : 1; p.aj = g.opA == OP_N ? 1 : g.lda;
     p.B = g.B; p.strideB = g.strideB; p.bi = g.opB == OP_N ? g.ldb : 1; p.bj = g.opB == OP_N ? 1 : g.ldb;
     p.tiles_m = (g.M + 127) / 128; p.tiles_n = (g.N + 127) / 128;
-    p.info = info;
+    p.info = info; p.least = least;
     *err = cudaFuncSetAttribute(i8_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I8_SMEM);
     if (*err != cudaSuccess) return true;
     i8_gemm_kernel<<<dim3((unsigned)(p.tiles_m * p.tiles_n), (unsigned)g.batch), I8_THREADS, I8_SMEM, stream>>>(p, a7, b7, a4, b4);

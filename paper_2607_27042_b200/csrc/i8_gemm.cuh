@@ -3,7 +3,7 @@
 //
 // Every row of op(A) and every column of op(B) is scaled by a power of two and written as I8_DIGITS signed base-256
 // digits; products of digit planes are exact in int32, and the planes whose weights stay within I8_DIGITS + 1 digits
-// are summed.  See i8_gemm.cu.
+// are summed.  Tiles that the digits do not suit are computed in fp64.  See i8_gemm.cu.
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -14,6 +14,7 @@ namespace gptq2d {
 
 constexpr int I8_DIGITS = 7;            // 56 bits below the largest entry of a row
 constexpr int I8_KCHUNK = 64;           // k-depth of a pipeline stage; planes are padded to a multiple of it
+constexpr double I8_LEAST = 0x1p-5, I8_LEAST_SETUP = 0x1p-9;
 constexpr int I8_MAX_K = 16384;         // 7 products of |digits| <= 128 per k: 7 * 2^14 * K < 2^31
 
 // The digit planes of `batch` matrices (rows x K each, K contiguous):
@@ -58,9 +59,15 @@ bool gemm_i8_pays(long M, long N, long K, long batch);
 // planes of that operand lack its diagonal, whose products are added in fp64 on the way out, from the operands in `g`.
 // A unit or dominant diagonal (triangular factors, their inverses, Cholesky bases) would otherwise set the scale of its
 // row, and the digits of all other entries with it.
+// `least`: a tile with a row or column whose largest entry is below `least` times the product of the largest entries of the two rows
+// that made it (each rounded up to a power of two that is two to four times as large) is computed in fp64 from the operands in `g`;
+// see i8_gemm.cu.  I8_LEAST: relative to the largest entry of its row or column in the tile no entry is further off than a chain of
+// fp64 additions leaves it.  I8_LEAST_SETUP: up to 16 times that in single tiles, for products that enter a factorisation, whose own
+// rounding is relative to the norms of whole rows; at 1/32 channel scales sent a third of the tiles of the inverse to fp64
+// (1100 x 4100: 4.5 -> 6.1 ms) for factors that came out no closer to 80-bit ones.
 // `info`: the call's status words (a bounded wait that runs out is reported there), may be NULL.
 // False: no tensor map can be had (no driver entry point); nothing was launched.
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
-                    bool diag_a = false, bool diag_b = false);
+                    bool diag_a = false, bool diag_b = false, double least = I8_LEAST);
 
 }  // namespace gptq2d

@@ -4,6 +4,8 @@ import numpy as np
 import pytest
 import torch
 
+import oracle as O
+
 pytestmark = pytest.mark.gpu
 
 
@@ -57,6 +59,93 @@ def test_rounding_is_within_the_digits_that_are_kept(g, K):
     top = np.abs(a).max(1, initial=0.0)[:, None] * np.abs(b).max(0, initial=0.0)[None, :]
     bound = K * 2.0 ** -52.9 * top + 2.0 ** -51 * np.abs(want).astype(np.float64)
     assert np.all(np.abs(c.cpu().numpy() - want) <= bound)
+
+
+@pytest.mark.parametrize("M,N,K", [(128, 128, 64), (5, 3, 2), (127, 129, 65), (257, 130, 191), (300, 100, 1000)])
+def test_integers_are_exact_in_all_layouts_where_tiles_fall_back_to_fp64(g, M, N, K):
+    # a large entry in every row of a that meets zeros only: the digits below it are of no use
+    rng = np.random.default_rng(M + N + K)
+    for transa in (False, True):
+        for transb in (False, True):
+            a = rng.integers(-8, 9, size=(M, K)).astype(np.float64)
+            b = rng.integers(-8, 9, size=(K, N)).astype(np.float64)
+            c0 = rng.integers(-8, 9, size=(M, N)).astype(np.float64)
+            a[:, K // 2], b[K // 2] = 2.0 ** 70, 0.0
+            for pitch in (padded, lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()):
+                for beta in (-1.0, 0.0, 1.0):
+                    c = pitch(c0)
+                    g.gptq2d_internal_gemm_split(pitch(a.T if transa else a), pitch(b.T if transb else b), c, transa=transa,
+                                                 transb=transb, alpha=2.0, beta=beta)
+                    assert np.array_equal(c.cpu().numpy(), 2.0 * (a @ b) + beta * c0), (transa, transb, beta)
+
+
+def product(g, a, b):
+    c = torch.empty((a.shape[0], b.shape[1]), dtype=torch.float64, device="cuda")
+    info = torch.full((4,), 9, dtype=torch.int32, device="cuda")
+    g.gptq2d_internal_gemm_split(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda(), c, info=info)
+    g.check_info(info)
+    return c.cpu().numpy()
+
+
+@pytest.mark.parametrize("outlier", [1e2, 1e4, 1e9])
+@pytest.mark.parametrize("K", [200, 256, 1000])
+@pytest.mark.parametrize("other", ["zero", "zero in some columns", "small in some columns", "there", "for half of the rows"])
+def test_outlier_channels_lose_no_digits(g, K, outlier, other):
+    # one k at which a is larger than elsewhere, and b is zero, small or like the rest there
+    rng = np.random.default_rng(int(outlier) + K)
+    M, N, k = 256, 384, K // 3
+    a, b = rng.standard_normal((M, K)), rng.uniform(-0.5, 0.5, (K, N))
+    a[:, k] *= outlier
+    if other == "zero":
+        b[k] = 0.0
+    elif other == "zero in some columns":
+        b[k, 100:200] = 0.0
+    elif other == "small in some columns":
+        b[k, 100:200] /= 50 * outlier
+    elif other == "for half of the rows":
+        a[:170, k] = 0.0
+    want = a.astype(np.longdouble) @ b.astype(np.longdouble)
+    error = np.abs(product(g, a, b) - want).astype(np.float64)
+    # Entries are cut 2^-57 below the largest of their row, so an entry of the product is moved by 2^-57.8 (|a| + |b|) with
+    # rows scaled to 1/2 at most (norms below 0.3 sqrt(K)), five times that in the worst of 10^5 entries; a tile is kept if its rows and
+    # columns, scaled in that way, reach 1/32: 3.8e-16 sqrt(K) of the largest entry of the row and of the column.  Other tiles: a
+    # chain of K additions in fp64, whose roundings add up to 0.2 * 2^-53 sqrt(K) (sum of (a b)^2)^(1/2), five times that in the worst.
+    scale = np.abs(a).max(1)[:, None] * np.abs(b).max(0)[None, :]
+    size, fp64 = np.abs(want).astype(np.float64) / scale, 2.0 ** -53 * np.sqrt(K) * np.sqrt((a * a) @ (b * b))
+    for i in range(0, M, 128):
+        for j in range(0, N, 128):
+            at = np.s_[i:i + 128, j:j + 128]
+            kept = 4e-16 * np.sqrt(K) * scale[at] * np.minimum(size[at].max(1)[:, None], size[at].max(0)[None, :])
+            assert np.all(error[at] <= np.maximum(kept, fp64[at])), (i, j)
+
+
+@pytest.mark.parametrize("outlier", [1e3, 1e9])
+def test_objective_with_an_outlier_channel_of_integers(g, outlier):
+    m = n = 1024
+    rng = np.random.default_rng(3)
+    a, b = (np.triu(rng.standard_normal((k, k)) / np.sqrt(2 * k), 1) + np.eye(k) for k in (m, n))
+    a[:, 300] *= outlier
+    x = 4.0 * rng.standard_normal((m, n))
+    x[300] = np.round(x[300])
+    z = np.round(x)
+    obj = g.gptq2d_objective(*(torch.from_numpy(v).cuda() for v in (x, z.astype(np.int32), a, b)))
+    r = (z - x).astype(np.longdouble)
+    want = float(np.square(a.astype(np.longdouble) @ r @ b.astype(np.longdouble)).sum())
+    # two products of 1024 terms in fp64 (1e-16 sqrt(1024) each, twice in a square), uncorrelated over 10^6 entries; plus their sum
+    assert abs(float(obj.cpu()[0]) - want) <= 1e-14 * want
+
+
+def test_set_up_of_a_basis_whose_large_entries_do_not_meet(g):
+    # one large entry a column, each in a row of its own: what couples two columns is 1e-8 of what their digits are spent on
+    k = 1100
+    rng = np.random.default_rng(4)
+    a = rng.standard_normal((k, k))
+    a[rng.permutation(k), np.arange(k)] += 1e8
+    L, _, _, _, info = g.gptq2d_factor(torch.from_numpy(a).cuda(), None, n=1)
+    g.check_info(info)
+    got, want = np.tril(L.cpu().numpy(), -1), np.tril(O.feedback_factors(a, np.eye(1))[0], -1)
+    # Gram, factor and inverse in fp64 with contractions of 1100, against the same in the oracle
+    assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
 
 
 def test_non_finite_entries_reach_their_row_and_column_only(g):

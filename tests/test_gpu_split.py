@@ -58,3 +58,20 @@ def test_status_words_name_the_first_anti_diagonal(g, where):
     i, j = min(where, key=lambda p: p[0] + p[1])
     # inside an 8 x 8 leaf a NaN reaches entries that exact arithmetic would spare: the anti-diagonal is known to a leaf's 15
     assert vals[0] == 6 and abs(vals[1] + vals[2] - i - j) < 15 and vals[3] == 0
+
+
+@pytest.mark.parametrize("m,n", [(300, 330), (515, 400)])
+def test_an_outlier_channel_of_integers_costs_no_digits(g, m, n):
+    # row 0 of X is whole numbers: its errors are zero, and so is what the large entries of column 0 of L are multiplied by
+    X, A, B = W.gaussian_like(m, n, 11)
+    L, U, _, _ = O.feedback_factors(A, B)
+    X[0] = np.round(X[0])
+    L[1:, 0] *= 1e6
+    dX, dL, dU = padded(X, 0), padded(L, 0), padded(U, 0)
+    Z, E, _, info = g.gptq2d_round(dX, dL, dU, want_E=True)
+    g.check_info(info)
+    g.gptq2d_internal_test_hook(7, 0)
+    Z1, E1, _, info = g.gptq2d_round(dX, dL, dU, want_E=True)
+    g.check_info(info)
+    # sums of at most 900 terms of order one in fp64, each side: 900 * 2^-53
+    assert torch.equal(Z, Z1) and float((E - E1).abs().max()) < 1e-13
