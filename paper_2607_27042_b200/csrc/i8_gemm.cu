@@ -65,6 +65,11 @@ __device__ __forceinline__ double i8_inner(const I8Inner &in, int b, int k, int 
 }
 
 // ---------------------------------------------------------------------------------------------
+// high word of |x|; not zero unless x is
+__device__ __forceinline__ unsigned i8_magnitude(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
+
 // Largest magnitude of every row (its high word: exponent and 20 bits are all that the scale needs; infinities and NaNs
 // come out above every finite number), and the range of k in which 128 rows have any entry.  A 64 x 64 block per CTA,
 // a thread's sixteen loads in flight together.  Memory bound.
@@ -88,14 +93,14 @@ __global__ void __launch_bounds__(256) i8_rowmax_kernel(I8Planes pl, const doubl
         const double f = i8_inner(inner, b, k0 + c, pl.K);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(v[i] * f) & 0x7fffffffu);
+            const unsigned m = __reduce_max_sync(0xffffffffu, i8_magnitude(v[i] * f));
             if ((tid & 31) == 0 && m) atomicMax(&s_max[(tid >> 6) + 4 * i], m);
         }
     } else {
         unsigned m = 0u;
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-            m = max(m, (unsigned)__double2hiint(v[i] * i8_inner(inner, b, k0 + (tid >> 6) + 4 * i, pl.K)) & 0x7fffffffu);
+            m = max(m, i8_magnitude(v[i] * i8_inner(inner, b, k0 + (tid >> 6) + 4 * i, pl.K)));
         if (m) atomicMax(&s_max[c], m);
     }
     __syncthreads();
@@ -117,6 +122,7 @@ __device__ __forceinline__ int i8_exponent(unsigned maxbits) {
     const int field = (int)((__double_as_longlong(top) >> 52) & 0x7ff);
     return max(field - 1022 + 1, -900);                                     // top < 2^(field - 1022); below 2^-900: one common scale
 }
+constexpr int I8_MAX_EXPONENT = 470;                                         // two scales 2^(e - 36) then multiply to 2^-1012 .. 2^868
 __device__ __forceinline__ double i8_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
 // Digit planes of a 64 x 64 block per CTA.  Padding rows and columns become zeros.
@@ -361,7 +367,8 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
         atomicExch(&s_abort, 1u);
     };
 
-    bool looked_at = false;                                    // row tid or column tid - 128 of the tile has an entry at all
+    // of row tid or column tid - 128 of the tile: has it an entry at all, and might its scale not multiply with any other to a normal number
+    bool looked_at = false, extreme = false;
     if (warp == 8) {
         if (lane == 0) {
             const int ra = (int)(bz * p.rowsA_pad) + m0, rb = (int)(bz * p.rowsB_pad) + n0;
@@ -454,8 +461,9 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
         bool ok = true;
         // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
         const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = (tall || !wide) && !p.sumsq_partials;
-        looked_at = (tid < 128 ? by_rows : by_cols) &&
-                    __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128) != 0u;
+        const unsigned top = __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128);
+        looked_at = top != 0u && (tid < 128 ? by_rows : by_cols);
+        extreme = top != 0u && abs(i8_exponent(top)) > I8_MAX_EXPONENT;
         if (!p.sumsq_partials && p.beta != 0.0 && !bulk_out) {  // the old values are needed at the end: ask for them now
             const int rows = out_rows, cols = out_cols;
             const double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
@@ -535,7 +543,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
                 atomicOr(&s_seen[4 + (c0 >> 5)], cols_seen[0]);
                 atomicOr(&s_seen[5 + (c0 >> 5)], cols_seen[1]);
             }
-            // (the scales are powers of two; that their product is one too is part of the check below)
+            // (the scales are powers of two; where their product might not be one the tile is computed again, see below)
             const double sa = __ldg(p.scaleA + (long)bz * p.rowsA_pad + m0 + row);
             const auto sb = [&](int c) { return __hiloint2double(s_scale[c0 + c], 0); };
             if (p.sumsq_partials) {
@@ -567,8 +575,8 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     // uniform entries.  So a tile is kept if the largest entry of each of its rows and columns is at least p.least, and computed in
     // fp64 otherwise.  1/32 (I8_LEAST) is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the
     // largest entry of a row; contractions of 128 and fewer, the corners of triangles, are kept from half of it on.  For a sum of
-    // squares the rows alone are looked at.
-    const bool in_fp64 = __syncthreads_or((looked_at && nchunk > 0 && !((s_seen[tid >> 5] >> lane) & 1u)));
+    // squares the rows alone are looked at.  Rows of extreme magnitude, whose scales might not multiply, take the same way.
+    const bool in_fp64 = __syncthreads_or(extreme || (looked_at && nchunk > 0 && !((s_seen[tid >> 5] >> lane) & 1u)));
     if (warp >= 8) return;                                     // (barriers below are met by the other eight)
     double sumsq = 0.0;
     if (in_fp64) {

@@ -148,6 +148,19 @@ def test_set_up_of_a_basis_whose_large_entries_do_not_meet(g):
     assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
 
 
+@pytest.mark.parametrize("ea,eb", [(-510, -505), (-1000, 900), (-1045, 1000), (600, -600), (700, 200), (500, 510)])
+def test_extreme_magnitudes(g, ea, eb):
+    # rows whose scales multiply to a subnormal number or to infinity, rows of subnormal numbers
+    rng = np.random.default_rng(ea + 2000)
+    a, b = rng.standard_normal((140, 100)), rng.uniform(-0.5, 0.5, (100, 150))
+    a[3], b[:, 9] = 0.0, 0.0
+    a, b = np.ldexp(a, ea), np.ldexp(b, eb)
+    want = a.astype(np.longdouble) @ b.astype(np.longdouble)
+    # 1e-16 sqrt(100) of the largest entry, and subnormal sums: half of 2^-1074 a term
+    bound = 4e-15 * np.abs(want).max() + 100 * 2.0 ** -1074
+    assert np.abs(want).max() < 2.0 ** 1023 and np.all(np.abs(product(g, a, b) - want) <= bound)
+
+
 def test_non_finite_entries_reach_their_row_and_column_only(g):
     rng = np.random.default_rng(1)
     a, b = rng.standard_normal((140, 70)), rng.standard_normal((70, 150))
