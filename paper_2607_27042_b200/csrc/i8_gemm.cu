@@ -311,7 +311,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
                const __grid_constant__ CUtensorMap mapA4, const __grid_constant__ CUtensorMap mapB4) {
     extern __shared__ __align__(16) unsigned char i8_raw[];
     __shared__ __align__(8) unsigned long long bar_full[I8_STAGES], bar_empty[I8_STAGES], bar_full2[I8_STAGES2], bar_empty2[I8_STAGES2], bar_acc, bar_drained;
-    __shared__ unsigned s_tmem, s_abort;
+    __shared__ unsigned s_tmem, s_abort, s_all_k;
     __shared__ double s_sum[8];
     __shared__ int s_scale[128];                               // of the tile's columns: high words (the low ones are zero)
     __shared__ unsigned s_seen[8];                             // bit per row (words 0 - 3) and column (4 - 7): it has an entry that is large enough, see below
@@ -368,6 +368,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     };
 
     // of row tid or column tid - 128 of the tile: has it an entry at all, and might its scale not multiply with any other to a normal number
+    const auto tile_top = [&]() { return __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128); };
     bool looked_at = false, extreme = false;
     if (warp == 8) {
         if (lane == 0) {
@@ -461,7 +462,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
         bool ok = true;
         // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
         const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = (tall || !wide) && !p.sumsq_partials;
-        const unsigned top = __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128);
+        const unsigned top = tile_top();
         looked_at = top != 0u && (tid < 128 ? by_rows : by_cols);
         extreme = top != 0u && abs(i8_exponent(top)) > I8_MAX_EXPONENT;
         if (!p.sumsq_partials && p.beta != 0.0 && !bulk_out) {  // the old values are needed at the end: ask for them now
@@ -580,9 +581,15 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     if (warp >= 8) return;                                     // (barriers below are met by the other eight)
     double sumsq = 0.0;
     if (in_fp64) {
+        // a factor of zero does not hide an infinity or a NaN: with one about, no chunk is skipped
+        if (tid == 0) s_all_k = 0u;
+        __syncthreads();
+        if (tile_top() >= 0x7ff00000u) s_all_k = 1u;
+        __syncthreads();
         int k_first = k_lo, k_hi = max(k_lo, min(p.K, k_lo + nchunk * I8_KCHUNK));
         if (p.diag_a) { k_first = min(k_first, m0); k_hi = max(k_hi, min(p.K, m0 + 128)); }     // the chunks count without the diagonals
         if (p.diag_b) { k_first = min(k_first, n0); k_hi = max(k_hi, min(p.K, n0 + 128)); }
+        if (s_all_k) { k_first = 0; k_hi = p.K; }
         double *tile = reinterpret_cast<double *>(stages);
         const bool a_kcontig = p.aj == 1, b_kcontig = p.bi == 1, sq = p.sumsq_partials != nullptr;
         if (a_kcontig) sumsq = b_kcontig ? i8_tile_in_fp64<true, true>(p, bz, m0, n0, k_first, k_hi, tile, sq) : i8_tile_in_fp64<true, false>(p, bz, m0, n0, k_first, k_hi, tile, sq);

@@ -172,3 +172,20 @@ def test_non_finite_entries_reach_their_row_and_column_only(g):
     assert np.all(~np.isfinite(c[7])) and np.all(~np.isfinite(c[:, 139]))
     c[7], c[:, 139], clean[7], clean[:, 139] = 0, 0, 0, 0
     assert np.max(np.abs(c - clean)) < 1e-13
+
+
+def test_infinities_and_nans_go_where_fp64_takes_them(g):
+    rng = np.random.default_rng(2)
+    a, b = rng.standard_normal((300, 400)), rng.standard_normal((400, 260))
+    a[7, 3], a[200, 399], a[130, 64] = np.inf, np.nan, -np.inf
+    b[3, :100], b[64, 5], b[399, 128:] = 0.0, np.inf, 0.0
+    a[:, 320:384] = 0.0                                        # a chunk without an entry in a, but with one in b
+    b[330, 140] = np.inf
+    with np.errstate(invalid="ignore"):
+        want = a @ b
+    got = product(g, a, b)
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+    inf = np.isinf(want)
+    assert np.array_equal(got[inf], want[inf]) and np.isnan(got).any() and inf.any()
+    fine = np.isfinite(want)
+    assert np.max(np.abs(got[fine] - want[fine])) < 1e-12
