@@ -489,9 +489,6 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     };
     // trailing update with the panel of block row K: rows [r0, r1) of the leading part,
     // G[r0:r1, 0:r1] -= P_K,r0:r1^T P_K,0:r1 (lower tiles only when the rows start at 0)
-    auto update = [&](const GemmArgs &t, cudaStream_t s) -> cudaError_t {
-        return (s == stream && t.lower_tiles_only) ? product(t, true) : launch_gemm(t, s);      // rows from 0 on: A and B are the same panel
-    };
     auto trailing = [&](int K, long r0, long r1, cudaStream_t s) -> int {
         const long k0 = (long)K * FB;
         const int bs = (int)((k - k0) < FB ? (k - k0) : FB);
@@ -507,7 +504,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.alpha = -1.0; t.beta = 1.0;
         t.A = G + k0 * ld + r0; t.lda = ld; t.B = G + k0 * ld; t.ldb = ld;
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
-        CK(update(t, s));
+        CK(launch_gemm(t, s));
         return GPTQ2D_OK;
     };
     // the same update with the panels of block rows [K0, K1) at once (contraction over all their rows), on the int8 tensor
