@@ -432,9 +432,10 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     auto product = [&](const GemmArgs &g, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
         if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
-            // few tiles: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the number of tiles)
+            // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
+            // number of tiles)
             const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
-            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && tiles <= 74;
+            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && 2 * tiles <= device_sms();
             return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
         }
         const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);

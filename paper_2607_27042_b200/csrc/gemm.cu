@@ -329,6 +329,12 @@ cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t stream) {
     return launch_t<false, false>(g, stream);
 }
 
+int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    return sms;
+}
+
 // ---------------------------------------------------------------------------------------------
 // One block row of the blocked Cholesky at a time: contraction of 128, output 128 x NT per CTA.  A 128 x 128 tile takes a CTA
 // 17 us of DMMA time whatever the number of tiles, and a block row has k0 / 128 of them (32 at order 4096, for 148 SMs);
@@ -414,7 +420,7 @@ cudaError_t launch_gemm_rank128(int M, int N, double alpha, const double *A, lon
                                 double *C, long ldc, cudaStream_t stream) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     // tiles of 16 columns while they fit the SMs in one wave, of 32 beyond
-    if ((long)(M / 128) * (N / 16) <= 148) return launch_rank128_t<16>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
+    if ((long)(M / 128) * (N / 16) <= device_sms()) return launch_rank128_t<16>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
     return launch_rank128_t<32>(M, N, alpha, A, lda, B, ldb, beta, C, ldc, stream);
 }
 

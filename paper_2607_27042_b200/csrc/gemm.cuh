@@ -27,6 +27,8 @@ struct GemmArgs {
                             // (the tile is then not written); NULL: nobody is told
 };
 
+// SMs of the current device (0 if it cannot be asked).
+int device_sms();
 // Enqueues the GEMM on `stream`.  Returns cudaSuccess or the launch error.
 cudaError_t launch_gemm(const GemmArgs &g, cudaStream_t stream);
 // C = alpha * A^T B + beta * C for a contraction of exactly 128 (A: 128 x M, B: 128 x N, row-major), M a multiple of 128,
