@@ -301,7 +301,7 @@ __device__ __noinline__ double i8_tile_in_fp64(const I8Params &p, int bz, int m0
         for (int b = 0; b < 4; ++b) {
             const double x0 = p.alpha * acc.v[a][b][0], x1 = p.alpha * acc.v[a][b][1];
             if (sumsq) s = fma(x1, x1, fma(x0, x0, s));        // (rows and columns that do not exist are zeros)
-            else *reinterpret_cast<double2 *>(smem + (wm * 64 + a * 8 + g) * I8_OUT_LD + wn * 32 + b * 8 + 2 * t) = double2{x0, x1};
+            else *reinterpret_cast<double2 *>(smem + CI((wm * 64 + a * 8 + g) * I8_OUT_LD + wn * 32 + b * 8 + 2 * t, 128 * I8_OUT_LD - 1, 302)) = double2{x0, x1};
         }
     return s;
 }
@@ -332,7 +332,8 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     const int bz = blockIdx.y;
     const int m0 = tm * 128, n0 = tn * 128;
     // chunks of k in which both operands have an entry (a triangular operand halves them)
-    const int *ra_ = p.rangeA + ((long)bz * (p.rowsA_pad / 128) + tm) * 2, *rb_ = p.rangeB + ((long)bz * (p.rowsB_pad / 128) + tn) * 2;
+    const int *ra_ = p.rangeA + ((long)bz * (p.rowsA_pad / 128) + CI(tm, p.rowsA_pad / 128, 303)) * 2;
+    const int *rb_ = p.rangeB + ((long)bz * (p.rowsB_pad / 128) + CI(tn, p.rowsB_pad / 128, 304)) * 2;
     const int all = (p.K + I8_KCHUNK - 1) / I8_KCHUNK;
     const int c_lo = all - min(ra_[0], rb_[0]), nchunk = max(0, min(ra_[1], rb_[1]) - c_lo);
     const int k_lo = c_lo * I8_KCHUNK;
@@ -557,7 +558,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 if (lane == 0) s_sum[warp] = s;
             } else {
-                double *out = reinterpret_cast<double *>(stages) + row * I8_OUT_LD + c0;
+                double *out = reinterpret_cast<double *>(stages) + CI(row * I8_OUT_LD + c0, 128 * I8_OUT_LD - 63, 301);
 #pragma unroll
                 for (int c = 0; c < 64; ++c) out[c] = p.alpha * (part[c] * (sa * sb(c)));
                 if (bulk_out) fence_proxy_async();             // the copy engine reads what was just written
@@ -648,7 +649,7 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
                         if (diag_a && gi < p.K) x = fma(p.alpha * Ab[gi * (p.ai + p.aj)], Bb[gi * p.bi + gj * p.bj], x);
                         if (diag_b && gj < p.K && !(diag_a && gi == gj))
                             x = fma(p.alpha * Ab[gi * p.ai + gj * p.aj], Bb[gj * (p.bi + p.bj)], x);
-                        Cb[(long)(r4 + i) * p.ldc + lane + 32 * j] = p.beta != 0.0 ? fma(p.beta, old[i][j], x) : x;
+                        Cb[CI((long)(r4 + i) * p.ldc + lane + 32 * j, (p.M - m0 - 1) * p.ldc + p.N - n0, 305)] = p.beta != 0.0 ? fma(p.beta, old[i][j], x) : x;
                     }
         }
     }

@@ -504,9 +504,9 @@ __device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKerne
             const bool lower = j < i, diag = (i & ~1) == j;
             const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
             if (!diag) cp_async16(dst + CI(i * QLD + j, QMAT - 1, 121), src, 16);
-            else cp_async8(dst + i * QLD + j + ((i & 1) ^ 1), (i & 1) ? src : src + 1, 8);
+            else cp_async8(dst + CI(i * QLD + j + ((i & 1) ^ 1), QMAT, 131), (i & 1) ? src : src + 1, 8);
         }
-        if (threadIdx.x < Q) dst[threadIdx.x * (QLD + 1)] = 0.0;
+        if (threadIdx.x < Q) dst[CI(threadIdx.x * (QLD + 1), QMAT, 132)] = 0.0;
         return;
     }
 #pragma unroll

@@ -1,6 +1,6 @@
 """The small parity cases once more under the CHECKED build of the library (libgptq2d_checked.so,
 -DGPTQ2D_CHECKED): every index that feeds a shared- or global-memory access of the tiled sweep, of its
-DMMA tile loop and of the blocked sweep is range-checked on the device, and a violation comes back through
+DMMA tile loop, of the blocked sweep and of the tiles of the int8 products is range-checked on the device, and a violation comes back through
 the status words as GPTQ2D_ERR_CHECK (nothing traps).  compute-sanitizer is not available where this library
 is developed; this is its stand-in.  Runs in a process of its own so that the two builds never share one."""
 import os
@@ -43,6 +43,12 @@ for k, (m, n) in enumerate([(1, 1), (17, 5), (65, 63), (129, 257), (200, 75), (2
     torch.cuda.synchronize()
     g.check_info(info)                                   # raises on GPTQ2D_ERR_CHECK (status 10)
     assert np.array_equal(Z.cpu().numpy().astype(np.int64), ref["Z"]), (m, n)
+    g.gptq2d_internal_test_hook(7, 129)                  # the same in 2 x 2 blocks, where there are two tiles each way
+    Z, E, mm, info = g.gptq2d_round(dX, dL, dU, want_E=True, want_margin=True)
+    torch.cuda.synchronize()
+    g.gptq2d_internal_test_hook(7, 0)
+    g.check_info(info)
+    assert np.array_equal(Z.cpu().numpy().astype(np.int64), ref["Z"]), (m, n)
     for w in (17, 64):
         Zb, _, _, ib = g.gptq2d_round_blocked(dX, dL, dU, w)
         torch.cuda.synchronize()
@@ -57,6 +63,17 @@ for z, c in zip(Zs, cases):
 hX, hL, hU = (c.cpu().pin_memory() for c in cases[6][:3])
 hZ, hinfo = g.gptq2d_round_host(hX, hL, hU)
 assert np.array_equal(hZ.numpy().astype(np.int64), cases[6][3])
+# a product on the int8 tensor cores whose tiles fall back to fp64 (a large entry that meets a zero), ragged, odd pitches
+a = torch.randint(-8, 9, (257, 191), device="cuda").double()
+b = torch.randint(-8, 9, (191, 131), device="cuda").double()
+for outlier in (False, True):
+    if outlier:
+        a[:, 90], b[90] = 2.0 ** 70, 0.0
+    c = torch.ones((257, 131), dtype=torch.float64, device="cuda")
+    info = torch.zeros(4, dtype=torch.int32, device="cuda")
+    g.gptq2d_internal_gemm_split(a, b, c, beta=1.0, info=info)
+    g.check_info(info)
+    assert np.array_equal(c.cpu().numpy(), a.cpu().numpy() @ b.cpu().numpy() + 1.0)
 print("checked build: %%d cases clean" %% len(cases))
 """
 

@@ -161,6 +161,36 @@ def test_extreme_magnitudes(g, ea, eb):
     assert np.abs(want).max() < 2.0 ** 1023 and np.all(np.abs(product(g, a, b) - want) <= bound)
 
 
+def test_the_largest_digit_sums_fit_int32(g):
+    # all digits at an end of their range and of one sign, K at its limit: seven pairs of 128 * 128 * 16384 in one sum
+    K = 16384
+    low = sum(256.0 ** -d for d in range(2, 8))
+    for x, y in ((126 / 256 + 127 * low, 126 / 256 + 127 * low), (-126 / 256 - 128 * low, 126 / 256 + 127 * low),
+                 (-126 / 256 - 128 * low, -126 / 256 - 128 * low)):
+        got = product(g, np.full((130, K), x), np.full((K, 5), y))
+        assert np.max(np.abs(got - K * x * y)) <= 2.0 ** -50 * abs(K * x * y)
+
+
+@pytest.mark.parametrize("k", [1100, 2200])
+def test_set_up_keeps_its_digits_under_channel_scales(g, k):
+    # Channel j scaled by 2^e_j scales L[i, j] by 2^(e_j - e_i), exactly.  Scales over 60 binary orders: without the scaling of the
+    # products of the inverse along k their digits would be spent on them.
+    rng = np.random.default_rng(k)
+    s = rng.standard_normal((2 * k, k))
+    a = np.linalg.cholesky(s.T @ s / (2 * k)).T
+    e = rng.integers(-30, 31, size=k)
+    plain, scaled = (g.gptq2d_factor(torch.from_numpy(np.ascontiguousarray(v)).cuda(), None, n=1) for v in (a, np.ldexp(a, e)))
+    g.check_info(plain[4])
+    g.check_info(scaled[4])
+    L = plain[0].cpu().numpy()
+    # against the oracle's: two fp64 factorisations of a Gram of condition 34 (1e-15 each measured)
+    assert np.max(np.abs(L - O.feedback_factors(a, np.eye(1))[0])) <= 1e-13
+    back = np.ldexp(scaled[0].cpu().numpy(), e[:, None] - e[None, :])
+    assert np.max(np.abs(back - L)) <= 1e-14
+    d = scaled[2].cpu().numpy() / np.ldexp(plain[2].cpu().numpy(), 2 * e)
+    assert np.max(np.abs(d - 1.0)) <= 1e-14
+
+
 def test_non_finite_entries_reach_their_row_and_column_only(g):
     rng = np.random.default_rng(1)
     a, b = rng.standard_normal((140, 70)), rng.standard_normal((70, 150))
