@@ -86,6 +86,9 @@ const char *gptq2d_status_string(int status);
  * dL (m) / dU (n), optional (NULL ok): 1/Lambda_L and 1/Lambda_U, so that
  * ||A (Z-X) B||_F^2 = sum_ij E_ij^2 dL_i dU_j for the local errors E.
  * A or B may be NULL, meaning the identity (L or U is then the identity).
+ * From order 1024 on the Gram, the rank-512 updates and the larger products of the triangular inverse run on the int8 tensor cores
+ * (fixed point as described at gptq2d_round, but a tile is kept from 1/512 on: an error of up to 16 times that of a chain of fp64
+ * additions in single tiles, relative to the largest entry of a row, below the rounding of the factorisation itself).
  * Device error: GPTQ2D_ERR_NOT_SPD when a Gram is numerically not positive definite
  * (A or B singular); L and U are then undefined.
  * Streams: everything is ordered after the work already on `stream`, and `stream` waits for all of it
@@ -110,8 +113,14 @@ int gptq2d_factor(int m, int n,
  *   is implied).  They must stay fixed during the call (Section 6, first caveat).
  * Initialisation (Y <- X, C <- 0; Algorithm 3 lines 4-5) is part of this call.
  * Device errors: NONFINITE, INT_OVERFLOW (Z is int32), DEVICE_TIMEOUT.
- * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 5632 run as four blocks in three kernels, with the
- * products between the blocks on the int8 tensor cores (error-free splitting, at least as exact), all on `stream`.
+ * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 5632 (and do not exceed 65536) run as four blocks in
+ * three kernels, with the products between the blocks on the int8 tensor cores, all on `stream`.  These products write each
+ * row of their operands in fixed point, 56 bits below its largest entry, and compute a 128 x 128 tile in fp64 instead where the
+ * largest entry of a row or column of the result is below 1/32 of what the largest entries of its operand rows
+ * could give: relative to the largest entry of a row of a tile the error stays within that of a chain of fp64 additions
+ * (1e-16 sqrt(K); 1e-17 sqrt(K) and less on normal and log-normal data), but an entry of its own may keep fewer digits than
+ * an fp64 sum would.  Sweeps through gptq2d_round_host are not cut into blocks, so on such sizes an entry within rounding
+ * (1e-13 and less) of a tie may fall differently there.
  * Calls on different streams must use different workspaces.
  */
 size_t gptq2d_round_workspace_bytes(int m, int n, int precision);
@@ -182,7 +191,7 @@ int gptq2d_round_batched(int count, const gptq2d_problem_t *problems,
 /* ---- the set-up of many matrices in one call (the factors that gptq2d_round_batched consumes) ----
  * For every problem the same L, U, dL, dU as gptq2d_factor (Section 3.1; Algorithm 3 lines 1-2).  The
  * problems whose bases both have order <= GPTQ2D_FACTOR_SMALL_MAX are factorised one CTA per side, all
- * in ONE launch, entirely in shared memory (Gram, Cholesky from the last index to the first, triangular
+ * in up to three launches (orders up to 64, 96 and 128), entirely in shared memory (Gram, Cholesky from the last index to the first, triangular
  * inverse, scaling); problems with a larger basis take the blocked route of gptq2d_factor, several of
  * them side by side on streams of the library's own (everything is ordered after the work already on
  * `stream`, and `stream` waits for all of it).
@@ -297,7 +306,8 @@ int gptq2d_round_blocked(int m, int n,
                          void *workspace, size_t workspace_bytes, int *info, void *stream);
 
 /* ---- the objective (Eq. 7): obj = || A (Z - X) B ||_F^2 ----
- * obj: device scalar.  A or B may be NULL (identity).
+ * obj: device scalar.  A or B may be NULL (identity).  Products of 0.9e9 multiplications and more run on the int8 tensor cores
+ * (see gptq2d_round; in the second product, whose entries are only squared and summed, the rows alone are looked at).
  */
 size_t gptq2d_objective_workspace_bytes(int m, int n);
 int gptq2d_objective(int m, int n,
@@ -342,7 +352,7 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
                          double beta, double *C, long ldc, void *stream);
 /* The same product on the int8 tensor cores by error-free splitting, as the set-up and the objective use it for their
  * large products: both operands are written as seven base-256 digit planes in the caller's workspace (256-byte aligned,
- * K <= 16384).  Exposed for tests. */
+ * K <= 16384); tiles that the digits do not suit are computed in fp64.  Exposed for tests. */
 size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K);
 int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha,
                                const double *A, long lda, const double *B, long ldb,
