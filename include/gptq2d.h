@@ -86,9 +86,10 @@ const char *gptq2d_status_string(int status);
  * dL (m) / dU (n), optional (NULL ok): 1/Lambda_L and 1/Lambda_U, so that
  * ||A (Z-X) B||_F^2 = sum_ij E_ij^2 dL_i dU_j for the local errors E.
  * A or B may be NULL, meaning the identity (L or U is then the identity).
- * From order 1024 on the Gram, the rank-512 updates and the larger products of the triangular inverse run on the int8 tensor cores
- * (fixed point as described at gptq2d_round, but a tile is kept from 1/512 on: an error of up to 16 times that of a chain of fp64
- * additions in single tiles, relative to the largest entry of a row, below the rounding of the factorisation itself).
+ * From order 1024 on the Gram, the rank-512 updates and the larger products of the triangular inverse run on the int8 tensor cores,
+ * in fixed point 56 bits below the largest entry of a column of the basis or factor: errors relative to the norms of whole columns, below the
+ * rounding of the factorisation itself.  A tile of the Gram or the inverse whose largest entries are below 1/512 of what its operand
+ * rows could give is computed in fp64.
  * Device error: GPTQ2D_ERR_NOT_SPD when a Gram is numerically not positive definite
  * (A or B singular); L and U are then undefined.
  * Streams: everything is ordered after the work already on `stream`, and `stream` waits for all of it
@@ -114,13 +115,14 @@ int gptq2d_factor(int m, int n,
  * Initialisation (Y <- X, C <- 0; Algorithm 3 lines 4-5) is part of this call.
  * Device errors: NONFINITE, INT_OVERFLOW (Z is int32), DEVICE_TIMEOUT.
  * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 5632 (and do not exceed 65536) run as four blocks in
- * three kernels, with the products between the blocks on the int8 tensor cores, all on `stream`.  These products write each
- * row of their operands in fixed point, 56 bits below its largest entry, and compute a 128 x 128 tile in fp64 instead where the
- * largest entry of a row or column of the result is below 1/32 of what the largest entries of its operand rows
- * could give: relative to the largest entry of a row of a tile the error stays within that of a chain of fp64 additions
- * (1e-16 sqrt(K); 1e-17 sqrt(K) and less on normal and log-normal data), but an entry of its own may keep fewer digits than
- * an fp64 sum would.  Sweeps through gptq2d_round_host are not cut into blocks, so on such sizes an entry within rounding
- * (1e-13 and less) of a tie may fall differently there.
+ * three kernels, with the products between the blocks on the int8 tensor cores, all on `stream`.  These products write the rows
+ * of their operands in fixed point, 56 bits below the largest entry, after a scaling along the contraction by powers of two that
+ * brings the largest entry of a row of the left operand to where the largest term of the row's sums is.  An entry of a product is
+ * then within 2^-57 sqrt(K) of the largest term in its row, less than what a chain of fp64 additions leaves in the worst entry of that row
+ * (1e-16 sqrt(K); measured 1e-17 sqrt(K) and less on normal and log-normal data); an entry far below the others of its row may keep
+ * fewer digits than an fp64 sum would give it.  Rows outside 2^-470 .. 2^470 and non-finite ones are multiplied in fp64.  Sweeps
+ * through gptq2d_round_host are not cut into blocks, so on such sizes an entry within rounding (1e-13 and less) of a tie may
+ * fall differently there.
  * Calls on different streams must use different workspaces.
  */
 size_t gptq2d_round_workspace_bytes(int m, int n, int precision);
@@ -307,7 +309,7 @@ int gptq2d_round_blocked(int m, int n,
 
 /* ---- the objective (Eq. 7): obj = || A (Z - X) B ||_F^2 ----
  * obj: device scalar.  A or B may be NULL (identity).  Products of 0.9e9 multiplications and more run on the int8 tensor cores
- * (see gptq2d_round; in the second product, whose entries are only squared and summed, the rows alone are looked at).
+ * (see gptq2d_round).
  */
 size_t gptq2d_objective_workspace_bytes(int m, int n);
 int gptq2d_objective(int m, int n,
@@ -352,7 +354,7 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
                          double beta, double *C, long ldc, void *stream);
 /* The same product on the int8 tensor cores by error-free splitting, as the set-up and the objective use it for their
  * large products: both operands are written as seven base-256 digit planes in the caller's workspace (256-byte aligned,
- * K <= 16384); tiles that the digits do not suit are computed in fp64.  Exposed for tests. */
+ * K <= 16384), scaled along k by the largest magnitudes of op(B); tiles with rows of extreme magnitude or infinities run in fp64.  Exposed for tests. */
 size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K);
 int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha,
                                const double *A, long lda, const double *B, long ldb,

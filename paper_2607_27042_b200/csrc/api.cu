@@ -599,7 +599,7 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
 
 size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K) {
     if (M < 1 || N < 1 || K < 1) return 0;
-    return i8_planes_bytes(M, K, 1) + i8_planes_bytes(N, K, 1);
+    return i8_planes_bytes(M, K, 1) + i8_planes_bytes(N, K, 1) + i8_inner_bytes(K);
 }
 
 int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha, const double *A, long lda,
@@ -619,8 +619,13 @@ int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, doub
     g.C = C; g.ldc = ldc; g.batch = 1;
     const I8Planes pa = i8_planes_at(workspace, M, K, 1);
     const I8Planes pb = i8_planes_at(static_cast<char *>(workspace) + i8_planes_bytes(M, K, 1), N, K, 1);
-    cudaError_t e = i8_split(pa, A, lda, 0, !transa, stream);
-    if (e == cudaSuccess) e = i8_split(pb, B, ldb, 0, transb != 0, stream);
+    I8Inner inner;
+    double *tops = reinterpret_cast<double *>(static_cast<char *>(workspace) + i8_planes_bytes(M, K, 1) + i8_planes_bytes(N, K, 1));
+    inner.p = tops;
+    cudaError_t e = i8_inner_tops(tops, B, K, N, transb ? 1 : ldb, transb ? ldb : 1, stream);
+    if (e == cudaSuccess) e = i8_split(pa, A, lda, 0, !transa, stream, inner);
+    inner.inverse = true;
+    if (e == cudaSuccess) e = i8_split(pb, B, ldb, 0, transb != 0, stream, inner);
     if (e != cudaSuccess || !launch_gemm_i8(g, pa, pb, info, stream, &e) || e != cudaSuccess) return GPTQ2D_ERR_CUDA;
     return GPTQ2D_OK;
 }

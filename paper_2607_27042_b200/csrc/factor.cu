@@ -531,7 +531,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
         const I8Planes pl = panel_planes(K0, K1);
         cudaError_t e = cudaSuccess;
-        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e, false, false, I8_LEAST_SETUP)) e = launch_gemm(t, s);
+        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
         CK(e);
         return GPTQ2D_OK;
     };

@@ -8,7 +8,7 @@
 // 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
 // entries: 4e-16 against 3e-15 of the fp64 tensor path).  The eight int32 sums (one per p + q) are put together in int64
 // and fp64.  An entry far below the largest of its row keeps fewer than its 53 bits, which matters where the largest one meets
-// a zero; a tile in which it does is recognised by its result and computed in fp64 instead (end of the kernel).
+// a zero: a scaling along k (i8_inner_tops) or a look at the result (end of the kernel) takes care of that.
 //
 // Kernel.  One CTA per 128 x 128 tile of C; tcgen05.mma kind::i8 (M 128, N 128, K 32), accumulators in tensor memory.
 // Four accumulators of 128 columns fill it, so a tile takes two passes over k: p + q = 6 .. 9 (24 products), then
@@ -56,6 +56,33 @@ I8Planes i8_planes_at(void *at, int rows, int K, int batch) {
     return p;
 }
 
+// high word of |x|; not zero unless x is
+__device__ __forceinline__ unsigned i8_magnitude(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
+
+size_t i8_inner_bytes(int K) { return up256((size_t)K * sizeof(double)); }
+
+// one CTA per 2048 entries of a k (memory bound; 134 MB in 25 us)
+__global__ void __launch_bounds__(256) i8_inner_tops_kernel(double *p, const double *src, int N, long sk, long sj) {
+    const double *row = src + (long)blockIdx.x * sk;
+    unsigned m = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const long j = (long)blockIdx.y * 2048 + i * 256 + threadIdx.x;
+        const unsigned h = j < N ? i8_magnitude(__ldg(row + j * sj)) : 0u;
+        m = max(m, h < 0x7ff00000u ? h : 0u);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) i8_raise_top(p, blockIdx.x, m);
+}
+cudaError_t i8_inner_tops(double *p, const double *src, int K, int N, long sk, long sj, cudaStream_t stream) {
+    const cudaError_t e = cudaMemsetAsync(p, 0, (size_t)K * sizeof(double), stream);
+    if (e != cudaSuccess) return e;
+    i8_inner_tops_kernel<<<dim3((unsigned)K, (unsigned)((N + 2047) / 2048)), 256, 0, stream>>>(p, src, N, sk, sj);
+    return cudaGetLastError();
+}
+
 // the power of two that entry k of every row of matrix b is multiplied by (1 if there is none): the binary order of p[k], or its inverse
 __device__ __forceinline__ double i8_inner(const I8Inner &in, int b, int k, int K) {
     if (!in.p || k >= K) return 1.0;
@@ -65,11 +92,6 @@ __device__ __forceinline__ double i8_inner(const I8Inner &in, int b, int k, int 
 }
 
 // ---------------------------------------------------------------------------------------------
-// high word of |x|; not zero unless x is
-__device__ __forceinline__ unsigned i8_magnitude(double x) {
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
-}
-
 // Largest magnitude of every row (its high word: exponent and 20 bits are all that the scale needs; infinities and NaNs
 // come out above every finite number), and the range of k in which 128 rows have any entry.  A 64 x 64 block per CTA,
 // a thread's sixteen loads in flight together.  Memory bound.
@@ -462,9 +484,9 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
         double part[64];
         bool ok = true;
         // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
-        const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = (tall || !wide) && !p.sumsq_partials;
+        const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = tall || !wide;
         const unsigned top = tile_top();
-        looked_at = top != 0u && (tid < 128 ? by_rows : by_cols);
+        looked_at = p.least > 0.0 && top != 0u && (tid < 128 ? by_rows : by_cols);
         extreme = top != 0u && abs(i8_exponent(top)) > I8_MAX_EXPONENT;
         if (!p.sumsq_partials && p.beta != 0.0 && !bulk_out) {  // the old values are needed at the end: ask for them now
             const int rows = out_rows, cols = out_cols;
@@ -529,21 +551,23 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
             // Which rows and columns have a digit sum of at least `least`, for the check below.  (High words compared as fp32 numbers: one
             // instruction with the absolute value.  The diagonal of a Gram, the same rows on both sides, says nothing about its
             // other entries and is left out.)
-            const float least = __int_as_float(__double2hiint(nchunk * I8_KCHUNK > 128 ? p.least * 0x1p72 : p.least * 0x1p71));     // (digit sums count 2^-72)
-            const int at_diagonal = tall && p.topA + bz * p.rowsA_pad + m0 == p.topB + bz * p.rowsB_pad + n0 ? row - c0 : -1;
-            bool row_seen = false;
-            unsigned cols_seen[2] = {0u, 0u};
+            if (p.least > 0.0) {
+                const float least = __int_as_float(__double2hiint(nchunk * I8_KCHUNK > 128 ? p.least * 0x1p72 : p.least * 0x1p71));     // (digit sums count 2^-72)
+                const int at_diagonal = tall && p.topA + bz * p.rowsA_pad + m0 == p.topB + bz * p.rowsB_pad + n0 ? row - c0 : -1;
+                bool row_seen = false;
+                unsigned cols_seen[2] = {0u, 0u};
 #pragma unroll
-            for (int c = 0; c < 64; ++c) {
-                const bool seen = fabsf(__int_as_float(__double2hiint(part[c]))) >= least && c != at_diagonal;
-                row_seen |= seen;
-                if (__any_sync(0xffffffffu, seen)) cols_seen[c >> 5] |= 1u << (c & 31);
-            }
-            const unsigned rows_seen = __ballot_sync(0xffffffffu, row_seen);
-            if (lane == 0) {
-                atomicOr(&s_seen[warp & 3], rows_seen);
-                atomicOr(&s_seen[4 + (c0 >> 5)], cols_seen[0]);
-                atomicOr(&s_seen[5 + (c0 >> 5)], cols_seen[1]);
+                for (int c = 0; c < 64; ++c) {
+                    const bool seen = fabsf(__int_as_float(__double2hiint(part[c]))) >= least && c != at_diagonal;
+                    row_seen |= seen;
+                    if (__any_sync(0xffffffffu, seen)) cols_seen[c >> 5] |= 1u << (c & 31);
+                }
+                const unsigned rows_seen = __ballot_sync(0xffffffffu, row_seen);
+                if (lane == 0) {
+                    atomicOr(&s_seen[warp & 3], rows_seen);
+                    atomicOr(&s_seen[4 + (c0 >> 5)], cols_seen[0]);
+                    atomicOr(&s_seen[5 + (c0 >> 5)], cols_seen[1]);
+                }
             }
             // (the scales are powers of two; where their product might not be one the tile is computed again, see below)
             const double sa = __ldg(p.scaleA + (long)bz * p.rowsA_pad + m0 + row);
@@ -572,12 +596,12 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     if (*(volatile unsigned *)&s_abort) return;                // the tile is not written
     // Do the digits suit the operands?  They cut every entry at the same distance below the largest of its row (of op(A) and of
     // op(B)^T), so where the large entries of a row meet zeros or small ones only, the result has lost digits that a product in fp64
-    // keeps: an outlier channel whose residuals happen to be zero.  The loss shows in the result.  With every row scaled to a largest
+    // keeps.  With p.least the loss is looked for in the result.  With every row scaled to a largest
     // entry of 1/4 to 1/2, the cut moves an entry by 2^-57.8 (|a| + |b|), norms of its two rows, below 2^-59 sqrt(K) for normal or
     // uniform entries.  So a tile is kept if the largest entry of each of its rows and columns is at least p.least, and computed in
-    // fp64 otherwise.  1/32 (I8_LEAST) is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the
-    // largest entry of a row; contractions of 128 and fewer, the corners of triangles, are kept from half of it on.  For a sum of
-    // squares the rows alone are looked at.  Rows of extreme magnitude, whose scales might not multiply, take the same way.
+    // fp64 otherwise: 1/32 is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the largest entry of a
+    // row.  Contractions of 128 and fewer, the corners of triangles, are kept from half of it on.
+    // Rows of extreme magnitude, whose scales might not multiply, and infinities and NaNs always take that way.
     const bool in_fp64 = __syncthreads_or(extreme || (looked_at && nchunk > 0 && !((s_seen[tid >> 5] >> lane) & 1u)));
     if (warp >= 8) return;                                     // (barriers below are met by the other eight)
     double sumsq = 0.0;

@@ -14,7 +14,7 @@ namespace gptq2d {
 
 constexpr int I8_DIGITS = 7;            // 56 bits below the largest entry of a row
 constexpr int I8_KCHUNK = 64;           // k-depth of a pipeline stage; planes are padded to a multiple of it
-constexpr double I8_LEAST = 0x1p-5, I8_LEAST_SETUP = 0x1p-9;
+constexpr double I8_LEAST_SETUP = 0x1p-9;
 constexpr int I8_MAX_K = 16384;         // 7 products of |digits| <= 128 per k: 7 * 2^14 * K < 2^31
 
 // The digit planes of `batch` matrices (rows x K each, K contiguous):
@@ -48,6 +48,15 @@ struct I8Inner {
     long stride = 0;
     bool inverse = false;
 };
+// Largest finite magnitude (its high word, as a double) of every k of a K x N operand, element (k, j) at src[k * sk + j * sj]: a p for
+// I8Inner, with which the other operand is multiplied and this one divided.  A row of op(A) then spends its digits on the k whose
+// terms are large, not on those where its own entry is (an outlier channel that meets zeros): whatever the operands, its result is
+// within 2^-57 sqrt(K) of the largest term |a_ik b_kj| of that row, which an fp64 chain loses as well.  i8_inner_bytes of memory.
+size_t i8_inner_bytes(int K);
+cudaError_t i8_inner_tops(double *p, const double *src, int K, int N, long sk, long sj, cudaStream_t stream);
+// the same for a matrix that is being written: rows' tops by atomicMax, from zeroed memory
+__device__ __forceinline__ void i8_raise_top(double *p, long k, unsigned high) { atomicMax(reinterpret_cast<unsigned *>(p + k) + 1, high); }
+
 // `skip_diagonal`: entries with k == r are left out (launch_gemm_i8 adds what they contribute).
 cudaError_t i8_split(const I8Planes &pl, const double *src, long ld, long stride, bool k_contig, cudaStream_t stream,
                      const I8Inner &inner = I8Inner(), bool skip_diagonal = false);
@@ -59,15 +68,15 @@ bool gemm_i8_pays(long M, long N, long K, long batch);
 // planes of that operand lack its diagonal, whose products are added in fp64 on the way out, from the operands in `g`.
 // A unit or dominant diagonal (triangular factors, their inverses, Cholesky bases) would otherwise set the scale of its
 // row, and the digits of all other entries with it.
-// `least`: a tile with a row or column whose largest entry is below `least` times the product of the largest entries of the two rows
+// `least` > 0: a tile with a row or column whose largest entry is below `least` times the product of the largest entries of the two rows
 // that made it (each rounded up to a power of two that is two to four times as large) is computed in fp64 from the operands in `g`;
-// see i8_gemm.cu.  I8_LEAST: relative to the largest entry of its row or column in the tile no entry is further off than a chain of
-// fp64 additions leaves it.  I8_LEAST_SETUP: up to 16 times that in single tiles, for products that enter a factorisation, whose own
-// rounding is relative to the norms of whole rows; at 1/32 channel scales sent a third of the tiles of the inverse to fp64
-// (1100 x 4100: 4.5 -> 6.1 ms) for factors that came out no closer to 80-bit ones.
+// see i8_gemm.cu.  For products in which both operands may be dominated by single entries (the Gram of a basis, joins of the inverse);
+// not where the result is small by cancellation, which costs fp64 the same digits (the objective of a rounded matrix: 2.2 -> 6.0 ms).
+// I8_LEAST_SETUP: at 1/32, where the cut meets what an fp64 chain loses, channel scales sent a third of the tiles of the inverse
+// to fp64 (1100 x 4100: 4.5 -> 6.1 ms) for factors that came out no closer to 80-bit ones.
 // `info`: the call's status words (a bounded wait that runs out is reported there), may be NULL.
 // False: no tensor map can be had (no driver entry point); nothing was launched.
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
-                    bool diag_a = false, bool diag_b = false, double least = I8_LEAST);
+                    bool diag_a = false, bool diag_b = false, double least = 0.0);
 
 }  // namespace gptq2d

@@ -6,11 +6,22 @@
 
 namespace gptq2d {
 
-__global__ void residual_kernel(int m, int n, const double *X, long ldx, const int *Z, long ldz, double *R, long ldr) {
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long)m * n) return;
-    int i = (int)(idx / n), j = (int)(idx % n);
-    R[(long)i * ldr + j] = (double)Z[(long)i * ldz + j] - X[(long)i * ldx + j];
+// R = Z - X, one CTA per 2048 entries of a row.  `tops` (optional, zeroed): the rows' largest finite magnitudes (i8_inner_tops).
+__global__ void __launch_bounds__(256) residual_kernel(int n, const double *X, long ldx, const int *Z, long ldz, double *R, long ldr, double *tops) {
+    const long i = blockIdx.x;
+    unsigned top = 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const long j = (long)blockIdx.y * 2048 + u * 256 + threadIdx.x;
+        if (j >= n) break;
+        const double r = (double)Z[i * ldz + j] - X[i * ldx + j];
+        R[i * ldr + j] = r;
+        const unsigned h = (unsigned)__double2hiint(r) & 0x7fffffffu;
+        top = max(top, h < 0x7ff00000u ? h : 0u);
+    }
+    if (!tops) return;
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0 && top) i8_raise_top(tops, i, top);
 }
 
 __global__ void __launch_bounds__(1024) sum_partials_kernel(const double *part, int count, double *out) {
@@ -35,7 +46,7 @@ static size_t objective_i8_bytes(int m, int n) {
     size_t b = 0;
     if (gemm_i8_pays(m, n, m, 1)) b = i8_planes_bytes(m, m, 1) + i8_planes_bytes(n, m, 1);
     if (gemm_i8_pays(m, n, n, 1)) b = std::max(b, i8_planes_bytes(m, n, 1) + i8_planes_bytes(n, n, 1));
-    return b;
+    return b ? b + i8_inner_bytes(std::max(m, n)) : 0;         // and the scaling along k
 }
 
 static size_t objective_f64_bytes(int m, int n) {
@@ -60,16 +71,27 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
     double *T1 = R + mat;
     double *part = T1 + mat;
     const int tiles = ((m + 127) / 128) * ((n + 127) / 128);
-    long tot = (long)m * n;
-    residual_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(m, n, X, ldx, Z, ldz, R, ld);
+    double *tops = reinterpret_cast<double *>(static_cast<char *>(ws) + objective_f64_bytes(m, n));
+    const bool first_split = A && planes && gemm_i8_pays(m, n, m, 1);
+    if (first_split) CK(cudaMemsetAsync(tops, 0, (size_t)m * sizeof(double), stream));
+    residual_kernel<<<dim3((unsigned)m, (unsigned)((n + 2047) / 2048)), 256, 0, stream>>>(n, X, ldx, Z, ldz, R, ld, first_split ? tops : nullptr);
     CK(cudaGetLastError());
-    auto product = [&](const GemmArgs &g) -> cudaError_t {
+    // Scaled along k by what the right operand has there: neither operand's digits are spent on a channel in which the other has
+    // nothing, as an outlier channel whose residuals are zero (not by a look at the result: a good rounding makes it small).
+    auto product = [&](const GemmArgs &g, bool tops_known) -> cudaError_t {
         if (!planes || !gemm_i8_pays(g.M, g.N, g.K, 1)) return launch_gemm(g, stream);
-        char *at = static_cast<char *>(ws) + objective_f64_bytes(m, n);
+        if (!tops_known) {
+            const cudaError_t e = i8_inner_tops(tops, g.B, g.K, g.N, g.ldb, 1, stream);
+            if (e != cudaSuccess) return e;
+        }
+        I8Inner inner, undo;
+        inner.p = undo.p = tops;
+        undo.inverse = true;
+        char *at = reinterpret_cast<char *>(tops) + i8_inner_bytes(std::max(m, n));
         const I8Planes pa = i8_planes_at(at, g.M, g.K, 1);
         const I8Planes pb = i8_planes_at(at + i8_planes_bytes(g.M, g.K, 1), g.N, g.K, 1);
-        cudaError_t e = i8_split(pa, g.A, g.lda, 0, true, stream);
-        if (e == cudaSuccess) e = i8_split(pb, g.B, g.ldb, 0, false, stream);
+        cudaError_t e = i8_split(pa, g.A, g.lda, 0, true, stream, inner);
+        if (e == cudaSuccess) e = i8_split(pb, g.B, g.ldb, 0, false, stream, undo);
         if (e != cudaSuccess) return e;
         if (!launch_gemm_i8(g, pa, pb, info, stream, &e)) return launch_gemm(g, stream);
         return e;
@@ -81,7 +103,7 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
         g.M = m; g.N = n; g.K = m;
         g.alpha = 1.0; g.beta = 0.0;
         g.A = A; g.lda = lda; g.B = R; g.ldb = ld; g.C = T1; g.ldc = ld; g.batch = 1;
-        CK(product(g));
+        CK(product(g, true));
         left = T1;
     }
     GemmArgs g{};   // sum of squares of left * B, or of left itself when B is the identity
@@ -91,7 +113,7 @@ int launch_objective(int m, int n, const double *X, long ldx, const int *Z, long
         g.alpha = 1.0; g.beta = 0.0;
         g.A = left; g.lda = ld; g.B = B; g.ldb = ldb; g.C = nullptr; g.ldc = ld; g.batch = 1;
         g.sumsq_partials = part;
-        CK(product(g));
+        CK(product(g, false));
         sum_partials_kernel<<<1, 1024, 0, stream>>>(part, tiles, obj);
     } else {
         // || left ||_F^2 directly

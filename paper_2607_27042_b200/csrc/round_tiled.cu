@@ -1425,8 +1425,13 @@ static int split_product(int M, int N, int K, int kparts, const double *A, long 
         g.M = (M + T - 1) / T * T; g.N = (N + T - 1) / T * T; g.K = kk;       // padding included: the planes hold zeros there
         g.alpha = 1.0; g.beta = k0 ? 1.0 : 0.0;
         g.A = A + k0; g.lda = lda; g.B = B + (long)k0 * ldb; g.ldb = ldb; g.C = C; g.ldc = ldc; g.batch = 1;
-        cudaError_t e = i8_split(pa, g.A, lda, 0, true, stream);
-        if (e == cudaSuccess) e = i8_split(pb, g.B, ldb, 0, false, stream);
+        I8Inner inner;                                         // a channel that E or U has nothing in must not cost L or C its digits
+        double *tops = reinterpret_cast<double *>(static_cast<char *>(at) + i8_planes_bytes(M, kk, 1) + i8_planes_bytes(N, kk, 1));
+        inner.p = tops;
+        cudaError_t e = i8_inner_tops(tops, g.B, kk, N, ldb, 1, stream);
+        if (e == cudaSuccess) e = i8_split(pa, g.A, lda, 0, true, stream, inner);
+        inner.inverse = true;
+        if (e == cudaSuccess) e = i8_split(pb, g.B, ldb, 0, false, stream, inner);
         if (e == cudaSuccess && !launch_gemm_i8(g, pa, pb, info, stream, &e)) return GPTQ2D_ERR_CUDA;
         if (e != cudaSuccess) return GPTQ2D_ERR_CUDA;
     }
@@ -1436,7 +1441,7 @@ static int split_product(int M, int N, int K, int kparts, const double *A, long 
 static int split_kparts(int M, int N, int K, size_t room) {
     for (int p = 1; p <= 8; ++p) {
         const int step = ((K + p - 1) / p + T - 1) / T * T;
-        if (step <= I8_MAX_K && i8_planes_bytes(M, step, 1) + i8_planes_bytes(N, step, 1) <= room) return p;
+        if (step <= I8_MAX_K && i8_planes_bytes(M, step, 1) + i8_planes_bytes(N, step, 1) + i8_inner_bytes(step) <= room) return p;
     }
     return 0;
 }

@@ -62,15 +62,19 @@ def test_rounding_is_within_the_digits_that_are_kept(g, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(128, 128, 64), (5, 3, 2), (127, 129, 65), (257, 130, 191), (300, 100, 1000)])
-def test_integers_are_exact_in_all_layouts_where_tiles_fall_back_to_fp64(g, M, N, K):
-    # a large entry in every row of a that meets zeros only: the digits below it are of no use
+@pytest.mark.parametrize("why", ["fp64", "scaled along k"])
+def test_integers_are_exact_in_all_layouts_where_digits_alone_do_not_do(g, M, N, K, why):
+    # "fp64": magnitudes that send every tile to the fp64 tensor path; "scaled along k": a large entry in every row of a that meets zeros
     rng = np.random.default_rng(M + N + K)
     for transa in (False, True):
         for transb in (False, True):
             a = rng.integers(-8, 9, size=(M, K)).astype(np.float64)
             b = rng.integers(-8, 9, size=(K, N)).astype(np.float64)
             c0 = rng.integers(-8, 9, size=(M, N)).astype(np.float64)
-            a[:, K // 2], b[K // 2] = 2.0 ** 70, 0.0
+            if why == "fp64":
+                a, b = a * 2.0 ** 600, b * 2.0 ** -600
+            else:
+                a[:, K // 2], b[K // 2] = 2.0 ** 70, 0.0
             for pitch in (padded, lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()):
                 for beta in (-1.0, 0.0, 1.0):
                     c = pitch(c0)
@@ -106,17 +110,11 @@ def test_outlier_channels_lose_no_digits(g, K, outlier, other):
         a[:170, k] = 0.0
     want = a.astype(np.longdouble) @ b.astype(np.longdouble)
     error = np.abs(product(g, a, b) - want).astype(np.float64)
-    # Entries are cut 2^-57 below the largest of their row, so an entry of the product is moved by 2^-57.8 (|a| + |b|) with
-    # rows scaled to 1/2 at most (norms below 0.3 sqrt(K)), five times that in the worst of 10^5 entries; a tile is kept if its rows and
-    # columns, scaled in that way, reach 1/32: 3.8e-16 sqrt(K) of the largest entry of the row and of the column.  Other tiles: a
-    # chain of K additions in fp64, whose roundings add up to 0.2 * 2^-53 sqrt(K) (sum of (a b)^2)^(1/2), five times that in the worst.
-    scale = np.abs(a).max(1)[:, None] * np.abs(b).max(0)[None, :]
-    size, fp64 = np.abs(want).astype(np.float64) / scale, 2.0 ** -53 * np.sqrt(K) * np.sqrt((a * a) @ (b * b))
-    for i in range(0, M, 128):
-        for j in range(0, N, 128):
-            at = np.s_[i:i + 128, j:j + 128]
-            kept = 4e-16 * np.sqrt(K) * scale[at] * np.minimum(size[at].max(1)[:, None], size[at].max(0)[None, :])
-            assert np.all(error[at] <= np.maximum(kept, fp64[at])), (i, j)
+    # Entries are cut 2^-57 below the largest of their row, and rows scaled along k have their largest where the largest term of the
+    # row's sums is: what that moves an entry by, 2^-57.8 (|a| + |b|) (five times in the worst of 10^5 entries), is below what a
+    # chain of K fp64 additions leaves in the worst column of the row, about 2^-53 sqrt(K) (sum of (a b)^2)^(1/2).
+    row = np.sqrt((a * a) @ (b * b)).max(1)[:, None]
+    assert np.all(error <= 2.0 ** -53 * np.sqrt(K) * row)
 
 
 @pytest.mark.parametrize("outlier", [1e3, 1e9])
