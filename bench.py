@@ -34,9 +34,10 @@ GRADED_SEED = {0: 0, 1: 0, 2: 0, 3: 0, 4: 1000}
 
 METRIC = "rounded entries/s (m*n / sweep time)"
 UNIT = "entries/s"
-SPLIT_MIN = 5632            # smaller order from which on a resident fp64 sweep runs in 2 x 2 blocks
 FP64_NOMINAL_TFLOPS = 37.2     # 148 SMs x 64 fp64 FMA/clk x 2 x 1.965 GHz; the run also measures the library's own 8192^3 product
 BF16_NOMINAL_TFLOPS = 2250.0
+# fp64-equivalent peak of the int8 products: 34 products of digit planes, one M128 N128 K32 MMA per 64 cycles and SM
+INT8_SPLIT_NOMINAL_TFLOPS = 148 * 2.0 * 128 * 128 * 32 / (34 * 64) * 1.965e9 / 1e12
 FP32_NOMINAL_TFLOPS = 74.4     # 148 SMs x 128 fp32 FMA/clk x 2 x 1.965 GHz
 
 
@@ -139,6 +140,19 @@ def workload(index, seed):
     from paper_2607_27042_b200 import workloads as W
     X, A, B = W.make_config(index, seed=seed)
     return X, A, B, W.CONFIG_NAMES[index]
+
+
+def flops_between_blocks(g, m, n):
+    """Flops of the products between the four blocks of a resident fp64 sweep, 0 if the library sweeps it whole."""
+    size = g.gptq2d_round_workspace_bytes(m, n)
+    g.gptq2d_internal_test_hook(7, 1 << 30)
+    whole = g.gptq2d_round_workspace_bytes(m, n)
+    g.gptq2d_internal_test_hook(7, 0)
+    if size == whole:
+        return 0.0
+    m0, n0 = ((-(-k // 128) + 1) // 2 * 128 for k in (m, n))
+    m1, n1 = m - m0, n - n0
+    return 2.0 * (m1 * n0 * m0 + m0 * n1 * n0 + m1 * n1 * (m0 + n0))
 
 
 def run_cuda(args):
@@ -255,10 +269,14 @@ def run_cuda(args):
     scaled_bf16 = peaks["bf16_tflops"] * FP64_NOMINAL_TFLOPS / BF16_NOMINAL_TFLOPS if peaks["bf16_tflops"] else None
     kernel_name = ("round_tiled_f32_kernel" if args.fp32 else "round_pull_kernel" if args.pull else
                    "round_fused_kernel" if args.fused else "round_tiled_kernel")
-    launches = 1
-    if kernel_name == "round_tiled_kernel" and min(m, n) >= SPLIT_MIN:
-        # four blocks: three sweeps, descriptors, status; four products of two operands each (two splitting kernels an operand)
-        kernel_name, launches = "round_tiled_kernel in 2x2 blocks + i8_gemm_kernel", 3 + 2 + 4 * (2 * 2 + 1)
+    launches, flops_i8 = 1, 0.0
+    if kernel_name == "round_tiled_kernel":
+        flops_i8 = flops_between_blocks(g, m, n)
+    # time that the flops take at the nominal rate of the pipe that they run on
+    peak = flops / ((flops - flops_i8) / FP64_NOMINAL_TFLOPS + flops_i8 / INT8_SPLIT_NOMINAL_TFLOPS)
+    if flops_i8:
+        # four blocks: three sweeps, descriptors, status; four products (scaling along k, two splitting kernels an operand, the product)
+        kernel_name, launches = "round_tiled_kernel in 2x2 blocks + i8_gemm_kernel", 3 + 2 + 4 * (1 + 2 * 2 + 1)
     traffic = None
     tp = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(tp):
@@ -286,13 +304,15 @@ def run_cuda(args):
     del ga, gb, gc
     peak_measured = 2.0 * gn ** 3 / (min(gts) * 1e-3) / 1e12
     roofline = {
-        "bound": "tensor", "achieved": achieved, "peak": FP64_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-        "frac": achieved / FP64_NOMINAL_TFLOPS, "traffic": traffic,
-        "kernel": kernel_name, "kernel_ms": kernel_ms, "flops_per_launch": flops,
-        "peak_note": "fp64 tensor (DMMA) peak: MEASURED_PEAKS.json has no fp64 figure; `peak` is nominal, 148 SMs x 64 "
-                     "FMA/clk x 2 x 1.965 GHz = 37.2; `peak_measured` is what the library's own 8192^3 fp64 product "
-                     "reached in this run (best of 5, CUDA events), a lower bound of the pipe's real peak",
-        "peak_measured": peak_measured, "frac_of_measured": achieved / peak_measured,
+        "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        "frac": achieved / peak, "traffic": traffic,
+        "kernel": kernel_name, "kernel_ms": kernel_ms, "flops_per_launch": flops, "flops_on_int8_pipe": flops_i8,
+        "peak_note": "nominal rates, MEASURED_PEAKS.json has no fp64 figure: fp64 tensor (DMMA) 148 SMs x 64 FMA/clk x 2 x "
+                     "1.965 GHz = 37.2; int8 products (34 products of digit planes each, splitting not counted) %.0f; `peak` is "
+                     "the rate at which this sweep's flops would run with each at its own pipe's rate; `peak_measured` is what the "
+                     "library's own 8192^3 fp64 product (DMMA) reached in this run (best of 5, CUDA events)" % INT8_SPLIT_NOMINAL_TFLOPS,
+        "peak_measured": peak_measured,
+        "frac_of_measured": achieved / (flops / ((flops - flops_i8) / peak_measured + flops_i8 / INT8_SPLIT_NOMINAL_TFLOPS)),
         "frac_of_scaled_measured_bf16": (achieved / scaled_bf16) if scaled_bf16 else None,
         "scaled_measured_bf16_peak": scaled_bf16, "peaks_source": peaks["source"],
         "hbm_compulsory_gbs": (8.0 * m * n + 4.0 * (m * m + n * n) + 4.0 * m * n) / (kernel_ms * 1e-3) / 1e9,
