@@ -18,8 +18,8 @@
 // the tensor pipe; pass 2 three of 64 KB, 1280 cycles each.
 //
 // Bound by the int8 tensor rate: an MMA takes 69 of its 64 cycles in pass 1 (in-kernel clocks).  Measured, splitting
-// included, against the fp64 tensor path (DMMA) of gemm.cu: 8192^3 12.5 ms (88 TFLOP/s) against 31.2, 4096^3 1.63 against
-// 3.91, 2048^3 0.27 against 0.57, rank-512 update of an 8192 x 8192 matrix 1.00 against 2.17.
+// included, against the fp64 tensor path (DMMA) of gemm.cu: 8192^3 13.5 ms (81 TFLOP/s) against 31.1, 4096^3 1.67 against
+// 4.0, 2048^3 0.29 against 0.57, rank-512 update of an 8192 x 8192 matrix 1.07 against 2.17.
 #include <cuda.h>
 #include "common.cuh"
 #include "dmma_tma.cuh"

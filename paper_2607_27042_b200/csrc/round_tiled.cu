@@ -1375,7 +1375,8 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
 // and they are plain matrix products of finished operands, so they run on the int8 tensor cores (i8_gemm.cu) at 80 TFLOP/s
 // where the far parts of the sweep run at 35.  Three sweeps (the middle one takes two blocks in one launch) replace one; each has
 // its own ramp, which is why small matrices are not cut.
-// 8192 x 8192: 38.0 -> 31.7 ms, 7168 x 7168 26.4 -> 23.4, 6144 x 6144 17.5 -> 16.3, 4096 x 4096 6.6 -> 8.0 (not cut).
+// 8192 x 8192: 38.0 -> 31.9 ms, 7168 x 7168 26.4 -> 23.4, 6144 x 6144 17.5 -> 16.3, 5632 x 24576 133 -> 107, 5632 x 5632 13.9 -> 14.0,
+// 4096 x 4096 6.6 -> 8.0 (not cut).
 // Nothing but the workspace is used: a product's digit planes lie in rows of Ebuf whose blocks have not been swept yet, or in
 // rows of Cbuf that nobody reads any more; where they do not fit at once k is cut.
 
