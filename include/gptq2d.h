@@ -339,6 +339,8 @@ int gptq2d_objective(int m, int n,
  *   key 6: how the fp32 mode's contraction gets its operand slabs.  0 (default): bulk tensor copies (TMA) where
  *          the driver offers tensor maps, cp.async otherwise; 1: cp.async always.  Comparison runs and tests.
  *   key 7: smaller order from which on resident fp64 sweeps run in 2 x 2 blocks (0: the default).  Workspace queries follow it.
+ *   key 8: most bits of a cell index in a batched sweep (0: what the number of matrices leaves); matrices with more cells of 32 x 32
+ *          are swept in launches of their own.  Tests.
  * Returns GPTQ2D_OK, or GPTQ2D_ERR_INVALID_ARG for an unknown key.
  */
 int gptq2d_internal_test_hook(int key, long value);

@@ -63,6 +63,8 @@ unsigned *round_tiled_rowdone(void *ws, int m, int n);
 int launch_round_tiled(const TiledParams &p, void *ws, size_t ws_bytes, cudaStream_t stream);
 // from which smaller order on resident matrices are swept in 2 x 2 blocks (tests; 0: the default)
 void round_split_set_min(long order);
+// most bits of a cell index in a batched launch; larger matrices are swept by themselves (tests; 0: the default)
+void round_batched_set_cell_bits(long bits);
 // The sixteen-warp kernel (round_fused.cu): far contractions and quadrant tasks side by side on every SM.
 // Modes: 0 never (default: it measures slower than the eight-warp kernel), 1 problems of at least 8 x 8
 // tiles, 2 whenever the operands allow it (tests, comparison runs).

@@ -10,33 +10,29 @@
 // so they run on the fp64 tensor path (dmma_gemm.cuh); tiles with equal I + J are independent.
 //
 // Scheduling.  Two kinds of work, one persistent cooperatively launched grid (one CTA per SM):
-//  * FAR parts.  Each tile's Cd and Rt contractions over every source tile EXCEPT the two nearest
+//  * FAR parts.  Each tile's Cd and Rt contractions over every source tile EXCEPT the nearest
 //    ones.  Listed wave by wave (I + J ascending) and claimed in that order from one atomic
 //    counter.  A far part waits (bounded) only on tiles three or more waves back, parks its
-//    partial sum in the tile's own workspace region and then announces it to the tile's four
-//    quadrant tasks; it is done long before they need it.  This is >90 % of the flops and runs on
-//    the fp64 tensor path.
-//  * QUADRANT tasks (64 x 64), the critical path.  In the grid of quadrants, (r, c) needs all
-//    quadrants above it in its column and to its left in its row.  What the quadrants of the two
-//    nearest tiles contribute (rows 2 I - 4 .. r - 2 of the grid, columns likewise) it pulls itself
-//    when it starts: up to eight 64^3 DMMA products.  The quadrant right above and the one right to
-//    the left are NOT waited for: every quadrant publishes its 8 x 8 leaves leaf-wave by leaf-wave
-//    (results to the workspace, a progress word per quadrant), and its two neighbours take them in
-//    as they come, running nine leaf-waves behind (block b of a neighbour is final after its
-//    leaf-wave 7 + b).  A task counts arrivals from the two far parts of its tile and from
-//    (r-1, c) and (r, c-1) beginning to sweep; the last arrival puts it on a global ready ring.  A
-//    running quadrant task waits -- bounded -- only on quadrants above it / to its left, which are
-//    running by then (or done).
+//    partial sum in the tile's own workspace region and then announces it to the tile's cells;
+//    it is done long before they need it.  This is most of the flops and runs on the fp64 tensor path.
+//  * CELLS (32 x 32), the critical path.  In the grid of cells, (r, c) needs all cells above it in
+//    its column and to its left in its row.  What the cells of the nearest tiles contribute
+//    it pulls itself when it starts: up to twenty 32^3 DMMA products.  The cell right above and the
+//    one right to the left are NOT waited for: every cell stores its 8 x 8 leaves in the workspace
+//    leaf-wave by leaf-wave, and its two neighbours take them in as they come, running four
+//    leaf-waves and a trip through L2 behind (block b of a neighbour is final after its leaf-wave
+//    3 + b).  A cell counts arrivals from the two far parts of its tile and from (r-1, c) and
+//    (r, c-1) begun; the last arrival puts it on a global ready ring.  A running cell
+//    waits -- bounded -- only on cells above it / to its left, which are running by then (or done).
 // Every CTA serves the ready ring first: at the top of its loop, while a far part waits, and
 // every 64 chunks of a far part (its accumulator stays in registers meanwhile).
 // A far part only ever waits on tiles of earlier waves, whose far parts were claimed earlier and
-// whose quadrant tasks wait on running tasks only, so the earliest unfinished work can always
-// progress.
+// whose cells wait on running tasks only, so the earliest unfinished work can always progress.
 //
-// In-tile sweep.  Inside a quadrant the anti-diagonal sweep runs on 8 x 8 leaves: each leaf of a
-// leaf-wave is swept by one warp (two entries per lane, errors exchanged through a 16-double
-// shared-memory buffer, branch-free pushes against zero-padded coefficient tables), and the
-// leaves' feedback to the remaining 8 x 8 blocks of the quadrant is m8n8k4 DMMA.
+// Inside a cell the anti-diagonal sweep runs on 8 x 8 leaves: each leaf of a leaf-wave is swept by
+// one warp (two entries per lane, errors exchanged through a shared-memory buffer, branch-free
+// pushes against zero-padded coefficient tables), and the leaves' feedback to the remaining
+// 8 x 8 blocks of the cell is m8n8k4 DMMA.
 #include <cstdio>
 #include "common.cuh"
 #include "dmma_gemm.cuh"
@@ -49,7 +45,7 @@
 
 namespace gptq2d {
 
-// optional in-kernel timing of the quadrant task (scratch builds only: -DTILED_STATS): cycles seen by lane 0 of
+// optional in-kernel timing of the cells (scratch builds only: -DTILED_STATS): cycles seen by lane 0 of
 // warp 0, which has a leaf in every leaf-wave, summed per phase over a CTA's tasks
 #ifdef TILED_STATS
 #define TS_MARK(slot)                                            \
@@ -66,17 +62,20 @@ namespace gptq2d {
     } while (0)
 __shared__ long long g_ts[16];
 __shared__ long long g_tlast;
-__shared__ long long g_sched[8];     // 0 quadrant tasks, 1 far main loop, 2 far park/unpark + flag scan, 3 idle, 4 looking for work, 5 far parts
+__shared__ long long g_sched[8];     // 0 cells, 1 far main loop, 2 far park/unpark + flag scan, 3 idle, 4 looking for work, 5 far parts
 #else
 #define TS_MARK(slot)
 #define TS_RESET()
 #endif
 
 constexpr int T = 128;           // tile edge
-constexpr int Q = 64;            // quadrant edge
-constexpr int QLD = 68;          // shared-memory row stride of quadrant matrices (68 mod 16 == 4)
-constexpr int QMAT = Q * QLD;    // doubles per quadrant matrix
-constexpr int TAB_LD = 24;       // row stride of the leaf coefficient tables (22 used)
+constexpr int S = 32;            // cell edge
+constexpr int TC = T / S;        // cells per tile edge
+constexpr int SLD = 36;          // shared-memory row stride of cell matrices (36 mod 16 == 4: conflict-free MMA fragments)
+constexpr int SMAT = S * SLD;    // doubles per cell matrix
+constexpr int TAB_LD = 28;       // row stride of the leaf coefficient tables (22 used; 28 mod 16 == 12: no two lanes of a half-warp meet in a bank)
+constexpr int NLEAF = S / 8;     // leaves per cell edge
+constexpr int PULL_STAGES = 3;   // buffers of the pulls: one multiplied, two on their way
 constexpr int BULK_NSTAGE = 4;
 constexpr int TILED_THREADS = 256;
 
@@ -90,12 +89,14 @@ struct TiledKernelParams {
     double *Euser; long lde;
     double *Ebuf, *Cbuf;
     unsigned *counter, *abort, *q_head, *q_tail, *tiles_done;
-    unsigned *q_slots;           // [qmask + 1] ready quadrant tasks
+    int *q_avail;                // ready cells that nobody has claimed yet
+    unsigned *q_slots;           // [qmask + 1] ready cells
     unsigned qmask;              // ring size - 1 (power of two)
+    int cell_bits;               // batched launches: bits of the cell index in a ring entry, the matrix index is above them
     unsigned *flagS;             // [ntm*ntn] tile swept
-    unsigned *quad_done;         // [ntm*ntn] swept quadrants of the tile (4 -> tile flag)
-    unsigned *qdep;              // [ntm*ntn][4] arrivals each quadrant task has received
-    unsigned *qprog;             // [ntm*ntn][4] leaf-waves each quadrant has published (15: complete)
+    unsigned *cells_done;        // [ntm*ntn] swept cells of the tile (all of them -> tile flag)
+    unsigned *cdep;              // [ntm*ntn][4] arrivals of the tile's cells, one byte each: word = row of cells, byte = column
+    unsigned char *cprog;        // [ntm*ntn][16] 1: the cell has taken its far sums, its results appear in their place; 2: all of them are there
     unsigned *rowdone;           // [ntm] tiles of each tile row that are swept (the host entry copies Z back row by row)
     double *max_abs_e;
     int *info;
@@ -103,6 +104,7 @@ struct TiledKernelParams {
     // a block of a larger matrix (launch_round_split): where it begins there (status words), and which far sums its regions of
     // Cbuf (bit 0) and Ebuf (bit 1) hold already when the launch begins: those of the blocks above and to the left
     int row_off, col_off, preloaded;
+    int near;                    // tiles above and to the left of its own from which a cell pulls itself; the far parts take the rest
     int report_index;            // matrix index in the status words
     // batched launches only (one descriptor per matrix in device memory; the kernel argument then
     // carries the shared scheduler words, the totals in ntasks / ntiles_total, and these tables)
@@ -118,564 +120,660 @@ struct TiledKernelParams {
 };
 static_assert(sizeof(TiledKernelParams) % 8 == 0, "descriptors are copied as 8-byte words");
 
-constexpr size_t SWEEP_SMEM = (size_t)(5 * QMAT + 2 * Q * TAB_LD + 2 * (64 * 12) + 2 * (8 * QLD)) * sizeof(double);
+// shared memory of a cell task, in doubles: W, C, both diagonal factor blocks, the factor blocks towards the cell above and the
+// cell to the left, the coefficient tables, the exchange buffers of the four sweeping warps, the integers, and the ring of the pulls
+constexpr int XCH_BUF = 160;     // one step's exchange: [0, 32) e by lane, [48, 80) C by lane, zeros around it (reached with zero coefficients)
+constexpr int CELL_TABS = 5 * SMAT, CELL_XCH = CELL_TABS + 2 * S * TAB_LD, CELL_Z = CELL_XCH + NLEAF * 2 * XCH_BUF, CELL_PULL = CELL_Z + S * S / 2;
+constexpr size_t SWEEP_SMEM = (size_t)(CELL_PULL + PULL_STAGES * 4 * SMAT) * sizeof(double);
 constexpr size_t BULK_SMEM = (size_t)BULK_NSTAGE * SlabLayout<true, false>::STAGE_DOUBLES * sizeof(double);
 constexpr size_t TILED_SMEM = SWEEP_SMEM > BULK_SMEM ? SWEEP_SMEM : BULK_SMEM;
 
 // ---------------------------------------------------------------------------------------------
-// workspace / factors -> shared memory.  The *_async loaders only issue cp.async copies; the caller
-// commits, waits and barriers once for all operands of a quadrant.
-__device__ __forceinline__ void load_quadrant_async(double *dst, const double *src, long ld) {
-    // dense 64 x 64 from a padded workspace buffer (always in range, 16-byte aligned); L2 only
+// factors -> shared memory.  The *_async loaders only issue cp.async copies; the caller commits and waits.
+// 32 x 32 block of a user matrix (k x k, leading dimension ld) whose top-left element is (r0, c0), 8 bytes at a time (odd pitches or
+// pointers); what is out of range becomes zero.
+__device__ __forceinline__ void load_factor_async(double *dst, const double *M, long ld, int k, int r0, int c0) {
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
-        int c = threadIdx.x + it * TILED_THREADS;
-        cp_async16(dst + CI((c >> 5) * QLD + (c & 31) * 2, QMAT - 1, 101), src + (long)(c >> 5) * ld + (c & 31) * 2, 16);
+    for (int it = 0; it < 4; ++it) {
+        const int c = threadIdx.x + it * TILED_THREADS, i = c >> 5, j = c & 31, gr = r0 + i, gc = c0 + j;
+        const bool take = gr < k && gc < k;
+        cp_async8(dst + CI(i * SLD + j, SMAT, 102), take ? M + CI((long)gr * ld + gc, (long)(k - 1) * ld + k, 103) : M, take ? 8 : 0);
     }
 }
-// 64 x 64 block of a user matrix (k x k, leading dimension ld) whose top-left element is
-// (r0, c0); mode 0: everything in range, 1: strictly lower part only, 2: strictly upper only
-// (relative to the matrix diagonal).  Out-of-range and masked elements become zero.
-__device__ __forceinline__ void load_factor_block_async(double *dst, const double *M, long ld, int k, int r0, int c0,
-                                                        int mode) {
+// 32 x 32 diagonal blocks of both factors into one shared-memory matrix: below the diagonal
+// L[r0 + i][r0 + k], above it U[c0 + k][c0 + j], zeros on it and outside the matrices.
+__device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKernelParams &p, int r0, int c0) {
+    if (p.l_al16 && p.u_al16 && r0 + S <= p.m && c0 + S <= p.n) {      // whole blocks in 16-byte pieces
 #pragma unroll
-    for (int it = 0; it < 16; ++it) {
-        int c = threadIdx.x + it * TILED_THREADS;
-        int r = c >> 6, cc = c & 63;
-        int gr = r0 + r, gc = c0 + cc;
-        bool take = gr < k && gc < k;
-        if (mode == 1) take = take && gc < gr;
-        if (mode == 2) take = take && gc > gr;
-        cp_async8(dst + CI(r * QLD + cc, QMAT, 102), take ? M + CI((long)gr * ld + gc, (long)(k - 1) * ld + k, 103) : M, take ? 8 : 0);
+        for (int it = 0; it < 2; ++it) {
+            const int c = threadIdx.x + it * TILED_THREADS, i = c >> 4, j = (c & 15) * 2;
+            // the piece that holds the diagonal: its off-diagonal entry only (from L if i is odd, from U if it is even)
+            const bool lower = j < i, diag = (i & ~1) == j;
+            const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
+            if (!diag) cp_async16(dst + CI(i * SLD + j, SMAT - 1, 121), src, 16);
+            else cp_async8(dst + CI(i * SLD + j + ((i & 1) ^ 1), SMAT, 131), (i & 1) ? src : src + 1, 8);
+        }
+        if (threadIdx.x < S) dst[CI(threadIdx.x * (SLD + 1), SMAT, 132)] = 0.0;
+        return;
     }
-}
-
-// Whole 64 x 64 block (no triangle mask) with 16-byte copies; needs M 16-byte aligned, ld and c0 even.
-__device__ __forceinline__ void load_full_block_async16(double *dst, const double *M, long ld, int k, int r0, int c0) {
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
-        int c = threadIdx.x + it * TILED_THREADS;
-        int r = c >> 5, cc = (c & 31) * 2;
-        int gr = r0 + r, gc = c0 + cc;
-        int nv = (gr < k) ? min(2, max(0, k - gc)) : 0;
-        cp_async16(dst + CI(r * QLD + cc, QMAT - 1, 104), nv ? M + CI((long)gr * ld + gc, (long)(k - 1) * ld + k - nv + 1, 105) : M, nv * 8);
+    for (int it = 0; it < 4; ++it) {
+        const int c = threadIdx.x + it * TILED_THREADS, i = c >> 5, j = c & 31;
+        const bool lower = j < i, upper = j > i;
+        const bool take = lower ? (r0 + i < p.m) : (upper && c0 + j < p.n);     // r0 + j < r0 + i, c0 + i < c0 + j
+        const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
+        cp_async8(dst + CI(i * SLD + j, SMAT, 121), take ? src : p.L, take ? 8 : 0);
     }
 }
 
-// 64 x 64 x 64 DMMA product on quadrant operands in shared memory: each warp owns a 16 x 32 piece
-// (2 x 4 fragments); element rows wr*16 + a*8 + (lane>>2), cols wc*32 + b*8 + (lane&3)*2 + {0,1}.
-struct QAcc {
-    double v[2][4][2];
-    __device__ __forceinline__ void zero() {
+// a copy that a warp makes or not, without a branch
+__device__ __forceinline__ void cp_async16_if(unsigned dst, const double *src, int src_bytes, bool on) {
+    asm volatile("{.reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q cp.async.cg.shared.global [%0], [%1], 16, %2;\n}" ::"r"(dst), "l"(src), "r"(src_bytes),
+                 "r"((unsigned)on) : "memory");
+}
+// acc += As (16 rows at wr, [m][k]) * Bs (16 columns at wc, [k][n]): one warp's quarter of a 32 x 32 x 32 product; element rows
+// wr + a*8 + (lane>>2), columns wc + b*8 + (lane&3)*2 + {0,1}.  copy(q), q = 0..7, asks for an eighth of a later step's operands,
+// between the MMAs.
+template <class Copy>
+__device__ __forceinline__ void quarter_mma(double (&acc)[2][2][2], bool mul, const double *As, const double *Bs, int wr, int wc, int g, int t, Copy copy) {
+    if (!mul) {
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) v[a][b][0] = v[a][b][1] = 0.0;
+        for (int q = 0; q < 8; ++q) copy(q);
+        return;
     }
-};
-// acc += As (64 x 64, [m][k]) * Bs (64 x 64, [k][n])
-__device__ __forceinline__ void quad_mma(QAcc &acc, const double *As, const double *Bs) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int wr = warp >> 1, wc = warp & 1;
-#pragma unroll 4
-    for (int kk = 0; kk < Q; kk += 4) {
-        double af[2], bf[4];
+    double af[2][2], bf[2][2];                              // of this and of the next k4-step: a copy ahead of them would hold up their loads
+    auto load = [&](int kk, int w) {
 #pragma unroll
-        for (int a = 0; a < 2; ++a) af[a] = As[CI((wr * 16 + a * 8 + g) * QLD + kk + t, QMAT, 106)];
+        for (int a = 0; a < 2; ++a) af[w][a] = As[CI((wr + a * 8 + g) * SLD + kk + t, SMAT, 135)];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) bf[b] = Bs[CI((kk + t) * QLD + wc * 32 + b * 8 + g, QMAT, 107)];
+        for (int b = 0; b < 2; ++b) bf[w][b] = Bs[CI((kk + t) * SLD + wc + b * 8 + g, SMAT, 136)];
+    };
+    load(0, 0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        if (q < 7) load(4 * q + 4, (q + 1) & 1);
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) dmma_m8n8k4(acc.v[a][b][0], acc.v[a][b][1], af[a], bf[b]);
+            for (int b = 0; b < 2; ++b) dmma_m8n8k4(acc[a][b][0], acc[a][b][1], af[q & 1][a], bf[q & 1][b]);
+        copy(q);
     }
 }
-// Leaf (a, b) of the quadrant collects, right before it is swept, all the feedback it is due from
-// the leaves already swept (left-looking): the downward pushes of the leaves above it through L,
-//     P = sum_{a' < a} L[a, a'] E[a', b]       (folded into C and pushed into Y)
-// and the rightward pushes of the leaves to its left through U,
-//     R = sum_{b' < b} C[a, b'] U[b', b]       (pushed into Y),
-// as m8n8k4 products on the warp's fragments (two independent accumulator chains each), then
-// Y += P + R, C += P in place.  E of a swept leaf lives where its Y was, its final C where its C
-// was.  Warp-uniform; all leaves of one leaf-wave do the same amount of work (a + b = lw).
-__device__ __forceinline__ void leaf_pull(double *Ys, double *Cs, const double *Ls, const double *Us, int a, int b,
-                                          int g, int t) {
+// Leaf (a, b) of the cell collects the feedback of leaves of its cell swept before it (left-looking): the downward pushes of leaves
+// a' < a1 above it through L, C += sum L[a, a'] E[a', b], and the rightward pushes of leaves b' < b1 to its left through U,
+// W += sum C[a, b'] U[b', b], as m8n8k4 products on the warp's fragments (two independent accumulator chains each).
+// E of a swept leaf lives where its W was, its final C where its C was.
+__device__ __forceinline__ void leaf_pull(double *Ws, double *Cs, const double *LU, int a, int b, int a1, int b1, int g, int t) {
+    double2 *wp = reinterpret_cast<double2 *>(Ws + CI((a * 8 + g) * SLD + b * 8 + t * 2, SMAT - 1, 108));
+    double2 *cp = reinterpret_cast<double2 *>(Cs + CI((a * 8 + g) * SLD + b * 8 + t * 2, SMAT - 1, 109));
     double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0, r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
-    const double *La = Ls + (a * 8 + g) * QLD + t;           // A fragments: row a*8+g, k = t (+4)
-    const double *Eb = Ys + t * QLD + b * 8 + g;             // B fragments: k = t (+4), col b*8+g
-#pragma unroll 2
-    for (int ap = 0; ap < a; ++ap) {
-        dmma_m8n8k4(p0, p1, La[ap * 8], Eb[(ap * 8) * QLD]);
-        dmma_m8n8k4(p2, p3, La[ap * 8 + 4], Eb[(ap * 8 + 4) * QLD]);
+    const double *La = LU + (a * 8 + g) * SLD + t, *Eb = Ws + t * SLD + b * 8 + g;          // A: row a*8+g, k = t (+4); B: k = t (+4), col b*8+g
+    const double *Ca = Cs + (a * 8 + g) * SLD + t, *Ub = LU + t * SLD + b * 8 + g;
+#pragma unroll 1
+    for (int ap = 0; ap < a1; ++ap) {
+        dmma_m8n8k4(p0, p1, La[ap * 8], Eb[(ap * 8) * SLD]);
+        dmma_m8n8k4(p2, p3, La[ap * 8 + 4], Eb[(ap * 8 + 4) * SLD]);
     }
-    const double *Ca = Cs + (a * 8 + g) * QLD + t;
-    const double *Ub = Us + t * QLD + b * 8 + g;
-#pragma unroll 2
-    for (int bp = 0; bp < b; ++bp) {
-        dmma_m8n8k4(r0, r1, Ca[bp * 8], Ub[(bp * 8) * QLD]);
-        dmma_m8n8k4(r2, r3, Ca[bp * 8 + 4], Ub[(bp * 8 + 4) * QLD]);
+#pragma unroll 1
+    for (int bp = 0; bp < b1; ++bp) {
+        dmma_m8n8k4(r0, r1, Ca[bp * 8], Ub[(bp * 8) * SLD]);
+        dmma_m8n8k4(r2, r3, Ca[bp * 8 + 4], Ub[(bp * 8 + 4) * SLD]);
     }
-    p0 += p2; p1 += p3;
-    double *yp = Ys + (a * 8 + g) * QLD + b * 8 + t * 2;
-    double *cp = Cs + (a * 8 + g) * QLD + b * 8 + t * 2;
-    double2 yv = *reinterpret_cast<double2 *>(yp), cv = *reinterpret_cast<double2 *>(cp);
-    cv.x += p0; cv.y += p1;
-    yv.x += p0 + (r0 + r2); yv.y += p1 + (r1 + r3);
-    *reinterpret_cast<double2 *>(yp) = yv;
-    *reinterpret_cast<double2 *>(cp) = cv;
+    if (a1 > 0) { double2 v = *cp; v.x += p0 + p2; v.y += p1 + p3; *cp = v; }
+    if (b1 > 0) { double2 w = *wp; w.x += r0 + r2; w.y += r1 + r3; *wp = w; }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Streaming between neighbouring quadrants.  A quadrant does not wait for the quadrant above it
-// (and the one to its left) to finish: column block b of the E above is final once that quadrant
-// has swept its leaf-waves 0 .. 7+b, row block a of the C to the left once leaf-waves 0 .. 7+a are
-// done, and leaf-wave lw of this quadrant needs exactly blocks 0 .. lw of both.  Every quadrant
-// therefore publishes its leaves wave by wave (E, C to the workspace, a progress word per
-// quadrant), and its two neighbours run nine leaf-waves behind it.
-constexpr int STG_E_LD = 12;                 // staged 64 x 8 column block of E, [k][n], 12 = 8 + 4 pad
-constexpr int STG_E = Q * STG_E_LD;          // doubles per staged E block
-constexpr int STG_C = 8 * QLD;               // staged 8 x 64 row block of C, [m][k]
+// Streaming between neighbouring cells.  A cell does not wait for the cell above it (and the one to its left) to finish: column
+// block b of the E above is final once that cell has swept its leaf-waves 0 .. 3+b, row block a of the C to the left once
+// leaf-waves 0 .. 3+a are done, and leaf-wave lw of this cell needs exactly blocks 0 .. lw of both.  The data are their own
+// flags: a task overwrites its regions of Ebuf and Cbuf with STREAM_EMPTY (a NaN) as soon as it has the far sums that they
+// held, says so once (cprog), and from then on its neighbours poll the entries themselves.  An entry is one 8-byte word that
+// is written once from then on, so nothing has to be ordered behind it; a flag with a fence before it and a load after it cost
+// two more trips to L2 on the critical path.  A result that happens to have this very bit pattern is stored with its last bit flipped
+// (a NaN either way).
+constexpr unsigned long long STREAM_EMPTY = 0xfff94d5a7c3e2b61ull;
+__device__ __forceinline__ double stream_value(double v) {
+    return __double_as_longlong(v) == (long long)STREAM_EMPTY ? __longlong_as_double((long long)(STREAM_EMPTY ^ 1)) : v;
+}
+__device__ __forceinline__ double ld_relaxed_f64(const double *p) {
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned ld_acquire_u8(const unsigned char *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u8 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_u8(unsigned char *p, unsigned v) {
+    asm volatile("st.release.gpu.global.u8 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;\n" ::: "memory"); }
 
-struct Stream {
-    const unsigned *prog_above, *prog_left;  // progress words of the two neighbours (NULL: none)
-    unsigned *prog_self;
-    const double *e_above;                   // Ebuf at (first row of the quadrant above, first column of this one)
-    const double *c_left;                    // Cbuf at (first row of this quadrant, first column of the one to the left)
-    int I, J, q;
-};
-
-// Called by one warp: lane 0 polls both neighbours' progress words until each has reached `need`
-// (bounded; on expiry the launch is aborted and the caller carries on with whatever is there).
-__device__ __forceinline__ void await_progress(const TiledKernelParams &p, const unsigned *wa, const unsigned *wl,
-                                               unsigned need) {
-    if ((threadIdx.x & 31) == 0) {
-        unsigned long long it = 0;
-        for (;;) {
-            const unsigned va = wa ? ld_acquire_u32(wa) : need, vl = wl ? ld_acquire_u32(wl) : need;
-            if (va >= need && vl >= need) break;
-            if (++it > p.spin_limit || ld_relaxed_u32(p.abort) != 0u) {
-                report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -8, (int)need, (int)blockIdx.x);
-                atomicExch(p.abort, 1u);
-                break;
-            }
-            __nanosleep(40);
-        }
+// One more poll of a bounded wait; true: give up (the launch is aborted and the caller carries on with whatever is there).
+__device__ __forceinline__ bool wait_expired(const TiledKernelParams &p, unsigned long long &it, int code, int what) {
+    if (++it > p.spin_limit || ((it & 15) == 0 && ld_relaxed_u32(p.abort) != 0u)) {
+        report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, code, what, (int)blockIdx.x);
+        atomicExch(p.abort, 1u);
+        return true;
     }
-    __syncwarp();
+    return false;
+}
+// Fragments v[0..7] of a neighbour's block, entry i at src + i * stride: all asked for at once, those that had not been written
+// are asked for again.
+__device__ __forceinline__ void stream_ask(double (&v)[8], const double *src, long stride) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = ld_relaxed_f64(src + i * stride);
+}
+__device__ __forceinline__ void stream_await(const TiledKernelParams &p, double &v0, double &v1, const double *src, long stride) {
+    unsigned long long it = 0;
+    for (;;) {
+        const bool here = __double_as_longlong(v0) != (long long)STREAM_EMPTY && __double_as_longlong(v1) != (long long)STREAM_EMPTY;
+        if (__all_sync(0xffffffffu, here)) return;
+        bool over = false;
+        if ((threadIdx.x & 31) == 0) over = wait_expired(p, it, -8, 1);
+        if (__any_sync(0xffffffffu, over)) return;
+        v0 = ld_relaxed_f64(src); v1 = ld_relaxed_f64(src + stride);
+    }
 }
 
-__device__ __forceinline__ void quadrant_arrive(const TiledKernelParams &p, int I, int J, int q);
+// ---------------------------------------------------------------------------------------------
+// Ready cells.
+// Global ring of ready cells (size a power of two).  It cannot overflow: a cell depends, directly or through others, on the cell
+// above it and on the one to its left, so the cells of one matrix that are ready at the same time lie on an anti-chain of its
+// 4 ntm x 4 ntn grid, at most 4 min(ntm, ntn) of them (E and C of 1024 x 1024 tiles would be 275 GB); each enters the ring once.
+// A batched launch sizes its ring from the sum over its matrices.
+constexpr unsigned QCAP = 4096;
 
-// Algorithm 3 on one 64 x 64 quadrant held in shared memory.
-//   Ys: in  Y (corrected values from everything but the two streaming neighbours); out E
-//   Cs: in  C likewise; out final C = L E rows of the quadrant
-//   LU: the 64 x 64 diagonal blocks of both factors in one matrix: strictly lower part from L,
-//       strictly upper part from U (the sweep never reads the other triangles)
-//   Lfa: L[rows of this quadrant, rows of the quadrant above];  Ufl: U[columns of the quadrant to
-//        the left, columns of this quadrant]
-//   stg: staging for the streamed blocks, two of each kind
-// row0/col0: global coordinates of the quadrant.
-//
-// Leaf-wave lw (leaves (a, lw - a), one per warp).  For lw <= 7, all warps first add what block lw
-// of the neighbours feeds into this quadrant (pull phase).  Then every leaf pulls the feedback of
-// the leaves swept before it (leaf_pull), runs the 15 anti-diagonal steps on its 8 x 8 entries and
-// stores its results, while warp 7 fetches block lw + 1 and warp 6 publishes the previous waves.
-__device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const double *LU, const double *Lfa,
-                                               const double *Ufl, double *stg, double *tabL, double *tabU, int row0,
-                                               int col0, const Stream &sm, const TiledKernelParams &p,
-                                               double &max_abs_e) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = lane >> 2, t = lane & 3;
-    __shared__ double xch[8 * 2 * 16];
-    __shared__ unsigned long long s_badkey;
-    const double *Ls = LU, *Us = LU;
-    // coefficient tables of the 8 diagonal leaves (see phase A); also clears the exchange buffers
-    for (int c = tid; c < Q * TAB_LD; c += blockDim.x) {
-        const int r = c / TAB_LD, k = c - r * TAB_LD;       // r: row (L) or column (U) inside the quadrant
-        const int src = k - 7, blk = r & ~7, in = r & 7;    // source index inside the leaf
-        const bool ok = src >= 0 && src < in;
-        tabL[c] = ok ? Ls[CI(r * QLD + blk + src, QMAT, 112)] : 0.0;
-        tabU[c] = ok ? Us[CI((blk + src) * QLD + r, QMAT, 113)] : 0.0;
-    }
-    if (tid < 8 * 2 * 16) xch[tid] = 0.0;
-    if (tid == 0) s_badkey = ~0ull;
-    unsigned long long badkey = ~0ull;
-    const bool fresh = sm.prog_above != nullptr || sm.prog_left != nullptr;
-    double *stgE = stg, *stgC = stg + 2 * STG_E;
-    // Warp 7 (idle in every leaf-wave but the eighth) is the streaming warp: it fetches the next block of
-    // the neighbours' results while the other warps sweep their leaves: 8 + 8 pieces of 16 bytes per lane.
-    auto fetch_block = [&](int blk) {
-        await_progress(p, sm.prog_above, sm.prog_left, (unsigned)(blk + 8));
-        if (sm.prog_above) {        // E above: 64 rows x 8 columns [8 blk, 8 blk + 8)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int piece = lane + 32 * i, r = piece >> 2, c2 = (piece & 3) * 2;
-                cp_async16(stgE + CI((blk & 1) * STG_E + r * STG_E_LD + c2, 2 * STG_E - 1, 108),
-                           p.Ebuf + CI((sm.e_above - p.Ebuf) + (long)r * p.np + blk * 8 + c2, (long)p.ntm * T * p.np - 1, 109), 16);
-            }
+// Multi-producer / multi-consumer ring in global memory; slot value 0 = empty.  *q_avail counts the entries that nobody has claimed:
+// a consumer takes one off it and puts it back if there was none, so that every step is a single atomic addition that
+// cannot fail.  (Claiming by compare-and-swap on the head let one consumer in 600 cycles through, however many there were, and sent
+// the others round again: with it, 64 matrices of 256 x 256 and 256 x 512 took 1850 us instead of 945.)
+// Pushing is in two parts, so that a caller can do something else during the trip to L2 of the first.
+__device__ __forceinline__ unsigned push_ticket(const TiledKernelParams &p) { return atomicAdd(p.q_tail, 1u); }
+__device__ __forceinline__ void push_entry(const TiledKernelParams &p, unsigned ticket, int r, int c) {
+    const unsigned cell = (unsigned)r * (unsigned)(TC * p.ntn) + (unsigned)c;
+    const unsigned entry = p.batch_index >= 0 ? ((unsigned)p.batch_index << p.cell_bits) | cell : cell;
+    fence_acq_rel();                                        // whoever takes the entry sees what all arrivals at the cell stand for
+    st_release_u32(p.q_slots + CI(ticket & p.qmask, (long)p.qmask + 1, 127), entry | 0x80000000u);
+    atomicAdd(p.q_avail, 1);
+}
+// One thread, after a look at *q_avail (many idle CTAs would otherwise keep taking one off and putting it back).  Returns 0 if there was
+// nothing after all (or on abort), else the entry (bit 31 set).
+__device__ __forceinline__ unsigned ready_pop(const TiledKernelParams &p) {
+    if (atomicAdd(p.q_avail, -1) <= 0) { atomicAdd(p.q_avail, 1); return 0u; }
+    const unsigned h = atomicAdd(p.q_head, 1u);
+    unsigned *slot = p.q_slots + (h & p.qmask);
+    unsigned long long spins = 0;
+    unsigned e;
+    while ((e = ld_acquire_u32(slot)) == 0u) {              // counted by a later ticket's producer; this one has not written yet
+        if (++spins > p.spin_limit || ld_relaxed_u32(p.abort) != 0u) {
+            report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -3, (int)h, (int)blockIdx.x);
+            atomicExch(p.abort, 1u);
+            return 0u;
         }
-        if (sm.prog_left) {         // C to the left: rows [8 blk, 8 blk + 8) x 64 columns
+    }
+    *slot = 0u;
+    return e;
+}
+
+// Arrivals that cell (r, c) waits for: the two far parts of its tile and the cells (r - 1, c) and (r, c - 1) begun.
+__device__ __forceinline__ unsigned cell_needed(int r, int c) { return 2u + (r >= 1 ? 1u : 0u) + (c >= 1 ? 1u : 0u); }
+// A cell that lies wholly outside the matrix (ragged last tile row / column) is never a task: arrivals at it are dropped here,
+// its region of the workspace keeps the zeros the far parts parked there, and nothing inside the matrix depends on it.
+__device__ __forceinline__ bool cell_exists(const TiledKernelParams &p, int r, int c) { return r * S < p.m && c * S < p.n; }
+__device__ __forceinline__ unsigned *cell_dep(const TiledKernelParams &p, int r, int I, int J) {
+    return p.cdep + CI(((long)I * p.ntn + J) * TC + r % TC, (long)TC * p.ntm * p.ntn, 125);
+}
+// A neighbour is in its task.  Nothing is ordered behind this: what the cell reads of that neighbour has flags of its own.
+__device__ __forceinline__ void cell_arrive(const TiledKernelParams &p, int r, int c) {
+    if (!cell_exists(p, r, c)) return;
+    const int sh = 8 * (c % TC);
+    if (((atomicAdd(cell_dep(p, r, r / TC, c / TC), 1u << sh) >> sh) & 255u) + 1u == cell_needed(r, c)) push_entry(p, push_ticket(p), r, c);
+}
+// a far part of tile (I, J) is done: all cells of the tile's row k of cells at once
+__device__ __forceinline__ void far_arrive(const TiledKernelParams &p, int I, int J, int k) {
+    const int r = I * TC + k;
+    fence_acq_rel();
+    const unsigned old = atomicAdd(cell_dep(p, r, I, J), 0x01010101u);
+    for (int q = 0; q < TC; ++q)
+        if (cell_exists(p, r, J * TC + q) && ((old >> (8 * q)) & 255u) + 1u == cell_needed(r, J * TC + q)) push_entry(p, push_ticket(p), r, J * TC + q);
+}
+
+// ---------------------------------------------------------------------------------------------
+// The 8 x 8 leaf at (a, b) of the cell, by one warp: the feedback of the two leaves swept last, then the 15 anti-diagonal steps.
+// Lane l owns entries (i0, j) and (i0 + 4, j) of the leaf, i0 = l & 3, j = l >> 2.  At step s the entries on anti-diagonal s are
+// rounded, their errors and final C values go to an exchange buffer, and after a warp barrier EVERY lane applies one downward
+// and one rightward push to both of its entries (Algorithm 3 lines 8-16 restricted to the leaf).  Y and C receive the same
+// downward pushes, so W = Y - C is kept, which receives the rightward ones only, and Y = W + C is formed to round; with the
+// integer z, E = z - Y and the final C + E = z - W come out side by side.
+// Nothing branches, and nothing is predicated: the push coefficients come from tables that hold zeros wherever no push is due (source
+// not on this anti-diagonal, or entry already rounded); a lane has at most one entry on an anti-diagonal and rounds and posts that
+// one, or one that is not due, which nobody uses.  After its own step an entry's W and C do not change any more, so the results
+// are formed from them after the last step.  Infinities, NaNs and values beyond 31 bits spoil this (0 * inf): then some lane has one
+// of them in the end, and the leaf is swept again with care.
+// A step is a chain of latencies (select 5, three adds and a subtraction 35, store to load 33, fma 10), to which every instruction of
+// the step adds its issue.  A leaf, one warp / four: 1463 / 1495 cycles; posting under predicates and keeping each entry's
+// integer at its step 1834 / 1863, both entries rounded at every step 1960 / 2016.
+__device__ __forceinline__ void sweep_leaf(double *Ws, double *Cs, int *Zs, const double *LU, const double *tabL, const double *tabU, double *exw, int a,
+                                           int b, int row0, int col0, const TiledKernelParams &p, unsigned long long &badkey) {
+    const int lane = threadIdx.x & 31, i0 = lane & 3, j = lane >> 2;
+    double *wp = Ws + CI((a * 8 + i0) * SLD + b * 8 + j, SMAT - 4 * SLD, 114);
+    double *cp = Cs + CI((a * 8 + i0) * SLD + b * 8 + j, SMAT - 4 * SLD, 115);
+    // tabL[row][7 + is] = L(row, is) for 0 <= is < row else 0; at step s, is = s - j
+    const double *tl0 = tabL + CI((a * 8 + i0) * TAB_LD + 7 - j, (S - 4) * TAB_LD - 14, 116);
+    const double *tl1 = tl0 + 4 * TAB_LD;
+    // tabU[col][7 + js] = U(js, col) for 0 <= js < col else 0; at step s, js = s - i
+    const double *tu0 = tabU + CI((b * 8 + j) * TAB_LD + 7 - i0 - 4, S * TAB_LD - 18, 117) + 4;
+    const double *tu1 = tu0 - 4;
+    double l0 = tl0[0], l1 = tl1[0], u0 = tu0[0], u1 = tu1[0];
+    double c0, c1, w0, w1;
+    // L[a, a-1] E[a-1, b] and C[a, b-1] U[b-1, b] as their transposes, with the rows in the order 0 4 1 5 2 6 3 7: fragment element
+    // (column j, rows i0 and i0 + 4) is the lane's own pair of entries, so nothing goes through shared memory
+    auto start = [&]() {
+        c0 = cp[0]; c1 = cp[4 * SLD]; w0 = wp[0]; w1 = wp[4 * SLD];
+        const int row = a * 8 + (j >> 1) + 4 * (j & 1);
+        double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0, x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
+        if (a > 0) {
+            const double *E = Ws + CI(((a - 1) * 8 + i0) * SLD + b * 8 + j, SMAT - 4 * SLD, 106), *L = LU + CI(row * SLD + (a - 1) * 8 + i0, SMAT - 4, 107);
+            dmma_m8n8k4(x0, x1, E[0], L[0]);
+            dmma_m8n8k4(p0, p1, E[4 * SLD], L[4]);
+        }
+        if (b > 0) {
+            const double *U = LU + CI(((b - 1) * 8 + i0) * SLD + b * 8 + j, SMAT - 4 * SLD, 110), *C = Cs + CI(row * SLD + (b - 1) * 8 + i0, SMAT - 4, 111);
+            dmma_m8n8k4(y0, y1, U[0], C[0]);
+            dmma_m8n8k4(q0, q1, U[4 * SLD], C[4]);
+        }
+        c0 += x0 + p0; c1 += x1 + p1; w0 += y0 + q0; w1 += y1 + q1;     // one rounding at the size of the sums, not one per product
+    };
+    start();
+    const int t0 = i0 + j, t1 = t0 + 4;
+    // the e of column j at step s is lane 4 j + (s - j) % 4's, the C of row i0 lane 4 (s - i0) + i0's, that of row i0 + 4 four columns before
+    double *pe = exw + lane, *pc = exw + 48 + lane;
+    const double *rc = exw + 48 - 3 * i0;
+    const double *re[4] = {exw + 4 * j + ((0 - j) & 3), exw + 4 * j + ((1 - j) & 3), exw + 4 * j + ((2 - j) & 3), exw + 4 * j + ((3 - j) & 3)};
+    // round half to even: adding and subtracting 1.5 * 2^52 leaves the integer, whose low word is the sum's
+    constexpr double MAGIC = 6755399441055744.0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int piece = lane + 32 * i, r = piece >> 5, c2 = (piece & 31) * 2;
-                cp_async16(stgC + CI((blk & 1) * STG_C + r * QLD + c2, 2 * STG_C - 1, 110),
-                           p.Cbuf + CI((sm.c_left - p.Cbuf) + (long)(blk * 8 + r) * p.np + c2, (long)p.ntm * T * p.np - 1, 111), 16);
+    for (int s = 0; s < 14; ++s) {
+        const bool first = s < 4 || (s < 11 && t0 >= s);
+        const double w = first ? w0 : w1, c = first ? c0 : c1;
+        const double v = w + c, z = (v + MAGIC) - MAGIC;
+        const int o = (s & 1) * XCH_BUF;
+        pe[o] = z - v; pc[o] = z - w;                           // lines 8-10: E = Z - Y; the fold, L_ii = 1: C + E = Z - W
+        __syncwarp();
+        const double ed = re[s & 3][o], cr0 = rc[o + 4 * s], cr1 = rc[o + 4 * s - 16];
+        double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;          // coefficients of the next step, asked for while the exchange is on its way
+        if (s < 13) { n0 = tl0[s + 1]; n1 = tl1[s + 1]; n2 = tu0[s + 1]; n3 = tu1[s + 1]; }
+        if (s < 10) { c0 = fma(l0, ed, c0); w0 = fma(cr0, u0, w0); }          // push down, push right
+        c1 = fma(l1, ed, c1);
+        if (s >= 4) w1 = fma(cr1, u1, w1);
+        l0 = n0; l1 = n1; u0 = n2; u1 = n3;
+    }
+    const double v0 = w0 + c0, v1 = w1 + c1, m0 = v0 + MAGIC, m1 = v1 + MAGIC, r0 = m0 - MAGIC, r1 = m1 - MAGIC;
+    const bool wild = __any_sync(0xffffffffu, max(__double2hiint(v0) & 0x7fffffff, __double2hiint(v1) & 0x7fffffff) >= 0x41dfffff);
+    double e0 = r0 - v0, e1 = r1 - v1;
+    int z0 = __double2loint(m0), z1 = __double2loint(m1);
+    c0 = r0 - w0; c1 = r1 - w1;
+    if (wild) {
+        // Again from the beginning, both entries rounded at every step; integer and high word of an entry are those of its own step.
+        start();
+        __syncwarp();
+        exw[lane] = 0.0;                                         // what the first pass left there may be infinite or NaN
+        int h0 = 0, h1 = 0;
+#pragma unroll 1
+        for (int s = 0; s < 15; ++s) {
+            const double x0 = w0 + c0, x1 = w1 + c1, k0 = x0 + MAGIC, k1 = x1 + MAGIC;
+            e0 = (k0 - MAGIC) - x0; e1 = (k1 - MAGIC) - x1;
+            const double f0 = (k0 - MAGIC) - w0, f1 = (k1 - MAGIC) - w1;
+            if (t0 == s) { z0 = __double2loint(k0); h0 = __double2hiint(x0); }
+            if (t1 == s) { z1 = __double2loint(k1); h1 = __double2hiint(x1); }
+            if (s == 14) { c0 = f0; c1 = f1; break; }
+            __syncwarp();
+            if (t0 == s) { exw[j] = e0; exw[8 + i0] = f0; }
+            if (t1 == s) { exw[j] = e1; exw[12 + i0] = f1; }
+            __syncwarp();
+            const double ed = exw[j], cr0 = exw[8 + i0], cr1 = exw[12 + i0];
+            c0 = fma(tl0[s], ed, c0); w0 = fma(cr0, tu0[s], w0);
+            c1 = fma(tl1[s], ed, c1); w1 = fma(cr1, tu1[s], w1);
+        }
+        // values that do not fit 32 bits: remember the first.  Either the high word is at or above that of 2^31 (infinities and NaNs
+        // are), or the value is within half of 2^31 and rounds to it: the low word of the sum is then that of -2^31
+        constexpr int TOP = (int)0x80000000;
+        auto look = [&](int h, int row, int &z) {
+            if ((h & 0x7fffffff) >= 0x41e00000) z = (int)__hiloint2double(h, 0);        // saturates
+            else if (z == TOP && h >= 0) z = 0x7fffffff;
+            else return;
+            const unsigned long long kr = row0 + a * 8 + row, kc = col0 + b * 8 + j;
+            const unsigned long long key = ((kr + kc) << 42) | (((h & 0x7fffffff) < 0x7ff00000 ? 1ull : 0ull) << 41) | (kr << 20) | kc;
+            if (kr < (unsigned long long)p.m && kc < (unsigned long long)p.n && key < badkey) badkey = key;
+        };
+        look(h0, i0, z0); look(h1, i0 + 4, z1);
+    }
+    wp[0] = e0; wp[4 * SLD] = e1; cp[0] = c0; cp[4 * SLD] = c1;
+    int *zp = Zs + CI((a * 8 + i0) * S + b * 8 + j, S * S - 4 * S, 118);
+    zp[0] = z0; zp[4 * S] = z1;
+}
+// E and C of the swept leaf (a, b) to the workspace, where the neighbours are waiting for them, by one warp
+__device__ __forceinline__ void post_leaf(const double *Ws, const double *Cs, int a, int b, double *eQ, double *cQ, long np) {
+    const int lane = threadIdx.x & 31, i = a * 8 + (lane >> 2), j = b * 8 + (lane & 3) * 2;
+    double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 133)), c = *reinterpret_cast<const double2 *>(Cs + i * SLD + j);
+    e.x = stream_value(e.x); e.y = stream_value(e.y); c.x = stream_value(c.x); c.y = stream_value(c.y);
+    *reinterpret_cast<double2 *>(eQ + i * np + j) = e;
+    *reinterpret_cast<double2 *>(cQ + i * np + j) = c;
+}
+// its Z (and the caller's E) to the output
+__device__ __forceinline__ void store_leaf(const double *Ws, const int *Zs, int a, int b, int row0, int col0, const TiledKernelParams &p, double &max_abs_e) {
+    const int lane = threadIdx.x & 31, i = a * 8 + (lane >> 2), j = b * 8 + (lane & 3) * 2, gr = row0 + i, gc = col0 + j;
+    if (gr >= p.m || gc >= p.n) return;
+    const double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 134));
+    const int2 z = *reinterpret_cast<const int2 *>(Zs + i * S + j);
+    const bool two = gc + 1 < p.n;
+    int *zo = p.Z + CI((long)gr * p.ldz + gc, (long)(p.m - 1) * p.ldz + p.n, 119);
+    zo[0] = z.x;
+    if (two) zo[1] = z.y;
+    if (p.Euser) {
+        double *eo = p.Euser + (long)gr * p.lde + gc;
+        eo[0] = e.x;
+        if (two) eo[1] = e.y;
+    }
+    max_abs_e = fmax(max_abs_e, fabs(e.x));
+    if (two) max_abs_e = fmax(max_abs_e, fabs(e.y));
+}
+
+// ---------------------------------------------------------------------------------------------
+// One 32 x 32 cell (r, c) of the matrix' grid of cells: the unit of work on the critical path.  On entry its part of Cbuf holds the
+// FAR part of Cd (all source tiles above except the nearest) and its part of Ebuf the FAR part of Rt.  The task
+//   1. pulls what the nearest tiles and its own tile contribute from cells that are COMPLETE (rows 4 (I - near) .. r - 2,
+//      columns 4 (J - near) .. c - 2 of the grid): up to ten 32^3 DMMA products a direction, warps 0-3 C, warps 4-7 W;
+//   2. sweeps the cell in seven leaf-waves.  Leaf (a, lw - a) of leaf-wave lw belongs to warp a (sweep_leaf).  Warps 4-7 do what can be
+//      done beside it: they store what the last leaf-wave left, take in block lw + 1 of the neighbours' results, straight from the
+//      workspace into fragments (warps 4 and 5 add La E_above[:, block] to C, warps 6 and 7 C_left[block, :] Ul to W), and
+//      pull for the leaves of leaf-wave lw + 1 from all leaves but the two swept last.
+// Why 32: the chain of leaf-waves is what bounds all but the largest matrices, and what a leaf-wave costs beside its 15 steps is
+// the streamed products (four times fewer than in a cell of 64, and off the chain: they share the fp64 pipe with the steps, of
+// which they take a sixth here but all of it there), the pulls of older leaves and the barriers.
+// `next` is called by one thread in the last leaf-wave: it looks for the CTA's next cell.
+template <class Next>
+__device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const TiledKernelParams &p, double &max_abs_e, Next next) {
+    double *Ws = smem, *Cs = smem + SMAT, *LU = smem + 2 * SMAT, *La = smem + 3 * SMAT, *Ul = smem + 4 * SMAT;
+    double *tabL = smem + CELL_TABS, *tabU = tabL + S * TAB_LD, *xch = smem + CELL_XCH, *ring = smem + CELL_PULL;
+    int *Zs = reinterpret_cast<int *>(smem + CELL_Z);
+    __shared__ unsigned long long s_badkey;
+    __shared__ int s_known[2];                                        // by parity of the step that reads it
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int row0 = r * S, col0 = c * S, I = r / TC, J = c / TC;
+    const long np = p.np;
+    double *eQ = p.Ebuf + (long)row0 * np + col0, *cQ = p.Cbuf + (long)row0 * np + col0;
+    TS_RESET();
+    // ---- 1. pulls.  Step i takes the source ns - i cells before the neighbour in both directions (the shorter one begins later), so
+    // the newest sources, (r - 2, c) and (r, c - 2), come last.  Those may still be in their last leaf-waves when this task starts
+    // (they are running: the neighbour between them and this cell could not have started otherwise); the others are almost
+    // always complete.
+    const int fa = max(0, TC * (I - p.near)), fl = max(0, TC * (J - p.near));
+    const int nsa = max(0, r - 1 - fa), nsl = max(0, c - 1 - fl), ns = max(nsa, nsl);
+    auto prog_of = [&](int rr, int cc) {
+        return p.cprog + CI(((long)(rr / TC) * p.ntn + cc / TC) * (TC * TC) + (rr % TC) * TC + cc % TC, (long)(TC * TC) * p.ntm * p.ntn, 124);
+    };
+    // Lanes 0-14 of warp 0 look at the sources above, lanes 16-30 at those to the left: the first step that lacks one.  Lanes 15 and 31
+    // look at the two neighbours, which must have taken their far sums before the sweep begins (as a step behind the last one).
+    const int skip_a = ns - nsa, skip_l = ns - nsl;                   // steps before the first source of a direction
+    const int my_step = (lane & 15) == 15 ? ns : lane < 16 ? skip_a + lane : skip_l + lane - 16;
+    const unsigned char *mine = nullptr;
+    if (warp == 0) {
+        if (lane == 15) { if (r > 0) mine = prog_of(r - 1, c); }
+        else if (lane == 31) { if (c > 0) mine = prog_of(r, c - 1); }
+        else if (lane < 16) { if (lane < nsa) mine = prog_of(fa + lane, c); }
+        else if (lane - 16 < nsl) mine = prog_of(r, fl + lane - 16);
+    }
+    const unsigned need = (lane & 15) == 15 ? 1u : 2u;
+    unsigned seen = mine ? ld_acquire_u8(mine) : 2u;
+    // A thread's share of the operands: with 16-byte pieces rows i16 and i16 + 16, columns j16 and j16 + 1 of each block.  The
+    // depth of every source lies inside the matrices, so what a thread has to fill with zeros is the same in every step.
+    const int i16 = tid >> 4, j16 = (tid & 15) * 2, d16 = i16 * SLD + j16;
+    const int lrow0 = min(row0 + i16, p.m - 1), lrow1 = min(row0 + i16 + 16, p.m - 1);
+    const int lz0 = row0 + i16 < p.m ? 16 : 0, lz1 = row0 + i16 + 16 < p.m ? 16 : 0, uz = 8 * min(2, max(0, p.n - col0 - j16));
+    const long np16 = 16 * np, ldu16 = 16 * p.ldu;
+    const bool l16 = p.l_al16, u16 = p.u_al16;
+    const double *lsrc0 = p.L + (long)lrow0 * p.ldl + j16, *lsrc1 = p.L + (long)lrow1 * p.ldl + j16;
+    const double *usrc = p.U + (long)i16 * p.ldu + (uz ? col0 + j16 : col0), *esrc = p.Ebuf + (long)i16 * np + col0 + j16;
+    const double *csrc = p.Cbuf + (long)(row0 + i16) * np + j16;
+    const unsigned smem_s = (unsigned)__cvta_generic_to_shared(smem) + d16 * 8;      // its place in matrix 0
+    constexpr unsigned MAT = SMAT * 8, HALF = 16 * SLD * 8;
+    // operands of the sweep, on their way during the pulls
+    if (r > 0) {
+        cp_async16_if(smem_s + 3 * MAT, lsrc0 + (row0 - S), lz0, l16); cp_async16_if(smem_s + 3 * MAT + HALF, lsrc1 + (row0 - S), lz1, l16);
+        if (!l16) load_factor_async(La, p.L, p.ldl, p.m, row0, row0 - S);
+    }
+    if (c > 0) {
+        const double *u = usrc + (long)(col0 - S) * p.ldu;
+        cp_async16_if(smem_s + 4 * MAT, u, uz, u16); cp_async16_if(smem_s + 4 * MAT + HALF, u + ldu16, uz, u16);
+        if (!u16) load_factor_async(Ul, p.U, p.ldu, p.n, col0 - S, col0);
+    }
+    cp_async16_if(smem_s + MAT, csrc + col0, 16, true); cp_async16_if(smem_s + MAT + HALF, csrc + col0 + np16, 16, true);
+    cp_async16_if(smem_s, esrc + row0 * np, 16, true); cp_async16_if(smem_s + HALF, esrc + row0 * np + np16, 16, true);
+    load_lu_diag_async(LU, p, row0, col0);
+    cp_async_commit();
+    // X in the layout of the accumulators of warps 4-7, zero outside the matrix
+    const int wr = ((warp >> 1) & 1) * 16, wc = (warp & 1) * 16;
+    double acc[2][2][2], xv[2][2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int gr = row0 + wr + a * 8 + g, gc = col0 + wc + b * 8 + t * 2 + h;
+                acc[a][b][h] = 0.0;
+                xv[a][b][h] = (warp >= 4 && gr < p.m && gc < p.n) ? __ldg(p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122)) : 0.0;
             }
+    // the copies of a step: `on` per direction; the pointers move on by one source
+    const double *lp0 = lsrc0 + fa * S, *lp1 = lsrc1 + fa * S, *ep = esrc + (long)fa * S * np, *qp = csrc + fl * S, *up = usrc + (long)fl * S * p.ldu;
+    unsigned dst = smem_s + CELL_PULL * 8, dst_end = dst + PULL_STAGES * 4 * MAT;
+    int asked = 0;                                                    // steps whose operands have been asked for
+    bool on_a = false, on_l = false;
+    auto ask_begin = [&](bool go) { on_a = go && asked >= skip_a; on_l = go && asked >= skip_l; };
+    auto copy = [&](int q) {                                          // operand q / 2 (L, E, C, U), upper or lower half
+        const unsigned at = dst + (q >> 1) * MAT + (q & 1) * HALF;
+        if (q < 2) cp_async16_if(at, q ? lp1 : lp0, q ? lz1 : lz0, on_a && l16);
+        else if (q < 4) cp_async16_if(at, q & 1 ? ep + np16 : ep, 16, on_a);
+        else if (q < 6) cp_async16_if(at, q & 1 ? qp + np16 : qp, 16, on_l);
+        else cp_async16_if(at, q & 1 ? up + ldu16 : up, uz, on_l && u16);
+    };
+    auto ask_end = [&](bool go) {
+        if (!(l16 && u16)) {                                          // odd pitches or pointers: 8 bytes at a time
+            double *buf = ring + (asked % PULL_STAGES) * 4 * SMAT;
+            if (on_a && !l16) load_factor_async(buf, p.L, p.ldl, p.m, row0, (r - 1 - ns + asked) * S);
+            if (on_l && !u16) load_factor_async(buf + 3 * SMAT, p.U, p.ldu, p.n, (c - 1 - ns + asked) * S, col0);
         }
         cp_async_commit();
-        cp_async_wait<0>();
+        if (on_a) { lp0 += S; lp1 += S; ep += 2 * np16; }
+        if (on_l) { qp += S; up += 2 * ldu16; }
+        if (go) { ++asked; dst = dst + 4 * MAT == dst_end ? smem_s + CELL_PULL * 8 : dst + 4 * MAT; }
     };
-    if (fresh && warp == 7) fetch_block(0);
-
-    TS_MARK(2);                                          // tables, first fetch
-    for (int lw = 0; lw < 15; ++lw) {
-        __syncthreads();
-        TS_MARK(lw <= 7 ? 3 : 9);                            // barrier at the top of the leaf-wave
-        if (fresh && lw <= 7) {
-            // ---- pull phase: warp w adds P = Lfa[row block w, :] E_above[:, block lw] to C and Y of leaf
-            // (w, lw), and R = C_left[block lw, :] Ufl[:, column block w] to Y of leaf (lw, w)
-            if (sm.prog_above) {
-                double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-                const double *A = Lfa + (warp * 8 + g) * QLD + t;
-                const double *B = stgE + (lw & 1) * STG_E + t * STG_E_LD + g;
-#pragma unroll 4
-                for (int kk = 0; kk < Q; kk += 8) {
-                    dmma_m8n8k4(p0, p1, A[kk], B[kk * STG_E_LD]);
-                    dmma_m8n8k4(p2, p3, A[kk + 4], B[(kk + 4) * STG_E_LD]);
-                }
-                p0 += p2; p1 += p3;
-                double2 *yq = reinterpret_cast<double2 *>(Ys + (warp * 8 + g) * QLD + lw * 8 + t * 2);
-                double2 *cq = reinterpret_cast<double2 *>(Cs + (warp * 8 + g) * QLD + lw * 8 + t * 2);
-                double2 yv = *yq, cv = *cq;
-                yv.x += p0; yv.y += p1; cv.x += p0; cv.y += p1;
-                *yq = yv; *cq = cv;
-            }
-            __syncwarp();
-            if (sm.prog_left) {
-                double r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
-                const double *A = stgC + (lw & 1) * STG_C + g * QLD + t;
-                const double *B = Ufl + t * QLD + warp * 8 + g;
-#pragma unroll 4
-                for (int kk = 0; kk < Q; kk += 8) {
-                    dmma_m8n8k4(r0, r1, A[kk], B[kk * QLD]);
-                    dmma_m8n8k4(r2, r3, A[kk + 4], B[(kk + 4) * QLD]);
-                }
-                r0 += r2; r1 += r3;
-                double2 *yq = reinterpret_cast<double2 *>(Ys + (lw * 8 + g) * QLD + warp * 8 + t * 2);
-                double2 yv = *yq;
-                yv.x += r0; yv.y += r1;
-                *yq = yv;
-            }
-            TS_MARK(4);                                      // streamed pull (own DMMAs)
-            __syncthreads();
-            TS_MARK(5);                                      // barrier after the pull
+    // warp 0: waits until the sources of all steps before `upto` are complete, and says how far it goes on from there
+    auto await_sources = [&](int upto, int slot) {
+        unsigned long long it = 0;
+        int known;
+        for (;;) {
+            known = __reduce_min_sync(0xffffffffu, seen >= need ? ns + 1 : my_step);
+            if (known >= upto) break;
+            bool over = false;
+            if (lane == 0) over = wait_expired(p, it, -8, 0);
+            if (__any_sync(0xffffffffu, over)) { known = ns + 1; break; }
+            if (seen < need) seen = ld_acquire_u8(mine);
         }
-        // ---- warp 7 fetches the next block of the neighbours; warp 6 (a leaf of its own only in leaf-waves
-        // 6 to 8) publishes what the previous leaf-waves stored: the barriers above order those stores
-        // before this thread's fence
-        if (warp == 7 && fresh && lw < 7) fetch_block(lw + 1);
-        if (tid == 6 * 32 && lw > 0) {
-            __threadfence();
-            st_release_u32(sm.prog_self, (unsigned)lw);
-        }
-        const int a_lo = max(0, lw - 7), a_hi = min(7, lw);
-        const int a = a_lo + warp, b = lw - a;
-        if (a <= a_hi) {
-            leaf_pull(Ys, Cs, Ls, Us, a, b, g, t);
-            __syncwarp();
-            TS_MARK(lw <= 7 ? 6 : 10);                       // leaf_pull
-            // Phase A.  Lane l owns entries (i0, j) and (i0 + 4, j) of the 8 x 8 leaf, i0 = l & 3, j = l >> 2.  At step s the
-            // entry on anti-diagonal s is rounded and its error (by column) and final C value (by row) go to a 16-double
-            // per-warp exchange buffer; after a warp barrier EVERY lane applies one downward and one rightward push to both
-            // of its entries (Algorithm 3 lines 8-16 restricted to the leaf).  Y and C receive the same downward pushes, so
-            // W = Y - C is kept, which receives the rightward ones only, and Y = W + C is formed to round.
-            // Nothing branches.  The push coefficients come from tables that hold zeros wherever no push is due (source
-            // not on this anti-diagonal, or entry already rounded), so stale exchange slots are multiplied by zero; and
-            // every lane rounds both entries at every step, of which only the values at the entry's own step are posted:
-            // before it W and C are incomplete, after it they do not change any more, so the last step leaves every lane's
-            // final values.  A step is a chain of latencies (add 8, round 16, subtract 8, add 8, store to load 35, fma 8);
-            // the branch around the rounding, with the range check in it, cost another 60 of 180 cycles (one warp
-            // alone, 8 x 8 leaf: 2696 -> 1808 cycles; eight warps 3087 -> 2762, where the shared-memory pipe is the bound).
-            const int i0 = lane & 3, j = lane >> 2;
-            double *yp = Ys + CI((a * 8 + i0) * QLD + b * 8 + j, QMAT - 4 * QLD, 114);
-            double *cp = Cs + CI((a * 8 + i0) * QLD + b * 8 + j, QMAT - 4 * QLD, 115);
-            double c0 = cp[0], c1 = cp[4 * QLD], w0 = yp[0] - c0, w1 = yp[4 * QLD] - c1;
-            double y0, y1, g0, g1;
-            // tabL[row][7 + is] = L(row, is) for 0 <= is < row else 0; at step s, is = s - j
-            const double *tl0 = tabL + CI((a * 8 + i0) * TAB_LD + 7 - j, (Q - 4) * TAB_LD - 14, 116);
-            const double *tl1 = tl0 + 4 * TAB_LD;
-            // tabU[col][7 + js] = U(js, col) for 0 <= js < col else 0; at step s, js = s - i
-            const double *tu0 = tabU + CI((b * 8 + j) * TAB_LD + 7 - i0 - 4, Q * TAB_LD - 18, 117) + 4;
-            const double *tu1 = tu0 - 4;
-            double *exw = xch + warp * 32;
-            int z0 = 0, z1 = 0;
-            const int t0 = i0 + j, t1 = t0 + 4;
-            // round half to even: adding and subtracting 1.5 * 2^52 leaves the integer, whose low word is the sum's; values that
-            // do not fit 32 bits are looked for after the leaf, by the words that each had at its own step (a NaN reaches
-            // entries rounded before it through the zero coefficients)
-            constexpr double MAGIC = 6755399441055744.0;
-            int h0 = 0, h1 = 0;
+        __syncwarp();
+        if (lane == 0) s_known[slot] = known;
+    };
+    if (warp == 0) await_sources(min(ns, PULL_STAGES - 1), 0);
+    if (tid == 0) s_badkey = ~0ull;
+    __syncthreads();
+    // The cells below and to the right may get ready: what they do first takes longer than the leaf-waves that they run behind this one
+    // (1024 x 4096: 1.79 ms; told when four / two pulls were left 2.01 / 2.25).  After the older sources have been seen, not before:
+    // otherwise whole diagonals of tasks wait for them on SMs that others could use (2.03).
+    if (tid == 2 * 32) cell_arrive(p, r + 1, c);
+    if (tid == 3 * 32) cell_arrive(p, r, c + 1);
 #pragma unroll
-            for (int s = 0; s < 15; ++s) {
-                const double v0 = w0 + c0, v1 = w1 + c1, r0 = v0 + MAGIC, r1 = v1 + MAGIC;
-                z0 = t0 == s ? __double2loint(r0) : z0; z1 = t1 == s ? __double2loint(r1) : z1;
-                h0 = t0 == s ? __double2hiint(v0) : h0; h1 = t1 == s ? __double2hiint(v1) : h1;
-                y0 = (r0 - MAGIC) - v0; y1 = (r1 - MAGIC) - v1;         // line 5: E = Z - Y
-                g0 = c0 + y0; g1 = c1 + y1;                             // fold, L_ii = 1
-                if (s == 14) break;
-                double *ex = exw + (s & 1) * 16;                        // [0..7] e by column, [8..15] C by row
-                const double l0 = tl0[s], l1 = tl1[s], u0 = tu0[s], u1 = tu1[s];
-                if (t0 == s || t1 == s) {
-                    ex[j] = t0 == s ? y0 : y1;
-                    ex[8 + i0 + (t0 == s ? 0 : 4)] = t0 == s ? g0 : g1;
-                }
-                __syncwarp();
-                const double ed = ex[j], cr0 = ex[8 + i0], cr1 = ex[12 + i0];
-                c0 = fma(l0, ed, c0); w0 = fma(cr0, u0, w0);            // push down, push right
-                c1 = fma(l1, ed, c1); w1 = fma(cr1, u1, w1);
+    for (int i = 0; i < PULL_STAGES - 1; ++i) {
+        const bool go = i < ns;
+        ask_begin(go);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) copy(q);
+        ask_end(go);
+    }
+    for (int k = tid; k < NLEAF * 2 * XCH_BUF; k += TILED_THREADS) xch[k] = 0.0;
+    // The operands of the sweep have landed, for all threads: the neighbours may look for results in the place of the far sums, and the
+    // coefficient tables of the diagonal leaves (see sweep_leaf) can be made.
+    auto prepare = [&]() {
+        const double empty = __longlong_as_double((long long)STREAM_EMPTY);
+        const double2 e2 = make_double2(empty, empty);
+        double *e = eQ + (long)i16 * np + j16, *q = cQ + (long)i16 * np + j16;
+        *reinterpret_cast<double2 *>(e) = e2; *reinterpret_cast<double2 *>(e + np16) = e2;
+        *reinterpret_cast<double2 *>(q) = e2; *reinterpret_cast<double2 *>(q + np16) = e2;
+        const int i = tid >> 3, blk = i & ~7, in = i & 7;             // i: row (L) or column (U) inside the cell
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int x = (tid & 7) + 8 * k, src = x - 7;             // source index inside the leaf
+            const bool ok = src >= 0 && src < in;
+            const int at = blk + (ok ? src : 0);
+            const double l = LU[CI(i * SLD + at, SMAT, 112)], u = LU[CI(at * SLD + i, SMAT, 113)];
+            if (x < TAB_LD) {
+                tabL[i * TAB_LD + x] = ok ? l : 0.0;
+                tabU[i * TAB_LD + x] = ok ? u : 0.0;
             }
-            c0 = g0; c1 = g1;
-            {   // values that do not fit 32 bits: remember the first.  Either the high word is at or above that of 2^31 (infinities and NaNs
-                // are), or the value is within half of 2^31 and rounds to it: the low word of the sum is then that of -2^31
-                constexpr int TOP = (int)0x80000000;
-                if (max(h0 & 0x7fffffff, h1 & 0x7fffffff) >= 0x41e00000 || (z0 == TOP && h0 >= 0) || (z1 == TOP && h1 >= 0)) {
-                    auto look = [&](int h, int row, int &z) {
-                        if ((h & 0x7fffffff) >= 0x41e00000) z = (int)__hiloint2double(h, 0);        // saturates
-                        else if (z == TOP && h >= 0) z = 0x7fffffff;
-                        else return;
-                        const unsigned long long gr = row0 + a * 8 + row, gc = col0 + b * 8 + j;
-                        const unsigned long long key = ((gr + gc) << 42) | (((h & 0x7fffffff) < 0x7ff00000 ? 1ull : 0ull) << 41) | (gr << 20) | gc;
-                        if (gr < (unsigned long long)p.m && gc < (unsigned long long)p.n && key < badkey) badkey = key;
-                    };
-                    look(h0, i0, z0); look(h1, i0 + 4, z1);
-                }
-            }
-            yp[0] = y0; yp[4 * QLD] = y1; cp[0] = c0; cp[4 * QLD] = c1;
-            TS_MARK(lw <= 7 ? 7 : 11);                       // the 15 anti-diagonal steps
-            // results of the leaf: E and C to the workspace (for the neighbours and for the far parts of
-            // later tiles), Z (and the caller's E) to the output
-            {
-                const int gr = row0 + a * 8 + i0, gc = col0 + b * 8 + j;
-                const long at = CI((long)gr * p.np + gc, (long)p.ntm * T * p.np - 4 * p.np, 118);
-                p.Ebuf[at] = y0; p.Ebuf[at + 4 * p.np] = y1;
-                p.Cbuf[at] = c0; p.Cbuf[at + 4 * p.np] = c1;
-                if (gc < p.n) {
-                    if (gr < p.m) {
-                        p.Z[CI((long)gr * p.ldz + gc, (long)(p.m - 1) * p.ldz + p.n, 119)] = z0;
-                        if (p.Euser) p.Euser[(long)gr * p.lde + gc] = y0;
-                        max_abs_e = fmax(max_abs_e, fabs(y0));
-                    }
-                    if (gr + 4 < p.m) {
-                        p.Z[CI((long)(gr + 4) * p.ldz + gc, (long)(p.m - 1) * p.ldz + p.n, 120)] = z1;
-                        if (p.Euser) p.Euser[(long)(gr + 4) * p.lde + gc] = y1;
-                        max_abs_e = fmax(max_abs_e, fabs(y1));
-                    }
-                }
-            }
-            TS_MARK(lw <= 7 ? 8 : 12);                       // stores of the leaf
         }
+    };
+    // A step's operands are asked for two steps ahead if its sources are known to be complete, one step ahead otherwise.
+    int last = -1, rd = 0;                                            // the step asked for in the previous iteration, the buffers of this one
+    for (int i = 0; i < ns; ++i) {
+        if (last == i) cp_async_wait<0>(); else cp_async_wait<PULL_STAGES - 2>();                  // step i's operands have landed
+        __syncthreads();
+        if (i == 0) TS_MARK(0);
+        const int known = s_known[i & 1];
+        const bool go = asked < ns && asked <= i + PULL_STAGES - 1 && asked < known;               // every warp is past product i - 1: its buffers are free
+        const double *As = ring + (rd * 4 + (warp < 4 ? 0 : 2)) * SMAT;
+        rd = rd == PULL_STAGES - 1 ? 0 : rd + 1;
+        last = go ? asked : -1;
+        ask_begin(go);
+        quarter_mma(acc, i >= (warp < 4 ? skip_a : skip_l), As, As + SMAT, wr, wc, g, t, copy);
+        ask_end(go);
+        if (i == 0) prepare();
+        // the step that has to be asked for in the next iteration; the barrier at its top tells the others
+        if (warp == 0) {
+            if ((i + 2 < ns && known <= i + 2) || (i == ns - 1 && known <= ns)) await_sources(min(i + 3, ns + 1), (i + 1) & 1);
+            else if (lane == 0) s_known[(i + 1) & 1] = known;
+        }
+    }
+    if (ns == 0) {
+        cp_async_wait<0>();
+        __syncthreads();
+        prepare();
+        if (warp == 0) await_sources(1, 0);
+    }
+    TS_MARK(1);
+    {   // C = far part + pulls; W = Y - C = X + Rt, far part and pulls likewise
+        double *dst = warp < 4 ? Cs : Ws;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                double2 *q = reinterpret_cast<double2 *>(dst + CI((wr + a * 8 + g) * SLD + wc + b * 8 + t * 2, SMAT - 1, 123)), v = *q;
+                v.x += acc[a][b][0] + xv[a][b][0]; v.y += acc[a][b][1] + xv[a][b][1];
+                *q = v;
+            }
     }
     __syncthreads();
-    TS_MARK(13);
-    if (tid == 0) {                      // everything is stored: the quadrant is complete
-        __threadfence();
-        st_release_u32(sm.prog_self, 15u);
+    if (tid == 3 * 32) st_release_u8(prog_of(r, c), 1u);              // STREAM_EMPTY is in place
+
+    // ---- 2. the sweep
+    unsigned long long badkey = ~0ull;
+    const int half = warp & 1;
+    // fragments of the neighbours: E above, k = 4 i + t, column g of the block (warps 4, 5); C to the left, row g of the block, k = 4 i + t (6, 7)
+    const bool down = warp < 6, fed = down ? r > 0 : c > 0;
+    const double *nsrc = down ? eQ + (long)(t - S) * np + g : cQ + (long)g * np - S + t;
+    const long nstep = down ? 4 * np : 4, nblk = down ? 8 : 8 * np;
+    double v[8];
+    auto stream_take = [&](int blk) {
+        const double *src = nsrc + blk * nblk;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        double2 *d0, *d1;
+        if (down) {
+            const double *A = La + (half * 16 + g) * SLD + t;
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                stream_await(p, v[i], v[i + 1], src + i * nstep, nstep);
+                dmma_m8n8k4(a0, a1, A[4 * i], v[i]);
+                dmma_m8n8k4(a2, a3, A[8 * SLD + 4 * i], v[i]);
+                dmma_m8n8k4(a0, a1, A[4 * i + 4], v[i + 1]);
+                dmma_m8n8k4(a2, a3, A[8 * SLD + 4 * i + 4], v[i + 1]);
+            }
+            d0 = reinterpret_cast<double2 *>(Cs + CI((half * 16 + g) * SLD + blk * 8 + t * 2, SMAT - 8 * SLD - 1, 126));
+            d1 = d0 + 8 * SLD / 2;
+        } else {
+            const double *B = Ul + t * SLD + half * 16 + g;
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                stream_await(p, v[i], v[i + 1], src + i * nstep, nstep);
+                dmma_m8n8k4(a0, a1, v[i], B[4 * i * SLD]);
+                dmma_m8n8k4(a2, a3, v[i], B[4 * i * SLD + 8]);
+                dmma_m8n8k4(a0, a1, v[i + 1], B[(4 * i + 4) * SLD]);
+                dmma_m8n8k4(a2, a3, v[i + 1], B[(4 * i + 4) * SLD + 8]);
+            }
+            d0 = reinterpret_cast<double2 *>(Ws + CI((blk * 8 + g) * SLD + half * 16 + t * 2, SMAT - 9, 128));
+            d1 = d0 + 4;
+        }
+        double2 x = *d0, y = *d1;
+        x.x += a0; x.y += a1; y.x += a2; y.y += a3;
+        *d0 = x; *d1 = y;
+    };
+    if (warp >= 4 && fed) {
+        stream_ask(v, nsrc, nstep);
+        stream_take(0);
     }
-    // status: the earliest (in sweep order) unrepresentable value of the quadrant, if any
+    TS_MARK(2);
+    for (int lw = 0; lw < 2 * NLEAF - 1; ++lw) {
+        __syncthreads();
+        TS_MARK(3);
+        if (warp < NLEAF) {
+            const int a = warp, b = lw - a;
+            if (b >= 0 && b < NLEAF) {
+                sweep_leaf(Ws, Cs, Zs, LU, tabL, tabU, xch + warp * 2 * XCH_BUF, a, b, row0, col0, p, badkey);
+                TS_MARK(5);
+            }
+        } else {
+            const bool take = fed && lw + 1 < NLEAF;
+            const int a = warp - 4, b = lw + 1 - a, done = b - 2;
+            if (done >= 0 && done < NLEAF) post_leaf(Ws, Cs, a, done, eQ, cQ, np);
+            if (take) stream_ask(v, nsrc + (lw + 1) * nblk, nstep);
+            if (b >= 0 && b < NLEAF) leaf_pull(Ws, Cs, LU, a, b, a - 1, b - 1, g, t);
+            if (done >= 0 && done < NLEAF) store_leaf(Ws, Zs, a, done, row0, col0, p, max_abs_e);
+            if (take) stream_take(lw + 1);
+            if (lw == 2 * NLEAF - 2 && tid == 5 * 32) next();
+        }
+    }
     if (badkey != ~0ull) atomicMin(&s_badkey, badkey);
     __syncthreads();
+    if (warp == 7) {
+        post_leaf(Ws, Cs, NLEAF - 1, NLEAF - 1, eQ, cQ, np);
+        __syncwarp();
+        if (lane == 0) st_release_u8(prog_of(r, c), 2u);              // E and C are complete: the cells two further on may pull
+    }
+    if (warp == 6) store_leaf(Ws, Zs, NLEAF - 1, NLEAF - 1, row0, col0, p, max_abs_e);
+    TS_MARK(6);
+    // status: the earliest (in sweep order) unrepresentable value of the cell, if any
     if (tid == 0 && s_badkey != ~0ull) {
         const unsigned long long k = s_badkey;
         report(p.info, ((k >> 41) & 1ull) ? GPTQ2D_ERR_INT_OVERFLOW : GPTQ2D_ERR_NONFINITE,
                (int)((k >> 20) & 0x1fffffull) + p.row_off, (int)(k & 0xfffffull) + p.col_off, p.report_index);
     }
-}
-
-// 64 x 64 diagonal blocks of both factors into one shared-memory matrix: below the diagonal
-// L[r0 + i][r0 + k], above it U[c0 + k][c0 + j], zeros on it and outside the matrices.
-__device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKernelParams &p, int r0, int c0) {
-    const bool vec = p.l_al16 && p.u_al16 && r0 + Q <= p.m && c0 + Q <= p.n;      // whole blocks in 16-byte pieces
-    if (vec) {
-#pragma unroll
-        for (int it = 0; it < 8; ++it) {
-            const int c = threadIdx.x + it * TILED_THREADS;
-            const int i = c >> 5, j = (c & 31) * 2;
-            // the piece that holds the diagonal: its off-diagonal entry only (from L if i is odd, from U if it is even)
-            const bool lower = j < i, diag = (i & ~1) == j;
-            const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
-            if (!diag) cp_async16(dst + CI(i * QLD + j, QMAT - 1, 121), src, 16);
-            else cp_async8(dst + CI(i * QLD + j + ((i & 1) ^ 1), QMAT, 131), (i & 1) ? src : src + 1, 8);
-        }
-        if (threadIdx.x < Q) dst[CI(threadIdx.x * (QLD + 1), QMAT, 132)] = 0.0;
-        return;
-    }
-#pragma unroll
-    for (int it = 0; it < 16; ++it) {
-        const int c = threadIdx.x + it * TILED_THREADS;
-        const int i = c >> 6, j = c & 63;
-        const bool lower = j < i, upper = j > i;
-        const bool take = lower ? (r0 + i < p.m) : (upper && c0 + j < p.n);     // r0 + j < r0 + i, c0 + i < c0 + j
-        const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
-        cp_async8(dst + CI(i * QLD + j, QMAT, 121), take ? src : p.L, take ? 8 : 0);
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// One 64 x 64 quadrant q (0: top-left, 1: top-right, 2: bottom-left, 3: bottom-right) of tile
-// (I, J): the unit of work on the critical path.  In the grid of quadrants it sits at
-// (r, c) = (2 I + q / 2, 2 J + q % 2).
-//
-// On entry the quadrant's part of the tile's Cbuf region holds the FAR part of Cd (all source
-// tiles above except the two nearest) and its Ebuf part the FAR part of Rt.  The task
-//   1. pulls what the two nearest tiles and its own tile contribute from quadrants that are COMPLETE
-//      (rows 2 I - 4 .. r - 2, columns 2 J - 4 .. c - 2 of the quadrant grid): up to eight 64^3 DMMA
-//      products;
-//   2. forms Y = X + Rt + Cd, C = Cd and runs Algorithm 3 on the quadrant, taking the contributions
-//      of the quadrant right above it and of the one right to its left block by block as they
-//      finish (quadrant_sweep), and publishing its own leaves wave by wave.
-__device__ __forceinline__ void sweep_quadrant(int I, int J, int q, double *smem, const TiledKernelParams &p,
-                                               double &max_abs_e) {
-    double *Ys = smem, *Cs = smem + QMAT, *LU = smem + 2 * QMAT, *Lfa = smem + 3 * QMAT, *Ufl = smem + 4 * QMAT;
-    double *tabL = smem + 5 * QMAT, *tabU = tabL + Q * TAB_LD;
-    double *stg = tabU + Q * TAB_LD;
-    const int tid = threadIdx.x;
-    const int qi = q >> 1, qj = q & 1;
-    const int row0 = I * T + qi * Q, col0 = J * T + qj * Q;
-    double *eQ = p.Ebuf + (long)row0 * p.np + col0;
-    double *cQ = p.Cbuf + (long)row0 * p.np + col0;
-
-    // ---- 1. pulls from complete quadrants: rows r' = max(0, 2 I - 4) .. r - 2 of the quadrant grid (the
-    // two tiles above, without the quadrant right above this one), columns likewise.  The far parts of the
-    // tile cover everything further away.  Oldest sources first; the two newest, (r - 2, c) and
-    // (r, c - 2), may still be sweeping their last leaves when this task starts and are waited for
-    // right before their blocks are requested (they are running: the neighbour between them and this
-    // quadrant could not have started otherwise).
-    QAcc accC, accR;
-    accC.zero();
-    accR.zero();
-    TS_RESET();
-    {   // X of the quadrant is read once, after the pulls, and comes from HBM: ask for it now (one 128-byte line per thread)
-        const int gr = row0 + (tid >> 2), gc = col0 + (tid & 3) * 16;
-        if (gr < p.m && gc < p.n) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.X + (long)gr * p.ldx + gc));
-    }
-    {
-        const int r = 2 * I + qi, c = 2 * J + qj;
-        const int fa = max(0, 2 * I - 4), fl = max(0, 2 * J - 4);
-        const int nsa = max(0, r - 1 - fa), nsl = max(0, c - 1 - fl), ns = nsa + nsl;
-        auto prog_of = [&](int rr, int cc) {
-            return p.qprog + CI(((long)(rr >> 1) * p.ntn + (cc >> 1)) * 4 + (rr & 1) * 2 + (cc & 1), 4L * p.ntm * p.ntn, 124);
-        };
-        // step i -> (direction, block): the older blocks of both directions first, then the newest of each
-        const int olda = max(0, nsa - 1), oldl = max(0, nsl - 1);
-        auto step_dir = [&](int i) {
-            return i < olda ? 0 : (i < olda + oldl ? 1 : ((i == olda + oldl && nsa > 0) ? 0 : 1));
-        };
-        auto step_blk = [&](int i) {
-            return i < olda ? fa + i : (i < olda + oldl ? fl + (i - olda) : (step_dir(i) == 0 ? r - 2 : c - 2));
-        };
-        // three buffer pairs: one being multiplied, two being filled; all unused until the sweep proper
-        auto bufA = [&](int j) { return j == 0 ? Lfa : (j == 1 ? LU : Ys); };
-        auto bufB = [&](int j) { return j == 0 ? Ufl : (j == 1 ? Cs : tabL); };
-        auto issue = [&](int i) {
-            double *Ab = bufA(i % 3), *Bb = bufB(i % 3);
-            const int dir = step_dir(i), blk = step_blk(i), k0 = blk * Q;
-            if (i >= olda + oldl) await_progress(p, dir == 0 ? prog_of(blk, c) : prog_of(r, blk), nullptr, 15u);
-            if (dir == 0) {
-                if (p.l_al16) load_full_block_async16(Ab, p.L, p.ldl, p.m, row0, k0);
-                else load_factor_block_async(Ab, p.L, p.ldl, p.m, row0, k0, 0);
-                load_quadrant_async(Bb, p.Ebuf + (long)k0 * p.np + col0, p.np);
-            } else {
-                load_quadrant_async(Ab, p.Cbuf + (long)row0 * p.np + k0, p.np);
-                if (p.u_al16) load_full_block_async16(Bb, p.U, p.ldu, p.n, k0, col0);
-                else load_factor_block_async(Bb, p.U, p.ldu, p.n, k0, col0, 0);
-            }
-            cp_async_commit();
-        };
-        // the older sources: one warp each makes sure its quadrant is complete (it almost always is)
-        {
-            const int w = threadIdx.x >> 5;
-            if (w < olda) await_progress(p, prog_of(fa + w, c), nullptr, 15u);
-            else if (w < olda + oldl) await_progress(p, prog_of(r, fl + (w - olda)), nullptr, 15u);
-        }
-        __syncthreads();
-        for (int i = 0; i < ns && i < 2; ++i) issue(i);
-        for (int i = 0; i < ns; ++i) {
-            if (i + 1 < ns) cp_async_wait<1>(); else cp_async_wait<0>();     // step i's operands have landed
-            __syncthreads();
-            // every warp is past product i - 1 now, so its buffer pair, (i + 2) % 3, can take step i + 2
-            if (i + 2 < ns) issue(i + 2);
-            if (step_dir(i) == 0) quad_mma(accC, bufA(i % 3), bufB(i % 3)); else quad_mma(accR, bufA(i % 3), bufB(i % 3));
-        }
-        __syncthreads();
-    }
-
-    TS_MARK(0);                                          // pulls from the two nearest tiles
-    if (tid == 7 * 32) {
-        // This quadrant is about to sweep: the one below it and the one to its right may start getting ready.  Told here, before
-        // this quadrant's own operand loads: what they do first (their pulls and loads, 60 thousand cycles) takes longer than the
-        // nine leaf-waves that they run behind this one (1024 x 4096: 2.76 -> 2.49 ms against telling them at the first leaf-wave).
-        if (qi == 0) quadrant_arrive(p, I, J, q + 2);
-        else if (I + 1 < p.ntm) quadrant_arrive(p, I + 1, J, q - 2);
-        if (qj == 0) quadrant_arrive(p, I, J, q + 1);
-        else if (J + 1 < p.ntn) quadrant_arrive(p, I, J + 1, q - 1);
-    }
-    // ---- 2. operands of the sweep
-    Stream sm;
-    sm.I = I; sm.J = J; sm.q = q;
-    const long tq = ((long)I * p.ntn + J) * 4;
-    sm.prog_self = p.qprog + tq + q;
-    sm.prog_above = nullptr; sm.prog_left = nullptr; sm.e_above = nullptr; sm.c_left = nullptr;
-    if (row0 > 0) {
-        sm.prog_above = qi ? p.qprog + tq + (q - 2) : p.qprog + ((long)(I - 1) * p.ntn + J) * 4 + (q + 2);
-        sm.e_above = p.Ebuf + (long)(row0 - Q) * p.np + col0;
-        if (p.l_al16) load_full_block_async16(Lfa, p.L, p.ldl, p.m, row0, row0 - Q);
-        else load_factor_block_async(Lfa, p.L, p.ldl, p.m, row0, row0 - Q, 0);
-    }
-    if (col0 > 0) {
-        sm.prog_left = qj ? p.qprog + tq + (q - 1) : p.qprog + ((long)I * p.ntn + (J - 1)) * 4 + (q + 1);
-        sm.c_left = p.Cbuf + (long)row0 * p.np + (col0 - Q);
-        if (p.u_al16) load_full_block_async16(Ufl, p.U, p.ldu, p.n, col0 - Q, col0);
-        else load_factor_block_async(Ufl, p.U, p.ldu, p.n, col0 - Q, col0, 0);
-    }
-    load_lu_diag_async(LU, p, row0, col0);
-    load_quadrant_async(Cs, cQ, p.np);
-    load_quadrant_async(Ys, eQ, p.np);
-    cp_async_commit();
-    // X of the quadrant, zero outside the matrix, in the layout of the accumulators (quad_mma)
-    const int xr = row0 + ((tid >> 6) * 16 + ((tid & 31) >> 2)), xc = col0 + ((tid >> 5) & 1) * 32 + (tid & 3) * 2;
-    double xv[2][4][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int gr = xr + a * 8, gc = xc + b * 8 + h;
-                xv[a][b][h] = (gr < p.m && gc < p.n) ? __ldg(p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122)) : 0.0;
-            }
-    cp_async_wait<0>();
-    __syncthreads();
-    // Cd = far part + pulls from complete quadrants; Rt likewise; Y = X + Rt + Cd
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int at = CI((xr - row0 + a * 8) * QLD + xc - col0 + b * 8, QMAT - 1, 123);
-            double2 *cq = reinterpret_cast<double2 *>(Cs + at), *yq = reinterpret_cast<double2 *>(Ys + at);
-            double2 cv = *cq, yv = *yq;
-            cv.x += accC.v[a][b][0]; cv.y += accC.v[a][b][1];
-            yv.x += accR.v[a][b][0]; yv.y += accR.v[a][b][1];
-            yv.x += xv[a][b][0] + cv.x; yv.y += xv[a][b][1] + cv.y;
-            *cq = cv; *yq = yv;
-        }
-    TS_MARK(1);                                          // operand loads, Y = X + Rt + Cd
-    quadrant_sweep(Ys, Cs, LU, Lfa, Ufl, stg, tabL, tabU, row0, col0, sm, p, max_abs_e);
     __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------------------
 // Far parts in claim order: wave by wave (I + J ascending); inside a wave the longest contractions
-// first (the Cd part of tile (I, J) has I - 2 chunks, the Rt part J - 2), so that a wave's far parts
+// first (the Cd part of tile (I, J) has I - near chunks, the Rt part J - near), so that a wave's far parts
 // finish close together instead of the long ones trailing.
 __device__ __forceinline__ void decode_task(int task, int ntm, int ntn, int &type, int &I, int &J) {
     int tt = task;
@@ -719,73 +817,16 @@ __device__ __forceinline__ void load_acc(Acc &acc, const double *srcT, long np, 
         }
 }
 
-// Global ring of ready quadrant tasks (size a power of two).  It cannot overflow: a quadrant depends,
-// directly or through others, on the quadrant above it and on the one to its left, so the quadrants
-// of one matrix that are ready at the same time lie on an anti-chain of its 2 ntm x 2 ntn quadrant
-// grid, at most 2 min(ntm, ntn) of them; each enters the ring once.  A single matrix therefore
-// needs at most 512 slots (ntm, ntn <= 256 tiles would be 32768 rows); a batched launch sizes its
-// ring from the sum over its matrices.
-constexpr unsigned QCAP = 4096;
 constexpr int FAR_RUN_CHUNKS = 64;      // a far part looks at the ready ring every this many K = 128 chunks
 constexpr unsigned IDLE_SLEEP_NS = 100; // pause of a CTA that found nothing to do (100 - 1600 ns and far runs of 8 - 64 chunks all time within 1 %)
-
-// multi-producer / multi-consumer ring in global memory; slot value 0 = empty.
-__device__ __forceinline__ void ready_push(const TiledKernelParams &p, unsigned entry) {
-    unsigned t = atomicAdd(p.q_tail, 1u);
-    st_release_u32(p.q_slots + CI(t & p.qmask, (long)p.qmask + 1, 127), entry | 0x80000000u);
-}
-// thread 0 only.  Returns 0 if the queue is empty (or on abort), else the entry (bit 31 set).
-__device__ __forceinline__ unsigned ready_pop(const TiledKernelParams &p) {
-    for (;;) {
-        unsigned h = ld_relaxed_u32(p.q_head), t = ld_relaxed_u32(p.q_tail);
-        if ((int)(t - h) <= 0) return 0u;
-        if (atomicCAS(p.q_head, h, h + 1u) != h) continue;
-        unsigned *slot = p.q_slots + (h & p.qmask);
-        unsigned long long spins = 0;
-        unsigned e;
-        while ((e = ld_acquire_u32(slot)) == 0u) {          // producer has the ticket but has not written yet
-            if (++spins > p.spin_limit || ld_relaxed_u32(p.abort) != 0u) {
-                report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -3, (int)h, (int)blockIdx.x);
-                atomicExch(p.abort, 1u);
-                return 0u;
-            }
-        }
-        *slot = 0u;
-        return e;
-    }
-}
-
-// Arrivals a quadrant task at (r, c) of the quadrant grid waits for: the two far parts of its tile and
-// the quadrants at (r - 1, c) and (r, c - 1) having begun to sweep.
-__device__ __forceinline__ unsigned quadrant_needed(int I, int J, int q) {
-    const int r = 2 * I + (q >> 1), c = 2 * J + (q & 1);
-    return 2u + (r >= 1 ? 1u : 0u) + (c >= 1 ? 1u : 0u);
-}
-// A quadrant that lies wholly outside the matrix (ragged last tile row / column) is never a task:
-// arrivals at it are dropped here, its region of the workspace keeps the zeros the far parts parked
-// there, and nothing inside the matrix depends on it.
-__device__ __forceinline__ bool quadrant_exists(const TiledKernelParams &p, int I, int J, int q) {
-    return I * T + (q >> 1) * Q < p.m && J * T + (q & 1) * Q < p.n;
-}
-__device__ __forceinline__ void quadrant_arrive(const TiledKernelParams &p, int I, int J, int q) {
-    if (!quadrant_exists(p, I, J, q)) return;
-    unsigned old = atomicAdd(p.qdep + CI(((long)I * p.ntn + J) * 4 + q, 4L * p.ntm * p.ntn, 125), 1u);
-    if (old + 1u == quadrant_needed(I, J, q)) {
-        // single matrix: q | I (14 bits) | J (15 bits); batched: q | matrix (13 bits) | I (8 bits) | J (8 bits)
-        const unsigned entry = p.batch_index >= 0
-            ? (((unsigned)q << 29) | ((unsigned)p.batch_index << 16) | ((unsigned)I << 8) | (unsigned)J | 0x80000000u)
-            : (((unsigned)q << 29) | ((unsigned)I << 15) | (unsigned)J | 0x80000000u);
-        __threadfence();
-        ready_push(p, entry);
-    }
-}
 
 constexpr int FAR_CTX = 2;       // far parts a CTA may hold at once (one live in registers, the others parked)
 
 // The persistent scheduler loop.  BATCHED = false: one matrix, described by the kernel argument
 // itself.  BATCHED = true: many matrices in one launch; the kernel argument holds what they share
 // (claim counter, ready ring, abort word, totals) and each task works on a shared-memory copy of
-// its matrix' descriptor (slots 0..FAR_CTX-1: the far contexts, slot FAR_CTX: the quadrant task).
+// its matrix' descriptor (slots 0..FAR_CTX-1: the far contexts, the two behind them: a cell and
+// the one after it).
 // PANELS = true (single matrix only): the inputs are still being copied in while the kernel runs, in
 // blocks of COPY_BLOCK_TILES x COPY_BLOCK_TILES tiles and in the order the wavefront needs them: step
 // s brings the blocks of X on block anti-diagonal s, the block row s of L and the block column s of
@@ -799,7 +840,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
     __shared__ int s_nctx, s_pick, s_state;
     __shared__ unsigned s_pop;
     __shared__ double s_red[TILED_THREADS / 32];
-    __shared__ TiledKernelParams s_view[BATCHED ? FAR_CTX + 1 : 1];
+    __shared__ TiledKernelParams s_view[BATCHED ? FAR_CTX + 2 : 1];
     static_assert(!BATCHED || FAR_CTX == 2, "view slots of far contexts are handed out as 0 / 1");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wm = warp >> 2, wn = warp & 3, g = lane >> 2, t = lane & 3;
@@ -821,13 +862,13 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
     if (tid == 0) {
         s_nctx = 0;
         if (BATCHED)
-            for (int k = 0; k <= FAR_CTX; ++k) s_view[k].batch_index = -1;
+            for (int k = 0; k < FAR_CTX + 2; ++k) s_view[k].batch_index = -1;
     }
 
     // the descriptor a task works on: the kernel argument itself for a single matrix (spelled so that the
     // compiler sees plain parameter accesses there), a shared-memory copy in a batched launch
 #define VIEW(slot) (BATCHED ? s_view[slot] : p)
-    auto load_view = [&](int slot, int b) {            // thread 0, before the barrier that publishes the task
+    auto load_view = [&](int slot, int b) {            // one thread, before a barrier that publishes the task
         if constexpr (BATCHED) {
             if (s_view[slot].batch_index != b) {
                 const unsigned long long *src = reinterpret_cast<const unsigned long long *>(p.probs + b);
@@ -840,8 +881,8 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
             }
         }
     };
-    auto entry_matrix = [&](unsigned e) { return (int)((e >> 16) & 0x1fffu); };
-    // thread 0.  Far parts poll (they have other things to do); a popped quadrant task waits, bounded:
+    auto entry_matrix = [&](unsigned e) { return BATCHED ? (int)((e & 0x7fffffffu) >> p.cell_bits) : 0; };
+    // thread 0.  Far parts poll (they have other things to do); a popped cell waits, bounded:
     // the copies make progress on their own.
     auto panels_arrived = [&](int need) -> bool {
         if constexpr (PANELS) return ld_acquire_u32(p.panels_ready) >= (unsigned)need;
@@ -850,8 +891,8 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
     auto await_panels = [&](unsigned e) -> unsigned {
         if constexpr (PANELS) {
             if (e == 0u) return e;
-            const int need = ((int)((e >> 15) & 0x3fffu) >> COPY_BLOCK_TILES_LOG2) +
-                             ((int)(e & 0x7fffu) >> COPY_BLOCK_TILES_LOG2) + 1;
+            const unsigned cell = e & 0x7fffffffu, nc = (unsigned)(TC * p.ntn);
+            const int need = (int)((cell / nc / TC) >> COPY_BLOCK_TILES_LOG2) + (int)((cell % nc / TC) >> COPY_BLOCK_TILES_LOG2) + 1;
             unsigned long long it = 0;
             while (!panels_arrived(need)) {
                 if (++it > p.panel_spin_limit || ld_relaxed_u32(p.abort) != 0u) {
@@ -871,15 +912,17 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
     };
 
     for (;;) {
-        // ---- thread 0 looks for work: a ready quadrant task first, else the oldest far part that can
+        // ---- thread 0 looks for work: a ready cell first, else the oldest far part that can
         // go on, else (room and tasks left) a new far part.  s_state: 0 run far part s_pick, 1 serve the
         // ring, 2 nothing to do right now, 3 all tiles swept, 4 abort.
         __syncthreads();
         if (tid == 0) {
             int state = 2, pick = -1;
             unsigned e = 0u;
+            const unsigned aborted = ld_relaxed_u32(p.abort), claimed = ld_relaxed_u32(p.counter);       // one trip to L2 for all three
+            const int avail = (int)ld_relaxed_u32(reinterpret_cast<unsigned *>(p.q_avail));
             // A far part of this CTA that is at most two chunks from done and can go on comes before
-            // everything else: the four quadrant tasks of its tile cannot start without it, and other
+            // everything else: the cells of its tile cannot start without it, and other
             // CTAs can serve the ring.
             for (int k = 0; k < s_nctx && pick < 0; ++k) {
                 const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
@@ -891,9 +934,9 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                     panels_arrived(((ty == 0 ? s_ctx[k][1] : s_ctx[k][2]) >> COPY_BLOCK_TILES_LOG2) + 1))
                     pick = k;
             }
-            if (ld_relaxed_u32(p.abort) != 0u) state = 4;
+            if (aborted != 0u) state = 4;
             else if (pick >= 0) state = 0;
-            else if ((e = await_panels(ready_pop(p))) != 0u) {
+            else if (avail > 0 && (e = await_panels(ready_pop(p))) != 0u) {
                 state = 1;
                 load_view(FAR_CTX, entry_matrix(e));
             } else {
@@ -908,7 +951,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                         panels_arrived(((ty == 0 ? s_ctx[k][1] : s_ctx[k][2]) >> COPY_BLOCK_TILES_LOG2) + 1))
                         pick = k;
                 }
-                if (pick < 0 && n < FAR_CTX && ld_relaxed_u32(p.counter) < (unsigned)p.ntasks) {
+                if (pick < 0 && n < FAR_CTX && claimed < (unsigned)p.ntasks) {
                     int task = (int)atomicAdd(p.counter, 1u);
                     if (task < p.ntasks) {
                         int ty, fi, fj, slot = 0;
@@ -922,7 +965,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                         }
                         const TiledKernelParams &pk = VIEW(slot);
                         s_ctx[n][0] = ty; s_ctx[n][1] = fi; s_ctx[n][2] = fj; s_ctx[n][3] = 0;
-                        s_ctx[n][4] = max(0, (ty == 0 ? fi : fj) - 2); s_ctx[n][5] = task; s_ctx[n][6] = slot;
+                        s_ctx[n][4] = max(0, (ty == 0 ? fi : fj) - pk.near); s_ctx[n][5] = task; s_ctx[n][6] = slot;
                         s_nctx = n + 1;
                         const unsigned *fl = ty == 0 ? pk.flagS + fj : pk.flagS + (long)fi * pk.ntn;
                         if ((s_ctx[n][4] == 0 || ld_acquire_u32(fl) != 0u) && panels_arrived(((ty == 0 ? fi : fj) >> COPY_BLOCK_TILES_LOG2) + 1))
@@ -930,7 +973,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                     }
                 }
                 if (pick >= 0) state = 0;
-                else if (s_nctx == 0 && ld_relaxed_u32(p.counter) >= (unsigned)p.ntasks &&
+                else if (s_nctx == 0 && claimed >= (unsigned)p.ntasks &&
                          ld_relaxed_u32(p.tiles_done) >= (unsigned)p.ntiles_total) state = 3;
             }
             s_state = state; s_pick = pick; s_pop = e;
@@ -954,15 +997,22 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         spins = 0;
 
         if (state == 1) {
-            // ================= A: quadrant tasks from the ready ring.  The accumulator of the live far part,
-            // if any, stays in its registers meanwhile: the quadrant task takes the shared memory only.
+            // ================= A: cells from the ready ring.  The accumulator of the live far part, if any, stays in
+            // its registers meanwhile: a cell takes the shared memory only.
             unsigned e = s_pop;
+            int vq = FAR_CTX;                                  // slot of the descriptor; the next cell's goes into the other one
             while (e != 0u) {
-                const TiledKernelParams &pq = VIEW(FAR_CTX);
-                const int q = (int)((e >> 29) & 3u);
-                const int I = BATCHED ? (int)((e >> 8) & 255u) : (int)((e >> 15) & 0x3fffu);
-                const int J = BATCHED ? (int)(e & 255u) : (int)(e & 0x7fffu);
-                sweep_quadrant(I, J, q, smem, pq, max_abs_e);
+                const TiledKernelParams &pq = VIEW(vq);
+                const unsigned cell = BATCHED ? e & ((1u << p.cell_bits) - 1u) : e & 0x7fffffffu, nc = (unsigned)(TC * pq.ntn);
+                const int r = (int)(cell / nc), c = (int)(cell % nc), I = r / TC, J = c / TC;
+                // one thread, in the last leaf-wave: the next cell.  With far parts in hand, back to the top of the loop after every cell (see there).
+                auto next = [&]() {
+                    unsigned en = 0u;
+                    if (s_nctx == 0 && (int)ld_relaxed_u32(reinterpret_cast<unsigned *>(p.q_avail)) > 0) en = ready_pop(p);
+                    if (en != 0u) load_view(2 * FAR_CTX + 1 - vq, entry_matrix(en));
+                    s_pop = en;
+                };
+                sweep_cell(r, c, smem, pq, max_abs_e, next);
 #ifdef TILED_STATS
                 if (tid == 0) g_ts[15] += 1;
 #endif
@@ -971,33 +1021,26 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                     if (lane == 0 && max_abs_e > 0.0) atomic_max_nonneg_double(pq.max_abs_e, max_abs_e);
                     max_abs_e = 0.0;
                 }
-                // arrivals at everything this quadrant feeds, one per thread (each is a dependent global
-                // atomic round trip); sweep_quadrant ended with a barrier, so each arriving thread's fence
-                // covers the whole CTA's results
-                if (tid < 8) {
+                // everything is stored: sweep_cell ended with a barrier, so a fence of one thread covers the whole CTA's results
+                if (tid == 3 * 32) {
                     __threadfence();
-                    if (tid == 6) {
-                        unsigned done = atomicAdd(pq.quad_done + (long)I * pq.ntn + J, 1u);
-                        const unsigned nquad = (pq.m - I * T > Q ? 2u : 1u) * (pq.n - J * T > Q ? 2u : 1u);
-                        if (done + 1u == nquad) {   // tile swept: far parts that list it as a source may go on
-                            __threadfence();
-                            st_release_u32(pq.flagS + CI((long)I * pq.ntn + J, (long)pq.ntm * pq.ntn, 129), 1u);
-                            atomicAdd(pq.rowdone + CI(I, pq.ntm, 130), 1u);
-                            atomicAdd(p.tiles_done, 1u);
-                        }
+                    const unsigned done = atomicAdd(pq.cells_done + (long)I * pq.ntn + J, 1u);
+                    const unsigned ncells = (unsigned)(min(TC, (pq.m - I * T + S - 1) / S) * min(TC, (pq.n - J * T + S - 1) / S));
+                    if (done + 1u == ncells) {   // tile swept: far parts that list it as a source may go on
+                        __threadfence();
+                        st_release_u32(pq.flagS + CI((long)I * pq.ntn + J, (long)pq.ntm * pq.ntn, 129), 1u);
+                        atomicAdd(pq.rowdone + CI(I, pq.ntm, 130), 1u);
+                        atomicAdd(p.tiles_done, 1u);
                     }
                 }
-                __syncthreads();
-                if (tid == 0) {
-                    // with far parts in hand, go back to the top of the loop after every task (see there)
-                    const unsigned en = s_nctx > 0 ? 0u : await_panels(ready_pop(p));
-                    if (en != 0u) load_view(FAR_CTX, entry_matrix(en));
-                    s_pop = en;
+                if constexpr (PANELS) {
+                    if (tid == 0) s_pop = await_panels(s_pop);
+                    __syncthreads();
                 }
-                __syncthreads();
                 e = s_pop;
+                vq = 2 * FAR_CTX + 1 - vq;
+                SC_MARK(0);
             }
-            SC_MARK(0);
             continue;
         }
 
@@ -1037,14 +1080,11 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
             new_pos = upto;
         }
         if (new_pos >= f_nfar) {
-            // far part complete: park the sum (zeros included: the quadrant tasks start from it) and
-            // announce it to the four quadrants of its tile; drop the context
+            // far part complete: park the sum (zeros included: the cells start from it) and
+            // announce it to the cells of its tile; drop the context
             store_acc(acc, tile_region(k), pk.np, wm, wn, g, t);
             __syncthreads();
-            if (tid < 4) {
-                __threadfence();
-                quadrant_arrive(pk, f_I, f_J, tid);
-            }
+            if (tid < TC) far_arrive(pk, f_I, f_J, tid);
             if (tid == 0) {
                 const int n = s_nctx;
                 for (int c = k; c + 1 < n; ++c)
@@ -1060,14 +1100,12 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
 
 #ifdef TILED_STATS
     if (tid == 0 && (blockIdx.x % 37) == 0)
-        printf("cta %3d scheduler: quadrant tasks %lld far main loop %lld far park/scan %lld idle %lld looking %lld\n", (int)blockIdx.x,
+        printf("cta %3d scheduler: cells %lld far main loop %lld far park/scan %lld idle %lld looking %lld\n", (int)blockIdx.x,
                g_sched[0], g_sched[1], g_sched[2], g_sched[3], g_sched[4]);
     if (tid == 0 && (blockIdx.x % 37) == 0 && g_ts[15] > 0) {
         const long long n_ = g_ts[15];
-        printf("cta %3d tasks %lld | per task: nearpull %lld load %lld tables %lld | lw0-7: barA %lld pull %lld barB %lld leafpull %lld "
-               "sweep %lld store %lld | lw8-14: bar %lld leafpull %lld sweep %lld store %lld | end %lld\n",
-               (int)blockIdx.x, n_, g_ts[0] / n_, g_ts[1] / n_, g_ts[2] / n_, g_ts[3] / n_, g_ts[4] / n_, g_ts[5] / n_, g_ts[6] / n_,
-               g_ts[7] / n_, g_ts[8] / n_, g_ts[9] / n_, g_ts[10] / n_, g_ts[11] / n_, g_ts[12] / n_, g_ts[13] / n_);
+        printf("cta %3d cells %lld | per cell: operands %lld pulls %lld finish + first block %lld | leaf-waves: barriers %lld sweep %lld | end %lld\n",
+               (int)blockIdx.x, n_, g_ts[0] / n_, g_ts[1] / n_, g_ts[2] / n_, g_ts[3] / n_, g_ts[5] / n_, g_ts[6] / n_);
     }
 #endif
     if constexpr (!BATCHED) {
@@ -1085,6 +1123,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
 #undef VIEW
 
 // ---------------------------------------------------------------------------------------------
+constexpr int NEAR_TILES = 2;       // 1 makes cells a fifth shorter, but a far part's last source then is swept just before it is needed (4096 x 4096: 6.58 -> 6.74 ms)
 static size_t pad256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct TiledLayout {
@@ -1100,8 +1139,8 @@ static TiledLayout tiled_layout(int m, int n) {
     l.q_off = 256;
     l.flags_off = l.q_off + 4096 * sizeof(unsigned);
     l.quad_off = l.flags_off + pad256(tiles * sizeof(unsigned));
-    l.qdep_off = l.quad_off + pad256(tiles * sizeof(unsigned));
-    l.qprog_off = l.qdep_off + pad256(4 * tiles * sizeof(unsigned));
+    l.qdep_off = l.quad_off + pad256(tiles * sizeof(unsigned));            // 16 cells a tile, a byte each
+    l.qprog_off = l.qdep_off + pad256(4 * tiles * sizeof(unsigned));       // likewise
     l.rowdone_off = l.qprog_off + pad256(4 * tiles * sizeof(unsigned));
     l.e_off = l.rowdone_off + pad256((size_t)l.ntm * sizeof(unsigned));
     l.c_off = l.e_off + pad256(mat);
@@ -1169,7 +1208,7 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
     TiledLayout l = tiled_layout(in.m, in.n);
     if (ws_bytes < l.total) return GPTQ2D_ERR_WORKSPACE;
     {
-        // large resident problems: far contractions and quadrant tasks side by side on every SM
+        // large resident problems: far contractions and quadrant tasks side by side on every SM (round_fused.cu)
         const int st = launch_round_fused(in, ws, ws_bytes, stream, false);
         if (st != -1) return st;
     }
@@ -1183,6 +1222,7 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
     p.ntasks = 2 * l.ntm * l.ntn;
     p.ntiles_total = l.ntm * l.ntn;
     p.batch_index = -1;
+    p.near = NEAR_TILES;
     p.np = (long)l.ntn * T;
     p.X = in.X; p.ldx = in.ldx; p.L = in.L; p.ldl = in.ldl; p.U = in.U; p.ldu = in.ldu;
     p.Z = in.Z; p.ldz = in.ldz; p.Euser = in.E; p.lde = in.lde;
@@ -1191,13 +1231,14 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
     p.q_head = reinterpret_cast<unsigned *>(w) + 2;
     p.q_tail = reinterpret_cast<unsigned *>(w) + 3;
     p.tiles_done = reinterpret_cast<unsigned *>(w) + 4;
+    p.q_avail = reinterpret_cast<int *>(w + 128);
     p.q_slots = reinterpret_cast<unsigned *>(w + l.q_off);
     p.qmask = QCAP - 1;
     p.max_abs_e = workspace_max_abs_e(ws);
     p.flagS = reinterpret_cast<unsigned *>(w + l.flags_off);
-    p.quad_done = reinterpret_cast<unsigned *>(w + l.quad_off);
-    p.qdep = reinterpret_cast<unsigned *>(w + l.qdep_off);
-    p.qprog = reinterpret_cast<unsigned *>(w + l.qprog_off);
+    p.cells_done = reinterpret_cast<unsigned *>(w + l.quad_off);
+    p.cdep = reinterpret_cast<unsigned *>(w + l.qdep_off);
+    p.cprog = reinterpret_cast<unsigned char *>(w + l.qprog_off);
     p.rowdone = reinterpret_cast<unsigned *>(w + l.rowdone_off);
     p.Ebuf = reinterpret_cast<double *>(w + l.e_off);
     p.Cbuf = reinterpret_cast<double *>(w + l.c_off);
@@ -1225,6 +1266,10 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
 
 
 // ---------------------------------------------------------------------------------------------
+// most bits of a cell index in a batched launch (tests; 31: no limit of its own)
+static std::atomic<long> g_batch_cell_bits{31};
+void round_batched_set_cell_bits(long bits) { g_batch_cell_bits.store(bits > 0 && bits < 31 ? bits : 31); }
+
 // Batched launch: every matrix keeps its own flags, counters and E / C buffers; claim counter,
 // ready ring and abort word are shared.  Workspace: [header | ring | max|E| per matrix | flags of
 // all matrices] (cleared per call) [descriptors | far-part table] (written per call from the
@@ -1286,6 +1331,17 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     unsigned *table = reinterpret_cast<unsigned *>(stage.data() + (l.table_off - l.desc_off));
     size_t foff = l.flags_off, boff = l.bufs_off;
     int max_waves = 0;
+    // A ring entry has 31 bits for matrix and cell.  With more than 2048 matrices the index of a cell may not fit beside that of the
+    // matrix; one that large (more than 2^18 cells, 16384 x 16384) fills the GPU and is swept in a launch of its own.
+    int cell_bits = 31, big = 0;
+    while (cell_bits > 0 && (1l << (31 - cell_bits)) < (long)count) --cell_bits;
+    cell_bits = std::min(cell_bits, (int)g_batch_cell_bits.load());
+    // With cells enough for every SM to have two at a time, no far part is urgent: cells pull from one tile back only (64 of 256 x 256
+    // and 256 x 512: 1 % faster; a single matrix: NEAR_TILES).
+    long ready = 0;
+    for (int b = 0; b < count; ++b) ready += TC * ((std::min(pr[b].m, pr[b].n) + T - 1) / T);
+    const int near = ready >= 296 ? 1 : NEAR_TILES;
+    auto alone = [&](const TiledKernelParams &d) { return (long)TC * d.ntm * TC * d.ntn > (1l << cell_bits); };
     for (int b = 0; b < count; ++b) {
         const TiledParams &in = pr[b];
         TiledLayout t = tiled_layout(in.m, in.n);
@@ -1298,12 +1354,13 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         d.X = in.X; d.ldx = in.ldx; d.L = in.L; d.ldl = in.ldl; d.U = in.U; d.ldu = in.ldu;
         d.Z = in.Z; d.ldz = in.ldz; d.Euser = in.E; d.lde = in.lde;
         d.counter = hdr; d.abort = hdr + 1; d.q_head = hdr + 2; d.q_tail = hdr + 3; d.tiles_done = hdr + 4;
+        d.q_avail = reinterpret_cast<int *>(w + 128);
         d.q_slots = reinterpret_cast<unsigned *>(w + 256);
         d.qmask = l.qcap - 1;
         d.flagS = reinterpret_cast<unsigned *>(w + foff); foff += pad256(tiles * sizeof(unsigned));
-        d.quad_done = reinterpret_cast<unsigned *>(w + foff); foff += pad256(tiles * sizeof(unsigned));
-        d.qdep = reinterpret_cast<unsigned *>(w + foff); foff += pad256(4 * tiles * sizeof(unsigned));
-        d.qprog = reinterpret_cast<unsigned *>(w + foff); foff += pad256(4 * tiles * sizeof(unsigned));
+        d.cells_done = reinterpret_cast<unsigned *>(w + foff); foff += pad256(tiles * sizeof(unsigned));
+        d.cdep = reinterpret_cast<unsigned *>(w + foff); foff += pad256(4 * tiles * sizeof(unsigned));
+        d.cprog = reinterpret_cast<unsigned char *>(w + foff); foff += pad256(4 * tiles * sizeof(unsigned));
         d.rowdone = reinterpret_cast<unsigned *>(w + foff); foff += pad256((size_t)t.ntm * sizeof(unsigned));
         d.Ebuf = reinterpret_cast<double *>(w + boff); boff += mat;
         d.Cbuf = reinterpret_cast<double *>(w + boff); boff += mat;
@@ -1312,10 +1369,13 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         d.l_al16 = ((reinterpret_cast<uintptr_t>(in.L) & 15) == 0) && ((in.ldl & 1) == 0);
         d.u_al16 = ((reinterpret_cast<uintptr_t>(in.U) & 15) == 0) && ((in.ldu & 1) == 0);
         d.batch_index = b;
+        d.cell_bits = cell_bits;
+        d.near = near;
         d.report_index = b;
         d.spin_limit = d.panel_spin_limit = SPIN_LIMIT;
         d.ntiles_total = (int)tiles;
         desc[b] = d;
+        if (alone(d)) { ++big; l.ntasks -= 2 * (long)tiles; l.ntiles -= (long)tiles; continue; }
         if (t.ntm + t.ntn - 1 > max_waves) max_waves = t.ntm + t.ntn - 1;
     }
     // claim order: tile-wave by tile-wave over all matrices; inside a matrix' wave as decode_task lists them
@@ -1323,7 +1383,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     for (int wv = 0; wv < max_waves; ++wv)
         for (int b = 0; b < count; ++b) {
             const int ntm = desc[b].ntm, ntn = desc[b].ntn;
-            if (wv >= ntm + ntn - 1) continue;
+            if (wv >= ntm + ntn - 1 || (big && alone(desc[b]))) continue;
             const int lo = wv - ntn + 1 > 0 ? wv - ntn + 1 : 0, hi = wv < ntm - 1 ? wv : ntm - 1;
             for (int k = 0; k <= hi - lo; ++k)
                 for (int type = 0; type < 2; ++type) {
@@ -1338,9 +1398,11 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     p.ntiles_total = (int)l.ntiles;
     p.batch_index = -1;
     p.counter = hdr; p.abort = hdr + 1; p.q_head = hdr + 2; p.q_tail = hdr + 3; p.tiles_done = hdr + 4;
+    p.q_avail = reinterpret_cast<int *>(w + 128);
     p.q_slots = reinterpret_cast<unsigned *>(w + 256);
     p.qmask = l.qcap - 1;
     p.info = info;
+    p.cell_bits = cell_bits;
     p.probs = reinterpret_cast<const TiledKernelParams *>(w + l.desc_off);
     p.far_tasks = reinterpret_cast<const unsigned *>(w + l.table_off);
     p.spin_limit = p.panel_spin_limit = SPIN_LIMIT;
@@ -1352,14 +1414,28 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
-    if (cudaFuncSetAttribute(round_tiled_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TILED_SMEM) != cudaSuccess)
-        return GPTQ2D_ERR_CUDA;
-    int grid = (long)sms < l.ntasks ? sms : (int)l.ntasks;
-    void *args[] = {&p};
-    if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<true, false>, dim3(grid), dim3(TILED_THREADS), args,
-                                    TILED_SMEM, stream) != cudaSuccess)
-        return GPTQ2D_ERR_CUDA;
+    for (int b = 0; big && b < count; ++b) {
+        TiledKernelParams d = desc[b];
+        if (!alone(d)) continue;
+        d.batch_index = -1;
+        if (cudaFuncSetAttribute(round_tiled_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess)
+            return GPTQ2D_ERR_CUDA;
+        void *own[] = {&d};
+        if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<false, false>, dim3(std::min(sms, d.ntasks)), dim3(TILED_THREADS), own,
+                                        TILED_SMEM, stream) != cudaSuccess)
+            return GPTQ2D_ERR_CUDA;
+        if (cudaMemsetAsync(w, 0, l.maxe_off, stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;      // scheduler words and ring
+    }
+    if (l.ntasks > 0) {
+        if (cudaFuncSetAttribute(round_tiled_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TILED_SMEM) != cudaSuccess)
+            return GPTQ2D_ERR_CUDA;
+        int grid = (long)sms < l.ntasks ? sms : (int)l.ntasks;
+        void *args[] = {&p};
+        if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<true, false>, dim3(grid), dim3(TILED_THREADS), args,
+                                        TILED_SMEM, stream) != cudaSuccess)
+            return GPTQ2D_ERR_CUDA;
+    }
     if (min_margin) {
         batched_margin_kernel<<<(count + 255) / 256, 256, 0, stream>>>(
             reinterpret_cast<const double *>(w + l.maxe_off), min_margin, count);
@@ -1483,17 +1559,19 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         d.Ebuf = E + r * np + c; d.Cbuf = C + r * np + c;
         unsigned *hdr = reinterpret_cast<unsigned *>(w + sl.hdr_off[launch]);
         d.counter = hdr; d.abort = hdr + 1; d.q_head = hdr + 2; d.q_tail = hdr + 3; d.tiles_done = hdr + 4;
+        d.q_avail = reinterpret_cast<int *>(hdr + 32);
         d.q_slots = hdr + 64; d.qmask = QCAP - 1;
         char *f = w + sl.flags_off[bi * 2 + bj];
         d.flagS = reinterpret_cast<unsigned *>(f); f += pad256(tiles * sizeof(unsigned));
-        d.quad_done = reinterpret_cast<unsigned *>(f); f += pad256(tiles * sizeof(unsigned));
-        d.qdep = reinterpret_cast<unsigned *>(f); f += pad256(4 * tiles * sizeof(unsigned));
-        d.qprog = reinterpret_cast<unsigned *>(f); f += pad256(4 * tiles * sizeof(unsigned));
+        d.cells_done = reinterpret_cast<unsigned *>(f); f += pad256(tiles * sizeof(unsigned));
+        d.cdep = reinterpret_cast<unsigned *>(f); f += pad256(4 * tiles * sizeof(unsigned));
+        d.cprog = reinterpret_cast<unsigned char *>(f); f += pad256(4 * tiles * sizeof(unsigned));
         d.rowdone = reinterpret_cast<unsigned *>(f);
         d.max_abs_e = workspace_max_abs_e(ws);
         d.info = reinterpret_cast<int *>(hdr + 8);
         d.l_al16 = ((reinterpret_cast<uintptr_t>(d.L) & 15) == 0) && ((in.ldl & 1) == 0);
         d.u_al16 = ((reinterpret_cast<uintptr_t>(d.U) & 15) == 0) && ((in.ldu & 1) == 0);
+        d.near = NEAR_TILES;
         d.row_off = (int)r; d.col_off = (int)c; d.preloaded = preloaded;
         d.batch_index = -1;
         d.spin_limit = d.panel_spin_limit = SPIN_LIMIT;
@@ -1514,6 +1592,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
     {
         TiledKernelParams a = block(0, 1, 1, 2), b = block(1, 0, 1, 1), p{};
         a.batch_index = 0; b.batch_index = 1;
+        a.cell_bits = b.cell_bits = p.cell_bits = 30;
         TiledKernelParams *desc = reinterpret_cast<TiledKernelParams *>(w + sl.desc_off);
         unsigned *table = reinterpret_cast<unsigned *>(w + sl.table_off);
         split_pair_kernel<<<1, 256, 0, stream>>>(a, b, desc, table);
@@ -1521,7 +1600,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         p.ntasks = a.ntasks + b.ntasks; p.ntiles_total = a.ntiles_total + b.ntiles_total;
         p.batch_index = -1;
         p.counter = a.counter; p.abort = a.abort; p.q_head = a.q_head; p.q_tail = a.q_tail; p.tiles_done = a.tiles_done;
-        p.q_slots = a.q_slots; p.qmask = a.qmask;
+        p.q_avail = a.q_avail; p.q_slots = a.q_slots; p.qmask = a.qmask;
         p.info = a.info;
         p.probs = desc; p.far_tasks = table;
         p.spin_limit = p.panel_spin_limit = SPIN_LIMIT;
