@@ -24,8 +24,8 @@
 //    3 + b).  A cell counts arrivals from the two far parts of its tile and from (r-1, c) and
 //    (r, c-1) begun; the last arrival puts it on a global ready ring.  A running cell
 //    waits -- bounded -- only on cells above it / to its left, which are running by then (or done).
-// Every CTA serves the ready ring first: at the top of its loop, while a far part waits, and
-// every 64 chunks of a far part (its accumulator stays in registers meanwhile).
+// A CTA holds one far part (its accumulator stays in registers) and goes on with it whenever a source
+// tile is there; otherwise it serves the ready ring.  It looks again every 16 chunks of a far part.
 // A far part only ever waits on tiles of earlier waves, whose far parts were claimed earlier and
 // whose cells wait on running tasks only, so the earliest unfinished work can always progress.
 //
@@ -817,16 +817,13 @@ __device__ __forceinline__ void load_acc(Acc &acc, const double *srcT, long np, 
         }
 }
 
-constexpr int FAR_RUN_CHUNKS = 64;      // a far part looks at the ready ring every this many K = 128 chunks
-constexpr unsigned IDLE_SLEEP_NS = 100; // pause of a CTA that found nothing to do (100 - 1600 ns and far runs of 8 - 64 chunks all time within 1 %)
-
-constexpr int FAR_CTX = 2;       // far parts a CTA may hold at once (one live in registers, the others parked)
+constexpr int FAR_RUN_CHUNKS = 16;      // a far part looks at its flags again every this many K = 128 chunks (4, 8, 16, 64 all time within 2 %)
+constexpr unsigned IDLE_SLEEP_NS = 50;  // pause of a CTA that found nothing to do (0 - 100 ns time within 1 %)
 
 // The persistent scheduler loop.  BATCHED = false: one matrix, described by the kernel argument
 // itself.  BATCHED = true: many matrices in one launch; the kernel argument holds what they share
 // (claim counter, ready ring, abort word, totals) and each task works on a shared-memory copy of
-// its matrix' descriptor (slots 0..FAR_CTX-1: the far contexts, the two behind them: a cell and
-// the one after it).
+// its matrix' descriptor (slot 0: the far part, 1 and 2: a cell and the one after it).
 // PANELS = true (single matrix only): the inputs are still being copied in while the kernel runs, in
 // blocks of COPY_BLOCK_TILES x COPY_BLOCK_TILES tiles and in the order the wavefront needs them: step
 // s brings the blocks of X on block anti-diagonal s, the block row s of L and the block column s of
@@ -836,17 +833,16 @@ template <bool BATCHED, bool PANELS>
 __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKernelParams p) {
     extern __shared__ __align__(16) double smem[];
     __shared__ int s_task[4];
-    __shared__ int s_ctx[FAR_CTX][7];      // far-part contexts, oldest first: type, I, J, pos, nfar, task, view slot
-    __shared__ int s_nctx, s_pick, s_state;
+    __shared__ int s_far[5];               // the CTA's far part: type, I, J, next source, number of sources
+    __shared__ int s_has, s_state;         // s_has: it holds one
     __shared__ unsigned s_pop;
     __shared__ double s_red[TILED_THREADS / 32];
-    __shared__ TiledKernelParams s_view[BATCHED ? FAR_CTX + 2 : 1];
-    static_assert(!BATCHED || FAR_CTX == 2, "view slots of far contexts are handed out as 0 / 1");
+    __shared__ TiledKernelParams s_view[BATCHED ? 3 : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wm = warp >> 2, wn = warp & 3, g = lane >> 2, t = lane & 3;
     CHECKED_SET_INFO(p.info);            // (checked builds: every CTA writes the same pointer before its first barrier)
     double max_abs_e = 0.0;
-    int cur = -1;                  // context whose accumulator is live in registers (uniform), -1: none
+    bool fresh = true;             // the next far part's accumulator is not set up yet (uniform)
     unsigned long long spins = 0;
     Acc acc;
     acc.zero();
@@ -860,9 +856,9 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
 #define SC_MARK(slot) do { if (tid == 0) { const long long n_ = clock64(); g_sched[slot] += n_ - sc_t; sc_t = n_; } } while (0)
 #endif
     if (tid == 0) {
-        s_nctx = 0;
+        s_has = 0;
         if (BATCHED)
-            for (int k = 0; k < FAR_CTX + 2; ++k) s_view[k].batch_index = -1;
+            for (int k = 0; k < 3; ++k) s_view[k].batch_index = -1;
     }
 
     // the descriptor a task works on: the kernel argument itself for a single matrix (spelled so that the
@@ -905,78 +901,55 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         }
         return e;
     };
-    auto tile_region = [&](int k) {
-        const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
-        return (s_ctx[k][0] == 0 ? pk.Cbuf : pk.Ebuf) +
-               CI((long)s_ctx[k][1] * T * pk.np + (long)s_ctx[k][2] * T, (long)(pk.ntm - 1) * T * pk.np + (long)(pk.ntn - 1) * T + 1, 128);
+    auto tile_region = [&]() {
+        const TiledKernelParams &pk = VIEW(0);
+        return (s_far[0] == 0 ? pk.Cbuf : pk.Ebuf) +
+               CI((long)s_far[1] * T * pk.np + (long)s_far[2] * T, (long)(pk.ntm - 1) * T * pk.np + (long)(pk.ntn - 1) * T + 1, 128);
+    };
+    // thread 0: the far part in hand can go on (a Cd part reads L in the block row of I, an Rt part U in the block column of J)
+    auto far_ready = [&]() -> bool {
+        const TiledKernelParams &pk = VIEW(0);
+        const int ty = s_far[0], pos = s_far[3];
+        const unsigned *fl = ty == 0 ? pk.flagS + (long)pos * pk.ntn + s_far[2] : pk.flagS + (long)s_far[1] * pk.ntn + pos;
+        return (pos >= s_far[4] || ld_acquire_u32(fl) != 0u) && panels_arrived(((ty == 0 ? s_far[1] : s_far[2]) >> COPY_BLOCK_TILES_LOG2) + 1);
     };
 
     for (;;) {
-        // ---- thread 0 looks for work: a ready cell first, else the oldest far part that can
-        // go on, else (room and tasks left) a new far part.  s_state: 0 run far part s_pick, 1 serve the
-        // ring, 2 nothing to do right now, 3 all tiles swept, 4 abort.
+        // ---- thread 0 looks for work: the CTA's far part if it can go on (the cells of its tile cannot start without it, and other CTAs
+        // can serve the ring), else a ready cell, else (none in hand and tasks left) a new far part.  One far part a CTA: with two or more it
+        // is often in a long run of one when the other, which cells wait for, could go on (1024 x 4096, cells first and two parts / far
+        // parts first and two / one: 1758 / 1640 / 1531 us; 4096 x 4096 6326 / 6225 / 6176).
+        // s_state: 0 run the far part, 1 serve the ring, 2 nothing to do right now, 3 all tiles swept, 4 abort.
         __syncthreads();
         if (tid == 0) {
-            int state = 2, pick = -1;
+            int state = 2;
             unsigned e = 0u;
             const unsigned aborted = ld_relaxed_u32(p.abort), claimed = ld_relaxed_u32(p.counter);       // one trip to L2 for all three
             const int avail = (int)ld_relaxed_u32(reinterpret_cast<unsigned *>(p.q_avail));
-            // A far part of this CTA that is at most two chunks from done and can go on comes before
-            // everything else: the cells of its tile cannot start without it, and other
-            // CTAs can serve the ring.
-            for (int k = 0; k < s_nctx && pick < 0; ++k) {
-                const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
-                const int ty = s_ctx[k][0], pos = s_ctx[k][3], left = s_ctx[k][4] - pos;
-                if (left < 1 || left > 2) continue;
-                const unsigned *fl = ty == 0 ? pk.flagS + (long)pos * pk.ntn + s_ctx[k][2]
-                                             : pk.flagS + (long)s_ctx[k][1] * pk.ntn + pos;
-                if (ld_acquire_u32(fl) != 0u &&
-                    panels_arrived(((ty == 0 ? s_ctx[k][1] : s_ctx[k][2]) >> COPY_BLOCK_TILES_LOG2) + 1))
-                    pick = k;
-            }
             if (aborted != 0u) state = 4;
-            else if (pick >= 0) state = 0;
+            else if (s_has && far_ready()) state = 0;
             else if (avail > 0 && (e = await_panels(ready_pop(p))) != 0u) {
                 state = 1;
-                load_view(FAR_CTX, entry_matrix(e));
-            } else {
-                int n = s_nctx;
-                for (int k = 0; k < n && pick < 0; ++k) {
-                    const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
-                    const int ty = s_ctx[k][0], pos = s_ctx[k][3];
-                    const unsigned *fl = ty == 0 ? pk.flagS + (long)pos * pk.ntn + s_ctx[k][2]
-                                                 : pk.flagS + (long)s_ctx[k][1] * pk.ntn + pos;
-                    // a Cd part reads L in the block row of I, an Rt part U in the block column of J
-                    if ((pos >= s_ctx[k][4] || ld_acquire_u32(fl) != 0u) &&
-                        panels_arrived(((ty == 0 ? s_ctx[k][1] : s_ctx[k][2]) >> COPY_BLOCK_TILES_LOG2) + 1))
-                        pick = k;
-                }
-                if (pick < 0 && n < FAR_CTX && claimed < (unsigned)p.ntasks) {
-                    int task = (int)atomicAdd(p.counter, 1u);
-                    if (task < p.ntasks) {
-                        int ty, fi, fj, slot = 0;
-                        if constexpr (BATCHED) {
-                            const unsigned ft = __ldg(p.far_tasks + task);
-                            ty = (int)((ft >> 16) & 1u); fi = (int)((ft >> 8) & 255u); fj = (int)(ft & 255u);
-                            slot = n == 0 ? 0 : 1 - s_ctx[0][6];
-                            load_view(slot, (int)(ft >> 17));
-                        } else {
-                            decode_task(task, p.ntm, p.ntn, ty, fi, fj);
-                        }
-                        const TiledKernelParams &pk = VIEW(slot);
-                        s_ctx[n][0] = ty; s_ctx[n][1] = fi; s_ctx[n][2] = fj; s_ctx[n][3] = 0;
-                        s_ctx[n][4] = max(0, (ty == 0 ? fi : fj) - pk.near); s_ctx[n][5] = task; s_ctx[n][6] = slot;
-                        s_nctx = n + 1;
-                        const unsigned *fl = ty == 0 ? pk.flagS + fj : pk.flagS + (long)fi * pk.ntn;
-                        if ((s_ctx[n][4] == 0 || ld_acquire_u32(fl) != 0u) && panels_arrived(((ty == 0 ? fi : fj) >> COPY_BLOCK_TILES_LOG2) + 1))
-                            pick = n;
+                load_view(1, entry_matrix(e));
+            } else if (!s_has) {
+                int task = p.ntasks;
+                if (claimed < (unsigned)p.ntasks) task = (int)atomicAdd(p.counter, 1u);
+                if (task < p.ntasks) {
+                    int ty, fi, fj;
+                    if constexpr (BATCHED) {
+                        const unsigned ft = __ldg(p.far_tasks + task);
+                        ty = (int)((ft >> 16) & 1u); fi = (int)((ft >> 8) & 255u); fj = (int)(ft & 255u);
+                        load_view(0, (int)(ft >> 17));
+                    } else {
+                        decode_task(task, p.ntm, p.ntn, ty, fi, fj);
                     }
-                }
-                if (pick >= 0) state = 0;
-                else if (s_nctx == 0 && claimed >= (unsigned)p.ntasks &&
-                         ld_relaxed_u32(p.tiles_done) >= (unsigned)p.ntiles_total) state = 3;
+                    s_far[0] = ty; s_far[1] = fi; s_far[2] = fj; s_far[3] = 0;
+                    s_far[4] = max(0, (ty == 0 ? fi : fj) - VIEW(0).near);
+                    s_has = 1;
+                    if (far_ready()) state = 0;
+                } else if (ld_relaxed_u32(p.tiles_done) >= (unsigned)p.ntiles_total) state = 3;
             }
-            s_state = state; s_pick = pick; s_pop = e;
+            s_state = state; s_pop = e;
         }
         __syncthreads();
         const int state = s_state;
@@ -985,12 +958,12 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         if (state == 2) {
             if (++spins > p.spin_limit) {
                 if (tid == 0) {
-                    report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -4, (int)blockIdx.x, s_nctx);
+                    report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -4, (int)blockIdx.x, s_has);
                     atomicExch(p.abort, 1u);
                 }
                 break;
             }
-            __nanosleep(s_nctx == 0 ? IDLE_SLEEP_NS : 100);
+            __nanosleep(IDLE_SLEEP_NS);
             SC_MARK(3);
             continue;
         }
@@ -1000,16 +973,16 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
             // ================= A: cells from the ready ring.  The accumulator of the live far part, if any, stays in
             // its registers meanwhile: a cell takes the shared memory only.
             unsigned e = s_pop;
-            int vq = FAR_CTX;                                  // slot of the descriptor; the next cell's goes into the other one
+            int vq = 1;                                        // slot of the descriptor; the next cell's goes into the other one
             while (e != 0u) {
                 const TiledKernelParams &pq = VIEW(vq);
                 const unsigned cell = BATCHED ? e & ((1u << p.cell_bits) - 1u) : e & 0x7fffffffu, nc = (unsigned)(TC * pq.ntn);
                 const int r = (int)(cell / nc), c = (int)(cell % nc), I = r / TC, J = c / TC;
-                // one thread, in the last leaf-wave: the next cell.  With far parts in hand, back to the top of the loop after every cell (see there).
+                // one thread, in the last leaf-wave: the next cell.  With a far part in hand, back to the top of the loop after every cell (see there).
                 auto next = [&]() {
                     unsigned en = 0u;
-                    if (s_nctx == 0 && (int)ld_relaxed_u32(reinterpret_cast<unsigned *>(p.q_avail)) > 0) en = ready_pop(p);
-                    if (en != 0u) load_view(2 * FAR_CTX + 1 - vq, entry_matrix(en));
+                    if (!s_has && (int)ld_relaxed_u32(reinterpret_cast<unsigned *>(p.q_avail)) > 0) en = ready_pop(p);
+                    if (en != 0u) load_view(3 - vq, entry_matrix(en));
                     s_pop = en;
                 };
                 sweep_cell(r, c, smem, pq, max_abs_e, next);
@@ -1038,22 +1011,20 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                     __syncthreads();
                 }
                 e = s_pop;
-                vq = 2 * FAR_CTX + 1 - vq;
+                vq = 3 - vq;
                 SC_MARK(0);
             }
             continue;
         }
 
-        // ================= B: far part s_pick (every source tile of the contraction except the two nearest)
-        const int k = s_pick;
-        const TiledKernelParams &pk = VIEW(s_ctx[k][6]);
-        if (k != cur) {
-            if (cur >= 0 && s_ctx[cur][3] > 0) store_acc(acc, tile_region(cur), VIEW(s_ctx[cur][6]).np, wm, wn, g, t);
-            if (s_ctx[k][3] > 0 || ((pk.preloaded >> s_ctx[k][0]) & 1)) load_acc(acc, tile_region(k), pk.np, wm, wn, g, t);
+        // ================= B: the far part (every source tile of the contraction except the nearest)
+        const TiledKernelParams &pk = VIEW(0);
+        const int f_type = s_far[0], f_I = s_far[1], f_J = s_far[2], f_pos = s_far[3], f_nfar = s_far[4];
+        if (fresh) {
+            if ((pk.preloaded >> f_type) & 1) load_acc(acc, tile_region(), pk.np, wm, wn, g, t);
             else acc.zero();
-            cur = k;
+            fresh = false;
         }
-        const int f_type = s_ctx[k][0], f_I = s_ctx[k][1], f_J = s_ctx[k][2], f_pos = s_ctx[k][3], f_nfar = s_ctx[k][4];
         int new_pos = f_pos;
         if (f_pos < f_nfar) {
             const unsigned *flags = f_type == 0 ? pk.flagS + f_J : pk.flagS + (long)f_I * pk.ntn;
@@ -1081,19 +1052,14 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         }
         if (new_pos >= f_nfar) {
             // far part complete: park the sum (zeros included: the cells start from it) and
-            // announce it to the cells of its tile; drop the context
-            store_acc(acc, tile_region(k), pk.np, wm, wn, g, t);
+            // announce it to the cells of its tile
+            store_acc(acc, tile_region(), pk.np, wm, wn, g, t);
             __syncthreads();
             if (tid < TC) far_arrive(pk, f_I, f_J, tid);
-            if (tid == 0) {
-                const int n = s_nctx;
-                for (int c = k; c + 1 < n; ++c)
-                    for (int f = 0; f < 7; ++f) s_ctx[c][f] = s_ctx[c + 1][f];
-                s_nctx = n - 1;
-            }
-            cur = -1;
+            if (tid == 0) s_has = 0;
+            fresh = true;
         } else if (tid == 0) {
-            s_ctx[k][3] = new_pos;
+            s_far[3] = new_pos;
         }
         SC_MARK(2);
     }
