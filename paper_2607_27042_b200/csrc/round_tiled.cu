@@ -241,6 +241,10 @@ __device__ __forceinline__ double ld_relaxed_f64(const double *p) {
     asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
     return v;
 }
+// what ld_relaxed_f64 polls: two entries in one store, each of them whole (a plain store beside polling loads would be a data race)
+__device__ __forceinline__ void st_relaxed_f64x2(double *p, double2 v) {
+    asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};\n" ::"l"(p), "d"(v.x), "d"(v.y) : "memory");
+}
 __device__ __forceinline__ unsigned ld_acquire_u8(const unsigned char *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u8 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
@@ -460,8 +464,8 @@ __device__ __forceinline__ void post_leaf(const double *Ws, const double *Cs, in
     const int lane = threadIdx.x & 31, i = a * 8 + (lane >> 2), j = b * 8 + (lane & 3) * 2;
     double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 133)), c = *reinterpret_cast<const double2 *>(Cs + i * SLD + j);
     e.x = stream_value(e.x); e.y = stream_value(e.y); c.x = stream_value(c.x); c.y = stream_value(c.y);
-    *reinterpret_cast<double2 *>(eQ + i * np + j) = e;
-    *reinterpret_cast<double2 *>(cQ + i * np + j) = c;
+    st_relaxed_f64x2(eQ + i * np + j, e);
+    st_relaxed_f64x2(cQ + i * np + j, c);
 }
 // its Z (and the caller's E) to the output
 __device__ __forceinline__ void store_leaf(const double *Ws, const int *Zs, int a, int b, int row0, int col0, const TiledKernelParams &p, double &max_abs_e) {
