@@ -499,7 +499,9 @@ __device__ __forceinline__ void store_leaf(const double *Ws, const int *Zs, int 
 // the streamed products (four times fewer than in a cell of 64, and off the chain: they share the fp64 pipe with the steps, of
 // which they take a sixth here but all of it there), the pulls of older leaves and the barriers.
 // `next` is called by one thread in the last leaf-wave: it looks for the CTA's next cell.
-template <class Next>
+// PANELS: X is still being copied in while the kernel runs (see round_tiled_kernel), so it must not be read through the read-only path,
+// which may go on serving a line whose other columns arrived later (with odd n a line spans two copy steps).
+template <bool PANELS, class Next>
 __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const TiledKernelParams &p, double &max_abs_e, Next next) {
     double *Ws = smem, *Cs = smem + SMAT, *LU = smem + 2 * SMAT, *La = smem + 3 * SMAT, *Ul = smem + 4 * SMAT;
     double *tabL = smem + CELL_TABS, *tabU = tabL + S * TAB_LD, *xch = smem + CELL_XCH, *ring = smem + CELL_PULL;
@@ -570,7 +572,11 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
             for (int h = 0; h < 2; ++h) {
                 const int gr = row0 + wr + a * 8 + g, gc = col0 + wc + b * 8 + t * 2 + h;
                 acc[a][b][h] = 0.0;
-                xv[a][b][h] = (warp >= 4 && gr < p.m && gc < p.n) ? __ldg(p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122)) : 0.0;
+                xv[a][b][h] = 0.0;
+                if (warp >= 4 && gr < p.m && gc < p.n) {
+                    const double *x = p.X + CI((long)gr * p.ldx + gc, (long)(p.m - 1) * p.ldx + p.n, 122);
+                    xv[a][b][h] = PANELS ? ld_relaxed_f64(x) : __ldg(x);
+                }
             }
     // the copies of a step: `on` per direction; the pointers move on by one source
     const double *lp0 = lsrc0 + fa * S, *lp1 = lsrc1 + fa * S, *ep = esrc + (long)fa * S * np, *qp = csrc + fl * S, *up = usrc + (long)fl * S * p.ldu;
@@ -989,7 +995,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                     if (en != 0u) load_view(3 - vq, entry_matrix(en));
                     s_pop = en;
                 };
-                sweep_cell(r, c, smem, pq, max_abs_e, next);
+                sweep_cell<PANELS>(r, c, smem, pq, max_abs_e, next);
 #ifdef TILED_STATS
                 if (tid == 0) g_ts[15] += 1;
 #endif
