@@ -253,6 +253,11 @@ __device__ __forceinline__ unsigned ld_acquire_u8(const unsigned char *p) {
 __device__ __forceinline__ void st_release_u8(unsigned char *p, unsigned v) {
     asm volatile("st.release.gpu.global.u8 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ unsigned exch_acquire_u32(unsigned *p, unsigned v) {
+    unsigned old;
+    asm volatile("atom.acquire.gpu.global.exch.b32 %0, [%1], %2;\n" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;\n" ::: "memory"); }
 
 // One more poll of a bounded wait; true: give up (the launch is aborted and the caller carries on with whatever is there).
@@ -294,31 +299,42 @@ constexpr unsigned QCAP = 4096;
 // a consumer takes one off it and puts it back if there was none, so that every step is a single atomic addition that
 // cannot fail.  (Claiming by compare-and-swap on the head let one consumer in 600 cycles through, however many there were, and sent
 // the others round again: with it, 64 matrices of 256 x 256 and 256 x 512 took 1850 us instead of 945.)
-// Pushing is in two parts, so that a caller can do something else during the trip to L2 of the first.
+// The bound above is one of entries, not of tickets: a consumer that is slow between its ticket and its slot may be overtaken by a
+// whole turn of the ring.  So an entry is put into an empty slot only and taken out by an exchange, whoever comes first: nothing is
+// lost or taken twice.
+// Pushing is in three parts, so that a caller can do something else during the trips to L2 of the first two.
+__device__ __forceinline__ unsigned *ring_slot(const TiledKernelParams &p, unsigned ticket) {
+    return p.q_slots + CI(ticket & p.qmask, (long)p.qmask + 1, 127);
+}
+struct PushedCell { unsigned ticket, entry, was; };         // was: what its slot held when the entry came; 0: the entry is in it
 __device__ __forceinline__ unsigned push_ticket(const TiledKernelParams &p) { return atomicAdd(p.q_tail, 1u); }
-__device__ __forceinline__ void push_entry(const TiledKernelParams &p, unsigned ticket, int r, int c) {
+__device__ __forceinline__ PushedCell push_entry(const TiledKernelParams &p, unsigned ticket, int r, int c) {
     const unsigned cell = (unsigned)r * (unsigned)(TC * p.ntn) + (unsigned)c;
-    const unsigned entry = p.batch_index >= 0 ? ((unsigned)p.batch_index << p.cell_bits) | cell : cell;
+    const unsigned entry = (p.batch_index >= 0 ? ((unsigned)p.batch_index << p.cell_bits) | cell : cell) | 0x80000000u;
     fence_acq_rel();                                        // whoever takes the entry sees what all arrivals at the cell stand for
-    st_release_u32(p.q_slots + CI(ticket & p.qmask, (long)p.qmask + 1, 127), entry | 0x80000000u);
+    const PushedCell e{ticket, entry, atomicCAS(ring_slot(p, ticket), 0u, entry)};
     atomicAdd(p.q_avail, 1);
+    return e;
+}
+__device__ __forceinline__ void push_finish(const TiledKernelParams &p, const PushedCell &e) {
+    unsigned long long it = 0;
+    for (unsigned was = e.was; was != 0u && !wait_expired(p, it, -3, (int)e.ticket);) was = atomicCAS(ring_slot(p, e.ticket), 0u, e.entry);
 }
 // One thread, after a look at *q_avail (many idle CTAs would otherwise keep taking one off and putting it back).  Returns 0 if there was
 // nothing after all (or on abort), else the entry (bit 31 set).
 __device__ __forceinline__ unsigned ready_pop(const TiledKernelParams &p) {
     if (atomicAdd(p.q_avail, -1) <= 0) { atomicAdd(p.q_avail, 1); return 0u; }
     const unsigned h = atomicAdd(p.q_head, 1u);
-    unsigned *slot = p.q_slots + (h & p.qmask);
+    unsigned *slot = ring_slot(p, h);
     unsigned long long spins = 0;
     unsigned e;
-    while ((e = ld_acquire_u32(slot)) == 0u) {              // counted by a later ticket's producer; this one has not written yet
+    while ((e = exch_acquire_u32(slot, 0u)) == 0u) {        // counted by a later ticket's producer; this one has not written yet
         if (++spins > p.spin_limit || ld_relaxed_u32(p.abort) != 0u) {
             report(p.info, GPTQ2D_ERR_DEVICE_TIMEOUT, -3, (int)h, (int)blockIdx.x);
             atomicExch(p.abort, 1u);
             return 0u;
         }
     }
-    *slot = 0u;
     return e;
 }
 
@@ -330,11 +346,13 @@ __device__ __forceinline__ bool cell_exists(const TiledKernelParams &p, int r, i
 __device__ __forceinline__ unsigned *cell_dep(const TiledKernelParams &p, int r, int I, int J) {
     return p.cdep + CI(((long)I * p.ntn + J) * TC + r % TC, (long)TC * p.ntm * p.ntn, 125);
 }
-// A neighbour is in its task.  Nothing is ordered behind this: what the cell reads of that neighbour has flags of its own.
-__device__ __forceinline__ void cell_arrive(const TiledKernelParams &p, int r, int c) {
-    if (!cell_exists(p, r, c)) return;
+// A neighbour is in its task.  Nothing is ordered behind this: what the cell reads of that neighbour has flags of its own.  The caller
+// finishes the push, if there was one.
+__device__ __forceinline__ PushedCell cell_arrive(const TiledKernelParams &p, int r, int c) {
     const int sh = 8 * (c % TC);
-    if (((atomicAdd(cell_dep(p, r, r / TC, c / TC), 1u << sh) >> sh) & 255u) + 1u == cell_needed(r, c)) push_entry(p, push_ticket(p), r, c);
+    if (cell_exists(p, r, c) && ((atomicAdd(cell_dep(p, r, r / TC, c / TC), 1u << sh) >> sh) & 255u) + 1u == cell_needed(r, c))
+        return push_entry(p, push_ticket(p), r, c);
+    return PushedCell{0u, 0u, 0u};
 }
 // a far part of tile (I, J) is done: all cells of the tile's row k of cells at once
 __device__ __forceinline__ void far_arrive(const TiledKernelParams &p, int I, int J, int k) {
@@ -342,7 +360,8 @@ __device__ __forceinline__ void far_arrive(const TiledKernelParams &p, int I, in
     fence_acq_rel();
     const unsigned old = atomicAdd(cell_dep(p, r, I, J), 0x01010101u);
     for (int q = 0; q < TC; ++q)
-        if (cell_exists(p, r, J * TC + q) && ((old >> (8 * q)) & 255u) + 1u == cell_needed(r, J * TC + q)) push_entry(p, push_ticket(p), r, J * TC + q);
+        if (cell_exists(p, r, J * TC + q) && ((old >> (8 * q)) & 255u) + 1u == cell_needed(r, J * TC + q))
+            push_finish(p, push_entry(p, push_ticket(p), r, J * TC + q));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -623,8 +642,9 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     // The cells below and to the right may get ready: what they do first takes longer than the leaf-waves that they run behind this one
     // (1024 x 4096: 1.79 ms; told when four / two pulls were left 2.01 / 2.25).  After the older sources have been seen, not before:
     // otherwise whole diagonals of tasks wait for them on SMs that others could use (2.03).
-    if (tid == 2 * 32) cell_arrive(p, r + 1, c);
-    if (tid == 3 * 32) cell_arrive(p, r, c + 1);
+    PushedCell pushed{0u, 0u, 0u};
+    if (tid == 2 * 32) pushed = cell_arrive(p, r + 1, c);
+    if (tid == 3 * 32) pushed = cell_arrive(p, r, c + 1);
 #pragma unroll
     for (int i = 0; i < PULL_STAGES - 1; ++i) {
         const bool go = i < ns;
@@ -634,6 +654,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
         ask_end(go);
     }
     for (int k = tid; k < NLEAF * 2 * XCH_BUF; k += TILED_THREADS) xch[k] = 0.0;
+    push_finish(p, pushed);
     // The operands of the sweep have landed, for all threads: the neighbours may look for results in the place of the far sums, and the
     // coefficient tables of the diagonal leaves (see sweep_leaf) can be made.
     auto prepare = [&]() {
@@ -1261,10 +1282,10 @@ static BatchedLayout batched_layout(int count, const TiledParams *pr) {
     long ready_bound = 1;
     for (int b = 0; b < count; ++b) {
         TiledLayout t = tiled_layout(pr[b].m, pr[b].n);
-        ready_bound += 2 * (t.ntm < t.ntn ? t.ntm : t.ntn);
+        ready_bound += TC * (t.ntm < t.ntn ? t.ntm : t.ntn);
     }
     l.qcap = QCAP;
-    while ((long)l.qcap < 2 * ready_bound) l.qcap *= 2;     // twice the bound: slots are never close to reuse
+    while ((long)l.qcap < ready_bound) l.qcap *= 2;
     l.maxe_off = 256 + (size_t)l.qcap * sizeof(unsigned);
     l.flags_off = l.maxe_off + pad256((size_t)count * sizeof(double));
     size_t off = l.flags_off, bufs = 0;
