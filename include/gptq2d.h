@@ -166,7 +166,9 @@ int gptq2d_round_host(int m, int n,
  * m + n - 1 stages (Section 2, Fig. 1) and few entries per stage.  Here the fp64 tiled sweeps of
  * all matrices share one persistent kernel, so the tiles that are ready in ANY matrix keep the SMs
  * busy.  Each matrix gets exactly the Z (and E, min_margin) that gptq2d_round with GPTQ2D_FP64
- * gives it alone; shapes may differ from matrix to matrix.
+ * gives it alone, whatever else is in the batch; shapes may differ from matrix to matrix.  Matrices large
+ * enough for gptq2d_round to sweep them in blocks (see there) are swept whole here: their sums are
+ * rounded elsewhere, so an entry within rounding (1e-13 and less) of a tie may fall differently.
  *   problems:   HOST array of `count` descriptors (device pointers inside, same rules as
  *               gptq2d_round); read before the call returns, the caller may free it afterwards.
  *   min_margin: optional DEVICE array of `count` doubles.

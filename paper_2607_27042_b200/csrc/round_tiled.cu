@@ -1334,11 +1334,6 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     int cell_bits = 31, big = 0;
     while (cell_bits > 0 && (1l << (31 - cell_bits)) < (long)count) --cell_bits;
     cell_bits = std::min(cell_bits, (int)g_batch_cell_bits.load());
-    // With cells enough for every SM to have two at a time, no far part is urgent: cells pull from one tile back only (64 of 256 x 256
-    // and 256 x 512: 1 % faster; a single matrix: NEAR_TILES).
-    long ready = 0;
-    for (int b = 0; b < count; ++b) ready += TC * ((std::min(pr[b].m, pr[b].n) + T - 1) / T);
-    const int near = ready >= 296 ? 1 : NEAR_TILES;
     auto alone = [&](const TiledKernelParams &d) { return (long)TC * d.ntm * TC * d.ntn > (1l << cell_bits); };
     for (int b = 0; b < count; ++b) {
         const TiledParams &in = pr[b];
@@ -1368,7 +1363,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         d.u_al16 = ((reinterpret_cast<uintptr_t>(in.U) & 15) == 0) && ((in.ldu & 1) == 0);
         d.batch_index = b;
         d.cell_bits = cell_bits;
-        d.near = near;
+        d.near = NEAR_TILES;                // as in a sweep of its own: it decides where the sums are cut, and so their last bits
         d.report_index = b;
         d.spin_limit = d.panel_spin_limit = SPIN_LIMIT;
         d.ntiles_total = (int)tiles;

@@ -145,3 +145,21 @@ def test_data_error_names_the_matrix(g):
     Zs, _, _ = run_batched(g, good)
     for b, (X, L, U) in enumerate(good):
         assert np.array_equal(Zs[b], cref.vec_sweep(X, L, U)["Z"])
+
+
+def test_a_matrix_of_a_large_batch_equals_the_single_call(g):
+    """However many matrices share the call: 40 of two tile rows and columns beside a few of three and more, aligned and with odd
+    pitches, give every matrix the bits that it gets alone."""
+    shapes = [(385, 515), (300, 640), (513, 390), (640, 641), (1030, 384)]
+    batch = make_batch(shapes, seed0=400)
+    rng = np.random.default_rng(4)
+    fill = [(rng.normal(0, 4, (256, 160)), *O.feedback_factors(*W.general_bases(256, 160, 500 + k)[1:])[:2]) for k in range(40)]
+    Zs, Es, mm = run_batched(g, fill[:20] + batch + fill[20:])
+    for k, (X, L, U) in enumerate(batch):
+        b = 20 + k
+        assert np.array_equal(Zs[b], cref.nested(X, L, U)["Z"]), shapes[k]
+        Z1, E1, m1, info = g.gptq2d_round(dev(X), dev(L), dev(U), want_E=True, want_margin=True)
+        torch.cuda.synchronize()
+        g.check_info(info)
+        assert np.array_equal(Z1.cpu().numpy(), Zs[b]) and np.array_equal(E1.cpu().numpy(), Es[b]), shapes[k]
+        assert float(m1.cpu()[0]) == mm[b], shapes[k]
