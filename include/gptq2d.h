@@ -114,7 +114,7 @@ int gptq2d_factor(int m, int n,
  *   is implied).  They must stay fixed during the call (Section 6, first caveat).
  * Initialisation (Y <- X, C <- 0; Algorithm 3 lines 4-5) is part of this call.
  * Device errors: NONFINITE, INT_OVERFLOW (Z is int32), DEVICE_TIMEOUT.
- * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 4096 (and do not exceed 65536) run as four blocks in
+ * GPTQ2D_FP64 runs as one kernel; resident matrices whose orders both reach 3969 (and do not exceed 65536) run as four blocks in
  * three kernels, with the products between the blocks on the int8 tensor cores, all on `stream`.  These products write the rows
  * of their operands in fixed point, 56 bits below the largest entry, after a scaling along the contraction by powers of two that
  * brings the largest entry of a row of the left operand to where the largest term of the row's sums is.  An entry of a product is

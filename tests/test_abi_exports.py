@@ -133,3 +133,20 @@ def test_long_matrices_are_not_swept_in_blocks():
         assert in_blocks(m, n), (m, n)
     for m, n in ((5632, 65537), (65537, 5632), (5632, 65664), (65664, 65664), (6000, 130000)):
         assert not in_blocks(m, n), (m, n)
+
+
+def test_blocks_begin_at_32_rows_and_columns_of_tiles():
+    from paper_2607_27042_b200 import gptq2d as g
+
+    def extra(m, n):
+        got = g.gptq2d_round_workspace_bytes(m, n)
+        g.gptq2d_internal_test_hook(7, 1 << 30)
+        try:
+            return got - g.gptq2d_round_workspace_bytes(m, n)
+        finally:
+            g.gptq2d_internal_test_hook(7, 0)
+
+    for m, n in ((3969, 3969), (3969, 65536), (65536, 3969), (4096, 4096)):
+        assert extra(m, n) > 0, (m, n)
+    for m, n in ((3968, 3968), (3968, 3969), (3968, 65536), (65536, 3968)):
+        assert extra(m, n) == 0, (m, n)

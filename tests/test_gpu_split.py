@@ -75,3 +75,37 @@ def test_an_outlier_channel_of_integers_costs_no_digits(g, m, n):
     g.check_info(info)
     # sums of at most 900 terms of order one in fp64, each side: 900 * 2^-53
     assert torch.equal(Z, Z1) and float((E - E1).abs().max()) < 1e-13
+
+
+def error(E, Z, X, L, U):
+    """2-norm of the error of E over that of E.  L E U = Z - X whatever the integers are: the residual in 64-bit significands, solved for."""
+    w = np.longdouble
+    R = (Z.astype(w) - X.astype(w) - (L.astype(w) @ E.astype(w)) @ U.astype(w)).astype(np.float64)
+    return np.linalg.norm(np.linalg.solve(L, np.linalg.solve(U.T, R.T).T)) / np.linalg.norm(E)
+
+
+@pytest.mark.parametrize("kind", ["plain", "scaled", "heavy", "spectrum"])
+def test_blocks_lose_no_precision(g, kind):
+    m, n = 640, 700
+    rng = np.random.default_rng(21)
+    sigma = {"plain": 0.0, "scaled": 1.0, "heavy": 1.5}
+
+    def basis(k):
+        if kind == "spectrum":
+            q = np.linalg.qr(rng.standard_normal((k, k)))[0]
+            s = (q * np.logspace(0, -6, k)) @ q.T
+        else:
+            s = rng.standard_normal((k, 2 * k)) * np.exp(sigma[kind] * rng.standard_normal((k, 1)))
+            s = s @ s.T / (2 * k)
+            s += 0.01 * np.mean(np.diag(s)) * np.eye(k)
+        return np.linalg.cholesky(0.5 * (s + s.T)).T.copy()
+    L, U, _, _ = O.feedback_factors(basis(m), basis(n))
+    X = 4.0 * rng.standard_normal((m, n))
+    err = []
+    for order in (1 << 30, 129):
+        g.gptq2d_internal_test_hook(7, order)
+        Z, E, _, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0), want_E=True)
+        g.check_info(info)
+        err.append(error(E.cpu().numpy(), Z.cpu().numpy(), X, L, U))
+    # the same sums, half of them rounded once instead of once a term
+    assert err[1] <= 1.05 * err[0], err
