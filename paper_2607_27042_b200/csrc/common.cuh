@@ -6,8 +6,8 @@
 
 namespace gptq2d {
 
-// Every device-side wait gives up after this many polls (each poll sleeps ~100 ns, so
-// about a second), records where it stopped and raises the abort word that all other
+// Every device-side wait gives up after this many polls (a poll is a trip to L2 or a pause, 0.1 to
+// 1 us: one to several seconds), records where it stopped and raises the abort word that all other
 // waits watch.  A kernel whose wait expired returns normally; the context stays usable.
 constexpr unsigned long long SPIN_LIMIT = 8ull * 1000 * 1000;
 
@@ -36,8 +36,9 @@ __device__ __forceinline__ void report(int *info, int status, int a, int b, int 
 }
 
 // ---- checked build (-DGPTQ2D_CHECKED) --------------------------------------------------------------
-// Every index that feeds a shared- or global-memory access of the sweep kernels goes through CI(index, limit,
-// site).  In a normal build that is the index itself.  In a checked build an index outside [0, limit) is
+// Every index that is computed from sizes, task numbers or lanes and feeds a shared- or global-memory access of
+// round_tiled.cu goes through CI(index, limit, site), of the other kernels those that a check names; every site
+// number stands in one place (a test looks).  In a normal build that is the index itself.  In a checked build an index outside [0, limit) is
 // recorded -- first one wins -- in the call's status words as GPTQ2D_ERR_CHECK with the site number, the
 // index and the limit, and the access is redirected to element 0 of its array: nothing traps, nothing faults,
 // and the host reads the violation like any other device-side error.  (compute-sanitizer is not available
@@ -51,9 +52,12 @@ __device__ __forceinline__ long checked_index(long idx, long limit, int site) {
     return 0;
 }
 #define CI(idx, limit, site) checked_index((long)(idx), (long)(limit), (site))
+// the same for a pointer that was carried on from access to access: it must lie in [base, base + limit)
+#define CIP(ptr, base, limit, site) ((base) + checked_index((long)((ptr) - (base)), (long)(limit), (site)))
 #define CHECKED_SET_INFO(ptr) do { g_chk_info = (ptr); } while (0)
 #else
 #define CI(idx, limit, site) (idx)
+#define CIP(ptr, base, limit, site) (ptr)
 #define CHECKED_SET_INFO(ptr) do { } while (0)
 #endif
 

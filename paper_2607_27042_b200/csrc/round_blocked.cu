@@ -63,16 +63,16 @@ __global__ void blocked_init_kernel(BlockedParams p) {
     const int m = p.m, n = p.n, w = p.w;
     for (long idx = tid0; idx < (long)m * n; idx += nthreads) {
         const int i = (int)(idx / n), j = (int)(idx % n);
-        p.Y[idx] = p.X[CI((long)i * p.ldx + j, (long)(m - 1) * p.ldx + n, 301)];
+        p.Y[idx] = p.X[CI((long)i * p.ldx + j, (long)(m - 1) * p.ldx + n, 401)];
         p.C[idx] = 0.0;
     }
     for (long idx = tid0; idx < (long)m * w; idx += nthreads) {
         const int i = (int)(idx / w), k = (int)(idx % w);
-        p.Lband[idx] = (k >= 1 && i - k >= 0) ? p.L[CI((long)i * p.ldl + (i - k), (long)(m - 1) * p.ldl + m, 302)] : 0.0;
+        p.Lband[idx] = (k >= 1 && i - k >= 0) ? p.L[CI((long)i * p.ldl + (i - k), (long)(m - 1) * p.ldl + m, 402)] : 0.0;
     }
     for (long idx = tid0; idx < (long)n * w; idx += nthreads) {
         const int j = (int)(idx / w), k = (int)(idx % w);
-        p.Uband[idx] = (k >= 1 && j - k >= 0) ? p.U[CI((long)(j - k) * p.ldu + j, (long)(n - 1) * p.ldu + n, 303)] : 0.0;
+        p.Uband[idx] = (k >= 1 && j - k >= 0) ? p.U[CI((long)(j - k) * p.ldu + j, (long)(n - 1) * p.ldu + n, 403)] : 0.0;
     }
 }
 
@@ -105,14 +105,14 @@ __global__ void __launch_bounds__(BLK_IN_THREADS) blocked_inblock_kernel(Blocked
 #pragma unroll
     for (int x = 0; x < BLK_WMAX / 4; ++x) {
         const int k = 1 + sub + 4 * x;
-        Lr[x] = (row_ok && k < w) ? p.Lband[CI((long)i * w + k, (long)p.m * w, 304)] : 0.0;
+        Lr[x] = (row_ok && k < w) ? p.Lband[CI((long)i * w + k, (long)p.m * w, 404)] : 0.0;
     }
 
     // columns of step 0: s0 - ibase - (BLK_ROWS - 1) .. s0 - ibase
     const int jtop = s0 - ibase;
     for (int idx = tid; idx < BLK_ROWS * w; idx += BLK_IN_THREADS) {
         const int j = jtop - (BLK_ROWS - 1) + idx / w, k = idx % w;
-        Us[CI((j & (BLK_RING - 1)) * BLK_LDB + k, BLK_RING * BLK_LDB, 305)] = (j >= 0 && j < n) ? p.Uband[CI((long)j * w + k, (long)n * w, 306)] : 0.0;
+        Us[CI((j & (BLK_RING - 1)) * BLK_LDB + k, BLK_RING * BLK_LDB, 405)] = (j >= 0 && j < n) ? p.Uband[CI((long)j * w + k, (long)n * w, 406)] : 0.0;
     }
     __syncthreads();
 
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(BLK_IN_THREADS) blocked_inblock_kernel(Blocked
         const int jj = s0 + tt - i;
         c = y = 0.0;
         if (row_ok && tt <= tmax && jj >= 0 && jj < n) {
-            c = p.C[CI((long)i * n + jj, (long)p.m * n, 307)];
+            c = p.C[CI((long)i * n + jj, (long)p.m * n, 407)];
             y = p.Y[(long)i * n + jj];
         }
     };
@@ -171,10 +171,10 @@ __global__ void __launch_bounds__(BLK_IN_THREADS) blocked_inblock_kernel(Blocked
                     report(p.info, isfinite(y) ? GPTQ2D_ERR_INT_OVERFLOW : GPTQ2D_ERR_NONFINITE, i, j, 0);
                     z = 0.0;
                 }
-                p.Z[CI((long)i * p.ldz + j, (long)(p.m - 1) * p.ldz + n, 308)] = (int)z;
-                p.Eb[CI((long)i * n + j, (long)p.m * n, 309)] = e;
+                p.Z[CI((long)i * p.ldz + j, (long)(p.m - 1) * p.ldz + n, 408)] = (int)z;
+                p.Eb[CI((long)i * n + j, (long)p.m * n, 409)] = e;
                 if (p.E) p.E[(long)i * p.lde + j] = e;
-                p.Cband[CI((long)i * w + t, (long)p.m * w, 310)] = c;
+                p.Cband[CI((long)i * w + t, (long)p.m * w, 410)] = c;
                 max_abs_e = fmax(max_abs_e, fabs(e));
             }
         }
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(FLUSH_THREADS, 2) blocked_flush_kernel(Blocked
             for (int x = 0; x < 2; ++x) {
                 const int j = jg0 + 2 * t + x;
                 if (i < m && j < n && i + j > s1) {
-                    const long idx = CI((long)i * n + j, (long)m * n, 311);
+                    const long idx = CI((long)i * n + j, (long)m * n, 411);
                     p.Y[idx] = yv[a4][x] + (accD[a][x] + accR[a][x]);
                     p.C[idx] = cv[a4][x] + accD[a][x];
                 }

@@ -149,7 +149,8 @@ __device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKerne
             const int c = threadIdx.x + it * TILED_THREADS, i = c >> 4, j = (c & 15) * 2;
             // the piece that holds the diagonal: its off-diagonal entry only (from L if i is odd, from U if it is even)
             const bool lower = j < i, diag = (i & ~1) == j;
-            const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
+            const double *src = lower ? p.L + CI((long)(r0 + i) * p.ldl + r0 + j, (long)(p.m - 1) * p.ldl + p.m - 1, 137)
+                                      : p.U + CI((long)(c0 + i) * p.ldu + c0 + j, (long)(p.n - 1) * p.ldu + p.n - 1, 138);
             if (!diag) cp_async16(dst + CI(i * SLD + j, SMAT - 1, 121), src, 16);
             else cp_async8(dst + CI(i * SLD + j + ((i & 1) ^ 1), SMAT, 131), (i & 1) ? src : src + 1, 8);
         }
@@ -162,7 +163,8 @@ __device__ __forceinline__ void load_lu_diag_async(double *dst, const TiledKerne
         const bool lower = j < i, upper = j > i;
         const bool take = lower ? (r0 + i < p.m) : (upper && c0 + j < p.n);     // r0 + j < r0 + i, c0 + i < c0 + j
         const double *src = lower ? p.L + (long)(r0 + i) * p.ldl + r0 + j : p.U + (long)(c0 + i) * p.ldu + c0 + j;
-        cp_async8(dst + CI(i * SLD + j, SMAT, 121), take ? src : p.L, take ? 8 : 0);
+        if (take) src = lower ? CIP(src, p.L, (long)(p.m - 1) * p.ldl + p.m, 139) : CIP(src, p.U, (long)(p.n - 1) * p.ldu + p.n, 140);
+        cp_async8(dst + CI(i * SLD + j, SMAT, 141), take ? src : p.L, take ? 8 : 0);
     }
 }
 
@@ -207,8 +209,9 @@ __device__ __forceinline__ void leaf_pull(double *Ws, double *Cs, const double *
     double2 *wp = reinterpret_cast<double2 *>(Ws + CI((a * 8 + g) * SLD + b * 8 + t * 2, SMAT - 1, 108));
     double2 *cp = reinterpret_cast<double2 *>(Cs + CI((a * 8 + g) * SLD + b * 8 + t * 2, SMAT - 1, 109));
     double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0, r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
-    const double *La = LU + (a * 8 + g) * SLD + t, *Eb = Ws + t * SLD + b * 8 + g;          // A: row a*8+g, k = t (+4); B: k = t (+4), col b*8+g
-    const double *Ca = Cs + (a * 8 + g) * SLD + t, *Ub = LU + t * SLD + b * 8 + g;
+    // A: row a*8+g, k = t (+4); B: k = t (+4), col b*8+g
+    const double *La = LU + CI((a * 8 + g) * SLD + t, SMAT - max(0, 8 * a1 - 4), 142), *Eb = Ws + CI(t * SLD + b * 8 + g, SMAT - max(0, 8 * a1 - 4) * SLD, 143);
+    const double *Ca = Cs + CI((a * 8 + g) * SLD + t, SMAT - max(0, 8 * b1 - 4), 144), *Ub = LU + CI(t * SLD + b * 8 + g, SMAT - max(0, 8 * b1 - 4) * SLD, 145);
 #pragma unroll 1
     for (int ap = 0; ap < a1; ++ap) {
         dmma_m8n8k4(p0, p1, La[ap * 8], Eb[(ap * 8) * SLD]);
@@ -413,9 +416,10 @@ __device__ __forceinline__ void sweep_leaf(double *Ws, double *Cs, int *Zs, cons
     start();
     const int t0 = i0 + j, t1 = t0 + 4;
     // the e of column j at step s is lane 4 j + (s - j) % 4's, the C of row i0 lane 4 (s - i0) + i0's, that of row i0 + 4 four columns before
-    double *pe = exw + lane, *pc = exw + 48 + lane;
-    const double *rc = exw + 48 - 3 * i0;
-    const double *re[4] = {exw + 4 * j + ((0 - j) & 3), exw + 4 * j + ((1 - j) & 3), exw + 4 * j + ((2 - j) & 3), exw + 4 * j + ((3 - j) & 3)};
+    double *pe = CIP(exw + lane, exw, XCH_BUF, 146), *pc = CIP(exw + 48 + lane, exw, XCH_BUF, 147);
+    const double *rc = CIP(exw + 48 - 3 * i0, exw, XCH_BUF - 52, 148);
+    const double *re[4] = {CIP(exw + 4 * j + ((0 - j) & 3), exw, 32, 149), CIP(exw + 4 * j + ((1 - j) & 3), exw, 32, 192),
+                           CIP(exw + 4 * j + ((2 - j) & 3), exw, 32, 193), CIP(exw + 4 * j + ((3 - j) & 3), exw, 32, 194)};
     // round half to even: adding and subtracting 1.5 * 2^52 leaves the integer, whose low word is the sum's
     constexpr double MAGIC = 6755399441055744.0;
 #pragma unroll
@@ -443,7 +447,7 @@ __device__ __forceinline__ void sweep_leaf(double *Ws, double *Cs, int *Zs, cons
         // Again from the beginning, both entries rounded at every step; integer and high word of an entry are those of its own step.
         start();
         __syncwarp();
-        exw[lane] = 0.0;                                         // what the first pass left there may be infinite or NaN
+        exw[CI(lane, XCH_BUF, 150)] = 0.0;                       // what the first pass left there may be infinite or NaN
         int h0 = 0, h1 = 0;
 #pragma unroll 1
         for (int s = 0; s < 15; ++s) {
@@ -454,10 +458,10 @@ __device__ __forceinline__ void sweep_leaf(double *Ws, double *Cs, int *Zs, cons
             if (t1 == s) { z1 = __double2loint(k1); h1 = __double2hiint(x1); }
             if (s == 14) { c0 = f0; c1 = f1; break; }
             __syncwarp();
-            if (t0 == s) { exw[j] = e0; exw[8 + i0] = f0; }
-            if (t1 == s) { exw[j] = e1; exw[12 + i0] = f1; }
+            if (t0 == s) { exw[CI(j, 8, 151)] = e0; exw[CI(8 + i0, 12, 152)] = f0; }
+            if (t1 == s) { exw[CI(j, 8, 195)] = e1; exw[CI(12 + i0, 16, 196)] = f1; }
             __syncwarp();
-            const double ed = exw[j], cr0 = exw[8 + i0], cr1 = exw[12 + i0];
+            const double ed = exw[CI(j, 8, 197)], cr0 = exw[CI(8 + i0, 12, 198)], cr1 = exw[CI(12 + i0, 16, 199)];
             c0 = fma(tl0[s], ed, c0); w0 = fma(cr0, tu0[s], w0);
             c1 = fma(tl1[s], ed, c1); w1 = fma(cr1, tu1[s], w1);
         }
@@ -481,23 +485,23 @@ __device__ __forceinline__ void sweep_leaf(double *Ws, double *Cs, int *Zs, cons
 // E and C of the swept leaf (a, b) to the workspace, where the neighbours are waiting for them, by one warp
 __device__ __forceinline__ void post_leaf(const double *Ws, const double *Cs, int a, int b, double *eQ, double *cQ, long np) {
     const int lane = threadIdx.x & 31, i = a * 8 + (lane >> 2), j = b * 8 + (lane & 3) * 2;
-    double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 133)), c = *reinterpret_cast<const double2 *>(Cs + i * SLD + j);
+    double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 133)), c = *reinterpret_cast<const double2 *>(Cs + CI(i * SLD + j, SMAT - 1, 153));
     e.x = stream_value(e.x); e.y = stream_value(e.y); c.x = stream_value(c.x); c.y = stream_value(c.y);
-    st_relaxed_f64x2(eQ + i * np + j, e);
-    st_relaxed_f64x2(cQ + i * np + j, c);
+    st_relaxed_f64x2(eQ + CI(i * np + j, (S - 1) * np + S - 1, 154), e);
+    st_relaxed_f64x2(cQ + CI(i * np + j, (S - 1) * np + S - 1, 155), c);
 }
 // its Z (and the caller's E) to the output
 __device__ __forceinline__ void store_leaf(const double *Ws, const int *Zs, int a, int b, int row0, int col0, const TiledKernelParams &p, double &max_abs_e) {
     const int lane = threadIdx.x & 31, i = a * 8 + (lane >> 2), j = b * 8 + (lane & 3) * 2, gr = row0 + i, gc = col0 + j;
     if (gr >= p.m || gc >= p.n) return;
     const double2 e = *reinterpret_cast<const double2 *>(Ws + CI(i * SLD + j, SMAT - 1, 134));
-    const int2 z = *reinterpret_cast<const int2 *>(Zs + i * S + j);
+    const int2 z = *reinterpret_cast<const int2 *>(Zs + CI(i * S + j, S * S - 1, 156));
     const bool two = gc + 1 < p.n;
     int *zo = p.Z + CI((long)gr * p.ldz + gc, (long)(p.m - 1) * p.ldz + p.n, 119);
     zo[0] = z.x;
     if (two) zo[1] = z.y;
     if (p.Euser) {
-        double *eo = p.Euser + (long)gr * p.lde + gc;
+        double *eo = p.Euser + CI((long)gr * p.lde + gc, (long)(p.m - 1) * p.lde + p.n, 157);
         eo[0] = e.x;
         if (two) eo[1] = e.y;
     }
@@ -530,7 +534,8 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int row0 = r * S, col0 = c * S, I = r / TC, J = c / TC;
     const long np = p.np;
-    double *eQ = p.Ebuf + (long)row0 * np + col0, *cQ = p.Cbuf + (long)row0 * np + col0;
+    const long buf = (long)(p.ntm * T - 1) * np + (long)p.ntn * T;     // entries from the first to the last of the matrix in Ebuf and Cbuf
+    double *eQ = p.Ebuf + CI((long)row0 * np + col0, buf - (S - 1) * np - (S - 1), 158), *cQ = p.Cbuf + CI((long)row0 * np + col0, buf - (S - 1) * np - (S - 1), 159);
     TS_RESET();
     // ---- 1. pulls.  Step i takes the source ns - i cells before the neighbour in both directions (the shorter one begins later), so
     // the newest sources, (r - 2, c) and (r, c - 2), come last.  Those may still be in their last leaf-waves when this task starts
@@ -566,18 +571,30 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     const double *csrc = p.Cbuf + (long)(row0 + i16) * np + j16;
     const unsigned smem_s = (unsigned)__cvta_generic_to_shared(smem) + d16 * 8;      // its place in matrix 0
     constexpr unsigned MAT = SMAT * 8, HALF = 16 * SLD * 8;
+    // a piece of an operand (checked builds look at both ends of a copy that is made; from: number of the site, base and entries of its matrix)
+    auto copy16 = [&](unsigned to, const double *src, int bytes, bool on, int from, const double *base, long count) {
+#ifdef GPTQ2D_CHECKED
+        if (on) {
+            const unsigned s0 = (unsigned)__cvta_generic_to_shared(smem);
+            to = s0 + (unsigned)CI((long)to - (long)s0, SWEEP_SMEM - 15, 160);
+            if (bytes > 0) src = CIP(src, base, count - bytes / 8 + 1, from);
+        }
+#endif
+        cp_async16_if(to, src, bytes, on);
+    };
+    const long lcount = (long)(p.m - 1) * p.ldl + p.m, ucount = (long)(p.n - 1) * p.ldu + p.n;
     // operands of the sweep, on their way during the pulls
     if (r > 0) {
-        cp_async16_if(smem_s + 3 * MAT, lsrc0 + (row0 - S), lz0, l16); cp_async16_if(smem_s + 3 * MAT + HALF, lsrc1 + (row0 - S), lz1, l16);
+        copy16(smem_s + 3 * MAT, lsrc0 + (row0 - S), lz0, l16, 161, p.L, lcount); copy16(smem_s + 3 * MAT + HALF, lsrc1 + (row0 - S), lz1, l16, 162, p.L, lcount);
         if (!l16) load_factor_async(La, p.L, p.ldl, p.m, row0, row0 - S);
     }
     if (c > 0) {
         const double *u = usrc + (long)(col0 - S) * p.ldu;
-        cp_async16_if(smem_s + 4 * MAT, u, uz, u16); cp_async16_if(smem_s + 4 * MAT + HALF, u + ldu16, uz, u16);
+        copy16(smem_s + 4 * MAT, u, uz, u16, 163, p.U, ucount); copy16(smem_s + 4 * MAT + HALF, u + ldu16, uz, u16, 164, p.U, ucount);
         if (!u16) load_factor_async(Ul, p.U, p.ldu, p.n, col0 - S, col0);
     }
-    cp_async16_if(smem_s + MAT, csrc + col0, 16, true); cp_async16_if(smem_s + MAT + HALF, csrc + col0 + np16, 16, true);
-    cp_async16_if(smem_s, esrc + row0 * np, 16, true); cp_async16_if(smem_s + HALF, esrc + row0 * np + np16, 16, true);
+    copy16(smem_s + MAT, csrc + col0, 16, true, 165, p.Cbuf, buf); copy16(smem_s + MAT + HALF, csrc + col0 + np16, 16, true, 166, p.Cbuf, buf);
+    copy16(smem_s, esrc + row0 * np, 16, true, 167, p.Ebuf, buf); copy16(smem_s + HALF, esrc + row0 * np + np16, 16, true, 168, p.Ebuf, buf);
     load_lu_diag_async(LU, p, row0, col0);
     cp_async_commit();
     // X in the layout of the accumulators of warps 4-7, zero outside the matrix
@@ -605,16 +622,16 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     auto ask_begin = [&](bool go) { on_a = go && asked >= skip_a; on_l = go && asked >= skip_l; };
     auto copy = [&](int q) {                                          // operand q / 2 (L, E, C, U), upper or lower half
         const unsigned at = dst + (q >> 1) * MAT + (q & 1) * HALF;
-        if (q < 2) cp_async16_if(at, q ? lp1 : lp0, q ? lz1 : lz0, on_a && l16);
-        else if (q < 4) cp_async16_if(at, q & 1 ? ep + np16 : ep, 16, on_a);
-        else if (q < 6) cp_async16_if(at, q & 1 ? qp + np16 : qp, 16, on_l);
-        else cp_async16_if(at, q & 1 ? up + ldu16 : up, uz, on_l && u16);
+        if (q < 2) copy16(at, q ? lp1 : lp0, q ? lz1 : lz0, on_a && l16, 169, p.L, lcount);
+        else if (q < 4) copy16(at, q & 1 ? ep + np16 : ep, 16, on_a, 170, p.Ebuf, buf);
+        else if (q < 6) copy16(at, q & 1 ? qp + np16 : qp, 16, on_l, 171, p.Cbuf, buf);
+        else copy16(at, q & 1 ? up + ldu16 : up, uz, on_l && u16, 172, p.U, ucount);
     };
     auto ask_end = [&](bool go) {
         if (!(l16 && u16)) {                                          // odd pitches or pointers: 8 bytes at a time
-            double *buf = ring + (asked % PULL_STAGES) * 4 * SMAT;
-            if (on_a && !l16) load_factor_async(buf, p.L, p.ldl, p.m, row0, (r - 1 - ns + asked) * S);
-            if (on_l && !u16) load_factor_async(buf + 3 * SMAT, p.U, p.ldu, p.n, (c - 1 - ns + asked) * S, col0);
+            double *to = ring + (asked % PULL_STAGES) * 4 * SMAT;
+            if (on_a && !l16) load_factor_async(to, p.L, p.ldl, p.m, row0, (r - 1 - ns + asked) * S);
+            if (on_l && !u16) load_factor_async(to + 3 * SMAT, p.U, p.ldu, p.n, (c - 1 - ns + asked) * S, col0);
         }
         cp_async_commit();
         if (on_a) { lp0 += S; lp1 += S; ep += 2 * np16; }
@@ -660,7 +677,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     auto prepare = [&]() {
         const double empty = __longlong_as_double((long long)STREAM_EMPTY);
         const double2 e2 = make_double2(empty, empty);
-        double *e = eQ + (long)i16 * np + j16, *q = cQ + (long)i16 * np + j16;
+        double *e = eQ + CI((long)i16 * np + j16, (S / 2 - 1) * np + S - 1, 173), *q = cQ + CI((long)i16 * np + j16, (S / 2 - 1) * np + S - 1, 174);
         *reinterpret_cast<double2 *>(e) = e2; *reinterpret_cast<double2 *>(e + np16) = e2;
         *reinterpret_cast<double2 *>(q) = e2; *reinterpret_cast<double2 *>(q + np16) = e2;
         const int i = tid >> 3, blk = i & ~7, in = i & 7;             // i: row (L) or column (U) inside the cell
@@ -671,8 +688,8 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
             const int at = blk + (ok ? src : 0);
             const double l = LU[CI(i * SLD + at, SMAT, 112)], u = LU[CI(at * SLD + i, SMAT, 113)];
             if (x < TAB_LD) {
-                tabL[i * TAB_LD + x] = ok ? l : 0.0;
-                tabU[i * TAB_LD + x] = ok ? u : 0.0;
+                tabL[CI(i * TAB_LD + x, S * TAB_LD, 175)] = ok ? l : 0.0;
+                tabU[CI(i * TAB_LD + x, S * TAB_LD, 176)] = ok ? u : 0.0;
             }
         }
     };
@@ -684,7 +701,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
         if (i == 0) TS_MARK(0);
         const int known = s_known[i & 1];
         const bool go = asked < ns && asked <= i + PULL_STAGES - 1 && asked < known;               // every warp is past product i - 1: its buffers are free
-        const double *As = ring + (rd * 4 + (warp < 4 ? 0 : 2)) * SMAT;
+        const double *As = ring + CI((rd * 4 + (warp < 4 ? 0 : 2)) * SMAT, (PULL_STAGES * 4 - 1) * SMAT, 177);
         rd = rd == PULL_STAGES - 1 ? 0 : rd + 1;
         last = go ? asked : -1;
         ask_begin(go);
@@ -725,13 +742,16 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     const bool down = warp < 6, fed = down ? r > 0 : c > 0;
     const double *nsrc = down ? eQ + (long)(t - S) * np + g : cQ + (long)g * np - S + t;
     const long nstep = down ? 4 * np : 4, nblk = down ? 8 : 8 * np;
+    auto block_src = [&](int blk) {
+        return down ? CIP(nsrc + blk * nblk, p.Ebuf, buf - 7 * nstep, 178) : CIP(nsrc + blk * nblk, p.Cbuf, buf - 7 * nstep, 179);
+    };
     double v[8];
     auto stream_take = [&](int blk) {
-        const double *src = nsrc + blk * nblk;
+        const double *src = block_src(blk);
         double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
         double2 *d0, *d1;
         if (down) {
-            const double *A = La + (half * 16 + g) * SLD + t;
+            const double *A = La + CI((half * 16 + g) * SLD + t, SMAT - 8 * SLD - 28, 180);
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
                 stream_await(p, v[i], v[i + 1], src + i * nstep, nstep);
@@ -743,7 +763,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
             d0 = reinterpret_cast<double2 *>(Cs + CI((half * 16 + g) * SLD + blk * 8 + t * 2, SMAT - 8 * SLD - 1, 126));
             d1 = d0 + 8 * SLD / 2;
         } else {
-            const double *B = Ul + t * SLD + half * 16 + g;
+            const double *B = Ul + CI(t * SLD + half * 16 + g, SMAT - 28 * SLD - 8, 181);
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
                 stream_await(p, v[i], v[i + 1], src + i * nstep, nstep);
@@ -760,7 +780,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
         *d0 = x; *d1 = y;
     };
     if (warp >= 4 && fed) {
-        stream_ask(v, nsrc, nstep);
+        stream_ask(v, block_src(0), nstep);
         stream_take(0);
     }
     TS_MARK(2);
@@ -777,7 +797,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
             const bool take = fed && lw + 1 < NLEAF;
             const int a = warp - 4, b = lw + 1 - a, done = b - 2;
             if (done >= 0 && done < NLEAF) post_leaf(Ws, Cs, a, done, eQ, cQ, np);
-            if (take) stream_ask(v, nsrc + (lw + 1) * nblk, nstep);
+            if (take) stream_ask(v, block_src(lw + 1), nstep);
             if (b >= 0 && b < NLEAF) leaf_pull(Ws, Cs, LU, a, b, a - 1, b - 1, g, t);
             if (done >= 0 && done < NLEAF) store_leaf(Ws, Zs, a, done, row0, col0, p, max_abs_e);
             if (take) stream_take(lw + 1);
@@ -833,7 +853,7 @@ __device__ __forceinline__ void store_acc(const Acc &acc, double *dstT, long np,
             double2 v;
             v.x = acc.v[a][b][0];
             v.y = acc.v[a][b][1];
-            *reinterpret_cast<double2 *>(dstT + CI((long)(wm * 64 + a * 8 + g) * np + wn * 32 + b * 8 + t * 2, 127L * np + T - 1, 126)) = v;
+            *reinterpret_cast<double2 *>(dstT + CI((long)(wm * 64 + a * 8 + g) * np + wn * 32 + b * 8 + t * 2, 127L * np + T - 1, 182)) = v;
         }
 }
 __device__ __forceinline__ void load_acc(Acc &acc, const double *srcT, long np, int wm, int wn, int g, int t) {
@@ -841,8 +861,7 @@ __device__ __forceinline__ void load_acc(Acc &acc, const double *srcT, long np, 
     for (int a = 0; a < 8; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            double2 v = __ldcg(reinterpret_cast<const double2 *>(srcT + (long)(wm * 64 + a * 8 + g) * np + wn * 32 +
-                                                                 b * 8 + t * 2));
+            double2 v = __ldcg(reinterpret_cast<const double2 *>(srcT + CI((long)(wm * 64 + a * 8 + g) * np + wn * 32 + b * 8 + t * 2, 127L * np + T - 1, 183)));
             acc.v[a][b][0] = v.x;
             acc.v[a][b][1] = v.y;
         }
@@ -863,7 +882,7 @@ constexpr unsigned IDLE_SLEEP_NS = 50;  // pause of a CTA that found nothing to 
 template <bool BATCHED, bool PANELS>
 __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKernelParams p) {
     extern __shared__ __align__(16) double smem[];
-    __shared__ int s_task[4];
+    __shared__ int s_upto;                 // the first source of the far part that is not swept yet
     __shared__ int s_far[5];               // the CTA's far part: type, I, J, next source, number of sources
     __shared__ int s_has, s_state;         // s_has: it holds one
     __shared__ unsigned s_pop;
@@ -935,14 +954,14 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
     auto tile_region = [&]() {
         const TiledKernelParams &pk = VIEW(0);
         return (s_far[0] == 0 ? pk.Cbuf : pk.Ebuf) +
-               CI((long)s_far[1] * T * pk.np + (long)s_far[2] * T, (long)(pk.ntm - 1) * T * pk.np + (long)(pk.ntn - 1) * T + 1, 128);
+               CI((long)s_far[1] * T * pk.np + (long)s_far[2] * T, (long)(pk.ntm - 1) * T * pk.np + (long)(pk.ntn - 1) * T + 1, 184);
     };
     // thread 0: the far part in hand can go on (a Cd part reads L in the block row of I, an Rt part U in the block column of J)
     auto far_ready = [&]() -> bool {
         const TiledKernelParams &pk = VIEW(0);
         const int ty = s_far[0], pos = s_far[3];
         const unsigned *fl = ty == 0 ? pk.flagS + (long)pos * pk.ntn + s_far[2] : pk.flagS + (long)s_far[1] * pk.ntn + pos;
-        return (pos >= s_far[4] || ld_acquire_u32(fl) != 0u) && panels_arrived(((ty == 0 ? s_far[1] : s_far[2]) >> COPY_BLOCK_TILES_LOG2) + 1);
+        return (pos >= s_far[4] || ld_acquire_u32(CIP(fl, pk.flagS, (long)pk.ntm * pk.ntn, 185)) != 0u) && panels_arrived(((ty == 0 ? s_far[1] : s_far[2]) >> COPY_BLOCK_TILES_LOG2) + 1);
     };
 
     for (;;) {
@@ -1028,7 +1047,7 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
                 // everything is stored: sweep_cell ended with a barrier, so a fence of one thread covers the whole CTA's results
                 if (tid == 3 * 32) {
                     __threadfence();
-                    const unsigned done = atomicAdd(pq.cells_done + (long)I * pq.ntn + J, 1u);
+                    const unsigned done = atomicAdd(pq.cells_done + CI((long)I * pq.ntn + J, (long)pq.ntm * pq.ntn, 186), 1u);
                     const unsigned ncells = (unsigned)(min(TC, (pq.m - I * T + S - 1) / S) * min(TC, (pq.n - J * T + S - 1) / S));
                     if (done + 1u == ncells) {   // tile swept: far parts that list it as a source may go on
                         __threadfence();
@@ -1062,19 +1081,19 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
             const long fstride = f_type == 0 ? pk.ntn : 1;
             // how many source tiles from f_pos on are swept already (the first one is)
             __syncthreads();
-            if (tid == 0) s_task[0] = f_nfar;
+            if (tid == 0) s_upto = f_nfar;
             __syncthreads();
             for (int idx = f_pos + tid; idx < f_nfar; idx += blockDim.x)
-                if (ld_acquire_u32(flags + (long)idx * fstride) == 0u) atomicMin(&s_task[0], idx);
+                if (ld_acquire_u32(CIP(flags + (long)idx * fstride, pk.flagS, (long)pk.ntm * pk.ntn, 187)) == 0u) atomicMin(&s_upto, idx);
             __syncthreads();
-            const int upto = min(s_task[0], f_pos + FAR_RUN_CHUNKS);
+            const int upto = min(s_upto, f_pos + FAR_RUN_CHUNKS);
             Operand a, b;
             if (f_type == 0) {
-                a.ptr = pk.L + CI((long)f_I * T * pk.ldl + (long)f_pos * T, (long)(pk.m - 1) * pk.ldl + pk.m, 131); a.ld = pk.ldl; a.mn_valid = min(T, pk.m - f_I * T); a.aligned16 = pk.l_al16;
-                b.ptr = pk.Ebuf + (long)f_J * T + (long)f_pos * T * pk.np; b.ld = pk.np; b.mn_valid = T; b.aligned16 = true;
+                a.ptr = pk.L + CI((long)f_I * T * pk.ldl + (long)f_pos * T, (long)(pk.m - 1) * pk.ldl + pk.m, 188); a.ld = pk.ldl; a.mn_valid = min(T, pk.m - f_I * T); a.aligned16 = pk.l_al16;
+                b.ptr = CIP(pk.Ebuf + (long)f_J * T + (long)f_pos * T * pk.np, pk.Ebuf, (long)(pk.ntm * T - 1) * pk.np + (long)pk.ntn * T, 190); b.ld = pk.np; b.mn_valid = T; b.aligned16 = true;
             } else {
-                a.ptr = pk.Cbuf + (long)f_I * T * pk.np + (long)f_pos * T; a.ld = pk.np; a.mn_valid = T; a.aligned16 = true;
-                b.ptr = pk.U + CI((long)f_J * T + (long)f_pos * T * pk.ldu, (long)(pk.n - 1) * pk.ldu + pk.n, 132); b.ld = pk.ldu; b.mn_valid = min(T, pk.n - f_J * T); b.aligned16 = pk.u_al16;
+                a.ptr = CIP(pk.Cbuf + (long)f_I * T * pk.np + (long)f_pos * T, pk.Cbuf, (long)(pk.ntm * T - 1) * pk.np + (long)pk.ntn * T, 191); a.ld = pk.np; a.mn_valid = T; a.aligned16 = true;
+                b.ptr = pk.U + CI((long)f_J * T + (long)f_pos * T * pk.ldu, (long)(pk.n - 1) * pk.ldu + pk.n, 189); b.ld = pk.ldu; b.mn_valid = min(T, pk.n - f_J * T); b.aligned16 = pk.u_al16;
             }
             SC_MARK(2);
             gemm_tile<true, false, BULK_NSTAGE>(acc, smem, a, b, (upto - f_pos) * T);

@@ -76,6 +76,49 @@ for scale in (1.0, 2.0 ** 600):
 print("checked build: %%d cases clean" %% len(cases))
 """
 
+CELLS = r"""
+import sys
+sys.path.insert(0, %r)
+sys.path.insert(0, %r)
+import numpy as np, torch
+from paper_2607_27042_b200 import gptq2d as g
+assert g.library_path().endswith("libgptq2d_checked.so")
+rng = np.random.default_rng(3)
+
+def padded(a, extra):
+    buf = torch.full((a.shape[0], a.shape[1] + extra), float("nan"), dtype=torch.float64, device="cuda")
+    buf[:, :a.shape[1]] = torch.from_numpy(a).cuda()
+    return buf[:, :a.shape[1]]
+
+# far parts in both directions, cells at both edges, a value that does not fit; operands in pieces of 16 and of 8 bytes
+for m, n in [(545, 399), (399, 545), (512, 640)]:
+    X = 4.0 * rng.standard_normal((m, n))
+    L, U = np.tril(rng.standard_normal((m, m)), -1) / m, np.triu(rng.standard_normal((n, n)), 1) / n
+    out = []
+    for extra in (0, 1):
+        E = padded(np.zeros((m, n)), 3)
+        for order in (1 << 30, 129):
+            g.gptq2d_internal_test_hook(7, order)
+            Z, _, _, info = g.gptq2d_round(padded(X, extra), padded(L, m %% 2 + extra), padded(U, n %% 2 + extra), E=E)
+            g.check_info(info)
+            out.append(Z.cpu())
+    assert all(torch.equal(z, out[0]) for z in out)
+    X[m - 1, n - 1] = 1e300
+    info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0))[3].cpu().tolist()
+    assert info[0] not in (0, 10), info
+g.gptq2d_internal_test_hook(7, 0)
+print("checked build: cells clean")
+"""
+
+
+def test_cells_under_the_checked_build():
+    from paper_2607_27042_b200 import build
+    build.build(checked=True)
+    env = dict(os.environ, GPTQ2D_LIBRARY="libgptq2d_checked.so")
+    r = subprocess.run([sys.executable, "-c", CELLS % (ROOT, os.path.join(ROOT, "tests"))], env=env, capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    assert "cells clean" in r.stdout
+
 
 def test_small_parity_cases_under_the_checked_build():
     from paper_2607_27042_b200 import build
