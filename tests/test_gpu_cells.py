@@ -64,9 +64,15 @@ def test_matrices_of_a_batch_swept_by_themselves(g):
 
 @pytest.mark.parametrize("i,j", [(0, 0), (40, 70), (150, 20)])
 def test_a_nan_that_looks_like_a_missing_entry_is_an_ordinary_nan(g, i, j):
+    mark = 0xfff94d5a7c3e2b61
     X, A, B = W.gaussian_like(160, 170, 5)
     L, U, _, _ = O.feedback_factors(A, B)
-    X[i, j] = np.array([0xfff94d5a7c3e2b61], dtype=np.uint64).view(np.float64)[0]
-    Z, E, mm, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0), want_E=True)
+    X[i, j] = np.array([mark], dtype=np.uint64).view(np.float64)[0]
+    ws = torch.zeros(g.gptq2d_round_workspace_bytes(160, 170) // 8, dtype=torch.int64, device="cuda")
+    Z, E, mm, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0), want_E=True, workspace=ws.view(torch.uint8))
     vals = info.cpu().tolist()
     assert vals[0] == 6 and abs(vals[1] + vals[2] - i - j) < 15            # known to a leaf's 15 anti-diagonals
+    # the caller's E is stored as computed: entries with the mark's bits did come up; none of them was posted with these bits
+    assert (E.cpu().numpy().view(np.uint64) == mark).any()
+    posted = ws.cpu().numpy().view(np.uint64)
+    assert not (posted == mark).any() and (posted == mark ^ 1).any()
