@@ -660,8 +660,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
     // (1024 x 4096: 1.79 ms; told when four / two pulls were left 2.01 / 2.25).  After the older sources have been seen, not before:
     // otherwise whole diagonals of tasks wait for them on SMs that others could use (2.03).
     PushedCell pushed{0u, 0u, 0u};
-    if (tid == 2 * 32) pushed = cell_arrive(p, r + 1, c);
-    if (tid == 3 * 32) pushed = cell_arrive(p, r, c + 1);
+    if (tid == 2 * 32 || tid == 3 * 32) pushed = cell_arrive(p, r + (tid == 2 * 32), c + (tid == 3 * 32));
 #pragma unroll
     for (int i = 0; i < PULL_STAGES - 1; ++i) {
         const bool go = i < ns;
@@ -671,7 +670,7 @@ __device__ __forceinline__ void sweep_cell(int r, int c, double *smem, const Til
         ask_end(go);
     }
     for (int k = tid; k < NLEAF * 2 * XCH_BUF; k += TILED_THREADS) xch[k] = 0.0;
-    push_finish(p, pushed);
+    push_finish(p, pushed);                                           // not later: the consumer may be a CTA whose cell this one waits for
     // The operands of the sweep have landed, for all threads: the neighbours may look for results in the place of the far sums, and the
     // coefficient tables of the diagonal leaves (see sweep_leaf) can be made.
     auto prepare = [&]() {
