@@ -3,15 +3,16 @@
 // Same restatement of Algorithm 3 on 128 x 128 tiles as round_tiled.cu (Eq. 11, Eq. 15-17): for tile
 // (I, J), Cd = sum_{I' < I} L[r, I'] E[I', c] and Rt = sum_{J' < J} C[r, J'] U[J', c] are dense
 // contractions, and Algorithm 3 on the tile alone, started from Y = X + Rt + Cd, C = Cd, gives the
-// tile's Z, E and C = L E.  There, one CTA of eight warps does either a far contraction or a 64 x 64
-// quadrant task at a time, so the fp64 tensor pipe of an SM idles for most of every quadrant task
+// tile's Z, E and C = L E.  There, one CTA of eight warps does either a far contraction or a task of
+// the sweep proper at a time (cells of 32 x 32 today; quadrants of 64 x 64 when this kernel was written, and it
+// keeps those), so the fp64 tensor pipe of an SM idles for most of every such task
 // (leaf sweeps are chains of dependent rint / add / fma steps).  Here a CTA has sixteen warps with two
 // fixed roles that share nothing but the device-wide scheduler words:
 //   * warps 0-7, the FAR group: claim far parts wave by wave from one atomic counter and run them as a
 //     DMMA contraction on a 128 x 64 register accumulator, operand slabs brought in by TMA
 //     (cp.async.bulk.tensor, 128-byte swizzle; every CTA fetches its own copy) through a three-stage mbarrier
 //     ring.  The group synchronises only with itself (mbarriers, one named barrier per far part).
-//   * warps 8-15, the QUADRANT group: serve the ready ring; a quadrant task is the one of round_tiled.cu
+//   * warps 8-15, the QUADRANT group: serve the ready ring; a quadrant task
 //     (pulls from the two nearest tiles, then 15 leaf-waves streamed from its two neighbours) on the
 //     group's own 150 KB of shared memory, synchronising on its own named barrier.
 // The warp schedulers interleave the two: while a leaf sweep waits on its dependent arithmetic the far
@@ -192,7 +193,7 @@ __device__ __forceinline__ void quad_load_from(QAcc &acc, const double *D, long 
             acc.v[a][b][1] = v.y;
         }
 }
-// left-looking feedback of the leaves already swept into leaf (a, b); see round_tiled.cu
+// left-looking feedback of the leaves already swept into leaf (a, b)
 __device__ __forceinline__ void leaf_pull(double *Ys, double *Cs, const double *Ls, const double *Us, int a, int b,
                                           int g, int t) {
     double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0, r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
@@ -246,7 +247,7 @@ __device__ __forceinline__ void await_progress(const FusedParams &p, const unsig
     __syncwarp();
 }
 
-// ---- ready ring and arrivals (same protocol as round_tiled.cu) --------------------------------
+// ---- ready ring and arrivals ------------------------------------------------------------------
 __device__ __forceinline__ void ready_push(const FusedParams &p, unsigned entry) {
     unsigned t = atomicAdd(p.q_tail, 1u);
     st_release_u32(p.q_slots + (t & p.qmask), entry | 0x80000000u);
@@ -287,8 +288,8 @@ __device__ __forceinline__ void quadrant_arrive(const FusedParams &p, int I, int
     }
 }
 
-// Algorithm 3 on one 64 x 64 quadrant in shared memory, streamed from its two neighbours; identical in
-// arithmetic and order to quadrant_sweep of round_tiled.cu.  The off-diagonal factor blocks that feed
+// Algorithm 3 on one 64 x 64 quadrant in shared memory, streamed from its two neighbours.  The order
+// of its sums is not that of the cells of round_tiled.cu, so last bits of E may differ between the two kernels.  The off-diagonal factor blocks that feed
 // the streamed pulls (L[rows, rows above], U[columns left, columns]) come as register fragments:
 // lfa[i] = L[row block `warp`, k = t + 4 i], ufl[i] = U[k = t + 4 i, column block `warp`].
 __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const double *LU, const double (&lfa)[16],
@@ -458,7 +459,7 @@ __device__ __forceinline__ void quadrant_sweep(double *Ys, double *Cs, const dou
     }
 }
 
-// One quadrant task (see round_tiled.cu, sweep_quadrant).  qs: the group's shared memory.
+// One quadrant task.  qs: the group's shared memory.
 __device__ __forceinline__ void sweep_quadrant(int I, int J, int q, double *qs, double *xch, unsigned long long *s_badkey,
                                                const FusedParams &p, double &max_abs_e, int qtid, volatile int *qsweeping) {
     double *Ys = qs, *Cs = qs + QMAT, *LU = qs + 2 * QMAT, *AUX = qs + 3 * QMAT;

@@ -65,7 +65,7 @@ int launch_round_tiled(const TiledParams &p, void *ws, size_t ws_bytes, cudaStre
 void round_split_set_min(long order);
 // most bits of a cell index in a batched launch; larger matrices are swept by themselves (tests; 0: the default)
 void round_batched_set_cell_bits(long bits);
-// The sixteen-warp kernel (round_fused.cu): far contractions and quadrant tasks side by side on every SM.
+// The sixteen-warp kernel (round_fused.cu): far contractions and 64 x 64 tasks side by side on every SM.
 // Modes: 0 never (default: it measures slower than the eight-warp kernel), 1 problems of at least 8 x 8
 // tiles, 2 whenever the operands allow it (tests, comparison runs).
 void round_fused_set_mode(int mode);
@@ -74,8 +74,8 @@ void round_tiled_f32_set_tma_mode(int mode);
 size_t round_tiled_f32_workspace_bytes(int m, int n);
 int launch_round_tiled_f32(const TiledParams &p, void *ws, size_t ws_bytes, cudaStream_t stream);
 // many matrices in one launch (fp64 tiled sweep); `info` is shared, `min_margin` (optional) gets one value per matrix
-constexpr int BATCH_MAX_COUNT = 8192;     // matrix index has 13 bits in a ready-ring entry
-constexpr int BATCH_MAX_DIM = 32768;      // tile coordinates have 8 bits there
+constexpr int BATCH_MAX_COUNT = 8192;     // the far-part table has 13 bits for the matrix index (a ring entry takes what the cell index leaves)
+constexpr int BATCH_MAX_DIM = 32768;      // and 8 bits for a tile coordinate
 size_t round_tiled_batched_workspace_bytes(int count, const TiledParams *problems);
 int launch_round_tiled_batched(int count, const TiledParams *problems, double *min_margin, int *info, void *ws,
                                size_t ws_bytes, cudaStream_t stream);

@@ -1140,7 +1140,10 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
 #undef VIEW
 
 // ---------------------------------------------------------------------------------------------
-constexpr int NEAR_TILES = 2;       // 1 makes cells a fifth shorter, but a far part's last source then is swept just before it is needed (4096 x 4096: 6.58 -> 6.74 ms)
+// 1 makes cells a fifth shorter, but a far part's last source then is swept just before it is needed; 3 makes them longer.  1 / 2 / 3:
+// 512 x 512 319 / 280 / 255 us, 1024 x 4096 1.81 / 1.57 / 1.80 ms, 2999 x 1803 2.19 / 2.17 / 2.21, 2048 x 3072 2.31 / 2.18 / 2.16,
+// 4096 x 4096 6.49 / 6.09 / 6.13, 64 matrices of 256 x 256 and 256 x 512 849 / 832 / 835 us.
+constexpr int NEAR_TILES = 2;
 static size_t pad256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct TiledLayout {
@@ -1187,8 +1190,8 @@ static SplitLayout split_layout(int m, int n) {
     const TiledLayout t = tiled_layout(m, n);
     l.total = t.total;
     if (std::min(m, n) < g_split_min.load() || t.ntm < 2 || t.ntn < 2) return l;
-    // The middle launch goes through the batched kernel, whose claim table and ready ring hold tile indices in 8 bits, so the
-    // first block (the largest) must stay within its limit.  Longer matrices are swept whole, with 14 and 15 bits.
+    // The middle launch goes through the batched kernel, whose claim table holds tile indices in 8 bits, so the first block (the
+    // largest) must stay within its limit.  Longer matrices are swept whole: a single launch needs no table.
     const int m0 = (t.ntm + 1) / 2 * T, n0 = (t.ntn + 1) / 2 * T;
     if (std::max(m0, n0) > BATCH_MAX_DIM) return l;
     l.m0 = m0; l.n0 = n0;
@@ -1228,7 +1231,7 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
     TiledLayout l = tiled_layout(in.m, in.n);
     if (ws_bytes < l.total) return GPTQ2D_ERR_WORKSPACE;
     {
-        // large resident problems: far contractions and quadrant tasks side by side on every SM (round_fused.cu)
+        // where it is asked for: far contractions and 64 x 64 tasks side by side on every SM (round_fused.cu)
         const int st = launch_round_fused(in, ws, ws_bytes, stream, false);
         if (st != -1) return st;
     }

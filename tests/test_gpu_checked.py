@@ -1,6 +1,6 @@
 """The small parity cases once more under the CHECKED build of the library (libgptq2d_checked.so,
--DGPTQ2D_CHECKED): every index that feeds a shared- or global-memory access of the tiled sweep, of its
-DMMA tile loop, of the blocked sweep and of the tiles of the int8 products is range-checked on the device, and a violation comes back through
+-DGPTQ2D_CHECKED): the computed indexes of every shared- and global-memory access of the tiled sweep, and the main ones
+of its DMMA tile loop, of the blocked sweep and of the tiles of the int8 products, are range-checked on the device, and a violation comes back through
 the status words as GPTQ2D_ERR_CHECK (nothing traps).  compute-sanitizer is not available where this library
 is developed; this is its stand-in.  Runs in a process of its own so that the two builds never share one."""
 import os

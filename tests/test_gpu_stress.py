@@ -1,5 +1,5 @@
 """Seeded random shapes through the tiled sweep: run-to-run bit-identity (a missing fence or a race in
-the streamed hand-over between quadrants would break it), agreement with the untiled Algorithm-3
+the streamed hand-over between cells would break it), agreement with the untiled Algorithm-3
 kernel (an independent implementation, itself checked against the oracle elsewhere), and the CPU
 oracle on a subset."""
 import numpy as np
