@@ -36,8 +36,8 @@ METRIC = "rounded entries/s (m*n / sweep time)"
 UNIT = "entries/s"
 FP64_NOMINAL_TFLOPS = 37.2     # 148 SMs x 64 fp64 FMA/clk x 2 x 1.965 GHz; the run also measures the library's own 8192^3 product
 BF16_NOMINAL_TFLOPS = 2250.0
-# fp64-equivalent peak of the int8 products: 34 products of digit planes, one M128 N128 K32 MMA per 64 cycles and SM
-INT8_SPLIT_NOMINAL_TFLOPS = 148 * 2.0 * 128 * 128 * 32 / (34 * 64) * 1.965e9 / 1e12
+# fp64-equivalent peak of the int8 products: sixteen products of residues, one M128 N128 K32 MMA per 64 cycles and SM
+INT8_SPLIT_NOMINAL_TFLOPS = 148 * 2.0 * 128 * 128 * 32 / (16 * 64) * 1.965e9 / 1e12
 FP32_NOMINAL_TFLOPS = 74.4     # 148 SMs x 128 fp32 FMA/clk x 2 x 1.965 GHz
 
 
@@ -308,7 +308,7 @@ def run_cuda(args):
         "frac": achieved / peak, "traffic": traffic,
         "kernel": kernel_name, "kernel_ms": kernel_ms, "flops_per_launch": flops, "flops_on_int8_pipe": flops_i8,
         "peak_note": "nominal rates, MEASURED_PEAKS.json has no fp64 figure: fp64 tensor (DMMA) 148 SMs x 64 FMA/clk x 2 x "
-                     "1.965 GHz = 37.2; int8 products (34 products of digit planes each, splitting not counted) %.0f; `peak` is "
+                     "1.965 GHz = 37.2; int8 products (16 products of residues each, splitting not counted) %.0f; `peak` is "
                      "the rate at which this sweep's flops would run with each at its own pipe's rate; `peak_measured` is what the "
                      "library's own 8192^3 fp64 product (DMMA) reached in this run (best of 5, CUDA events)" % INT8_SPLIT_NOMINAL_TFLOPS,
         "peak_measured": peak_measured,

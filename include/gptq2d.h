@@ -15,9 +15,12 @@
  *     Part of that size may only serve speed, and a workspace without that part is accepted too; the results are the same
  *     to rounding.  The set-up needs three square matrices of order k rounded up to 16, k rounded up to 32 values and 256
  *     bytes a side, the objective two m x n matrices (rows rounded up to 16) and a value per 128 x 128 tile; what the
- *     query returns on top holds the digit planes of large products (7 (k + 512) min(k + 512, 16384) bytes a side from
+ *     query returns on top holds the residue planes of large products (16 (k + 512) min(k + 512, 16384) bytes a side from
  *     order 1024 on), without which all products run on the fp64 tensor path.  A sweep needs two m x n matrices
- *     (both sizes rounded up to 128) and its bookkeeping; less than 1 MB more lets a large one run in blocks.
+ *     (both sizes rounded up to 128) and its bookkeeping; what lets a large one run in blocks, up to 258 MB, comes on top
+ *     (less than 1 MB at order 8192, 136 MB at 4096).
+ *     The library itself holds 78 MB on every GPU where it is loaded, in which running products keep what does not fit on chip
+ *     (i8_gemm.cu); calls on any number of streams share it.
  *   - `stream` is a cudaStream_t passed as void* (NULL = default stream).  Calls
  *     enqueue work and return; they do not synchronise.
  *   - The return value reports argument / launch errors found on the host
@@ -343,6 +346,7 @@ int gptq2d_objective(int m, int n,
  *   key 7: smaller order from which on resident fp64 sweeps run in 2 x 2 blocks (0: the default).  Workspace queries follow it.
  *   key 8: most bits of a cell index in a batched sweep (0: what the number of matrices leaves); matrices with more cells of 32 x 32
  *          are swept in launches of their own.  Tests.
+ *   key 9: columns of a tile of the products on the int8 tensor cores, 128 or 256 (0: by their size).  Tests.
  * Returns GPTQ2D_OK, or GPTQ2D_ERR_INVALID_ARG for an unknown key.
  */
 int gptq2d_internal_test_hook(int key, long value);
@@ -357,7 +361,7 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
                          const double *A, long lda, const double *B, long ldb,
                          double beta, double *C, long ldc, void *stream);
 /* The same product on the int8 tensor cores by error-free splitting, as the set-up and the objective use it for their
- * large products: both operands are written as seven base-256 digit planes in the caller's workspace (256-byte aligned,
+ * large products: both operands are written as residues modulo sixteen numbers in the caller's workspace (256-byte aligned,
  * K <= 16384), scaled along k by the largest magnitudes of op(B); tiles with rows of extreme magnitude or infinities run in fp64.  Exposed for tests. */
 size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K);
 int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, double alpha,

@@ -571,6 +571,7 @@ int gptq2d_internal_test_hook(int key, long value) {
     if (key == 4) { round_fused_set_mode((int)value); return GPTQ2D_OK; }
     if (key == 6) { round_tiled_f32_set_tma_mode((int)value); return GPTQ2D_OK; }
     if (key == 7) { round_split_set_min(value); return GPTQ2D_OK; }
+    if (key == 9) { i8_set_tile((int)value); return GPTQ2D_OK; }
     if (key == 8) { round_batched_set_cell_bits(value); return GPTQ2D_OK; }
 #ifdef GPTQ2D_CHECKED
     if (key == 5) {          // value: device int[5]; [0..3] receive the status words, [4] the redirected index

@@ -387,7 +387,7 @@ int launch_factor_small(const int (&counts)[3], const FactorSmallSide *dev_sides
 
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
 
-// Digit planes of the operands of one large product at a time (i8_gemm.cuh).  The largest is the Gram's one k x k operand;
+// Residue planes of the operands of one large product at a time (i8_gemm.cuh).  The largest is the Gram's one k x k operand;
 // the two of a product of the inverse have at most k rows together, plus padding.  Contractions end at I8_MAX_K.
 constexpr int FACTOR_I8_MIN = 1024;      // orders below keep the fp64 product: their products have few tiles
 static size_t factor_i8_bytes(int k) { return k < FACTOR_I8_MIN ? 0 : i8_planes_bytes(k + 512, std::min(k + 512, I8_MAX_K), 1); }

@@ -12,7 +12,7 @@ struct FactorLookahead {
     cudaEvent_t fork, join, panel, t2[2];
 };
 
-// `planes`: with room for the digit planes of its large products (i8_gemm.cuh); without, all products are fp64 ones
+// `planes`: with room for the residue planes of its large products (i8_gemm.cuh); without, all products are fp64 ones
 size_t factor_workspace_bytes(int m, int n, bool planes);
 size_t factor_side_workspace_bytes(int k, bool planes);
 // side 0: S = M^T M -> out = F (unit lower).  side 1: S = M M^T -> out = F^T (unit upper).

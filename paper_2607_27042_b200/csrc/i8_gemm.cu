@@ -1,45 +1,120 @@
-// fp64 products on the int8 tensor cores: splitting into digit planes, and the tcgen05 kernel that multiplies them.
+// fp64 products on the int8 tensor cores: splitting into residue planes, and the tcgen05 kernel that multiplies them.
 //
-// Arithmetic.  A row with largest entry below 2^e is written as x = 2^e (d1/256 + d2/256^2 + .. + d7/256^7) with signed
-// digits (rounded to 56 bits below 2^e).  sum_k a_k b_k is then sum over p, q of 256^-(p+q) sum_k a_p b_q; the sums over
-// k are exact in int32 (K <= 16384), and the pairs with p + q <= 9 are kept: 34 of 49.  (Without p + q = 9 the dropped
-// pairs outweigh the rounding of the digits in rows with one dominant entry, such as those of a triangular factor: the
-// set-up at order 8192 was 9e-14 off instead of 1e-15.)  What the last digit rounds off is of the order
-// 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
-// entries: 4e-16 against 3e-15 of the fp64 tensor path).  The eight int32 sums (one per p + q) are put together in int64
-// and fp64.  An entry far below the largest of its row keeps fewer than its 53 bits, which matters where the largest one meets
+// Arithmetic (Ozaki, Uchino, Imamura, "Ozaki Scheme II: a GEMM-oriented emulation of floating-point matrix multiplication using an
+// integer modular technique", 2025).  A row with largest entry below 2^e is rounded to integers x' = x 2^(56 - e), |x'| < 2^55.
+// The integer product S = sum_k a'_k b'_k has |S| <= K 2^110 <= 2^124 (K <= 16384); it is known from its residues modulo sixteen
+// coprime numbers p_i <= 256 whose product P exceeds 2^125.3.  A residue of S is the residue of one int8 product of the residues
+// of a' and b', exact in int32: sixteen int8 products, where the signed base-256 digits that stood here before took 34
+// for the same 56 bits.  S / P is the fractional part of sum_i (S mod p_i) u_i / p_i with u_i = (P / p_i)^-1 mod p_i; it is summed in 80-bit fixed
+// point (the weights cut at 2^-80: S is off by 2^53 or so and at most 2^57, 2^-57 of the largest term, sixteen times less than what the 56 bits round off) and multiplied by P.  What the 56 bits round
+// off is of the order 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
+// entries: 4e-16 against 3e-15 of the fp64 tensor path).  Rows whose integers end in zero bits (integers, fp32 data) give an S that
+// ends in as many: it is rounded there, which makes such products exact.
+// An entry far below the largest of its row keeps fewer than its 53 bits, which matters where the largest one meets
 // a zero: a scaling along k (i8_inner_tops) or a look at the result (end of the kernel) takes care of that.
 //
-// Kernel.  One CTA per 128 x 128 tile of C; tcgen05.mma kind::i8 (M 128, N 128, K 32), accumulators in tensor memory.
-// Four accumulators of 128 columns fill it, so a tile takes two passes over k: p + q = 6 .. 9 (24 products), then
-// p + q = 2 .. 5 (10 products of the first four planes only).  One warp issues the TMA loads (one three-dimensional box
-// per operand and stage: 64 bytes of k, 128 rows, 7 or 4 planes), one issues the MMAs, eight hold the partial tile
-// between the passes and write C through shared memory.  Pass 1 has two stages of 112 KB, each 48 x 64 = 3072 cycles of
-// the tensor pipe; pass 2 three of 64 KB, 1280 cycles each.
+// Kernel.  A pair of CTAs per 256 x 256 (or 256 x 128) tile of C: tcgen05.mma cta_group::2 kind::i8, M 256, K 32; each CTA loads half of
+// the rows of A and half of those of B^T and holds 128 x 256 sums in its tensor memory, twice, so that one residue's sums are
+// reduced to bytes while the next residue's are computed.  One warp issues the TMA loads (256 bytes of k a stage), one (of the
+// pair's first CTA) the MMAs, sixteen reduce.  The bytes, 16 an entry, wait in a slot that a CTA holds while it runs (512 KB,
+// written and read by the same threads, in L2) until the sixteen are there.
 //
-// Bound by the int8 tensor rate: an MMA takes 69 of its 64 cycles in pass 1 (in-kernel clocks).  Measured, splitting
-// included, against the fp64 tensor path (DMMA) of gemm.cu: 8192^3 13.5 ms (81 TFLOP/s) against 31.1, 4096^3 1.67 against
-// 4.0, 2048^3 0.29 against 0.57, rank-512 update of an 8192 x 8192 matrix 1.07 against 2.17.
+// Bound, at K = 4096, by the loads of a stage (32 KB a CTA and 128 of k: 611 cycles against the 513 of the tensor pipe), then by power; at K = 512
+// by the reduction and by putting the entries together, some 45 thousand cycles of a tile each.  Measured, without the splitting, against
+// the 34 products of digits that stood here before: 8192^3 5.8 ms (189 TFLOP/s) against 12.5, 4096^3 0.86 against 1.38, 2048^3 0.126 against
+// 0.208, rank-512 update of an 8192 x 8192 matrix 0.90 against 1.07.
 #include <cuda.h>
 #include "common.cuh"
 #include "dmma_tma.cuh"
 #include "tma_host.cuh"
 #include "i8_gemm.cuh"
+#include <algorithm>
+#include <atomic>
 
 namespace gptq2d {
 
-static_assert(I8_DIGITS == 7, "the kernel's two passes and the digit extraction are laid out for seven planes");
+// The moduli and what follows from them.
+constexpr int I8_WEIGHT_BYTES = 10;                            // 80-bit fixed point
+constexpr int I8_SNAP = 58;                                    // S is off by less than 2^57: multiples of 2^58 and more are found by rounding
+struct I8Tables {
+    int p[I8_MODULI];
+    int inv0[I8_MODULI], inv6[I8_MODULI];                      // ceil(2^32 / p), ceil(2^38 / p): floor(s / p) for |s| <= 2^24, 2^28 but for negative multiples of p
+    unsigned digit_lo[I8_MODULI], digit_hi[I8_MODULI];         // 256^j mod p as signed bytes, j = 0 .. 3, 4 .. 6
+    float pf[I8_MODULI], invf[I8_MODULI];                      // p, 1 / p
+    unsigned weight[I8_WEIGHT_BYTES][I8_MODULI / 4];           // byte b of round(2^80 u_i / p_i), four i to a word
+    double product_hi, product_lo;                             // P 2^-80 2^-40 in two parts
+};
+constexpr I8Tables i8_tables() {
+    I8Tables t{};
+    const int p[I8_MODULI] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+    unsigned __int128 product = 1;
+    for (int i = 0; i < I8_MODULI; ++i) product *= (unsigned)p[i];
+    for (int i = 0; i < I8_MODULI; ++i) {
+        const unsigned q = (unsigned)p[i];
+        t.p[i] = p[i];
+        t.inv0[i] = (int)(((1ull << 32) + q - 1) / q);
+        t.inv6[i] = (int)(((1ull << 38) + q - 1) / q);
+        t.pf[i] = (float)p[i]; t.invf[i] = 1.0f / (float)p[i];
+        unsigned power = 1;
+        for (int j = 0; j < 7; ++j) {
+            const unsigned byte = (power > q / 2 ? power - q : power) & 0xffu;
+            if (j < 4) t.digit_lo[i] |= byte << (8 * j);
+            else t.digit_hi[i] |= byte << (8 * (j - 4));
+            power = power * 256 % q;
+        }
+        const unsigned rest = (unsigned)((product / q) % q);
+        unsigned u = 1;
+        while (rest * u % q != 1) ++u;
+        unsigned __int128 w = ((((unsigned __int128)u) << (8 * I8_WEIGHT_BYTES)) + q / 2) / q;
+        for (int b = 0; b < I8_WEIGHT_BYTES; ++b, w >>= 8) t.weight[b][i / 4] |= (unsigned)(w & 0xff) << (8 * (i % 4));
+    }
+    // P < 2^126: its top 53 bits and the rest, as doubles
+    const unsigned __int128 top = product >> 73 << 73;
+    double hi = (double)(unsigned long long)(top >> 73), lo = (double)(unsigned long long)((product - top) >> 20);
+    for (int k = 0; k < 73; ++k) hi *= 2.0;
+    for (int k = 0; k < 20; ++k) lo *= 2.0;
+    for (int k = 0; k < 8 * I8_WEIGHT_BYTES + 40; ++k) { hi *= 0.5; lo *= 0.5; }
+    t.product_hi = hi; t.product_lo = lo;
+    return t;
+}
+__constant__ const I8Tables I8_TAB = i8_tables();
+static_assert([] {                                             // pairwise coprime, and P > 2 * 2^14 * 2^110
+    const I8Tables t = i8_tables();
+    unsigned __int128 product = 1;
+    for (int i = 0; i < I8_MODULI; ++i) {
+        product *= (unsigned)t.p[i];
+        for (int j = 0; j < i; ++j) {
+            int a = t.p[i], b = t.p[j];
+            while (b) { const int r = a % b; a = b; b = r; }
+            if (a != 1) return false;
+        }
+    }
+    return product >> 125 != 0;
+}(), "the residues determine the sum");
+
+static std::atomic<int> g_i8_tile{0};                          // tests: 128 or 256 columns a tile
+void i8_set_tile(int columns) { g_i8_tile.store(columns == 128 || columns == 256 ? columns : 0); }
 
 static inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 static long i8_rows_pad(int rows) { return (rows + 127L) / 128 * 128; }
-static long i8_k_pad(int K) { return (K + I8_KCHUNK - 1L) / I8_KCHUNK * I8_KCHUNK; }
+static long i8_k_pad(int K) { return (K + 127L) / 128 * 128; }
 
-size_t i8_planes_bytes(int rows, int K, int batch) {
+size_t i8_residue_bytes(int rows, int K, int batch) { return up256((size_t)i8_rows_pad(rows) * batch * (size_t)i8_k_pad(K) * I8_MODULI); }
+size_t i8_rows_bytes(int rows, int batch) {
     const size_t r = (size_t)i8_rows_pad(rows) * batch;
-    return up256(r * (size_t)i8_k_pad(K) * I8_DIGITS) + up256(r * sizeof(double)) + up256(r * sizeof(unsigned) + r / 128 * 2 * sizeof(int));
+    return up256(r * sizeof(double)) + up256(r * (sizeof(unsigned long long) + sizeof(unsigned)) + r / 128 * 2 * sizeof(int));
 }
+size_t i8_planes_bytes(int rows, int K, int batch) { return i8_residue_bytes(rows, K, batch) + i8_rows_bytes(rows, batch); }
 
-I8Planes i8_planes_at(void *at, int rows, int K, int batch) {
+// Where the CTAs of products keep residues until the sixteen of an entry are there: a slot for every CTA that runs at a time (one on an
+// SM, for its shared memory), taken and given back by the CTA itself, so that the products of all calls, streams and threads share them.  On a GPU
+// with more SMs CTAs would wait for a slot.  Not in the workspaces: a sweep's has no room for them beside the planes.
+constexpr size_t I8_SLOT_BYTES = (size_t)I8_MODULI * 128 * 256;
+constexpr int I8_SLOTS = 148;
+static __device__ unsigned i8_slot_busy[I8_SLOTS];
+static __device__ __align__(256) unsigned char i8_slot_bytes[I8_SLOTS * I8_SLOT_BYTES];
+
+I8Planes i8_planes_at(void *at, int rows, int K, int batch, void *rows_at) {
     I8Planes p{};
     p.rows = rows; p.K = K; p.batch = batch;
     p.rows_pad = i8_rows_pad(rows);
@@ -47,10 +122,11 @@ I8Planes i8_planes_at(void *at, int rows, int K, int batch) {
     const size_t r = (size_t)p.rows_pad * batch;
     char *w = static_cast<char *>(at);
     p.planes = reinterpret_cast<int8_t *>(w);
-    w += up256(r * (size_t)p.k_pad * I8_DIGITS);
+    w = rows_at ? static_cast<char *>(rows_at) : w + i8_residue_bytes(rows, K, batch);
     p.scale = reinterpret_cast<double *>(w);
     w += up256(r * sizeof(double));
-    p.maxbits = reinterpret_cast<unsigned *>(w);
+    p.bits = reinterpret_cast<unsigned long long *>(w);
+    p.maxbits = reinterpret_cast<unsigned *>(p.bits + r);
     p.plane_rows = (long)r;
     p.range = reinterpret_cast<int *>(p.maxbits + r);
     return p;
@@ -132,7 +208,7 @@ __global__ void __launch_bounds__(256) i8_rowmax_kernel(I8Planes pl, const doubl
         any = __reduce_max_sync(0xffffffffu, any);
         if ((tid & 31) == 0 && any) {
             int *range = pl.range + ((long)b * (pl.rows_pad / 128) + (r0 >> 7)) * 2;
-            atomicMax(range, (int)(pl.k_pad / I8_KCHUNK) - (int)blockIdx.x);
+            atomicMax(range, (int)gridDim.x - (int)blockIdx.x);
             atomicMax(range + 1, (int)blockIdx.x + 1);
         }
     }
@@ -147,24 +223,42 @@ __device__ __forceinline__ int i8_exponent(unsigned maxbits) {
 constexpr int I8_MAX_EXPONENT = 470;                                         // two scales 2^(e - 36) then multiply to 2^-1012 .. 2^868
 __device__ __forceinline__ double i8_pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// Digit planes of a 64 x 64 block per CTA.  Padding rows and columns become zeros.
+// Chunks of k (of I8_KCHUNK) in which the 128-row blocks [blk, blk + count) of an operand have an entry: [lo, hi), hi = 0 if none.
+__device__ __forceinline__ void i8_chunks(const int *range, int blk, int count, int blocks, int all, int &lo, int &hi) {
+    lo = all; hi = 0;
+    for (int b = blk; b < min(blk + count, blocks); ++b) {
+        lo = min(lo, all - __ldg(range + 2 * b));
+        hi = max(hi, __ldg(range + 2 * b + 1));
+    }
+}
+
+// Residues of 32 rows x 64 k per CTA.  Padding rows and columns become zeros; stages of the product (128 k) in which a pair of 128-row blocks
+// has no entry are never read (i8_where) and are left as they are.  A CTA loads, then computes (some twelve instructions a residue): many small
+// ones overlap the two (4096 x 4096: 64 rows a CTA 133 us; bytes 62).
 template <bool KCONTIG>
-__global__ void __launch_bounds__(256) i8_split_kernel(I8Planes pl, const double *src, long ld, long stride, I8Inner inner,
-                                                       int skip_diagonal) {
-    __shared__ double tile[64][65];
-    const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 64, b = blockIdx.z, tid = threadIdx.x;
+__global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const double *src, long ld, long stride, I8Inner inner,
+                                                          int skip_diagonal) {
+    __shared__ double tile[32][65];
+    const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32, b = blockIdx.z, tid = threadIdx.x;
+    {
+        const int blocks = (int)(pl.rows_pad / 128), all = (pl.K + I8_KCHUNK - 1) / I8_KCHUNK, pair = r0 / 256 * 2;
+        int lo, hi;
+        i8_chunks(pl.range + (long)b * blocks * 2, pair, 2, blocks, all, lo, hi);
+        const int per = 128 / I8_KCHUNK;
+        if ((k0 / 128 < lo / per || k0 / 128 >= (hi + per - 1) / per) && blockIdx.x > 0) return;      // (the first column of CTAs writes the scales)
+    }
     const double *S = src + (long)b * stride;
     double v[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-        const int c = tid & 63, o = (tid >> 6) + 4 * i;                     // c runs along memory
-        const int r = r0 + (KCONTIG ? o : c), k = k0 + (KCONTIG ? c : o);
+        const int o = KCONTIG ? (tid >> 6) + 2 * i : tid & 31, c = KCONTIG ? tid & 63 : (tid >> 5) + 4 * i;       // row and k; neighbours run along memory
+        const int r = r0 + o, k = k0 + c;
         v[i] = (r < pl.rows && k < pl.K && !(skip_diagonal && k == r)) ? (KCONTIG ? S[(long)r * ld + k] : S[(long)k * ld + r]) * i8_inner(inner, b, k, pl.K) : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-        const int c = tid & 63, o = (tid >> 6) + 4 * i;
-        tile[KCONTIG ? o : c][KCONTIG ? c : o] = v[i];
+        const int o = KCONTIG ? (tid >> 6) + 2 * i : tid & 31, c = KCONTIG ? tid & 63 : (tid >> 5) + 4 * i;
+        tile[o][c] = v[i];
     }
     __syncthreads();
     const int rr = tid >> 2, kk = (tid & 3) * 16, r = r0 + rr;
@@ -173,136 +267,182 @@ __global__ void __launch_bounds__(256) i8_split_kernel(I8Planes pl, const double
     const bool finite = mb < 0x7ff00000u;
     const int e = i8_exponent(mb);
     if (blockIdx.x == 0 && (tid & 3) == 0)
-        // (half of the weight 256^-8 of the last kept digit pair, 256^-9, is folded in on either side)
+        // (the product's sums count 2^-72: 2^-36 is folded in on either side)
         pl.scale[row] = finite ? i8_pow2(e - 36) : __longlong_as_double(0x7ff8000000000000ll);
     const double up = i8_pow2(min(56 - e, 1000));                           // e >= -900: at most 2^956, exact
-    uint4 out[I8_DIGITS];
+    unsigned lo[16], hi[16];
+    unsigned long long bits = 0ull;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        unsigned lo[4], hi[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const double x = finite ? tile[rr][kk + 4 * w + i] : 0.0;
-            // 56-bit fixed point, then balanced digits: adding 128 to every digit and flipping the top bits back
-            const long long f = __double2ll_rn(x * up);
-            const unsigned long long y = ((unsigned long long)f + 0x0080808080808080ull) ^ 0x0080808080808080ull;
-            lo[i] = (unsigned)y; hi[i] = (unsigned)(y >> 32);
-        }
-        // byte j of the four words -> one word (4 x 4 byte transposes); byte 0 is the least significant digit, plane 6
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned *q = h ? hi : lo;
-            const unsigned a = __byte_perm(q[0], q[1], 0x5140), c = __byte_perm(q[2], q[3], 0x5140);
-            const unsigned d = __byte_perm(q[0], q[1], 0x7362), f = __byte_perm(q[2], q[3], 0x7362);
-            const unsigned t0 = __byte_perm(a, c, 0x5410), t1 = __byte_perm(a, c, 0x7632);
-            const unsigned t2 = __byte_perm(d, f, 0x5410), t3 = __byte_perm(d, f, 0x7632);
-            const unsigned t[4] = {t0, t1, t2, t3};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int plane = 6 - (4 * h + j);
-                if (plane >= 0) {
-                    if (w == 0) out[plane].x = t[j];
-                    else if (w == 1) out[plane].y = t[j];
-                    else if (w == 2) out[plane].z = t[j];
-                    else out[plane].w = t[j];
-                }
-            }
-        }
+    for (int i = 0; i < 16; ++i) {
+        const double x = finite ? tile[rr][kk + i] : 0.0;
+        // 56-bit integer, then balanced base-256 digits: adding 128 to every digit and flipping the top bits back
+        const long long f = __double2ll_rn(x * up);
+        bits |= (unsigned long long)f;
+        const unsigned long long y = ((unsigned long long)f + 0x0080808080808080ull) ^ 0x0080808080808080ull;
+        lo[i] = (unsigned)y; hi[i] = (unsigned)(y >> 32);
     }
+    bits |= __shfl_xor_sync(0xffffffffu, bits, 1);
+    bits |= __shfl_xor_sync(0xffffffffu, bits, 2);
+    if ((tid & 3) == 0 && bits) atomicOr(pl.bits + row, bits);
     const long plane_bytes = pl.plane_rows * pl.k_pad;
-    int8_t *dst = pl.planes + row * pl.k_pad + k0 + kk;
+    int8_t *dst = pl.planes + ((long)(k0 / 128) * pl.plane_rows + row) * 128 + (k0 & 64) + kk;
+#pragma unroll 4
+    for (int d = 0; d < I8_MODULI; ++d, dst += plane_bytes) {
+        const int wl = (int)I8_TAB.digit_lo[d], wh = (int)I8_TAB.digit_hi[d];
+        const float p = I8_TAB.pf[d], inv = I8_TAB.invf[d];
+        unsigned w[4];
 #pragma unroll
-    for (int d = 0; d < I8_DIGITS; ++d) *reinterpret_cast<uint4 *>(dst + d * plane_bytes) = out[d];
+        for (int q = 0; q < 4; ++q) {
+            unsigned t[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // x' mod p from its digits' residues, as their sum s added to the bits of 1.5 * 2^23 (raw = 1.5 * 2^23 + s, f = s); |s| <= 7 * 128 * 127 < 2^17, so s and the nearest
+                // multiple of p are found exactly in fp32 (s / p is off by 2^-13 at most, 1 / 2p from a tie) and |s - q p| <= p / 2
+                const float raw = __int_as_float(__dp4a((int)lo[4 * q + i], wl, __dp4a((int)hi[4 * q + i], wh, 0x4b400000))), f = raw - 12582912.0f;
+                const float k = fmaf(f, inv, 12582912.0f) - 12582912.0f;
+                t[i] = (unsigned)__float_as_int(fmaf(-k, p, raw));
+            }
+            w[q] = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
+        }
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
 }
 
 cudaError_t i8_split(const I8Planes &pl, const double *src, long ld, long stride, bool k_contig, cudaStream_t stream,
                      const I8Inner &inner, bool skip_diagonal) {
     const size_t r = (size_t)pl.rows_pad * pl.batch;
-    cudaError_t e = cudaMemsetAsync(pl.maxbits, 0, r * sizeof(unsigned) + r / 128 * 2 * sizeof(int), stream);
+    cudaError_t e = cudaMemsetAsync(pl.bits, 0, r * (sizeof(unsigned long long) + sizeof(unsigned)) + r / 128 * 2 * sizeof(int), stream);
     if (e != cudaSuccess) return e;
     const dim3 gm((pl.K + 63) / 64, (pl.rows + 63) / 64, pl.batch);
-    const dim3 gs((unsigned)(pl.k_pad / 64), (unsigned)(pl.rows_pad / 64), pl.batch);
+    const dim3 gs((unsigned)(pl.k_pad / 64), (unsigned)(pl.rows_pad / 32), pl.batch);
     if (k_contig) {
         i8_rowmax_kernel<true><<<gm, 256, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
-        i8_split_kernel<true><<<gs, 256, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
+        i8_split_kernel<true><<<gs, 128, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
     } else {
         i8_rowmax_kernel<false><<<gm, 256, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
-        i8_split_kernel<false><<<gs, 256, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
+        i8_split_kernel<false><<<gs, 128, 0, stream>>>(pl, src, ld, stride, inner, skip_diagonal ? 1 : 0);
     }
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
-constexpr int I8_TILE_BYTES = 128 * I8_KCHUNK;                 // one plane of one operand in a stage: 8 KB
-constexpr int I8_STAGE_BYTES = 2 * I8_DIGITS * I8_TILE_BYTES;  // 112 KB
-constexpr int I8_STAGES = 2;
-constexpr int I8_TOP = 4;                                      // planes of the second pass (p + q <= 5)
-constexpr int I8_STAGE2_BYTES = 2 * I8_TOP * I8_TILE_BYTES;    // 64 KB
-constexpr int I8_STAGES2 = 3;
-static_assert(I8_STAGES2 * I8_STAGE2_BYTES <= I8_STAGES * I8_STAGE_BYTES, "pass 2 reuses the memory of pass 1");
-constexpr int I8_OUT_LD = 130;                                 // row pitch (doubles) of the tile on its way out: rows start on 16 bytes
-constexpr size_t I8_SMEM = (size_t)I8_STAGES * I8_STAGE_BYTES + 1024;       // (leaves 2 KB of a CTA's 227 for what is declared in the kernel)
-static_assert(128 * I8_OUT_LD * 8 <= I8_STAGES * I8_STAGE_BYTES, "the output tile reuses the stages");
-constexpr int I8_THREADS = 320;                                // warps 0-7 epilogue, 8 TMA, 9 MMA and tensor memory
+constexpr int I8_STAGE_K = 128;                                // bytes of k in a stage: one swizzle row
+constexpr int I8_A_BYTES = 128 * I8_STAGE_K;                   // 128 rows of op(A): 16 KB
+constexpr int I8_STAGES = 3;
+constexpr int I8_DEEP = 2;                                     // pieces of I8_STAGE_K a stage
+constexpr int I8_OUT_LD = 130;                                 // row pitch (doubles) of a tile computed in fp64: rows start on 16 bytes
+constexpr int I8_WARPS = 16;                                   // warps that reduce and write
+constexpr int I8_THREADS = (I8_WARPS + 2) * 32;                // then one for TMA, one for the MMAs and tensor memory
+template <int TN> struct I8Tile {
+    static constexpr int B_BYTES = TN / 2 * I8_STAGE_K;        // half of the columns of the tile
+    static constexpr int PIECE = I8_A_BYTES + B_BYTES, STAGE = I8_DEEP * PIECE;
+    static constexpr size_t SMEM = (size_t)I8_STAGES * STAGE + 1024;
+    static constexpr size_t SMEM_MIN = 128 * I8_OUT_LD * 8 + 1024;         // a tile in fp64 reuses the stages
+};
+static_assert(I8Tile<256>::SMEM <= 227 * 1024 - 1024 && I8Tile<128>::SMEM >= I8Tile<128>::SMEM_MIN, "shared memory of a CTA");
+// one CTA on an SM: the slots of residue bytes are counted on it
+static_assert(2 * I8Tile<128>::SMEM > 227 * 1024, "a slot of residue bytes per SM");
 
-// K-major operand tile of 128 rows x 64 bytes in the 64-byte swizzle: eight-row groups 512 bytes apart
+// K-major operand tile of rows of 128 bytes in the 128-byte swizzle: eight-row groups 1024 bytes apart
 __device__ __forceinline__ unsigned long long i8_smem_desc(unsigned addr) {
-    return (unsigned long long)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((unsigned long long)(512 >> 4) << 32) |
-           (1ull << 46) | (4ull << 61);
+    return (unsigned long long)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((unsigned long long)(1024 >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
 }
-// instruction descriptor: s32 accumulator, s8 operands, both K-major, N = 128, M = 128
-constexpr unsigned I8_IDESC = (2u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-
+// instruction descriptor: s32 accumulator, s8 operands, both K-major, N = TN, M = 256
+template <int TN>
 __device__ __forceinline__ void i8_mma(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned accumulate) {
+    constexpr unsigned IDESC = (2u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(TN >> 3) << 17) | ((256u >> 4) << 24);
     asm volatile(
         "{\n"
         ".reg .pred p;\n"
         "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem), "l"(a), "l"(b), "r"(I8_IDESC), "r"(accumulate)
+        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem), "l"(a), "l"(b), "r"(IDESC), "r"(accumulate)
         : "memory");
 }
+// arrives at this barrier of both CTAs when every MMA issued so far has completed
 __device__ __forceinline__ void i8_commit(unsigned long long *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(smem_u32(bar)),
+                 "h"((unsigned short)3)
+                 : "memory");
 }
-__device__ __forceinline__ void i8_tmem_ld4(int (&v)[4], unsigned addr) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+// address of the same variable in the pair's first CTA
+__device__ __forceinline__ unsigned i8_in_first(const void *p) {
+    unsigned a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(a) : "r"(smem_u32(p)));
+    return a;
+}
+// (relaxed: what it orders are reads of tensor memory, which have arrived in registers and are fenced by tcgen05.fence; a release would
+// wait for the warp's stores to reach L2 every time: 2900 cycles a residue)
+__device__ __forceinline__ void i8_arrive_first(unsigned bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+// 3-D tiled copy global -> this CTA's shared memory, its bytes reported to a barrier of the pair's first CTA
+__device__ __forceinline__ void i8_load(void *dst, const CUtensorMap *map, int x, int y, int z, unsigned bar_in_first) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5}], [%2];\n" ::"r"(
+            smem_u32(dst)),
+        "l"(map), "r"(bar_in_first), "r"(x), "r"(y), "r"(z)
+        : "memory");
+}
+__device__ __forceinline__ void i8_pair_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+__device__ __forceinline__ void i8_tmem_ld32(int (&v)[32], unsigned addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+                   "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
+                   "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),
+                   "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                  : "r"(addr));
 }
 __device__ __forceinline__ void i8_tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void i8_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void i8_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-
-// (double)v for |v| < 2^51, by the bits of 1.5 * 2^52 + v: an integer addition and one fp64 addition (the conversion
-// instruction runs at a quarter of the fp64 rate)
-__device__ __forceinline__ double i8_to_double(long long v) {
-    return __longlong_as_double(v + 0x4338000000000000ll) - 6755399441055744.0;
+// barrier of the warps that reduce, and the same with the disjunction of a flag
+__device__ __forceinline__ void i8_reducers() { asm volatile("barrier.cta.sync 1, %0;\n" ::"n"(I8_WARPS * 32) : "memory"); }
+__device__ __forceinline__ bool i8_reducers_or(bool flag) {
+    unsigned r;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.u32 p, %1, 0;\n"
+        "barrier.cta.red.or.pred q, 1, %2, p;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n"
+        : "=r"(r)
+        : "r"((unsigned)flag), "n"(I8_WARPS * 32)
+        : "memory");
+    return r != 0u;
 }
 
 struct I8Params {
-    int M, N, K;
+    int M, N, K, k_blocks;
     double alpha, beta;
     double *C; long ldc, strideC;
     double *sumsq_partials;
     const double *scaleA, *scaleB;
     long rowsA_pad, rowsB_pad;
     const int *rangeA, *rangeB;
-    int lower_tiles_only, tiles_m, tiles_n;
+    int lower_tiles_only, tiles_m, tiles_n, tiles, batch;      // tiles of 256 x TN, those of one matrix
     // diagonals left out of the planes: op(A)[i][j] = A[i * ai + j * aj], op(B)[i][j] = B[i * bi + j * bj]
     int diag_a, diag_b;
     const double *A; long ai, aj, strideA;
     const double *B; long bi, bj, strideB;
     const unsigned *topA, *topB;                               // high words of the largest magnitude of every row of either operand's planes
+    const unsigned long long *bitsA, *bitsB;                   // all bits that occur in a row's integers
     int rowsA, rowsB;                                          // rows that exist there
     double least;
     int *info;
 };
 
 // The tile once more in fp64, for operands that its digits do not suit (see below): alpha * op(A) op(B) over [k_lo, k_hi) into the output
-// tile in shared memory, or the sum of its squares.  Warps 0 - 7, the others have left.  The loop is gemm.cu's, at its speed.
+// tile in shared memory, or the sum of its squares.  All sixteen warps, 32 x 32 entries each; the copies are gemm.cu's.
 template <bool A_KCONTIG, bool B_KCONTIG>
 __device__ __noinline__ double i8_tile_in_fp64(const I8Params &p, int bz, int m0, int n0, int k_lo, int k_hi, double *smem, bool sumsq) {
+    using SL = SlabLayout<A_KCONTIG, B_KCONTIG>;
+    constexpr int STAGES = 3;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wm = warp >> 2, wn = warp & 3, g = lane >> 2, t = lane & 3;
     Operand A, B;
     A.ptr = p.A + (long)bz * p.strideA + (long)m0 * p.ai + (long)k_lo * p.aj;
@@ -313,76 +453,329 @@ __device__ __noinline__ double i8_tile_in_fp64(const I8Params &p, int bz, int m0
     B.ld = B_KCONTIG ? p.bj : p.bi;
     B.mn_valid = min(128, p.rowsB - n0);
     B.aligned16 = ((reinterpret_cast<uintptr_t>(B.ptr) & 15) == 0) && ((B.ld & 1) == 0);
-    Acc acc;
-    acc.zero();
-    gemm_tile<A_KCONTIG, B_KCONTIG, 3>(acc, smem, A, B, k_hi - k_lo);
+    const int K = k_hi - k_lo, nk = (K + BK - 1) / BK;
+    auto load = [&](int slab) {
+        if (slab < nk && tid < GEMM_THREADS) {
+            double *st = smem + (slab % STAGES) * SL::STAGE_DOUBLES;
+            load_slab<A_KCONTIG>(st, A, slab * BK, K, tid);
+            load_slab<B_KCONTIG>(st + SL::A_DOUBLES, B, slab * BK, K, tid);
+        }
+        cp_async_commit();
+    };
+    double c[4][4][2];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) c[a][b][0] = c[a][b][1] = 0.0;
+    for (int i = 0; i < STAGES - 1; ++i) load(i);
+    for (int kt = 0; kt < nk; ++kt) {
+        cp_async_wait<STAGES - 2>();
+        __syncthreads();
+        load(kt + STAGES - 1);
+        const double *As = smem + (kt % STAGES) * SL::STAGE_DOUBLES, *Bs = As + SL::A_DOUBLES;
+#pragma unroll
+        for (int kk = 0; kk < BK; kk += 4) {
+            double af[4], bf[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int r = wm * 32 + a * 8 + g, q = wn * 32 + a * 8 + g;
+                af[a] = A_KCONTIG ? As[r * LDK + kk + t] : As[(kk + t) * LDN + r];
+                bf[a] = B_KCONTIG ? Bs[q * LDK + kk + t] : Bs[(kk + t) * LDN + q];
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) dmma_m8n8k4(c[a][b][0], c[a][b][1], af[a], bf[b]);
+        }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
     double s = 0.0;
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const double x0 = p.alpha * acc.v[a][b][0], x1 = p.alpha * acc.v[a][b][1];
+            const double x0 = p.alpha * c[a][b][0], x1 = p.alpha * c[a][b][1];
             if (sumsq) s = fma(x1, x1, fma(x0, x0, s));        // (rows and columns that do not exist are zeros)
-            else *reinterpret_cast<double2 *>(smem + CI((wm * 64 + a * 8 + g) * I8_OUT_LD + wn * 32 + b * 8 + 2 * t, 128 * I8_OUT_LD - 1, 302)) = double2{x0, x1};
+            else *reinterpret_cast<double2 *>(smem + CI((wm * 32 + a * 8 + g) * I8_OUT_LD + wn * 32 + b * 8 + 2 * t, 128 * I8_OUT_LD - 1, 302)) = double2{x0, x1};
         }
     return s;
 }
 
-__global__ void __launch_bounds__(I8_THREADS, 1)
-i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUtensorMap mapA7, const __grid_constant__ CUtensorMap mapB7,
-               const __grid_constant__ CUtensorMap mapA4, const __grid_constant__ CUtensorMap mapB4) {
-    extern __shared__ __align__(16) unsigned char i8_raw[];
-    __shared__ __align__(8) unsigned long long bar_full[I8_STAGES], bar_empty[I8_STAGES], bar_full2[I8_STAGES2], bar_empty2[I8_STAGES2], bar_acc, bar_drained;
-    __shared__ unsigned s_tmem, s_abort, s_all_k;
-    __shared__ double s_sum[8];
-    __shared__ int s_scale[128];                               // of the tile's columns: high words (the low ones are zero)
-    __shared__ unsigned s_seen[8];                             // bit per row (words 0 - 3) and column (4 - 7): it has an entry that is large enough, see below
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    CHECKED_SET_INFO(p.info);
-    // Tiles in groups of sixteen tile rows, column by column inside a group, so that the CTAs that run at one time share
-    // operand tiles in L2; the last rows first, which have the longest contractions where there are lower triangles.
-    int tm, tn;
-    {
-        constexpr int GROUP = 16;
-        const int id = blockIdx.x, per = GROUP * p.tiles_n, grp = id / per, first = grp * GROUP;
-        const int rows = min(GROUP, p.tiles_m - first), in = id - grp * per;
-        tn = in / rows;
-        tm = first + (in - tn * rows);
-        tm = p.tiles_m - 1 - tm;
+// One tile of the product, as every warp of the pair sees it.
+struct I8Where {
+    int bz, m0, n0;                                            // first row and column of the tile
+    int k_lo, stages;                                          // contraction: pieces of I8_STAGE_K
+};
+// Tiles in groups of eight tile rows, column by column inside a group, so that the CTAs that run at one time share
+// operand tiles in L2.  The rows and columns with the longer contractions first, where an operand is a triangle (4096 x 4096 with a triangular
+// left operand, rows in the wrong order: 0.70 ms).  false: a tile above the diagonal that fills up a group.
+template <int TN>
+__device__ __forceinline__ bool i8_where(const I8Params &p, int id, I8Where &w) {
+    constexpr int GROUP = 8, PER = I8_STAGE_K / I8_KCHUNK;
+    const int all = (p.K + I8_KCHUNK - 1) / I8_KCHUNK, blocksA = (int)(p.rowsA_pad / 128), blocksB = (int)(p.rowsB_pad / 128);
+    w.bz = p.batch > 1 ? id / p.tiles : 0;
+    const int *rangeA = p.rangeA + (long)w.bz * blocksA * 2, *rangeB = p.rangeB + (long)w.bz * blocksB * 2;
+    int in = id - w.bz * p.tiles, hi = p.tiles_m, tm = 0, tn = 0;            // rows [lo, hi) of the group
+    while (hi > 0) {
+        const int lo = max(0, hi - GROUP), rows = hi - lo;
+        const int cols = p.lower_tiles_only ? min(p.tiles_n, hi * (256 / TN)) : p.tiles_n;
+        if (in < rows * cols) {
+            tn = in / rows;
+            tm = hi - 1 - (in - tn * rows);
+            break;
+        }
+        in -= rows * cols;
+        hi = lo;
     }
-    if (p.lower_tiles_only && tn > tm) return;
-    const int bz = blockIdx.y;
-    const int m0 = tm * 128, n0 = tn * 128;
+    int la, ha, lb, hb, lc, hc;
+    if (!p.lower_tiles_only) {
+        i8_chunks(rangeA, 0, 2, blocksA, all, la, ha);
+        i8_chunks(rangeA, blocksA - 1, 1, blocksA, all, lc, hc);
+        if (ha - la > hc - lc) tm = p.tiles_m - 1 - tm;
+        i8_chunks(rangeB, 0, 2, blocksB, all, lb, hb);
+        i8_chunks(rangeB, blocksB - 1, 1, blocksB, all, lc, hc);
+        if (hb - lb < hc - lc) tn = p.tiles_n - 1 - tn;
+    }
+    w.m0 = tm * 256; w.n0 = tn * TN;
+    if (p.lower_tiles_only && w.n0 > w.m0 + 255) return false;
     // chunks of k in which both operands have an entry (a triangular operand halves them)
-    const int *ra_ = p.rangeA + ((long)bz * (p.rowsA_pad / 128) + CI(tm, p.rowsA_pad / 128, 303)) * 2;
-    const int *rb_ = p.rangeB + ((long)bz * (p.rowsB_pad / 128) + CI(tn, p.rowsB_pad / 128, 304)) * 2;
-    const int all = (p.K + I8_KCHUNK - 1) / I8_KCHUNK;
-    const int c_lo = all - min(ra_[0], rb_[0]), nchunk = max(0, min(ra_[1], rb_[1]) - c_lo);
-    const int k_lo = c_lo * I8_KCHUNK;
+    i8_chunks(rangeA, w.m0 / 128, 2, blocksA, all, la, ha);
+    i8_chunks(rangeB, w.n0 / 128, TN / 128, blocksB, all, lb, hb);
+    const int c_lo = max(la, lb), c_hi = min(ha, hb);
+    w.k_lo = c_lo / PER * I8_STAGE_K;
+    w.stages = c_hi > c_lo ? (c_hi + PER - 1) / PER - c_lo / PER : 0;
+    return true;
+}
+
+// S * 2^-40 of four columns from their residues, x[i] the four columns' bytes of residue i: see the head of this file.
+__device__ __forceinline__ void i8_from_residues(double (&v)[4], const unsigned (&x)[I8_MODULI]) {
+    unsigned r[4][I8_MODULI / 4];                              // column j: residues 4 g .. 4 g + 3 in one word
+#pragma unroll
+    for (int g = 0; g < I8_MODULI / 4; ++g) {
+        const unsigned a = __byte_perm(x[4 * g], x[4 * g + 1], 0x5140), c = __byte_perm(x[4 * g + 2], x[4 * g + 3], 0x5140);
+        const unsigned d = __byte_perm(x[4 * g], x[4 * g + 1], 0x7362), f = __byte_perm(x[4 * g + 2], x[4 * g + 3], 0x7362);
+        r[0][g] = __byte_perm(a, c, 0x5410); r[1][g] = __byte_perm(a, c, 0x7632);
+        r[2][g] = __byte_perm(d, f, 0x5410); r[3][g] = __byte_perm(d, f, 0x7632);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        unsigned d[I8_WEIGHT_BYTES];                           // sums for every byte of the weights, below 2^20
+#pragma unroll
+        for (int b = 0; b < I8_WEIGHT_BYTES; ++b) {
+            d[b] = 0u;
+#pragma unroll
+            for (int g = 0; g < I8_MODULI / 4; ++g) d[b] = __dp4a(r[j][g], I8_TAB.weight[b][g], d[b]);
+        }
+        // the sum modulo 2^80, as a signed number: hi 2^64 + mid 2^32 + lo
+        const unsigned long long x0 = (unsigned long long)(d[0] + (d[1] << 8)) + ((unsigned long long)(d[2] + (d[3] << 8)) << 16);
+        const unsigned long long x1 = (unsigned long long)(d[4] + (d[5] << 8)) + ((unsigned long long)(d[6] + (d[7] << 8)) << 16) + (x0 >> 32);
+        const unsigned x2 = d[8] + (d[9] << 8) + (unsigned)(x1 >> 32);
+        const int hi = (int)(x2 << 16) >> 16;
+        // (an unsigned number x as the low word of 2^52 + x)
+        const double fl = __hiloint2double(0x43300000, (int)(unsigned)x0) - 4503599627370496.0;
+        const double fm = __hiloint2double(0x43300000, (int)(unsigned)x1) - 4503599627370496.0;
+        const double fh = __hiloint2double(0x43300000, hi ^ 0x80000000) - 4503601774854144.0;
+        const double s = fma(fh, 18446744073709551616.0, fma(fm, 4294967296.0, fl));
+        v[j] = fma(s, I8_TAB.product_hi, s * I8_TAB.product_lo);
+    }
+}
+__device__ __forceinline__ void i8_load4(double (&v)[4], const double *src) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];\n" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(src) : "memory");
+}
+__device__ __forceinline__ void i8_store4(double *dst, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(dst), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
+}
+
+// Sums modulo p, a byte each: COLS columns of a warp's 32 rows from tensor memory to its words.  inv >> shift: ceil(2^(32 + shift) / p).  (Bound
+// by the multiplications, six cycles of their pipe a sum; a function of its own for its registers' sake, like the next.)
+template <int COLS>
+__device__ __noinline__ void i8_reduce(unsigned tmem, unsigned *words, int p, int inv, int shift) {
+#pragma unroll
+    for (int c = 0; c < COLS; c += 32) {
+        int v[32];
+        i8_tmem_ld32(v, tmem + c);
+        i8_tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+            unsigned r[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[e] = (unsigned)(v[j + e] - (__mulhi(v[j + e], inv) >> shift) * p);
+            __stcg(words + (c + j) / 4 * 128, __byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410));
+        }
+    }
+}
+
+// The entries of a lane's row from its residues, where they are scaled and written only: columns [0, cols) of the warp's, four at a time, to
+// dst (NULL: the row does not exist).  `scale`: the row's, with alpha; column_scale: high words of the columns'.  A function of its own, so
+// that the sixteen words on their way for the next four columns keep their registers (spilled, every load was waited for).
+template <int MOD_STRIDE>
+__device__ __noinline__ void i8_entries(const unsigned *bytes, double *dst, int cols, bool vec, double scale, const int *column_scale, double beta) {
+    unsigned x[I8_MODULI];
+#pragma unroll
+    for (int i = 0; i < I8_MODULI; ++i) x[i] = __ldcg(bytes + i * MOD_STRIDE);
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 4) {
+        const bool four = vec && c + 4 <= cols;
+        double old[4], v[4];
+        if (beta != 0.0 && dst) {
+            if (four) i8_load4(old, dst + c);
+            else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) old[j] = c + j < cols ? dst[c + j] : 0.0;
+            }
+        }
+        unsigned now[I8_MODULI];
+#pragma unroll
+        for (int i = 0; i < I8_MODULI; ++i) now[i] = x[i];
+        if (c + 4 < cols) {
+            bytes += 128;
+#pragma unroll
+            for (int i = 0; i < I8_MODULI; ++i) x[i] = __ldcg(bytes + i * MOD_STRIDE);
+        }
+        i8_from_residues(v, now);
+        const int4 cs = *reinterpret_cast<const int4 *>(column_scale + c);
+        v[0] *= scale * __hiloint2double(cs.x, 0); v[1] *= scale * __hiloint2double(cs.y, 0);
+        v[2] *= scale * __hiloint2double(cs.z, 0); v[3] *= scale * __hiloint2double(cs.w, 0);
+        if (!dst) continue;
+        if (beta != 0.0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = fma(beta, old[j], v[j]);
+        }
+        if (four) i8_store4(dst + c, v);
+        else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < cols) dst[c + j] = v[j];
+        }
+    }
+}
+
+// The same with all that a product may ask for: columns [0, cols) from first_col on of row gi.  words: NULL where every sum is zero.  za: zero bits
+// at the end of the row's integers, -100 if no sum is rounded; least > 0: rows and columns with an entry of that size leave a bit in seen (four
+// words of rows, four of columns, the warp's from at on), the entry of column at_diagonal does not count.  Returns the sum of squares if asked for.
+template <int MOD_STRIDE>
+__device__ __noinline__ double i8_entries_general(const I8Params &p, int bz, const unsigned *words, int gi, int first_col, int cols, bool vec, double sa,
+                                                  const int *column_scale, int za, double least, int at_diagonal, unsigned *seen, int at) {
+    const int lane = threadIdx.x & 31;
+    const bool there = gi < p.M, load_old = p.beta != 0.0 && !p.sumsq_partials;
+    double *dst = p.C + (long)bz * p.strideC + CI(there ? (long)gi * p.ldc + first_col : 0, (p.M - 1) * p.ldc + p.N, 305);
+    const double *Ab = p.A + (long)bz * p.strideA, *Bb = p.B + (long)bz * p.strideB;
+    const double scale = p.alpha * sa;
+    // the diagonals' products: row gi of op(B) and of op(A), walked along the columns
+    const bool row_diag = p.diag_a && gi < p.K && there;
+    const double a_gg = row_diag ? p.alpha * Ab[(long)gi * (p.ai + p.aj)] : 0.0;
+    const double *b_row = Bb + (long)gi * p.bi + (long)first_col * p.bj, *a_row = Ab + (long)gi * p.ai + (long)first_col * p.aj;
+    double sq = 0.0;
+    bool row_seen = false;
+    unsigned col_bits = 0u, x[I8_MODULI];
+    if (words) {
+#pragma unroll
+        for (int i = 0; i < I8_MODULI; ++i) x[i] = __ldcg(words + i * MOD_STRIDE);
+    }
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 4) {
+        const bool four = vec && c + 4 <= cols;
+        double old[4], v[4];
+        if (load_old && there) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) old[j] = c + j < cols ? dst[c + j] : 0.0;
+        }
+        if (words) {
+            unsigned now[I8_MODULI];
+#pragma unroll
+            for (int i = 0; i < I8_MODULI; ++i) now[i] = x[i];
+            if (c + 4 < cols) {
+                words += 128;
+#pragma unroll
+                for (int i = 0; i < I8_MODULI; ++i) x[i] = __ldcg(words + i * MOD_STRIDE);
+            }
+            i8_from_residues(v, now);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = 0.0;
+        }
+        if (za > -100) {                                       // (a row of zeros has no bits, and sums that are zero as they are)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned long long b = __ldg(p.bitsB + (long)bz * p.rowsB_pad + min((long)first_col + c + j, p.rowsB_pad - 1));
+                const int z = b ? za + __ffsll((long long)b) - 1 : -100;
+                if (z >= I8_SNAP) v[j] = i8_pow2(z - 40) * rint(v[j] * i8_pow2(40 - z));
+            }
+        }
+        if (least > 0.0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool s = fabs(v[j]) >= least && at + c + j != at_diagonal;
+                row_seen |= s;
+                if (__any_sync(0xffffffffu, s)) col_bits |= 1u << ((c + j) & 31);
+            }
+            if ((c & 31) == 28 || c + 4 >= cols) {
+                if (lane == 0) atomicOr(seen + 4 + ((at + c) >> 5), col_bits);
+                col_bits = 0u;
+            }
+        }
+        const int4 cs = *reinterpret_cast<const int4 *>(column_scale + c);
+        v[0] *= scale * __hiloint2double(cs.x, 0); v[1] *= scale * __hiloint2double(cs.y, 0);
+        v[2] *= scale * __hiloint2double(cs.z, 0); v[3] *= scale * __hiloint2double(cs.w, 0);
+        if (!there) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int gj = first_col + c + j;
+            if (c + j >= cols) continue;
+            if (p.sumsq_partials) { sq = fma(v[j], v[j], sq); continue; }
+            if (row_diag) v[j] = fma(a_gg, b_row[(c + j) * p.bj], v[j]);
+            if (p.diag_b && gj < p.K && !(p.diag_a && gi == gj)) v[j] = fma(p.alpha * a_row[(c + j) * p.aj], Bb[(long)gj * (p.bi + p.bj)], v[j]);
+            if (load_old) v[j] = fma(p.beta, old[j], v[j]);
+        }
+        if (p.sumsq_partials) continue;
+        if (four) i8_store4(dst + c, v);
+        else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < cols) dst[c + j] = v[j];
+        }
+    }
+    if (least > 0.0) {
+        const unsigned rows = __ballot_sync(0xffffffffu, row_seen);
+        if (lane == 0) atomicOr(seen + (((threadIdx.x >> 5) & 3)), rows);
+    }
+    return sq;
+}
+
+template <int TN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(I8_THREADS, 1)
+i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB) {
+    extern __shared__ __align__(16) unsigned char i8_raw[];
+    __shared__ __align__(8) unsigned long long bar_full[I8_STAGES], bar_empty[I8_STAGES], bar_acc[2], bar_drained[2], bar_done;
+    __shared__ unsigned s_tmem, s_abort, s_all_k, s_fix;
+    __shared__ int s_slot;
+    __shared__ double s_sum[I8_WARPS];
+    __shared__ __align__(16) int s_scale[TN];                  // of the tile's columns: high words (the low ones are zero, or those of a NaN that nobody sees)
+    __shared__ unsigned s_seen[2][8];                          // per 128 columns: bit per row (words 0 - 3) and column (4 - 7) with an entry that is large enough
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x & 1;
+    CHECKED_SET_INFO(p.info);
+    I8Where w;
+    if (!i8_where<TN>(p, (int)(blockIdx.x >> 1), w)) return;   // (both CTAs of the pair)
     unsigned char *stages = i8_raw + ((1024u - (smem_u32(i8_raw) & 1023u)) & 1023u);
 
     if (tid == 0) {
         for (int s = 0; s < I8_STAGES; ++s) { mbar_init(bar_full + s, 1); mbar_init(bar_empty + s, 1); }
-        for (int s = 0; s < I8_STAGES2; ++s) { mbar_init(bar_full2 + s, 1); mbar_init(bar_empty2 + s, 1); }
-        mbar_init(&bar_acc, 1);
-        mbar_init(&bar_drained, 8);
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_acc + s, 1); mbar_init(bar_drained + s, 2 * I8_WARPS); }
+        mbar_init(&bar_done, 1);
         mbar_init_fence();
         s_abort = 0u;
+        s_fix = 0u;
+        s_slot = -1;
     }
-    if (tid < 8) s_seen[tid] = 0u;
-    if (tid < 128) s_scale[tid] = __double2hiint(__ldg(p.scaleB + (long)bz * p.rowsB_pad + n0 + tid));
-    // Rows that start on 16 bytes leave as bulk copies, or bulk additions where beta = 1: the tile's old values then never
-    // come to this SM, and the next CTA starts while L2 is still adding (rank-512 update of an 8192 x 8192 matrix: the
-    // load-add-store loop took 21.6 of a tile's 76 thousand cycles).
-    const int out_rows = min(128, p.M - m0), out_cols = min(128, p.N - n0);
-    const bool bulk_out = !p.sumsq_partials && !p.diag_a && !p.diag_b && (p.beta == 0.0 || p.beta == 1.0) && ((p.ldc | out_cols | p.strideC) & 1) == 0 &&
-                          (reinterpret_cast<uintptr_t>(p.C) & 15) == 0;
-    if (warp == 9) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(&s_tmem)) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    if (tid < 16) s_seen[tid >> 3][tid & 7] = 0u;
+    if (warp == I8_WARPS + 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(&s_tmem)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n");
     }
     i8_fence_before();
     __syncthreads();
+    i8_pair_barrier();                                         // the other CTA's barriers exist
     i8_fence_after();
     const unsigned tmem = s_tmem;
     auto give_up = [&](int code) {                             // a bounded wait ran out: tell everybody, return normally
@@ -390,340 +783,330 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
         atomicExch(&s_abort, 1u);
     };
 
-    // of row tid or column tid - 128 of the tile: has it an entry at all, and might its scale not multiply with any other to a normal number
-    const auto tile_top = [&]() { return __ldg(tid < 128 ? p.topA + (long)bz * p.rowsA_pad + m0 + tid : p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128); };
-    bool looked_at = false, extreme = false;
-    if (warp == 8) {
+    if (warp == I8_WARPS) {
         if (lane == 0) {
-            const int ra = (int)(bz * p.rowsA_pad) + m0, rb = (int)(bz * p.rowsB_pad) + n0;
-            int issued = 0, issued2 = 0;
+            // (One thread's instructions bound a stage as well as the tensor pipe does, at 4096 x 4096 with 128 of k a stage: 750 cycles where
+            // the slots were found by division, 630 with what is left, against 513 of the pipe.  So a stage is 256 of k.)
+            int slot = 0, lap = 0, issued = 0;                 // next slot of the ring, times it has been around, stages issued (those in flight at most)
             bool ok = true;
-            for (int s = 0; s < nchunk && ok; ++s) {
-                const int slot = s % I8_STAGES, k = k_lo + s * I8_KCHUNK;
-                if (s >= I8_STAGES && !mbar_wait(bar_empty + slot, (unsigned)((s / I8_STAGES - 1) & 1), &s_abort)) { give_up(-20); ok = false; break; }
-                unsigned char *st = stages + slot * I8_STAGE_BYTES;
-                mbar_arrive_expect_tx(bar_full + slot, I8_STAGE_BYTES);
-                tma_load_3d(st, &mapA7, k, ra, 0, bar_full + slot);
-                tma_load_3d(st + I8_DIGITS * I8_TILE_BYTES, &mapB7, k, rb, 0, bar_full + slot);
-                issued = s + 1;
-            }
-            // the stages of pass 2 lie over those of pass 1: every MMA of pass 1 has to be done with them
-            for (int s = max(0, nchunk - I8_STAGES); s < nchunk && ok; ++s)
-                if (!mbar_wait(bar_empty + s % I8_STAGES, (unsigned)((s / I8_STAGES) & 1), &s_abort)) { give_up(-25); ok = false; }
-            for (int s = 0; s < nchunk && ok; ++s) {
-                const int slot = s % I8_STAGES2, k = k_lo + s * I8_KCHUNK;
-                if (s >= I8_STAGES2 && !mbar_wait(bar_empty2 + slot, (unsigned)((s / I8_STAGES2 - 1) & 1), &s_abort)) { give_up(-26); ok = false; break; }
-                unsigned char *st = stages + slot * I8_STAGE2_BYTES;
-                mbar_arrive_expect_tx(bar_full2 + slot, I8_STAGE2_BYTES);
-                tma_load_3d(st, &mapA4, k, ra, 0, bar_full2 + slot);
-                tma_load_3d(st + I8_TOP * I8_TILE_BYTES, &mapB4, k, rb, 0, bar_full2 + slot);
-                issued2 = s + 1;
-            }
-            if (*(volatile unsigned *)&s_abort) {              // copies still in flight land before the CTA leaves
-                for (int s = max(0, issued - I8_STAGES); s < issued; ++s)
-                    mbar_wait(bar_full + s % I8_STAGES, (unsigned)((s / I8_STAGES) & 1), nullptr, 100000);
-                for (int s = max(0, issued2 - I8_STAGES2); s < issued2; ++s)
-                    mbar_wait(bar_full2 + s % I8_STAGES2, (unsigned)((s / I8_STAGES2) & 1), nullptr, 100000);
-            }
+            const int ra = (int)(w.bz * p.rowsA_pad) + w.m0 + 128 * rank, rb = (int)(w.bz * p.rowsB_pad) + w.n0 + TN / 2 * rank;
+            const int z0 = w.k_lo / I8_STAGE_K;
+            for (int i = 0; i < I8_MODULI && ok; ++i)
+                for (int z = i * p.k_blocks + z0, end = z + w.stages; z < end; z += I8_DEEP) {
+                    if (lap > 0 && !mbar_wait(bar_empty + slot, (unsigned)((lap - 1) & 1), &s_abort)) { give_up(-20); ok = false; break; }
+                    unsigned char *st = stages + slot * I8Tile<TN>::STAGE;
+                    const unsigned bar = i8_in_first(bar_full + slot);
+                    const int pieces = min(I8_DEEP, end - z);
+                    if (rank == 0) mbar_arrive_expect_tx(bar_full + slot, pieces * 2 * I8Tile<TN>::PIECE);
+                    for (int q = 0; q < pieces; ++q, st += I8Tile<TN>::PIECE) {
+                        i8_load(st, &mapA, 0, ra, z + q, bar);
+                        i8_load(st + I8_A_BYTES, &mapB, 0, rb, z + q, bar);
+                    }
+                    issued = min(issued + 1, I8_STAGES);
+                    if (++slot == I8_STAGES) { slot = 0; ++lap; }
+                }
+            if (rank == 0 && *(volatile unsigned *)&s_abort)   // copies still in flight land before the pair leaves
+                for (int k = 0; k < issued; ++k) {
+                    if (--slot < 0) { slot = I8_STAGES - 1; --lap; }
+                    mbar_wait(bar_full + slot, (unsigned)(lap & 1), nullptr, 100000);
+                }
         }
         __syncwarp();
-    } else if (warp == 9) {
-        if (lane == 0) {
+    } else if (warp == I8_WARPS + 1) {
+        if (lane == 0 && rank == 0) {
+            const unsigned long long desc = i8_smem_desc(smem_u32(stages));      // (14 bits of address: the stages end below 2^18)
+            int slot = 0, lap = 0;
             bool ok = true;
-            for (int s = 0; s < nchunk && ok; ++s) {
-                const int slot = s % I8_STAGES;
-                if (!mbar_wait(bar_full + slot, (unsigned)((s / I8_STAGES) & 1), &s_abort)) { give_up(-22); ok = false; break; }
+            for (int i = 0; i < I8_MODULI && ok && w.stages > 0; ++i) {
+                const int buf = i & 1;
+                if (i >= 2 && !mbar_wait(bar_drained + buf, (unsigned)((i / 2 - 1) & 1), &s_abort)) { give_up(-21); ok = false; break; }
                 i8_fence_after();
-                const unsigned st = smem_u32(stages + slot * I8_STAGE_BYTES);
-                const unsigned long long da = i8_smem_desc(st), db = i8_smem_desc(st + I8_DIGITS * I8_TILE_BYTES);
+                for (int s = 0; s < w.stages; s += I8_DEEP) {
+                    if (!mbar_wait(bar_full + slot, (unsigned)(lap & 1), &s_abort)) { give_up(-22); ok = false; break; }
+                    const unsigned long long d = desc + (unsigned)(slot * (I8Tile<TN>::STAGE >> 4));
 #pragma unroll
-                for (int kk = 0; kk < I8_KCHUNK / 32; ++kk)
+                    for (int q = 0; q < I8_DEEP; ++q)
+                        if (q == 0 || s + q < w.stages) {
 #pragma unroll
-                    for (int gsum = 6; gsum <= 9; ++gsum)
-#pragma unroll
-                        for (int pp = (gsum > 8 ? gsum - 7 : 1); pp < gsum && pp <= 7; ++pp)
-                            i8_mma(tmem + (gsum - 6) * 128, da + (unsigned)(((pp - 1) * I8_TILE_BYTES + kk * 32) >> 4),
-                                   db + (unsigned)(((gsum - pp - 1) * I8_TILE_BYTES + kk * 32) >> 4),
-                                   (s > 0 || kk > 0 || pp > (gsum > 8 ? gsum - 7 : 1)) ? 1u : 0u);
-                i8_commit(bar_empty + slot);                   // completes when every MMA issued so far has
+                            for (int kk = 0; kk < I8_STAGE_K / 32; ++kk)
+                                i8_mma<TN>(tmem + buf * 256, d + (unsigned)((q * I8Tile<TN>::PIECE + kk * 32) >> 4),
+                                           d + (unsigned)((q * I8Tile<TN>::PIECE + I8_A_BYTES + kk * 32) >> 4), (s > 0 || q > 0 || kk > 0) ? 1u : 0u);
+                        }
+                    i8_commit(bar_empty + slot);           // completes when every MMA issued so far has
+                    if (++slot == I8_STAGES) { slot = 0; ++lap; }
+                }
+                if (ok) i8_commit(bar_acc + buf);
             }
-            if (nchunk > 0) {
-                i8_commit(&bar_acc);
-                // pass 2 reuses the accumulators: pass 1 must have been read out
-                if (ok && !mbar_wait(&bar_drained, 0u, &s_abort)) { give_up(-21); ok = false; }
-                i8_fence_after();
-            }
-            for (int s = 0; s < nchunk && ok; ++s) {
-                const int slot = s % I8_STAGES2;
-                if (!mbar_wait(bar_full2 + slot, (unsigned)((s / I8_STAGES2) & 1), &s_abort)) { give_up(-27); ok = false; break; }
-                i8_fence_after();
-                const unsigned st = smem_u32(stages + slot * I8_STAGE2_BYTES);
-                const unsigned long long da = i8_smem_desc(st), db = i8_smem_desc(st + I8_TOP * I8_TILE_BYTES);
-#pragma unroll
-                for (int kk = 0; kk < I8_KCHUNK / 32; ++kk)
-#pragma unroll
-                    for (int gsum = 2; gsum <= 5; ++gsum)
-#pragma unroll
-                        for (int pp = 1; pp < gsum; ++pp)
-                            i8_mma(tmem + (gsum - 2) * 128, da + (unsigned)(((pp - 1) * I8_TILE_BYTES + kk * 32) >> 4),
-                                   db + (unsigned)(((gsum - pp - 1) * I8_TILE_BYTES + kk * 32) >> 4),
-                                   (s > 0 || kk > 0 || pp > 1) ? 1u : 0u);
-                i8_commit(bar_empty2 + slot);
-            }
-            if (nchunk > 0) {
-                i8_commit(&bar_acc);
-                // after a failure: MMAs in flight finish before tensor memory is given back (bounded)
-                if (!ok) mbar_wait(&bar_acc, 1u, nullptr, 100000);
-            }
+            i8_commit(&bar_done);
         }
+        __syncwarp();
+        // tensor memory is given back, and the stages are used again, when no MMA is left (bounded)
+        if (lane == 0) mbar_wait(&bar_done, 0u, nullptr, 1000000);
         __syncwarp();
     } else {
-        // ---- epilogue warps: lane = row of the tile (its quarter), 64 columns each
-        const int row = (warp & 3) * 32 + lane, c0 = (warp >> 2) * 64;
-        const unsigned lane_base = tmem + ((unsigned)((warp & 3) * 32) << 16) + (unsigned)c0;
-        double part[64];
+        // ---- the warps that reduce: lane = row of this CTA's half of the tile, a quarter of its columns each
+        const int quarter = warp & 3, row = quarter * 32 + lane, c0 = (warp >> 2) * (TN / 4);
+        const unsigned lane_base = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)c0;
+        const int half = c0 >> 7;                              // of 128 columns
+        constexpr int HALVES = TN / 128;
         bool ok = true;
-        // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
-        const bool wide = p.rowsB - n0 >= 32, tall = p.rowsA - m0 >= 32, by_rows = wide || !tall, by_cols = tall || !wide;
-        const unsigned top = tile_top();
-        looked_at = p.least > 0.0 && top != 0u && (tid < 128 ? by_rows : by_cols);
-        extreme = top != 0u && abs(i8_exponent(top)) > I8_MAX_EXPONENT;
-        if (!p.sumsq_partials && p.beta != 0.0 && !bulk_out) {  // the old values are needed at the end: ask for them now
-            const int rows = out_rows, cols = out_cols;
-            const double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = (tid >> 3) + 32 * i, c = (tid & 7) * 16;
-                if (r < rows && c < cols) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Cb + (long)r * p.ldc + c));
+        if (tid == 0) {
+            // a slot for residue bytes: there is one for every CTA that can run, so a free one is found in one round; bounded all the same
+            unsigned at;
+            asm volatile("mov.u32 %0, %%smid;\n" : "=r"(at));
+            at %= (unsigned)I8_SLOTS;
+            for (int t = 0; t < 10000 * I8_SLOTS; ++t) {
+                if (atomicExch(i8_slot_busy + at, 1u) == 0u) { s_slot = (int)at; break; }
+                at = at + 1 < (unsigned)I8_SLOTS ? at + 1 : 0u;
             }
+            if (s_slot < 0) give_up(-25);
+            __threadfence();
         }
-        if (nchunk > 0) {
-            ok = mbar_wait(&bar_acc, 0u, &s_abort);
-            if (!ok && lane == 0) give_up(-23);
-            __syncwarp();
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) {
-                i8_fence_after();
+        i8_reducers();
+        const int slot_index = s_slot;
+        if (slot_index < 0) ok = false;
+        constexpr long MOD_STRIDE = TN / 4 * 128;              // words of four columns: [residue][four columns][row]
+        unsigned *bytes = reinterpret_cast<unsigned *>(i8_slot_bytes + (size_t)max(slot_index, 0) * I8_SLOT_BYTES) + CI((long)(c0 / 4) * 128 + row, MOD_STRIDE, 306);
+        const int m0 = w.m0 + 128 * rank, bz = w.bz, n0 = w.n0 + 128 * half;             // this CTA's rows, this warp's 128 columns
+        // (a row is judged by the columns that it meets and a column by the rows: by 32 at least, unless the tile has no more of either)
+        const auto top = [&](int q, int h) -> unsigned {   // row q of the 128, or column q - 128 of half h
+            if (q >= 256) return 0u;
+            const long at = q < 128 ? m0 + q : w.n0 + 128 * h + q - 128;
+            if (at >= (q < 128 ? p.rowsA_pad : p.rowsB_pad)) return 0u;
+            return q < 128 ? __ldg(p.topA + (long)bz * p.rowsA_pad + at) : __ldg(p.topB + (long)bz * p.rowsB_pad + at);
+        };
+        // rows of extreme magnitude, whose scales might not multiply, infinities and NaNs: not written here
+        bool in_fp64 = false;
 #pragma unroll
-                for (int c = 0; c < 64; c += 4) {              // exact: |sums| < 2^31
-                    int g6[4], g7[4], g8[4], g9[4];
-                    i8_tmem_ld4(g6, lane_base + c);
-                    i8_tmem_ld4(g7, lane_base + 128 + c);
-                    i8_tmem_ld4(g8, lane_base + 256 + c);
-                    i8_tmem_ld4(g9, lane_base + 384 + c);
-                    i8_tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        part[c + j] = fma(i8_to_double(g6[j]), 16777216.0, i8_to_double(g9[j] + g8[j] * 256ll + g7[j] * 65536ll));
-                }
-                i8_fence_before();
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bar_drained);
-            if (ok) {
-                ok = mbar_wait(&bar_acc, 1u, &s_abort);
-                if (!ok && lane == 0) give_up(-24);
+        for (int h = 0; h < HALVES; ++h) {
+            const unsigned t = top(tid, h);
+            const bool any = i8_reducers_or(t != 0u && abs(i8_exponent(t)) > I8_MAX_EXPONENT);
+            if (any && tid == 0) s_fix |= 1u << h;
+            if (h == half) in_fp64 = any;
+        }
+        // (the next barrier comes before the entries)
+        if (tid < TN) s_scale[tid] = w.n0 + tid < p.rowsB_pad ? __double2hiint(__ldg(p.scaleB + (long)bz * p.rowsB_pad + w.n0 + tid)) : 0;
+        const bool skip = in_fp64 || m0 >= p.M || n0 >= p.N || (p.lower_tiles_only && n0 > m0);
+        double sq = 0.0;
+        const int all_chunks = (p.K + I8_KCHUNK - 1) / I8_KCHUNK;
+        const bool tall = p.rowsA - m0 >= 32;
+        const int my_row = min(m0 + row, (int)p.rowsA_pad - 1);
+        const double sa = __ldg(p.scaleA + (long)bz * p.rowsA_pad + my_row);
+        // zero bits at the end of a row's integers: the sum's last bit lies at their product
+        const unsigned long long bits = __ldg(p.bitsA + (long)bz * p.rowsA_pad + my_row);
+        const int za = bits ? __ffsll((long long)bits) - 1 : -100, za_max = __reduce_max_sync(0xffffffffu, za);
+        // Which rows and columns have an entry of at least `least`, for the check below.  (The diagonal of a Gram, the same rows
+        // on both sides, says nothing about its other entries and is left out.)
+        int la, ha, lb, hb;
+        i8_chunks(p.rangeA + bz * (p.rowsA_pad / 128) * 2, m0 / 128, 1, (int)(p.rowsA_pad / 128), all_chunks, la, ha);
+        i8_chunks(p.rangeB + bz * (p.rowsB_pad / 128) * 2, n0 / 128, 1, (int)(p.rowsB_pad / 128), all_chunks, lb, hb);
+        const int chunks = max(0, min(ha, hb) - max(la, lb));
+        const double least = chunks * I8_KCHUNK > 128 ? p.least * 0x1p72 : p.least * 0x1p71;      // (entries count 2^-72)
+        // zero bits at the end of the integers of this warp's columns, the most of them
+        int zb_max = -100;
+        for (int c = lane; c < TN / 4; c += 32) {
+            const int col = w.n0 + c0 + c;
+            const unsigned long long b = col < p.rowsB_pad ? __ldg(p.bitsB + (long)bz * p.rowsB_pad + col) : 0ull;
+            if (b) zb_max = max(zb_max, __ffsll((long long)b) - 1);
+        }
+        const bool snap = za_max + __reduce_max_sync(0xffffffffu, zb_max) >= I8_SNAP;
+        // ---- sixteen times: sums -> residues modulo p_i, a byte each
+        if (w.stages > 0)
+            for (int i = 0; i < I8_MODULI && ok; ++i) {
+                const int buf = i & 1;
+                ok = mbar_wait(bar_acc + buf, (unsigned)((i / 2) & 1), &s_abort);
+                if (!ok && lane == 0) give_up(-23);
                 __syncwarp();
                 ok = __all_sync(0xffffffffu, ok);
-            }
-            if (ok) {
+                if (!ok) break;
                 i8_fence_after();
-#pragma unroll
-                for (int c = 0; c < 64; c += 4) {
-                    int g2[4], g3[4], g4[4], g5[4];
-                    i8_tmem_ld4(g2, lane_base + c);
-                    i8_tmem_ld4(g3, lane_base + 128 + c);
-                    i8_tmem_ld4(g4, lane_base + 256 + c);
-                    i8_tmem_ld4(g5, lane_base + 384 + c);
-                    i8_tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const double hi = fma(i8_to_double(g2[j]), 16777216.0, i8_to_double(g5[j] + g4[j] * 256ll + g3[j] * 65536ll));
-                        part[c + j] = fma(hi, 4294967296.0, part[c + j]);
-                    }
-                }
+                const int md = I8_TAB.p[i], shift = w.stages > 8 ? 6 : 0, inv = w.stages > 8 ? I8_TAB.inv6[i] : I8_TAB.inv0[i];
+                i8_reduce<TN / 4>(lane_base + buf * 256, bytes + i * MOD_STRIDE, md, inv, shift);
+                i8_fence_before();
+                __syncwarp();
+                if (lane == 0) i8_arrive_first(i8_in_first(bar_drained + buf));
             }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 64; ++c) part[c] = 0.0;
-        }
-        if (ok) {
-            // Which rows and columns have a digit sum of at least `least`, for the check below.  (High words compared as fp32 numbers: one
-            // instruction with the absolute value.  The diagonal of a Gram, the same rows on both sides, says nothing about its
-            // other entries and is left out.)
-            if (p.least > 0.0) {
-                const float least = __int_as_float(__double2hiint(nchunk * I8_KCHUNK > 128 ? p.least * 0x1p72 : p.least * 0x1p71));     // (digit sums count 2^-72)
-                const int at_diagonal = tall && p.topA + bz * p.rowsA_pad + m0 == p.topB + bz * p.rowsB_pad + n0 ? row - c0 : -1;
-                bool row_seen = false;
-                unsigned cols_seen[2] = {0u, 0u};
-#pragma unroll
-                for (int c = 0; c < 64; ++c) {
-                    const bool seen = fabsf(__int_as_float(__double2hiint(part[c]))) >= least && c != at_diagonal;
-                    row_seen |= seen;
-                    if (__any_sync(0xffffffffu, seen)) cols_seen[c >> 5] |= 1u << (c & 31);
-                }
-                const unsigned rows_seen = __ballot_sync(0xffffffffu, row_seen);
-                if (lane == 0) {
-                    atomicOr(&s_seen[warp & 3], rows_seen);
-                    atomicOr(&s_seen[4 + (c0 >> 5)], cols_seen[0]);
-                    atomicOr(&s_seen[5 + (c0 >> 5)], cols_seen[1]);
-                }
+        ok = !i8_reducers_or(!ok);                         // all go on or none: barriers follow
+        // ---- the entries
+        if (ok && !skip) {
+            const bool look = p.least > 0.0 && chunks > 0;
+            const int at_diagonal = tall && p.topA + bz * p.rowsA_pad + m0 == p.topB + bz * p.rowsB_pad + n0 ? row : -1;
+            double *Cb = p.C + (long)bz * p.strideC;
+            const long gi = m0 + row;
+            const bool there = gi < p.M;
+            // four entries of a row at a time; 32 bytes where they start on a boundary of that
+            const bool vec = ((reinterpret_cast<uintptr_t>(p.C) & 31) | (p.ldc & 3) | (p.strideC & 3)) == 0;
+            const int first_col = w.n0 + c0, cols = min(TN / 4, p.N - first_col);
+            const unsigned *words = w.stages > 0 ? bytes : nullptr;
+            if (cols > 0) {
+                if (words && !(snap || look || p.diag_a || p.diag_b || p.sumsq_partials))
+                    i8_entries<(int)MOD_STRIDE>(words, there ? Cb + CI(gi * p.ldc + first_col, (p.M - 1) * p.ldc + p.N, 308) : nullptr, cols, vec, p.alpha * sa, s_scale + c0, p.beta);
+                else
+                    sq = i8_entries_general<(int)MOD_STRIDE>(p, bz, words, (int)gi, first_col, cols, vec, sa, s_scale + c0, snap ? za : -100, look ? least : 0.0,
+                                                             at_diagonal, &s_seen[half][0], c0 & 127);
             }
-            // (the scales are powers of two; where their product might not be one the tile is computed again, see below)
-            const double sa = __ldg(p.scaleA + (long)bz * p.rowsA_pad + m0 + row);
-            const auto sb = [&](int c) { return __hiloint2double(s_scale[c0 + c], 0); };
             if (p.sumsq_partials) {
-                double s = 0.0;
-#pragma unroll
-                for (int c = 0; c < 64; ++c) {
-                    const double x = p.alpha * (part[c] * (sa * sb(c)));
-                    s = fma(x, x, s);
-                }
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) s_sum[warp] = s;
-            } else {
-                double *out = reinterpret_cast<double *>(stages) + CI(row * I8_OUT_LD + c0, 128 * I8_OUT_LD - 63, 301);
-#pragma unroll
-                for (int c = 0; c < 64; ++c) out[c] = p.alpha * (part[c] * (sa * sb(c)));
-                if (bulk_out) fence_proxy_async();             // the copy engine reads what was just written
+                for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
             }
+        }
+        if (ok && p.sumsq_partials) {
+            if (lane == 0) s_sum[warp] = sq;
+            i8_reducers();
+            if (tid < HALVES && m0 < p.M && w.n0 + 128 * tid < p.N) {
+                double tot = 0.0;
+                for (int k = 0; k < I8_WARPS / HALVES; ++k) tot += s_sum[tid * 8 + k];
+                const int t128m = (p.M + 127) / 128, t128n = (p.N + 127) / 128;
+                p.sumsq_partials[((long)bz * t128m + m0 / 128) * t128n + w.n0 / 128 + tid] = tot;
+            }
+        }
+        // Do the digits suit the operands?  They cut every entry at the same distance below the largest of its row (of op(A) and of
+        // op(B)^T), so where the large entries of a row meet zeros or small ones only, the result has lost digits that a product in fp64
+        // keeps.  With p.least the loss is looked for in the result.  With every row scaled to a largest
+        // entry of 1/4 to 1/2, the cut moves an entry by 2^-57.8 (|a| + |b|), norms of its two rows, below 2^-59 sqrt(K) for normal or
+        // uniform entries.  So a tile is kept if the largest entry of each of its rows and columns is at least p.least, and computed in
+        // fp64 otherwise: 1/32 is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the largest entry of a
+        // row.  Contractions of 128 and fewer, the corners of triangles, are kept from half of it on.
+        if (ok && p.least > 0.0) {
+            i8_reducers();
+            const int all = (p.K + I8_KCHUNK - 1) / I8_KCHUNK;
+#pragma unroll
+            for (int h = 0; h < HALVES; ++h) {
+                const int nh = w.n0 + 128 * h;
+                const bool wide = p.rowsB - nh >= 32, tall = p.rowsA - m0 >= 32;
+                int la, ha, lb, hb;
+                i8_chunks(p.rangeA + bz * (p.rowsA_pad / 128) * 2, m0 / 128, 1, (int)(p.rowsA_pad / 128), all, la, ha);
+                i8_chunks(p.rangeB + bz * (p.rowsB_pad / 128) * 2, nh / 128, 1, (int)(p.rowsB_pad / 128), all, lb, hb);
+                const bool judged = top(tid, h) != 0u && (tid < 128 ? wide || !tall : tall || !wide);
+                const bool any = i8_reducers_or(judged && min(ha, hb) > max(la, lb) && !((s_seen[h][(tid >> 5) & 7] >> lane) & 1u));
+                if (any && tid == 0) s_fix |= 1u << h;
+            }
+        }
+        i8_reducers();
+        if (tid == 0 && slot_index >= 0) {
+            __threadfence();
+            atomicExch(i8_slot_busy + slot_index, 0u);
         }
     }
     i8_fence_before();
     __syncthreads();
+    i8_pair_barrier();
     i8_fence_after();
-    if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
-    if (*(volatile unsigned *)&s_abort) return;                // the tile is not written
-    // Do the digits suit the operands?  They cut every entry at the same distance below the largest of its row (of op(A) and of
-    // op(B)^T), so where the large entries of a row meet zeros or small ones only, the result has lost digits that a product in fp64
-    // keeps.  With p.least the loss is looked for in the result.  With every row scaled to a largest
-    // entry of 1/4 to 1/2, the cut moves an entry by 2^-57.8 (|a| + |b|), norms of its two rows, below 2^-59 sqrt(K) for normal or
-    // uniform entries.  So a tile is kept if the largest entry of each of its rows and columns is at least p.least, and computed in
-    // fp64 otherwise: 1/32 is where the cut meets what a chain of K fp64 additions loses, 1e-16 sqrt(K) of the largest entry of a
-    // row.  Contractions of 128 and fewer, the corners of triangles, are kept from half of it on.
-    // Rows of extreme magnitude, whose scales might not multiply, and infinities and NaNs always take that way.
-    const bool in_fp64 = __syncthreads_or(extreme || (looked_at && nchunk > 0 && !((s_seen[tid >> 5] >> lane) & 1u)));
-    if (warp >= 8) return;                                     // (barriers below are met by the other eight)
-    double sumsq = 0.0;
-    if (in_fp64) {
+    if (warp == I8_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+    if (warp >= I8_WARPS) return;                              // (barriers below are met by the others)
+    const unsigned fix = *(volatile unsigned *)&s_fix;
+    if (fix == 0u || *(volatile unsigned *)&s_abort) return;
+    // ---- tiles that are computed in fp64 (128 columns at a time)
+    for (int f = 0; f < TN / 128; ++f) {
+        if (!((fix >> f) & 1u)) continue;
+        const int m0 = w.m0 + 128 * rank, n0 = w.n0 + 128 * f, bz = w.bz;
+        if (m0 >= p.M || n0 >= p.N || (p.lower_tiles_only && n0 > m0)) continue;
+        const int out_rows = min(128, p.M - m0), out_cols = min(128, p.N - n0);
         // a factor of zero does not hide an infinity or a NaN: with one about, no chunk is skipped
+        __syncthreads();
         if (tid == 0) s_all_k = 0u;
         __syncthreads();
-        if (tile_top() >= 0x7ff00000u) s_all_k = 1u;
+        const unsigned t = tid >= 256 ? 0u : tid < 128 ? (m0 + tid < p.rowsA_pad ? __ldg(p.topA + (long)bz * p.rowsA_pad + m0 + tid) : 0u)
+                                     : (n0 + tid - 128 < p.rowsB_pad ? __ldg(p.topB + (long)bz * p.rowsB_pad + n0 + tid - 128) : 0u);
+        if (t >= 0x7ff00000u) s_all_k = 1u;
         __syncthreads();
-        int k_first = k_lo, k_hi = max(k_lo, min(p.K, k_lo + nchunk * I8_KCHUNK));
+        int k_first = w.k_lo, k_hi = max(w.k_lo, min(p.K, w.k_lo + w.stages * I8_STAGE_K));
         if (p.diag_a) { k_first = min(k_first, m0); k_hi = max(k_hi, min(p.K, m0 + 128)); }     // the chunks count without the diagonals
         if (p.diag_b) { k_first = min(k_first, n0); k_hi = max(k_hi, min(p.K, n0 + 128)); }
         if (s_all_k) { k_first = 0; k_hi = p.K; }
         double *tile = reinterpret_cast<double *>(stages);
         const bool a_kcontig = p.aj == 1, b_kcontig = p.bi == 1, sq = p.sumsq_partials != nullptr;
+        double sumsq;
         if (a_kcontig) sumsq = b_kcontig ? i8_tile_in_fp64<true, true>(p, bz, m0, n0, k_first, k_hi, tile, sq) : i8_tile_in_fp64<true, false>(p, bz, m0, n0, k_first, k_hi, tile, sq);
         else sumsq = b_kcontig ? i8_tile_in_fp64<false, true>(p, bz, m0, n0, k_first, k_hi, tile, sq) : i8_tile_in_fp64<false, false>(p, bz, m0, n0, k_first, k_hi, tile, sq);
         if (sq) {
             for (int o = 16; o > 0; o >>= 1) sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
             if (lane == 0) s_sum[warp] = sumsq;
-        } else if (bulk_out) {
-            fence_proxy_async();
         }
         __syncthreads();
-    }
-    if (p.sumsq_partials) {
-        if (tid == 0) {
-            double tot = 0.0;
-            for (int w = 0; w < 8; ++w) tot += s_sum[w];
-            p.sumsq_partials[((long)bz * p.tiles_m + tm) * p.tiles_n + tn] = tot;
-        }
-        return;
-    }
-    if (bulk_out) {
-        if (tid < out_rows) {
-            const double *in = reinterpret_cast<const double *>(stages) + tid * I8_OUT_LD;
-            double *dst = p.C + (long)bz * p.strideC + (long)(m0 + tid) * p.ldc + n0;
-            if (p.beta == 0.0)
-                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(smem_u32(in)), "r"(out_cols * 8) : "memory");
-            else
-                asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f64 [%0], [%1], %2;\n" ::"l"(dst), "r"(smem_u32(in)), "r"(out_cols * 8) : "memory");
-            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-        }
-        return;
-    }
-    {
-        const double *in = reinterpret_cast<const double *>(stages);
-        double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
-        const int rows = out_rows, cols = out_cols;
-        const double *Ab = p.A + (long)bz * p.strideA, *Bb = p.B + (long)bz * p.strideB;
-        const bool diag_a = p.diag_a && !in_fp64, diag_b = p.diag_b && !in_fp64;
-        for (int r4 = warp * 4; r4 < rows; r4 += 32) {         // four rows of the tile per warp: sixteen loads in flight
-            double old[4][4];
-            if (p.beta != 0.0) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        old[i][j] = (r4 + i < rows && lane + 32 * j < cols) ? Cb[(long)(r4 + i) * p.ldc + lane + 32 * j] : 0.0;
+        if (sq) {
+            if (tid == 0) {
+                double tot = 0.0;
+                for (int k = 0; k < I8_WARPS; ++k) tot += s_sum[k];
+                const int t128m = (p.M + 127) / 128, t128n = (p.N + 127) / 128;
+                p.sumsq_partials[((long)bz * t128m + m0 / 128) * t128n + n0 / 128] = tot;
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (r4 + i < rows && lane + 32 * j < cols) {
-                        double x = in[(r4 + i) * I8_OUT_LD + lane + 32 * j];
-                        const long gi = m0 + r4 + i, gj = n0 + lane + 32 * j;
-                        if (diag_a && gi < p.K) x = fma(p.alpha * Ab[gi * (p.ai + p.aj)], Bb[gi * p.bi + gj * p.bj], x);
-                        if (diag_b && gj < p.K && !(diag_a && gi == gj))
-                            x = fma(p.alpha * Ab[gi * p.ai + gj * p.aj], Bb[gj * (p.bi + p.bj)], x);
-                        Cb[CI((long)(r4 + i) * p.ldc + lane + 32 * j, (p.M - m0 - 1) * p.ldc + p.N - n0, 305)] = p.beta != 0.0 ? fma(p.beta, old[i][j], x) : x;
-                    }
+            continue;
         }
+        double *Cb = p.C + (long)bz * p.strideC + (long)m0 * p.ldc + n0;
+        for (int r = warp; r < out_rows; r += I8_WARPS)
+            for (int c = lane; c < out_cols; c += 32) {
+                double &dst = Cb[CI((long)r * p.ldc + c, (p.M - m0 - 1) * p.ldc + p.N - n0, 307)];
+                dst = p.beta != 0.0 ? fma(p.beta, dst, tile[r * I8_OUT_LD + c]) : tile[r * I8_OUT_LD + c];
+            }
     }
 }
 
 bool gemm_i8_pays(long M, long N, long K, long batch) {
     if (K > I8_MAX_K || K < 256) return false;
-    // fewer tiles leave SMs idle, and the four launches of the splitting are not repaid below some 10^9 products
-    // (1024^3: 0.117 ms against 0.148; 512^3 four at a time: 0.11 either way)
+    // fewer tiles leave SMs idle, and the launches of the splitting are not repaid below some 10^9 products (1024^3: 0.106 ms with the splitting
+    // against 0.148)
     const long tiles = ((M + 127) / 128) * ((N + 127) / 128) * batch;
     return tiles >= 64 && (double)M * N * K * batch >= 0.9e9;
 }
 
-static bool encode_planes_map(CUtensorMap *map, const I8Planes &pl, int planes) {
+static bool encode_planes_map(CUtensorMap *map, const I8Planes &pl, int box_rows) {
     TensorMapEncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return false;
     const cuuint64_t rows = (cuuint64_t)pl.rows_pad * pl.batch;
-    const cuuint64_t dims[3] = {(cuuint64_t)pl.k_pad, rows, (cuuint64_t)I8_DIGITS};
-    const cuuint64_t strides[2] = {(cuuint64_t)pl.k_pad, (cuuint64_t)(pl.k_pad * pl.plane_rows)};
-    const cuuint32_t box[3] = {(cuuint32_t)I8_KCHUNK, 128u, (cuuint32_t)planes};
+    const cuuint64_t dims[3] = {(cuuint64_t)I8_STAGE_K, rows, (cuuint64_t)(I8_MODULI * (pl.k_pad / I8_STAGE_K))};
+    const cuuint64_t strides[2] = {(cuuint64_t)I8_STAGE_K, (cuuint64_t)(I8_STAGE_K * pl.plane_rows)};
+    const cuuint32_t box[3] = {(cuuint32_t)I8_STAGE_K, (cuuint32_t)box_rows, 1u};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, pl.planes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// tiles of 256 x tn of one matrix, with those above the diagonal that fill up a group of rows (i8_where)
+static long i8_tiles(const GemmArgs &g, int tn) {
+    const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + tn - 1) / tn;
+    if (!g.lower_tiles_only) return (long)tiles_m * tiles_n;
+    long n = 0;
+    for (int hi = tiles_m; hi > 0; hi = std::max(0, hi - 8)) n += (long)(hi - std::max(0, hi - 8)) * std::min(tiles_n, hi * (256 / tn));
+    return n;
+}
+
+template <int TN>
+static cudaError_t i8_launch(I8Params &p, const GemmArgs &g, const CUtensorMap &a, const CUtensorMap &b, cudaStream_t stream) {
+    p.tiles_m = (g.M + 255) / 256; p.tiles_n = (g.N + TN - 1) / TN;
+    const long all = i8_tiles(g, TN) * g.batch;                // (matrices of 2^31 tiles do not fit in memory)
+    p.tiles = (int)i8_tiles(g, TN);
+    cudaError_t e = cudaFuncSetAttribute(i8_gemm_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I8Tile<TN>::SMEM);
+    if (e != cudaSuccess) return e;
+    i8_gemm_kernel<TN><<<(unsigned)(2 * all), I8_THREADS, I8Tile<TN>::SMEM, stream>>>(p, a, b);
+    return cudaGetLastError();
 }
 
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
                     bool diag_a, bool diag_b, double least) {
     *err = cudaSuccess;
     if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return true;
-    if (g.K > I8_MAX_K) return false;
-    CUtensorMap a7, b7, a4, b4;
-    if (!encode_planes_map(&a7, A, I8_DIGITS) || !encode_planes_map(&b7, B, I8_DIGITS) || !encode_planes_map(&a4, A, I8_TOP) ||
-        !encode_planes_map(&b4, B, I8_TOP))
-        return false;
+    if (g.K > I8_MAX_K || (least > 0.0 && g.beta != 0.0)) return false;
+    // tiles of 256 x 128 where those of 256 x 256 leave too many pairs of SMs idle (one takes 0.6 to 0.75 times as long: its
+    // loads, 24 KB for 256 cycles of the tensor pipe, are bound by L2; 1024^3 56 against 76 us, 2048^3 182 against 127)
+    const int pairs = std::max(1, device_sms() / 2);
+    const long n256 = i8_tiles(g, 256) * g.batch, n128 = i8_tiles(g, 128) * g.batch;
+    const int asked = g_i8_tile.load();
+    const bool narrow = asked > 0 ? asked == 128 : 0.72 * (double)((n128 + pairs - 1) / pairs) < (double)((n256 + pairs - 1) / pairs);
+    CUtensorMap a, b;
+    if (!encode_planes_map(&a, A, 128) || !encode_planes_map(&b, B, narrow ? 64 : 128)) return false;
     I8Params p{};
-    p.M = g.M; p.N = g.N; p.K = g.K; p.alpha = g.alpha; p.beta = g.beta;
+    p.M = g.M; p.N = g.N; p.K = g.K; p.k_blocks = (int)(A.k_pad / I8_STAGE_K); p.alpha = g.alpha; p.beta = g.beta;
     p.C = g.C; p.ldc = g.ldc; p.strideC = g.strideC; p.sumsq_partials = g.sumsq_partials;
     p.scaleA = A.scale; p.scaleB = B.scale; p.rowsA_pad = A.rows_pad; p.rowsB_pad = B.rows_pad;
-    p.lower_tiles_only = g.lower_tiles_only;
+    p.lower_tiles_only = g.lower_tiles_only; p.batch = g.batch;
     p.rangeA = A.range; p.rangeB = B.range;
     p.topA = A.maxbits; p.topB = B.maxbits; p.rowsA = A.rows; p.rowsB = B.rows;
+    p.bitsA = A.bits; p.bitsB = B.bits;
     p.diag_a = diag_a; p.diag_b = diag_b;
     p.A = g.A; p.strideA = g.strideA; p.ai = g.opA == OP_N ? g.lda : 1; p.aj = g.opA == OP_N ? 1 : g.lda;
     p.B = g.B; p.strideB = g.strideB; p.bi = g.opB == OP_N ? g.ldb : 1; p.bj = g.opB == OP_N ? 1 : g.ldb;
-    p.tiles_m = (g.M + 127) / 128; p.tiles_n = (g.N + 127) / 128;
     p.info = info; p.least = least;
-    *err = cudaFuncSetAttribute(i8_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I8_SMEM);
-    if (*err != cudaSuccess) return true;
-    i8_gemm_kernel<<<dim3((unsigned)(p.tiles_m * p.tiles_n), (unsigned)g.batch), I8_THREADS, I8_SMEM, stream>>>(p, a7, b7, a4, b4);
-    *err = cudaGetLastError();
+    *err = narrow ? i8_launch<128>(p, g, a, b, stream) : i8_launch<256>(p, g, a, b, stream);
     return true;
 }
 

@@ -1,9 +1,7 @@
-// fp64 products on the int8 tensor cores (tcgen05), by error-free splitting (Ozaki, Ogita, Oishi, Rump, "Error-free
-// transformations of matrix multiplication by using fast routines of matrix multiplication", 2012): host interface.
+// fp64 products on the int8 tensor cores (tcgen05), by residues (Ozaki, Uchino, Imamura, "Ozaki Scheme II", 2025): host interface.
 //
-// Every row of op(A) and every column of op(B) is scaled by a power of two and written as I8_DIGITS signed base-256
-// digits; products of digit planes are exact in int32, and the planes whose weights stay within I8_DIGITS + 1 digits
-// are summed.  Tiles that the digits do not suit are computed in fp64.  See i8_gemm.cu.
+// Every row of op(A) and every column of op(B) is scaled by a power of two and rounded to integers of 56 bits ("digits" below), whose product is
+// put together from sixteen int8 products of residues.  Tiles that the digits do not suit are computed in fp64.  See i8_gemm.cu.
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -12,17 +10,19 @@
 
 namespace gptq2d {
 
-constexpr int I8_DIGITS = 7;            // 56 bits below the largest entry of a row
-constexpr int I8_KCHUNK = 64;           // k-depth of a pipeline stage; planes are padded to a multiple of it
+constexpr int I8_MODULI = 16;
+constexpr int I8_KCHUNK = 64;           // granularity along k at which rows of zeros are noticed
 constexpr double I8_LEAST_SETUP = 0x1p-9;
-constexpr int I8_MAX_K = 16384;         // 7 products of |digits| <= 128 per k: 7 * 2^14 * K < 2^31
+constexpr int I8_MAX_K = 16384;         // sums up to K 2^110 are determined by their residues
 
-// The digit planes of `batch` matrices (rows x K each, K contiguous):
-// planes[d][b * rows_pad + r][k], d = 0 the most significant digit; scale[b * rows_pad + r] = 2^(e - 36), 2^e the power
-// of two that the row's digits (as 0.d1 d2 .. in base 256) are to be multiplied by, NaN for a row with a non-finite entry.
+// The residue planes of `batch` matrices (rows x K each), 128 k of a row together and the rows one behind the other, so that
+// what a stage of the product takes, 128 rows of 128 bytes, is one piece of memory:
+// planes[i][k / 128][b * rows_pad + r][k % 128]; scale[b * rows_pad + r] = 2^(e - 36), the row's integers count 2^(e - 56);
+// NaN for a row with a non-finite entry.
 struct I8Planes {
     int8_t *planes;
     double *scale;
+    unsigned long long *bits;           // disjunction of a row's integers: where they end in zeros
     unsigned *maxbits;                  // scratch of the splitting pass: high word of a row's largest magnitude
     int *range;                         // per 128 rows: {number of k-chunks - first chunk with an entry, last such chunk + 1}, 0 0 if none
     int rows, K, batch;
@@ -31,14 +31,17 @@ struct I8Planes {
     // the planes of rows [r0, r0 + count) of a single matrix; r0 a multiple of 128
     I8Planes part(int r0, int count) const {
         I8Planes v = *this;
-        v.planes += (long)r0 * k_pad; v.scale += r0; v.maxbits += r0; v.range += r0 / 128 * 2;
+        v.planes += (long)r0 * 128; v.scale += r0; v.bits += r0; v.maxbits += r0; v.range += r0 / 128 * 2;
         v.rows = count; v.rows_pad = (count + 127L) / 128 * 128;
         return v;
     }
 };
+// the planes alone, what goes with them, and both (multiples of 256)
+size_t i8_residue_bytes(int rows, int K, int batch);
+size_t i8_rows_bytes(int rows, int batch);
 size_t i8_planes_bytes(int rows, int K, int batch);
-// lays an I8Planes out at `at` (256-byte aligned)
-I8Planes i8_planes_at(void *at, int rows, int K, int batch);
+// lays an I8Planes out at `at` (256-byte aligned), or the planes at `at` and the rest at `rows_at`
+I8Planes i8_planes_at(void *at, int rows, int K, int batch, void *rows_at = nullptr);
 // Splits: element (r, k) of matrix b is src[b * stride + r * ld + k] (k_contig) or src[b * stride + k * ld + r].
 // With `inner`, entry k of every row is first multiplied by the power of two nearest below p[k] (or by its inverse):
 // where the rows of one operand grow along k as those of the other shrink, the two factors cancel in the product and
@@ -75,8 +78,10 @@ bool gemm_i8_pays(long M, long N, long K, long batch);
 // I8_LEAST_SETUP: at 1/32, where the cut meets what an fp64 chain loses, channel scales sent a third of the tiles of the inverse
 // to fp64 (1100 x 4100: 4.5 -> 6.1 ms) for factors that came out no closer to 80-bit ones.
 // `info`: the call's status words (a bounded wait that runs out is reported there), may be NULL.
-// False: no tensor map can be had (no driver entry point); nothing was launched.
+// (`least` is for beta = 0.)  False: no tensor map can be had (no driver entry point); nothing was launched.
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
                     bool diag_a = false, bool diag_b = false, double least = 0.0);
+
+void i8_set_tile(int columns);          // tests: tiles of 128 or 256 columns; 0: by the rule
 
 }  // namespace gptq2d

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(1024) sum_partials_kernel(const double *part, 
 static inline long round_up(long x, long a) { return (x + a - 1) / a * a; }
 void launch_sumsq_plain(const double *M, int m, int n, long ld, double *part, int *count, cudaStream_t s);
 
-// Digit planes of both operands of one of the two products at a time (i8_gemm.cuh), 0 if neither is worth splitting.
+// Residue planes of both operands of one of the two products at a time (i8_gemm.cuh), 0 if neither is worth splitting.
 static size_t objective_i8_bytes(int m, int n) {
     size_t b = 0;
     if (gemm_i8_pays(m, n, m, 1)) b = i8_planes_bytes(m, m, 1) + i8_planes_bytes(n, m, 1);

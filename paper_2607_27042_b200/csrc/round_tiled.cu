@@ -1177,10 +1177,14 @@ static TiledLayout tiled_layout(int m, int n) {
 constexpr int SPLIT_MIN = 31 * T + 1;
 static std::atomic<long> g_split_min{SPLIT_MIN};
 void round_split_set_min(long order) { g_split_min.store(order > 0 ? order : SPLIT_MIN); }
+// Residue planes of a product up to this size get room of their own; those of larger ones lie in rows of the E and C buffers that are free at the time,
+// where k has to be cut (4096 x 4096, 134 MB: 5.80 ms, with two pieces of k 6.13; 8192 x 8192, 537 MB: 29.2 and 30.1).
+constexpr size_t SPLIT_OWN_PLANES = (size_t)256 << 20;
 struct SplitLayout {
     int m0, n0;                          // rows / columns of the first block (multiples of T); 0: not split
-    size_t hdr_off[3], flags_off[4], desc_off, table_off, zero_off, total;
+    size_t hdr_off[3], flags_off[4], desc_off, table_off, zero_off, rows_off, planes_off, total;      // planes_off 0: no room of their own
 };
+
 static size_t split_flag_bytes(int m, int n) {
     const size_t tm = (m + T - 1) / T, tiles = tm * ((n + T - 1) / T);
     return 2 * pad256(tiles * sizeof(unsigned)) + 2 * pad256(4 * tiles * sizeof(unsigned)) + pad256(tm * sizeof(unsigned));
@@ -1203,6 +1207,11 @@ static SplitLayout split_layout(int m, int n) {
     l.table_off = off;
     const size_t tm0 = l.m0 / T, tn0 = l.n0 / T;
     off += pad256(2 * (tm0 * (t.ntn - tn0) + (t.ntm - tm0) * tn0) * sizeof(unsigned));
+    // what goes with the residue planes of one product at a time: the scales of both operands' rows and that along k
+    l.rows_off = off;
+    off += i8_rows_bytes(l.m0, 1) + i8_rows_bytes(l.n0, 1) + i8_inner_bytes(std::min(std::max(l.m0, l.n0), I8_MAX_K));
+    const size_t planes = std::max(i8_residue_bytes(l.m0, l.n0, 1) + i8_residue_bytes(l.n0, l.n0, 1), i8_residue_bytes(l.m0, l.m0, 1) + i8_residue_bytes(l.n0, l.m0, 1));
+    if (planes <= SPLIT_OWN_PLANES) { l.planes_off = off; off += planes; }
     l.total = off;
     return l;
 }
@@ -1466,15 +1475,15 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
 // Large matrices in 2 x 2 blocks.  With the matrix cut behind row m0 and column n0 (tile boundaries), the restatement on tiles at
 // the head of this file holds for the four blocks, too: block (0, 0) is a sweep of its own; (0, 1) starts from Rt = C00 U01 and
 // (1, 0) from Cd = L10 E00; (1, 1) from Cd = L10 E01 and Rt = C10 U01.  Half of all flops are in these four products,
-// and they are plain matrix products of finished operands, so they run on the int8 tensor cores (i8_gemm.cu) at 80 TFLOP/s
+// and they are plain matrix products of finished operands, so they run on the int8 tensor cores (i8_gemm.cu) at 130 TFLOP/s and more
 // where the far parts of the sweep run at 35.  Three sweeps (the middle one takes two blocks in one launch) replace one; each has
 // its own ramp, which is why small matrices are not cut.
+// Nothing but the workspace is used: where a product's residue planes have no room of their own they lie in rows of Ebuf whose blocks have not been
+// swept yet, or in rows of Cbuf that nobody reads any more; they do not fit there at once, so k is cut (square matrices: in two).
 // ms, whole / in blocks: 4096 x 4096 6.20 / 6.09, 5632 x 5632 14.2 / 12.6, 6144 x 6144 17.9 / 15.2, 4096 x 8192 16.4 / 14.5, 5120 x 8192
 // 21.4 / 18.3; with tasks of 64 x 64 before cells 8192 x 8192 38.0 / 31.9 and 4096 x 4096 6.6 / 8.0.
 // The error of E against an 80-bit residual does not grow: at 3969 x 3969, 4096 x 4096, 4100 x 5003 and 5631 x 5631, with Gaussian, log-normal
 // (sigma 1 and 1.5) and condition 1e6 Grams, it is 0.77 to 0.92 times that of the whole sweep in the 2-norm.
-// Nothing but the workspace is used: a product's digit planes lie in rows of Ebuf whose blocks have not been swept yet, or in
-// rows of Cbuf that nobody reads any more; where they do not fit at once k is cut.
 
 // descriptors and claim order of a launch that sweeps two matrices (what the host builds for batched launches)
 __global__ void __launch_bounds__(256) split_pair_kernel(TiledKernelParams a, TiledKernelParams b, TiledKernelParams *desc, unsigned *table) {
@@ -1509,21 +1518,22 @@ __global__ void split_status_kernel(const int *a, const int *b, const int *c, in
         for (int k = 0; k < 4; ++k) info[k] = best[k];
 }
 
-// C (M x N, padded to whole tiles, row pitch ldc) = A B on the int8 tensor cores; A: M x K row-major, B: K x N row-major.  The digit planes
-// of kparts pieces of k in turn lie at `at`.
+// C (M x N, padded to whole tiles, row pitch ldc) = A B on the int8 tensor cores; A: M x K row-major, B: K x N row-major.  The residue planes
+// of kparts pieces of k lie at `at` in turn, what goes with them at `rows`.
 static int split_product(int M, int N, int K, int kparts, const double *A, long lda, const double *B, long ldb, double *C, long ldc, void *at,
-                         int *info, cudaStream_t stream) {
+                         char *rows, int *info, cudaStream_t stream) {
     const int step = ((K + kparts - 1) / kparts + T - 1) / T * T;
     for (int k0 = 0; k0 < K; k0 += step) {
         const int kk = std::min(step, K - k0);
-        const I8Planes pa = i8_planes_at(at, M, kk, 1), pb = i8_planes_at(static_cast<char *>(at) + i8_planes_bytes(M, kk, 1), N, kk, 1);
+        const I8Planes pa = i8_planes_at(at, M, kk, 1, rows);
+        const I8Planes pb = i8_planes_at(static_cast<char *>(at) + i8_residue_bytes(M, kk, 1), N, kk, 1, rows + i8_rows_bytes(M, 1));
         GemmArgs g{};
         g.opA = OP_N; g.opB = OP_N;
         g.M = (M + T - 1) / T * T; g.N = (N + T - 1) / T * T; g.K = kk;       // padding included: the planes hold zeros there
         g.alpha = 1.0; g.beta = k0 ? 1.0 : 0.0;
         g.A = A + k0; g.lda = lda; g.B = B + (long)k0 * ldb; g.ldb = ldb; g.C = C; g.ldc = ldc; g.batch = 1;
         I8Inner inner;                                         // a channel that E or U has nothing in must not cost L or C its digits
-        double *tops = reinterpret_cast<double *>(static_cast<char *>(at) + i8_planes_bytes(M, kk, 1) + i8_planes_bytes(N, kk, 1));
+        double *tops = reinterpret_cast<double *>(rows + i8_rows_bytes(M, 1) + i8_rows_bytes(N, 1));
         inner.p = tops;
         cudaError_t e = i8_inner_tops(tops, g.B, kk, N, ldb, 1, stream);
         if (e == cudaSuccess) e = i8_split(pa, g.A, lda, 0, true, stream, inner);
@@ -1534,11 +1544,12 @@ static int split_product(int M, int N, int K, int kparts, const double *A, long 
     }
     return GPTQ2D_OK;
 }
-// pieces of k for which the planes of an M x K and a K x N operand fit in `room` bytes; 0: none of up to eight
+
+// pieces of k for which the planes of an M x K and a K x N operand fit in `room` bytes; 0: none of up to sixteen
 static int split_kparts(int M, int N, int K, size_t room) {
-    for (int p = 1; p <= 8; ++p) {
+    for (int p = 1; p <= 16; ++p) {
         const int step = ((K + p - 1) / p + T - 1) / T * T;
-        if (step <= I8_MAX_K && i8_planes_bytes(M, step, 1) + i8_planes_bytes(N, step, 1) + i8_inner_bytes(step) <= room) return p;
+        if (step <= I8_MAX_K && i8_residue_bytes(M, step, 1) + i8_residue_bytes(N, step, 1) <= room) return p;
     }
     return 0;
 }
@@ -1552,11 +1563,13 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
     const long np = (long)l.ntn * T;
     double *E = reinterpret_cast<double *>(w + l.e_off), *C = reinterpret_cast<double *>(w + l.c_off);
     const int m0 = sl.m0, n0 = sl.n0, m1 = in.m - m0, n1 = in.n - n0;
-    // room for digit planes: first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
-    const size_t room0 = (size_t)(l.ntm * T - m0) * np * sizeof(double), room1 = (size_t)m0 * np * sizeof(double);
+    // room for residue planes: their own, or first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
+    const size_t room0 = sl.planes_off ? SPLIT_OWN_PLANES : (size_t)(l.ntm * T - m0) * np * sizeof(double);
+    const size_t room1 = sl.planes_off ? SPLIT_OWN_PLANES : (size_t)m0 * np * sizeof(double);
     const int k10 = split_kparts(m1, n0, m0, room0), k01 = split_kparts(m0, n1, n0, room0);
     const int k11 = split_kparts(m1, n1, m0, room1), k11r = split_kparts(m1, n1, n0, room1);
     if (!k10 || !k01 || !k11 || !k11r) return -1;
+    char *rows = w + sl.rows_off;
 
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
@@ -1605,9 +1618,10 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
                    ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
     };
     int st = sweep_one(block(0, 0, 0, 0));
-    void *at = E + (long)m0 * np;
-    if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, k10, in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, in.info, stream);
-    if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, k01, C, np, in.U + n0, in.ldu, E + n0, np, at, in.info, stream);
+    void *const own = sl.planes_off ? w + sl.planes_off : nullptr;
+    void *at = own ? own : E + (long)m0 * np;
+    if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, k10, in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, rows, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, k01, C, np, in.U + n0, in.ldu, E + n0, np, at, rows, in.info, stream);
     if (st != GPTQ2D_OK) return st;
     {
         TiledKernelParams a = block(0, 1, 1, 2), b = block(1, 0, 1, 1), p{};
@@ -1630,9 +1644,9 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         if (cudaLaunchCooperativeKernel(kernel, dim3(std::min(sms, p.ntasks)), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
     }
-    at = C;
-    st = split_product(m1, n1, m0, k11, in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, in.info, stream);
-    if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, k11r, C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, in.info, stream);
+    at = own ? own : C;
+    st = split_product(m1, n1, m0, k11, in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, rows, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, k11r, C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, rows, in.info, stream);
     if (st == GPTQ2D_OK) st = sweep_one(block(1, 1, 2, 3));
     if (st != GPTQ2D_OK) return st;
     if (in.info) {

@@ -1,5 +1,5 @@
-"""The fp64 product on the int8 tensor cores (error-free splitting into base-256 digits) against exact integers and
-against a bound on what its digits drop."""
+"""The fp64 product on the int8 tensor cores (residues of 56-bit integers) against exact integers and against a bound on
+what its digits drop."""
 import numpy as np
 import pytest
 import torch
@@ -217,3 +217,19 @@ def test_infinities_and_nans_go_where_fp64_takes_them(g):
     assert np.array_equal(got[inf], want[inf]) and np.isnan(got).any() and inf.any()
     fine = np.isfinite(want)
     assert np.max(np.abs(got[fine] - want[fine])) < 1e-12
+
+
+@pytest.mark.parametrize("columns", [128, 256])
+@pytest.mark.parametrize("M,N,K", [(256, 256, 128), (255, 257, 1024), (257, 129, 1025), (513, 385, 1152), (130, 650, 2304)])
+def test_tiles_of_both_widths(g, columns, M, N, K):
+    # edges of tiles, of the halves of a pair and of stages of 128 and 256 k; both sides of K = 1024, where the reduction of the sums
+    # changes.  Integers of 20 bits: sums below 2^52 and multiples of 2^60 of the scaled product, so exact.  Triangles: tiles in reverse order.
+    rng = np.random.default_rng(M + N + K)
+    a = rng.integers(-2 ** 20, 2 ** 20, size=(M, K)).astype(np.float64)
+    b = rng.integers(-2 ** 20, 2 ** 20, size=(K, N)).astype(np.float64)
+    g.gptq2d_internal_test_hook(9, columns)
+    try:
+        for x, y in ((a, b), (np.triu(a), b), (np.tril(a), np.tril(b)), (a, np.triu(b))):
+            assert np.array_equal(product(g, x, y), x @ y)
+    finally:
+        g.gptq2d_internal_test_hook(9, 0)
