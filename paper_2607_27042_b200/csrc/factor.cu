@@ -26,225 +26,284 @@ constexpr int FB = 128;
 
 // Cholesky factor and inverse of one block, in shared memory, by one CTA of 256 threads.  Orders up to NP (64, 96 or 128: the
 // block is padded to NP x NP with the identity).  a[NP][NP + 4]: row pitch == 4 mod 16 doubles, so that the 8 x 4 fragments of
-// the fp64 tensor path touch sixteen different 8-byte banks.  w: packed lower triangle.
-__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
+// the fp64 tensor path touch sixteen different 8-byte banks.  Behind it the diagonal of the inverse, the inverse of the 16 x 16 block in hand and
+// two rows of it.
 template <int NP>
 struct CholBlock {
-    static constexpr int LD = NP + 4;
-    static constexpr size_t SMEM = (size_t)(NP * LD + NP * (NP + 1) / 2) * sizeof(double);
+    static constexpr int LD = NP + 4, LDV = 20;
+    static constexpr size_t SMEM = (size_t)(NP * LD + NP + 16 * LDV + 32) * sizeof(double);
+    // W = P^{-1}: entry (i, j), i > j, lies above the diagonal of a
+    static __device__ __forceinline__ double inverse(const double *a, int i, int j) { return i > j ? a[j * LD + i] : a[NP * LD + i]; }
 };
 
-// X21 = -W22 (P21 W11) for PAIRS pairs of blocks (b1 and b2 rows, `step` rows apart, the first at 0), on the fp64 tensor path.  A warp
-// takes a row of 8 x 8 fragments of a pair (a 1 / CP part of its columns), all of them at once: one fragment of the left
-// operand is loaded for FU products in flight.  The temporary product lies, transposed, above the diagonal of a.
-template <int NP, int PAIRS, int B1, int B2, int CP>
-__device__ __forceinline__ void inverse_join(double *a, double *w, int step) {
-    constexpr int LD = CholBlock<NP>::LD, FU = B1 / 8 / CP, ROWS = PAIRS * (B2 / 8);
-    static_assert(ROWS * CP <= 8, "one unit per warp");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int row = warp / CP, pr = row / (B2 / 8), fr = row - pr * (B2 / 8), s0 = pr * step, f0 = (warp - row * CP) * FU;
-    const bool on = row < ROWS;
-    double c[FU][2];
-#pragma unroll
-    for (int f = 0; f < FU; ++f) c[f][0] = c[f][1] = 0.0;
-    if (on) {                                                  // T = P21 W11
-        for (int kk = 8 * f0; kk < B1; kk += 4) {              // W11[k][c] = 0 for k < c
-            const int k = kk + t;
-            const double af = a[(s0 + B1 + 8 * fr + g) * LD + s0 + k];
-#pragma unroll
-            for (int f = 0; f < FU; ++f) {
-                const int cc = 8 * (f0 + f) + g;
-                const double bf = k >= cc ? w[tri(s0 + k, s0 + min(cc, k))] : 0.0;         // index clamped: stays inside the array
-                dmma_m8n8k4(c[f][0], c[f][1], af, bf);
-            }
-        }
-#pragma unroll
-        for (int f = 0; f < FU; ++f) {
-            double *dst = a + (s0 + 8 * (f0 + f) + 2 * t) * LD + s0 + B1 + 8 * fr + g;
-            dst[0] = c[f][0];
-            dst[LD] = c[f][1];
-            c[f][0] = c[f][1] = 0.0;
-        }
+// 1 / sqrt(d) and 1 / d to the last bit or two.  NORMAL: by the approximations of the hardware (1e-6 off at most; zeros for subnormal numbers) and a
+// step of third order, then for the root a Newton step.  On a dependent chain 1 / d takes 41 cycles, 1 / sqrt(d) 73 (91 with rsqrt()).
+template <bool NORMAL>
+__device__ __forceinline__ double chol_rsqrt(double d) {
+    double r;
+    if (NORMAL) {
+        asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
+        const double e = fma(-(d * r), r, 1.0);
+        r = fma(r * e, fma(0.375, e, 0.5), r);
+    } else {
+        r = rsqrt(d);
     }
-    __syncthreads();
-    if (on) {                                                  // W21 = -W22 T
-        const int rr = 8 * fr + g;
-        for (int kk = 0; kk < 8 * fr + 8; kk += 4) {           // W22[r][k] = 0 for k > r
-            const int k = kk + t;
-            const double af = k <= rr ? w[tri(s0 + B1 + rr, s0 + B1 + min(k, rr))] : 0.0;
-#pragma unroll
-            for (int f = 0; f < FU; ++f) dmma_m8n8k4(c[f][0], c[f][1], af, a[(s0 + 8 * (f0 + f) + g) * LD + s0 + B1 + k]);
-        }
-#pragma unroll
-        for (int f = 0; f < FU; ++f) {
-            double *dst = w + tri(s0 + B1 + rr, s0 + 8 * (f0 + f) + 2 * t);
-            dst[0] = -c[f][0];
-            dst[1] = -c[f][1];
-        }
-    }
-    __syncthreads();
+    return r * fma(-0.5 * d, r * r, 1.5);
+}
+template <bool NORMAL>
+__device__ __forceinline__ double chol_rcp(double d) {
+    if (!NORMAL) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// a holds the lower triangle of a Schur complement (bs rows are real); on return its lower triangle is P (S = P^T P, Cholesky from
-// the last index to the first) and w is the packed lower triangle of W = P^{-1}.  Ends with a barrier.
-// err_c: what a non-positive pivot reports in info[3], beside its index and the side.
+// The 16 x 16 block at r, r of a, by one warp: elimination in [S_RR | I], last row first, column j of either in lanes j and 16 + j.  The block's lower
+// triangle becomes P_RR, above it comes W_RR = P_RR^{-1}, transposed, and V holds P_RR^{-T}.  Returns the largest index of a pivot that was not positive,
+// -1 if there is none.  NORMAL: no pivot is near an end of the range.
+// The chain is 57 cycles a pivot (inverse 41, multiply 8, multiply-add 8): pivots follow from each other as in an L D L^T factorisation, the roots
+// are taken behind them, each in a lane of its own, and a row goes to all lanes through shared memory while its pivot is inverted; with the issue of some thirty fp64 operations a
+// pivot takes 130 cycles (by shuffles, with the root on the chain, 185; in a loop over two times eight rows 260, inlined into its caller 330).
+template <int NP, bool NORMAL>
+__device__ __noinline__ int chol_block(int r) {
+    constexpr int LD = CholBlock<NP>::LD, LDV = CholBlock<NP>::LDV;
+    extern __shared__ __align__(16) double sm[];               // (by this name the accesses are known to be to shared memory)
+    double *s = sm + r * LD + r, *inv = sm + NP * LD + r, *V = sm + NP * LD + NP, *rows = V + 16 * LDV;
+    const int lane = threadIdx.x & 31, j = lane & 15;
+    double x[16], d, mine = 1.0;                               // mine: the pivot of row j
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = lane < 16 ? s[i * LD + j] : (i == j ? 1.0 : 0.0);      // (rows above j of lanes 0 - 15 are never used)
+    d = __shfl_sync(0xffffffffu, x[15], 15);
+    int bad = -1;
+#pragma unroll
+    for (int kk = 15; kk >= 0; --kk) {
+        mine = j == kk ? d : mine;
+        // (by its high word: positive, and not infinite or a NaN; the smallest subnormal numbers have none)
+        const bool positive = NORMAL ? (unsigned)__double2hiint(d) - 1u < 0x7fefffffu : d > 0.0 && isfinite(d);
+        bad = positive ? bad : max(bad, kk);
+        if (kk == 0) break;
+        double *row = rows + 16 * (kk & 1);
+        if (lane < 16) row[j] = x[kk];
+        __syncwarp();
+        const double before = __shfl_sync(0xffffffffu, x[kk > 0 ? kk - 1 : 0], kk > 0 ? kk - 1 : 0), rc = chol_rcp<NORMAL>(d);
+        double2 y[8];
+#pragma unroll
+        for (int h = 0; h < (kk + 1) / 2; ++h) y[h] = *reinterpret_cast<const double2 *>(row + 2 * h);
+        const double p = ((kk - 1) & 1) ? y[(kk - 1) / 2].y : y[(kk - 1) / 2].x;
+        // the next pivot, in every lane; a repeated channel (p = before = d) leaves zero, not a rounding error of either sign
+        const bool same = p == d && before == d;
+        const double pn = same ? 0.0 : p, next = fma(-(pn * rc), pn, same ? 0.0 : before);
+        double m = x[kk] * rc;
+        m = fma(fma(-m, d, x[kk]), rc, m);                      // x[kk] / d, rounded as a division is (1 where they are the same)
+#pragma unroll
+        for (int i = kk - 1; i >= 0; --i) x[i] = fma(-((i & 1) ? y[i / 2].y : y[i / 2].x), m, x[i]);
+        d = next;
+    }
+    // the roots, all at once
+    const double root = chol_rsqrt<NORMAL>(mine);
+    if (lane < 16) inv[j] = root;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        const double2 rk = *reinterpret_cast<const double2 *>(inv + i);
+        x[i] *= rk.x;
+        x[i + 1] *= rk.y;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        if (lane < 16 ? i > j : i < j) s[i * LD + j] = x[i];
+        if (lane >= 16) V[i * LDV + j] = i <= j ? x[i] : 0.0;
+    }
+    // (P's diagonal is the inverse of W's: closer than sqrt(d) = d rk is, and F = W diag(P) keeps the difference)
+    const double p = mine * root;
+    if (lane < 16) s[j * LD + j] = fma(p, fma(-p, root, 1.0), p);
+    return bad;
+}
+
+// a, the dynamic shared memory, holds the lower triangle of a Schur complement (bs rows are real, the others identity); on return its lower triangle is P (S = P^T P,
+// Cholesky from the last index to the first) and above its diagonal lies W = P^{-1} (CholBlock::inverse), of the rows below the next multiple of 16.
+// Ends with a barrier.  err_c: what a non-positive pivot reports in info[3], beside its index and the side.
+//
+// Sixteen rows R = [r, r + 16) at a time, from the last block to the first.  Between two barriers
+//   warp 0 brings the block's own 16 x 16 part up to date and eliminates in [S_RR | I], a column per lane in registers: lanes 0 - 15 end with
+//     P_RR, lanes 16 - 31 with the columns of V = P_RR^{-T};
+//   the warps of the other three quarters of the SM take the updates of the block before to the rows above, and U = W22 P2R (2: the rows below R);
+// then P_R,0:r = P_RR^{-T} S_R,0:r by substitution, a thread per column (products with V would be off by a third more under channel scales), and
+// W_2R = -U V^T.  Updates and W are 8 x 8 fragments on the fp64 tensor path.
+// In the set-up of 1100 x 4100 a block of 128 takes 28 us with its loads and stores, where solves after an elimination of all sixteen rows, updates after them
+// and the inverse by doubling at the end took 44; 256 sides of order 96 52 us against 62.
 template <int NP>
-__device__ __forceinline__ void chol_inverse(double *a, double *w, int bs, int *info, int side, int k0, int err_c) {
-    constexpr int LD = CholBlock<NP>::LD;
+__device__ __forceinline__ void chol_inverse(double *a, int bs, int *info, int side, int k0, int err_c) {
+    constexpr int LD = CholBlock<NP>::LD, LDV = CholBlock<NP>::LDV;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    // Blocked, sixteen rows R = [r_lo, r_hi) at a time from the last block to the first, three barriers a block:
-    //  (1) warp 0 factors the block's own 16 x 16 part, a column per lane in registers (lanes 16 - 31 repeat lanes 0 - 15);
-    //  (2) every column j < r_lo of the block's rows is a triangular solve of its own, one thread per column, sixteen
-    //      values in registers:  P[k][j] = (A[k][j] - sum_{k' in R, k' > k} P[k'][k] P[k'][j]) / P[k][k],  k descending;
-    //  (3) the rows above the block receive the block's sixteen rank-one updates at once, as 8 x 8 fragments of the
-    //      lower triangle on the fp64 tensor path (four m8n8k4 products each), two rows of fragments per warp.
-    // Rows from bs on are identity padding: they factor to the identity and contribute nothing.
-    // The whole is a chain of latencies.  In (1) a step's chain is: reciprocal square root of the pivot, scaling of the lane's entry
-    // of row k, update of the next pivot by the lane that owns it, one shuffle to all; the other updates of the step fill
-    // the time of the next square root.  Order 128, thousands of cycles (with the loads and stores around it 84 -> 45 us): (1) 62 -> 34,
-    // (3) 30 -> 13 (fragments were decoded one by one), inverse 49 -> 16 (one chain per column of 32, one fragment at a time).
-    __shared__ double s_rk[16];
-    for (int kb = (bs - 1) >> 4; kb >= 0; --kb) {
-        const int r_lo = 16 * kb;
+    double *wd = a + NP * LD, *V = wd + NP;
+    const int last = (bs - 1) >> 4, end = 16 * last + 16;
+    for (int kb = last; kb >= 0; --kb) {
+        const int r = 16 * kb, q = r + 16;                      // this block's rows [r, q); the block before, if any, is [q, q + 16)
         if (warp == 0) {
-            const int j = lane & 15;
-            double x[16];
+            if (kb < last) {
+                double c[3][2] = {};                            // fragments (0, 0), (1, 0), (1, 1)
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = a[(r_lo + i) * LD + r_lo + j];              // rows i < j: never used
-            double d = __shfl_sync(0xffffffffu, x[15], 15), rmine = 0.0;
-            int bad = -1;
+                for (int kk = 0; kk < 16; kk += 4) {
+                    const double lo = a[(q + kk + t) * LD + r + g], hi = a[(q + kk + t) * LD + r + 8 + g];
+                    dmma_m8n8k4(c[0][0], c[0][1], lo, lo);
+                    dmma_m8n8k4(c[1][0], c[1][1], hi, lo);
+                    dmma_m8n8k4(c[2][0], c[2][1], hi, hi);
+                }
 #pragma unroll
-            for (int kk = 15; kk >= 0; --kk) {
-                if (!(d > 0.0) || !isfinite(d)) { bad = max(bad, kk); d = 1.0; }
-                double rk = rsqrt(d);
-                rk = rk * fma(-0.5 * d, rk * rk, 1.5);         // one Newton step: 1 / sqrt(d) to the last bit or two
-                const double pk = x[kk] * rk;                  // P[k][j], j < k
-                if (kk > 0) {
-                    x[kk - 1] = fma(-__shfl_sync(0xffffffffu, pk, kk - 1), pk, x[kk - 1]);
-                    const double dn = __shfl_sync(0xffffffffu, x[kk - 1], kk - 1);
+                for (int f = 0; f < 3; ++f) {
+                    double2 *dst = reinterpret_cast<double2 *>(a + (r + 8 * ((f + 1) >> 1) + g) * LD + r + 8 * (f >> 1) + 2 * t);
+                    const double2 o = *dst;
+                    *dst = double2{o.x - c[f][0], o.y - c[f][1]};
+                }
+                __syncwarp();
+            }
+            // pivots lie below the diagonal, and a factor of 2^60 below it they are rounding errors: where the diagonal is far from either end of the
+            // range all of them are
+            const int i = r + (lane & 15);
+            const unsigned top = (unsigned)__double2hiint(a[i * LD + i]);
+            const bool normal = __all_sync(0xffffffffu, top > (1023u - 900u) << 20 && top < (1023u + 900u) << 20);
+            const int bad = normal ? chol_block<NP, true>(r) : chol_block<NP, false>(r);
+            if (bad >= 0 && lane == 0) report(info, GPTQ2D_ERR_NOT_SPD, k0 + r + bad, side, err_c);
+        } else if (warp != 4) {
+            const int w = warp - 1 - (warp > 4);                // 0 .. 5
+            // rows above this block's and its own: -= P_Q,:^T P_Q,: with the block Q = [q, q + 16) before; warp 0 has the 16 x 16 part
+            const int nb = kb < last ? 2 * kb + 2 : 0;
+            for (int h = 0; 6 * h < nb; ++h) {
+                const int bi = nb - 1 - 6 * h - ((h & 1) ? 5 - w : w);
+                if (bi < 0) continue;
+                const int ri = 8 * bi + g, stop = min(bi, nb - 3);
+                double af[4];
 #pragma unroll
-                    for (int i = kk - 2; i >= 0; --i) x[i] = fma(-__shfl_sync(0xffffffffu, pk, i), pk, x[i]);
-                    x[kk] = j == kk ? d * rk : pk;
-                    if (j == kk) rmine = rk;
-                    d = dn;
-                } else {
-                    x[0] = j == 0 ? d * rk : pk;
-                    if (j == 0) rmine = rk;
+                for (int kk = 0; kk < 4; ++kk) af[kk] = a[(q + 4 * kk + t) * LD + ri];
+                for (int bj = 0; bj <= stop; bj += 2) {         // (fragments on the diagonal reach above it, where no W lies yet)
+                    const bool two = bj < stop;
+                    const int c1 = two ? bj + 1 : bj;
+                    double c[2][2] = {};
+                    double2 *dst = reinterpret_cast<double2 *>(a + ri * LD + 8 * bj + 2 * t), *dst1 = reinterpret_cast<double2 *>(a + ri * LD + 8 * c1 + 2 * t);
+                    const double2 o = *dst, o1 = *dst1;
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        dmma_m8n8k4(c[0][0], c[0][1], af[kk], a[(q + 4 * kk + t) * LD + 8 * bj + g]);
+                        dmma_m8n8k4(c[1][0], c[1][1], af[kk], a[(q + 4 * kk + t) * LD + 8 * c1 + g]);
+                    }
+                    *dst = double2{o.x - c[0][0], o.y - c[0][1]};
+                    if (two) *dst1 = double2{o1.x - c[1][0], o1.y - c[1][1]};
                 }
             }
-            if (bad >= 0 && lane == 0) report(info, GPTQ2D_ERR_NOT_SPD, k0 + r_lo + bad, side, err_c);
-            if (lane < 16) {
-                s_rk[j] = rmine;
+            // U = W22 P2R, eight rows at a time, into the place of W2R
+            const int nu = (end - q) >> 3;
+            for (int h = 0; 6 * h < nu; ++h) {
+                const int fr = nu - 1 - 6 * h - ((h & 1) ? w : 5 - w);
+                if (fr < 0) continue;
+                const int i0 = q + 8 * fr, i = i0 + g;
+                double c[4][2][2] = {};                         // four chains
+                const auto step = [&](double (&x)[2][2], double af, int k) {
+                    dmma_m8n8k4(x[0][0], x[0][1], af, a[k * LD + r + g]);
+                    dmma_m8n8k4(x[1][0], x[1][1], af, a[k * LD + r + 8 + g]);
+                };
+                int k = q;
+                for (; k + 8 < i0; k += 16) {                   // (i0 - q is a multiple of eight: eight rows are left over, or none)
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (i >= j) a[(r_lo + i) * LD + r_lo + j] = x[i];
+                    for (int h2 = 0; h2 < 4; ++h2) step(c[h2], a[(k + 4 * h2 + t) * LD + i], k + 4 * h2 + t);
+                }
+                if (k < i0) {
+#pragma unroll
+                    for (int h2 = 0; h2 < 2; ++h2) step(c[h2], a[(k + 4 * h2 + t) * LD + i], k + 4 * h2 + t);
+                }
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) {                // the 8 x 8 part on the diagonal of W
+                    const int kt = i0 + 4 * h2 + t;
+                    step(c[2 + h2], kt < i ? a[kt * LD + i] : (kt == i ? wd[i] : 0.0), kt);
+                }
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    a[(r + 8 * f + 2 * t) * LD + i] = (c[0][f][0] + c[1][f][0]) + (c[2][f][0] + c[3][f][0]);
+                    a[(r + 8 * f + 2 * t + 1) * LD + i] = (c[0][f][1] + c[1][f][1]) + (c[2][f][1] + c[3][f][1]);
+                }
             }
         }
         __syncthreads();
-        if (kb > 0) {
-            if (tid < r_lo) {
-                double x[16];
+        // P_R,0:r in place, from the last threads on: their warps have no part in the next step's elimination
+        const int col = 255 - tid;
+        if (col < r) {
+            double x[16];
 #pragma unroll
-                for (int kk = 0; kk < 16; ++kk) x[kk] = a[(r_lo + kk) * LD + tid];
+            for (int kk = 0; kk < 16; ++kk) x[kk] = a[(r + kk) * LD + col];
 #pragma unroll
-                for (int kk = 15; kk >= 0; --kk) {
-                    double sum = x[kk];
+            for (int kk = 15; kk >= 0; --kk) {
+                x[kk] *= wd[r + kk];
 #pragma unroll
-                    for (int k2 = 15; k2 > kk; --k2) sum = fma(-a[(r_lo + k2) * LD + r_lo + kk], x[k2], sum);
-                    x[kk] = sum * s_rk[kk];
+                for (int k2 = 0; k2 < kk; k2 += 2) {
+                    const double2 p = *reinterpret_cast<const double2 *>(a + (r + kk) * LD + r + k2);      // P[kk][k2], P[kk][k2 + 1]
+                    x[k2] = fma(-p.x, x[kk], x[k2]);
+                    if (k2 + 1 < kk) x[k2 + 1] = fma(-p.y, x[kk], x[k2 + 1]);
                 }
-#pragma unroll
-                for (int kk = 0; kk < 16; ++kk) a[(r_lo + kk) * LD + tid] = x[kk];
+                a[(r + kk) * LD + col] = x[kk];
             }
-            __syncthreads();
-            // leading (16 kb) x (16 kb) lower triangle -= P[R, :]^T P[R, :]
-            const int nb = 2 * kb;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int bi = nb - 1 - (h ? 15 - warp : warp);                // a long row of fragments and a short one
-                if (bi < 0) continue;
-                double af[4];
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) af[kk] = a[(r_lo + 4 * kk + t) * LD + 8 * bi + g];
-                const int ri = 8 * bi + g;
-#pragma unroll 2
-                for (int bj = 0; bj <= bi; ++bj) {
-                    const int cj = 8 * bj + 2 * t;
-                    double c0 = 0.0, c1 = 0.0;
-                    const double o0 = a[ri * LD + cj], o1 = a[ri * LD + cj + 1];
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) dmma_m8n8k4(c0, c1, af[kk], a[(r_lo + 4 * kk + t) * LD + 8 * bj + g]);
-                    if (cj <= ri) a[ri * LD + cj] = o0 - c0;
-                    if (cj + 1 <= ri) a[ri * LD + cj + 1] = o1 - c1;
-                }
-            }
-            __syncthreads();
         }
-    }
-    // ---- W = P^{-1}.  Level 0: the 16 x 16 diagonal blocks, one column per thread, in registers.
-    if (tid < NP) {
-        const int r0 = tid & ~15, j = tid & 15;
-        const double inv = 1.0 / a[(r0 + j) * LD + r0 + j];
-        double y[16];
+        // W_2R = -U V^T in place, eight rows a unit, from the first warps on
+        for (int u = warp; u < (end - q) >> 3; u += 8) {
+            const int i0 = q + 8 * u;
+            double c[2][2] = {}, af[4];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            double s0 = 0.0, s1 = 0.0;
+            for (int kk = 0; kk < 4; ++kk) af[kk] = a[(r + 4 * kk + t) * LD + i0 + g];
+            __syncwarp();
 #pragma unroll
-            for (int k = 0; k < i; ++k) {
-                if (k & 1) s1 = fma(a[(r0 + i) * LD + r0 + k], y[k], s1);
-                else s0 = fma(a[(r0 + i) * LD + r0 + k], y[k], s0);
+            for (int kk = 0; kk < 4; ++kk) {                    // (V^T)[k][n] = V[n][k], zero for n > k
+                dmma_m8n8k4(c[0][0], c[0][1], af[kk], V[g * LDV + 4 * kk + t]);
+                if (kk >= 2) dmma_m8n8k4(c[1][0], c[1][1], af[kk], V[(8 + g) * LDV + 4 * kk + t]);
             }
-            const double ii = __shfl_sync(0xffffffffu, inv, i, 16);
-            y[i] = i > j ? -(s0 + s1) * ii : (i == j ? inv : 0.0);
-            if (i >= j) w[tri(r0 + i, r0 + j)] = y[i];
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                a[(r + 8 * f + 2 * t) * LD + i0 + g] = -c[f][0];
+                a[(r + 8 * f + 2 * t + 1) * LD + i0 + g] = -c[f][1];
+            }
         }
-    }
-    __syncthreads();
-    // ---- then pairs of blocks: 16, 32 and 64 rows
-    if (NP == 128) {
-        inverse_join<NP, NP == 128 ? 4 : 1, 16, 16, 1>(a, w, 32);
-        inverse_join<NP, NP == 128 ? 2 : 1, 32, 32, 1>(a, w, 64);
-        inverse_join<NP, 1, 64, NP == 128 ? 64 : 32, 1>(a, w, 0);
-    } else if (NP == 96) {
-        inverse_join<NP, NP == 96 ? 3 : 1, 16, 16, 1>(a, w, 32);
-        inverse_join<NP, 1, 32, 32, 2>(a, w, 0);
-        inverse_join<NP, 1, 64, 32, 2>(a, w, 0);
-    } else {
-        inverse_join<NP, 2, 16, 16, 2>(a, w, 32);
-        inverse_join<NP, 1, 32, 32, 2>(a, w, 0);
+        __syncthreads();
     }
 }
 
 __global__ void __launch_bounds__(256) factor_diag_kernel(double *S, long lds, int bs, double *W, long ldw,
                                                           double *pdiag, int *info, int side, int k0) {
     constexpr int LD = CholBlock<128>::LD;
-    extern __shared__ double sm[];
-    double *a = sm;               // [128][LD]: P in the lower triangle, scratch above it
-    double *w = sm + 128 * LD;    // packed lower triangle of W
-    const int tid = threadIdx.x;
-    // the block, padded with the identity: the kernel sits on the serial spine of the set-up, so a thread's 64 loads
-    // are issued in two batches of 32 (entry idx = 256 u + tid: a warp reads 32 consecutive columns of one row)
-    for (int base = 0; base < 128 * 128; base += 32 * 256) {
-        double v[32];
+    extern __shared__ __align__(16) double sm[];
+    double *a = sm;               // [128][LD]: P in the lower triangle, its inverse above it
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // the block, padded with the identity; it sits on the serial spine of the set-up, so all copies are in flight at once
+    // (S and lds come from the workspace: rows start on 16 bytes)
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            const int idx = base + u * 256 + tid, i = idx >> 7, j = idx & 127;
-            v[u] = (j <= i && i < bs) ? S[(long)i * lds + j] : (i == j ? 1.0 : 0.0);
-        }
+    for (int u = 0; u < 16; ++u) {
+        const int i = warp + 8 * u;
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            const int idx = base + u * 256 + tid, i = idx >> 7, j = idx & 127;
-            if (j <= i) a[i * LD + j] = v[u];
+        for (int h = 0; h < 2; ++h) {
+            const int j = 64 * h + 2 * lane;
+            if (i < bs && j <= i) cp_async16(a + i * LD + j, S + (long)i * lds + j, 16);
+            else if (i >= bs && j <= i) *reinterpret_cast<double2 *>(a + i * LD + j) = double2{j == i ? 1.0 : 0.0, j + 1 == i ? 1.0 : 0.0};
         }
     }
+    cp_async_commit();
+    cp_async_wait<0>();
     __syncthreads();
-    chol_inverse<128>(a, w, bs, info, side, k0, 0);
-#pragma unroll 8
-    for (int u = 0; u < 64; ++u) {
-        const int idx = u * 256 + tid, i = idx >> 7, j = idx & 127;
-        if (i < bs && j <= i) {                                // (W's block has been cleared: nothing to write above its diagonal)
-            S[(long)i * lds + j] = a[i * LD + j];
-            W[(long)i * ldw + j] = w[tri(i, j)];
+    chol_inverse<128>(a, bs, info, side, k0, 0);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+        const int i = warp + 8 * u;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int j = 32 * h + lane;
+            if (i < bs && j <= i) S[(long)i * lds + j] = a[i * LD + j];
+        }
+    }
+    // (W's block has been cleared: nothing to write above its diagonal; eight rows of four columns a warp, whose entries lie in sixteen banks)
+#pragma unroll 4
+    for (int h = 0; h < 16; ++h) {
+        const int i = 8 * h + (lane >> 2);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = 4 * (warp + 8 * u) + (lane & 3);
+            if (i < bs && j <= i) W[(long)i * ldw + j] = CholBlock<128>::inverse(a, i, j);
         }
     }
     for (int i = tid; i < bs; i += blockDim.x) pdiag[i] = a[i * LD + i];
@@ -294,13 +353,12 @@ __global__ void identity_kernel(double *out, long ldo, int k, double *dinv) {
 // factorisation and inverse (chol_inverse), the unit triangular factor and 1/Lambda.  For the set-up of many small matrices
 // at once, where one launch sequence per matrix would cost far more than the arithmetic.  NP = 64, 96 or 128: what a CTA
 // does is a chain of latencies, so the smaller orders, whose blocks leave room for four or two CTAs on an SM, run that many
-// at once (256 sides of order 96: 192 -> 68 us, with the shorter chain of chol_inverse).
+// at once (256 sides of order 96: 192 -> 52 us, with the shorter chain of chol_inverse).
 template <int NP>
 __global__ void __launch_bounds__(256, NP == 64 ? 4 : (NP == 96 ? 2 : 1)) factor_small_kernel(const FactorSmallSide *sides, int *info) {
     constexpr int LD = CholBlock<NP>::LD, F = NP / 16;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     double *a = sm;               // [NP][LD]
-    double *w = sm + NP * LD;     // packed lower triangle of W
     const FactorSmallSide q = sides[blockIdx.x];
     const int k = q.k, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     if (!q.M) {                                           // identity basis
@@ -355,12 +413,12 @@ __global__ void __launch_bounds__(256, NP == 64 ? 4 : (NP == 96 ? 2 : 1)) factor
             if (j <= i) a[i * LD + j] = i < k ? acc[ii][jj] : (i == j ? 1.0 : 0.0);
         }
     __syncthreads();
-    chol_inverse<NP>(a, w, k, info, q.side, 0, q.index);
+    chol_inverse<NP>(a, k, info, q.side, 0, q.index);
     // F = W diag(P): unit lower (side 0) or, transposed on the way out, unit upper (side 1)
 #pragma unroll 4
     for (int idx = tid; idx < NP * NP; idx += 256) {
         const int r = idx / NP, c = idx - r * NP, i = q.side == 0 ? r : c, j = q.side == 0 ? c : r;      // writes run along memory
-        if (r < k && c < k) q.out[(long)r * q.ldo + c] = i > j ? w[tri(i, j)] * a[j * LD + j] : (i == j ? 1.0 : 0.0);
+        if (r < k && c < k) q.out[(long)r * q.ldo + c] = i > j ? CholBlock<NP>::inverse(a, i, j) * a[j * LD + j] : (i == j ? 1.0 : 0.0);
     }
     if (q.dinv)
         for (int j = tid; j < k; j += blockDim.x) q.dinv[j] = a[j * LD + j] * a[j * LD + j];

@@ -135,3 +135,26 @@ def test_the_multi_stream_set_up_is_bit_identical_to_the_one_stream_set_up(g):
             torch.cuda.synchronize()
             g.check_info(info)
             assert torch.equal(L, L0) and torch.equal(U, U0) and torch.equal(dL, dL0) and torch.equal(dU, dU0), k
+
+
+@pytest.mark.parametrize("e", [470, -490])
+@pytest.mark.parametrize("k", [1, 16, 17, 64, 97, 128, 150])
+def test_diagonal_blocks_near_the_ends_of_the_range(g, k, e):
+    # pivots of 2^940 and 2^-980, where the approximate inverses are not taken; a power of two changes no digit of L but for those
+    rng = np.random.default_rng(k)
+    a = rng.standard_normal((k, k)) / np.sqrt(4 * k) + np.eye(k)
+    plain, scaled = (g.gptq2d_factor(dev(v), None, n=1) for v in (a, np.ldexp(a, e)))
+    g.check_info(plain[4])
+    g.check_info(scaled[4])
+    # two factorisations of a Gram of condition below 100: 128 roundings of 1e-16 times that
+    assert float((scaled[0] - plain[0]).abs().max()) <= 2e-12
+    assert np.max(np.abs(np.ldexp(scaled[2].cpu().numpy(), -2 * e) / plain[2].cpu().numpy() - 1.0)) <= 2e-12
+
+
+@pytest.mark.parametrize("k,i,j", [(40, 5, 6), (40, 0, 15), (40, 18, 29), (40, 33, 39), (128, 112, 127), (96, 7, 13)])
+def test_a_repeated_channel_is_a_zero_pivot(g, k, i, j):
+    # two equal columns of one block of sixteen: what is left of the first after the second is zero, not a rounding error of either sign
+    for seed in range(4):
+        a = np.random.default_rng(seed).standard_normal((k, k))
+        a[:, i] = a[:, j]
+        assert g.gptq2d_factor_batched([dev(a)], [dev(np.eye(1))])[4].cpu().tolist() == [5, i, 0, 0]
