@@ -508,17 +508,25 @@ struct I8Where {
     int k_lo, stages;                                          // contraction: pieces of I8_STAGE_K
 };
 // Tiles in groups of eight tile rows, column by column inside a group, so that the CTAs that run at one time share
-// operand tiles in L2.  The rows and columns with the longer contractions first, where an operand is a triangle (4096 x 4096 with a triangular
-// left operand, rows in the wrong order: 0.70 ms).  false: a tile above the diagonal that fills up a group.
+// operand tiles in L2; where an operand is a triangle by the length of its contractions instead, longest first: row by row for the left one,
+// column by column for the right one (the Gram at order 4100 580 us in groups; 4096 x 4096 with a triangular left operand, rows in the
+// wrong order, 0.70 ms).  false: no tile.
 template <int TN>
 __device__ __forceinline__ bool i8_where(const I8Params &p, int id, I8Where &w) {
-    constexpr int GROUP = 8, PER = I8_STAGE_K / I8_KCHUNK;
+    constexpr int PER = I8_STAGE_K / I8_KCHUNK;
     const int all = (p.K + I8_KCHUNK - 1) / I8_KCHUNK, blocksA = (int)(p.rowsA_pad / 128), blocksB = (int)(p.rowsB_pad / 128);
     w.bz = p.batch > 1 ? id / p.tiles : 0;
     const int *rangeA = p.rangeA + (long)w.bz * blocksA * 2, *rangeB = p.rangeB + (long)w.bz * blocksB * 2;
+    int la, ha, lb, hb, lc, hc, ld, hd;
+    i8_chunks(rangeA, 0, 2, blocksA, all, la, ha);
+    i8_chunks(rangeA, blocksA - 1, 1, blocksA, all, lc, hc);
+    i8_chunks(rangeB, 0, 2, blocksB, all, lb, hb);
+    i8_chunks(rangeB, blocksB - 1, 1, blocksB, all, ld, hd);
+    const int more_a = (ha - la) - (hc - lc), more_b = (hb - lb) - (hd - ld);                // of the first block against the last
+    const int group = p.lower_tiles_only || abs(more_a) > all / 4 ? 1 : (abs(more_b) > all / 4 ? p.tiles_m : 8);
     int in = id - w.bz * p.tiles, hi = p.tiles_m, tm = 0, tn = 0;            // rows [lo, hi) of the group
     while (hi > 0) {
-        const int lo = max(0, hi - GROUP), rows = hi - lo;
+        const int lo = max(0, hi - group), rows = hi - lo;
         const int cols = p.lower_tiles_only ? min(p.tiles_n, hi * (256 / TN)) : p.tiles_n;
         if (in < rows * cols) {
             tn = in / rows;
@@ -528,14 +536,9 @@ __device__ __forceinline__ bool i8_where(const I8Params &p, int id, I8Where &w) 
         in -= rows * cols;
         hi = lo;
     }
-    int la, ha, lb, hb, lc, hc;
     if (!p.lower_tiles_only) {
-        i8_chunks(rangeA, 0, 2, blocksA, all, la, ha);
-        i8_chunks(rangeA, blocksA - 1, 1, blocksA, all, lc, hc);
-        if (ha - la > hc - lc) tm = p.tiles_m - 1 - tm;
-        i8_chunks(rangeB, 0, 2, blocksB, all, lb, hb);
-        i8_chunks(rangeB, blocksB - 1, 1, blocksB, all, lc, hc);
-        if (hb - lb < hc - lc) tn = p.tiles_n - 1 - tn;
+        if (more_a > 0) tm = p.tiles_m - 1 - tm;
+        if (more_b < 0) tn = p.tiles_n - 1 - tn;
     }
     w.m0 = tm * 256; w.n0 = tn * TN;
     if (p.lower_tiles_only && w.n0 > w.m0 + 255) return false;
@@ -666,6 +669,8 @@ __device__ __noinline__ double i8_entries_general(const I8Params &p, int bz, con
     const bool row_diag = p.diag_a && gi < p.K && there;
     const double a_gg = row_diag ? p.alpha * Ab[(long)gi * (p.ai + p.aj)] : 0.0;
     const double *b_row = Bb + (long)gi * p.bi + (long)first_col * p.bj, *a_row = Ab + (long)gi * p.ai + (long)first_col * p.aj;
+    // (a lane's own row: 32 bytes at a time where they start on a boundary of that)
+    const bool a_vec = p.aj == 1 && (reinterpret_cast<uintptr_t>(a_row) & 31) == 0, b_vec = p.bj == 1 && (reinterpret_cast<uintptr_t>(b_row) & 31) == 0;
     double sq = 0.0;
     bool row_seen = false;
     unsigned col_bits = 0u, x[I8_MODULI];
@@ -719,16 +724,40 @@ __device__ __noinline__ double i8_entries_general(const I8Params &p, int bz, con
         v[0] *= scale * __hiloint2double(cs.x, 0); v[1] *= scale * __hiloint2double(cs.y, 0);
         v[2] *= scale * __hiloint2double(cs.z, 0); v[3] *= scale * __hiloint2double(cs.w, 0);
         if (!there) continue;
+        if (p.sumsq_partials) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gj = first_col + c + j;
-            if (c + j >= cols) continue;
-            if (p.sumsq_partials) { sq = fma(v[j], v[j], sq); continue; }
-            if (row_diag) v[j] = fma(a_gg, b_row[(c + j) * p.bj], v[j]);
-            if (p.diag_b && gj < p.K && !(p.diag_a && gi == gj)) v[j] = fma(p.alpha * a_row[(c + j) * p.aj], Bb[(long)gj * (p.bi + p.bj)], v[j]);
-            if (load_old) v[j] = fma(p.beta, old[j], v[j]);
+            for (int j = 0; j < 4; ++j)
+                if (c + j < cols) sq = fma(v[j], v[j], sq);
+            continue;
         }
-        if (p.sumsq_partials) continue;
+        if (row_diag) {
+            double b[4];
+            if (b_vec && c + 4 <= cols) i8_load4(b, b_row + c);
+            else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) b[j] = c + j < cols ? b_row[(c + j) * p.bj] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = fma(a_gg, b[j], v[j]);
+        }
+        if (p.diag_b) {
+            double x[4];
+            const bool whole = c + 4 <= cols && first_col + c + 4 <= p.K;
+            if (a_vec && whole) i8_load4(x, a_row + c);
+            else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x[j] = c + j < cols && first_col + c + j < p.K ? a_row[(c + j) * p.aj] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int gj = first_col + c + j;
+                if (c + j < cols && gj < p.K && !(p.diag_a && gi == gj)) v[j] = fma(p.alpha * x[j], Bb[(long)gj * (p.bi + p.bj)], v[j]);
+            }
+        }
+        if (load_old) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = fma(p.beta, old[j], v[j]);
+        }
         if (four) i8_store4(dst + c, v);
         else {
 #pragma unroll
@@ -1061,12 +1090,12 @@ static bool encode_planes_map(CUtensorMap *map, const I8Planes &pl, int box_rows
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// tiles of 256 x tn of one matrix, with those above the diagonal that fill up a group of rows (i8_where)
+// tiles of 256 x tn of one matrix, with those above the diagonal that a row of tiles reaches (i8_where)
 static long i8_tiles(const GemmArgs &g, int tn) {
     const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + tn - 1) / tn;
     if (!g.lower_tiles_only) return (long)tiles_m * tiles_n;
     long n = 0;
-    for (int hi = tiles_m; hi > 0; hi = std::max(0, hi - 8)) n += (long)(hi - std::max(0, hi - 8)) * std::min(tiles_n, hi * (256 / tn));
+    for (int hi = 1; hi <= tiles_m; ++hi) n += std::min(tiles_n, hi * (256 / tn));
     return n;
 }
 
