@@ -1071,6 +1071,19 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         // ================= B: the far part (every source tile of the contraction except the nearest)
         const TiledKernelParams &pk = VIEW(0);
         const int f_type = s_far[0], f_I = s_far[1], f_J = s_far[2], f_pos = s_far[3], f_nfar = s_far[4];
+        if (f_nfar == 0) {
+            // no sources: the cells start from zeros, or from what is there already
+            if (!((pk.preloaded >> f_type) & 1)) {
+                double *dst = tile_region();
+#pragma unroll 4
+                for (int k = tid; k < T * T / 2; k += TILED_THREADS)
+                    *reinterpret_cast<double2 *>(dst + CI((long)(k / (T / 2)) * pk.np + k % (T / 2) * 2, 127L * pk.np + T - 1, 200)) = double2{0.0, 0.0};
+            }
+            __syncthreads();
+            if (tid < TC) far_arrive(pk, f_I, f_J, tid);
+            if (tid == 0) s_has = 0;
+            continue;
+        }
         if (fresh) {
             if ((pk.preloaded >> f_type) & 1) load_acc(acc, tile_region(), pk.np, wm, wn, g, t);
             else acc.zero();
@@ -1150,6 +1163,11 @@ struct TiledLayout {
     int ntm, ntn;
     size_t q_off, flags_off, quad_off, qdep_off, qprog_off, rowdone_off, e_off, c_off, total;
 };
+// CTAs of a launch: one for every cell, up to one an SM.  One a far part, as there were when a tile had four tasks of its own, leaves the cells of small
+// matrices waiting for each other's CTAs (us, a CTA a far part / four / a cell: 64 x 64 44.5 / 38.1 / 38.0, 128 x 128 120 / 62.5 / 63.1, 256 x 256
+// 156 / 112 / 111, 512 x 512 259 / 237 / 235).
+static long cells_of(int m, int n) { return (long)((m + S - 1) / S) * ((n + S - 1) / S); }
+static int tiled_grid(int sms, long cells) { return (int)std::max(2l, std::min((long)sms, cells)); }
 static TiledLayout tiled_layout(int m, int n) {
     TiledLayout l;
     l.ntm = (m + T - 1) / T;
@@ -1289,7 +1307,7 @@ int launch_round_tiled(const TiledParams &in, void *ws, size_t ws_bytes, cudaStr
                                          : (const void *)round_tiled_kernel<false, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess)
         return GPTQ2D_ERR_CUDA;
-    int grid = sms < p.ntasks ? sms : p.ntasks;
+    const int grid = tiled_grid(sms, cells_of(p.m, p.n));
     void *args[] = {&p};
     if (cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
         return GPTQ2D_ERR_CUDA;
@@ -1363,6 +1381,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
     unsigned *table = reinterpret_cast<unsigned *>(stage.data() + (l.table_off - l.desc_off));
     size_t foff = l.flags_off, boff = l.bufs_off;
     int max_waves = 0;
+    long ncells = 0;
     // A ring entry has 31 bits for matrix and cell.  With more than 2048 matrices the index of a cell may not fit beside that of the
     // matrix; one that large (more than 2^18 cells, 16384 x 16384) fills the GPU and is swept in a launch of its own.
     int cell_bits = 31, big = 0;
@@ -1403,6 +1422,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         d.ntiles_total = (int)tiles;
         desc[b] = d;
         if (alone(d)) { ++big; l.ntasks -= 2 * (long)tiles; l.ntiles -= (long)tiles; continue; }
+        ncells += cells_of(in.m, in.n);
         if (t.ntm + t.ntn - 1 > max_waves) max_waves = t.ntm + t.ntn - 1;
     }
     // claim order: tile-wave by tile-wave over all matrices; inside a matrix' wave as decode_task lists them
@@ -1448,7 +1468,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         if (cudaFuncSetAttribute(round_tiled_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
         void *own[] = {&d};
-        if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<false, false>, dim3(std::min(sms, d.ntasks)), dim3(TILED_THREADS), own,
+        if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<false, false>, dim3(tiled_grid(sms, cells_of(d.m, d.n))), dim3(TILED_THREADS), own,
                                         TILED_SMEM, stream) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
         if (cudaMemsetAsync(w, 0, l.maxe_off, stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;      // scheduler words and ring
@@ -1457,7 +1477,7 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
         if (cudaFuncSetAttribute(round_tiled_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)TILED_SMEM) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
-        int grid = (long)sms < l.ntasks ? sms : (int)l.ntasks;
+        const int grid = tiled_grid(sms, ncells);
         void *args[] = {&p};
         if (cudaLaunchCooperativeKernel((const void *)round_tiled_kernel<true, false>, dim3(grid), dim3(TILED_THREADS), args,
                                         TILED_SMEM, stream) != cudaSuccess)
@@ -1614,7 +1634,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         const void *kernel = (const void *)round_tiled_kernel<false, false>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess) return GPTQ2D_ERR_CUDA;
         void *args[] = {&p};
-        return cudaLaunchCooperativeKernel(kernel, dim3(std::min(sms, p.ntasks)), dim3(TILED_THREADS), args, TILED_SMEM, stream) == cudaSuccess
+        return cudaLaunchCooperativeKernel(kernel, dim3(tiled_grid(sms, cells_of(p.m, p.n))), dim3(TILED_THREADS), args, TILED_SMEM, stream) == cudaSuccess
                    ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
     };
     int st = sweep_one(block(0, 0, 0, 0));
@@ -1641,7 +1661,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         const void *kernel = (const void *)round_tiled_kernel<true, false>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILED_SMEM) != cudaSuccess) return GPTQ2D_ERR_CUDA;
         void *args[] = {&p};
-        if (cudaLaunchCooperativeKernel(kernel, dim3(std::min(sms, p.ntasks)), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
+        if (cudaLaunchCooperativeKernel(kernel, dim3(tiled_grid(sms, cells_of(a.m, a.n) + cells_of(b.m, b.n))), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
     }
     at = own ? own : C;
