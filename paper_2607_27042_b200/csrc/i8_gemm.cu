@@ -40,7 +40,8 @@ struct I8Tables {
     int p[I8_MODULI];
     int inv0[I8_MODULI], inv6[I8_MODULI];                      // ceil(2^32 / p), ceil(2^38 / p): floor(s / p) for |s| <= 2^24, 2^28 but for negative multiples of p
     unsigned digit_lo[I8_MODULI], digit_hi[I8_MODULI];         // 256^j mod p as signed bytes, j = 0 .. 3, 4 .. 6
-    float pf[I8_MODULI], invf[I8_MODULI];                      // p, 1 / p
+    int lift[I8_MODULI];                                       // bits of B, the least float from 2^23 + 2^17 that is a multiple of 256 p
+    float less_p[I8_MODULI], invf[I8_MODULI], lifted[I8_MODULI];                   // -p, 1 / p, -(1.5 * 2^23 + B / p)
     unsigned weight[I8_WEIGHT_BYTES][I8_MODULI / 4];           // byte b of round(2^80 u_i / p_i), four i to a word
     double product_hi, product_lo;                             // P 2^-80 2^-40 in two parts
 };
@@ -54,7 +55,9 @@ constexpr I8Tables i8_tables() {
         t.p[i] = p[i];
         t.inv0[i] = (int)(((1ull << 32) + q - 1) / q);
         t.inv6[i] = (int)(((1ull << 38) + q - 1) / q);
-        t.pf[i] = (float)p[i]; t.invf[i] = 1.0f / (float)p[i];
+        const int lift = ((1 << 23) + (1 << 17) + 256 * p[i] - 1) / (256 * p[i]) * 256;
+        t.lift[i] = 0x4b000000 + lift * p[i] - (1 << 23);
+        t.less_p[i] = -(float)p[i]; t.invf[i] = 1.0f / (float)p[i]; t.lifted[i] = -(12582912.0f + (float)lift);
         unsigned power = 1;
         for (int j = 0; j < 7; ++j) {
             const unsigned byte = (power > q / 2 ? power - q : power) & 0xffu;
@@ -232,13 +235,44 @@ __device__ __forceinline__ void i8_chunks(const int *range, int blk, int count, 
     }
 }
 
+// x' mod p from its digits' residues: their sum s, |s| <= 7 * 128 * 128 < 2^17, comes added to the bits of the float B = 2^23 + 2^17 + ..., a multiple of
+// 256 p, so that the float's value is B + s.  Its quotient by p, rounded to k by adding 1.5 * 2^23, less B / p (`lifted` takes both away again) leaves
+// B + s - k p, whose last byte is the residue.  fp32 finds every s (the product with 1 / p is off by 0.0027 at most, and k by one from the nearest only
+// where that is near a tie, of p = 255: -128 then stands for 127).  Two at a time (f32x2).
+__device__ __forceinline__ unsigned long long i8_twice(float x) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(x));
+    return v;
+}
+__device__ __forceinline__ void i8_reduce_two(unsigned &a, unsigned &b, unsigned long long less_p, unsigned long long inv, unsigned long long lifted) {
+    constexpr unsigned long long MAGIC = 0x4b4000004b400000ull;
+    asm("{\n"
+        ".reg .b64 raw, k;\n"
+        "mov.b64 raw, {%0, %1};\n"
+        "fma.rn.f32x2 k, raw, %3, %5;\n"
+        "add.rn.f32x2 k, k, %4;\n"
+        "fma.rn.f32x2 raw, k, %2, raw;\n"
+        "mov.b64 {%0, %1}, raw;\n"
+        "}\n"
+        : "+r"(a), "+r"(b)
+        : "l"(less_p), "l"(inv), "l"(lifted), "l"(MAGIC));
+}
+
+__device__ __forceinline__ void i8_fetch(double *dst, const double *src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void i8_fetched() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
 // Residues of 32 rows x 64 k per CTA.  Padding rows and columns become zeros; stages of the product (128 k) in which a pair of 128-row blocks
-// has no entry are never read (i8_where) and are left as they are.  A CTA loads, then computes (some twelve instructions a residue): many small
-// ones overlap the two (4096 x 4096: 64 rows a CTA 133 us; bytes 62).
+// has no entry are never read (i8_where) and are left as they are.  The entries come by cp.async, all sixteen of a thread in flight whatever the
+// bounds checks: eight CTAs on an SM then overlap their loads and their residues, which loads into registers did not.
+// Bound by its instructions (two dp4a, one and a half packed fp32, three quarters of a permutation a residue; bytes 62 us): 4096 x 4096 dense 84 us,
+// 129 with loads into registers and fp32 one at a time; planes four at a time 89, all sixteen unrolled 84.
 template <bool KCONTIG>
 __global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const double *src, long ld, long stride, I8Inner inner,
                                                           int skip_diagonal) {
-    __shared__ double tile[32][65];
+    constexpr int PITCH = 81;                                                // sixteen k, then four unused: no two of a half warp's in a bank, written or read
+    __shared__ double tile[32][PITCH], factor[80];
     const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32, b = blockIdx.z, tid = threadIdx.x;
     {
         const int blocks = (int)(pl.rows_pad / 128), all = (pl.K + I8_KCHUNK - 1) / I8_KCHUNK, pair = r0 / 256 * 2;
@@ -248,19 +282,14 @@ __global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const dou
         if ((k0 / 128 < lo / per || k0 / 128 >= (hi + per - 1) / per) && blockIdx.x > 0) return;      // (the first column of CTAs writes the scales)
     }
     const double *S = src + (long)b * stride;
-    double v[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int o = KCONTIG ? (tid >> 6) + 2 * i : tid & 31, c = KCONTIG ? tid & 63 : (tid >> 5) + 4 * i;       // row and k; neighbours run along memory
         const int r = r0 + o, k = k0 + c;
-        v[i] = (r < pl.rows && k < pl.K && !(skip_diagonal && k == r)) ? (KCONTIG ? S[(long)r * ld + k] : S[(long)k * ld + r]) * i8_inner(inner, b, k, pl.K) : 0.0;
+        const bool in = r < pl.rows && k < pl.K && !(skip_diagonal && k == r);
+        i8_fetch(&tile[o][c + (c >> 4) * 4], in ? S + (KCONTIG ? (long)r * ld + k : (long)k * ld + r) : S, in);
     }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int o = KCONTIG ? (tid >> 6) + 2 * i : tid & 31, c = KCONTIG ? tid & 63 : (tid >> 5) + 4 * i;
-        tile[o][c] = v[i];
-    }
-    __syncthreads();
+    if (inner.p && tid < 64) factor[tid + (tid >> 4) * 4] = i8_inner(inner, b, k0 + tid, pl.K);
     const int rr = tid >> 2, kk = (tid & 3) * 16, r = r0 + rr;
     const long row = (long)b * pl.rows_pad + r;
     const unsigned mb = r < pl.rows ? pl.maxbits[row] : 0u;
@@ -270,11 +299,14 @@ __global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const dou
         // (the product's sums count 2^-72: 2^-36 is folded in on either side)
         pl.scale[row] = finite ? i8_pow2(e - 36) : __longlong_as_double(0x7ff8000000000000ll);
     const double up = i8_pow2(min(56 - e, 1000));                           // e >= -900: at most 2^956, exact
+    i8_fetched();
+    __syncthreads();
     unsigned lo[16], hi[16];
     unsigned long long bits = 0ull;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-        const double x = finite ? tile[rr][kk + i] : 0.0;
+        double x = finite ? tile[rr][(tid & 3) * 20 + i] : 0.0;
+        if (inner.p) x *= factor[(tid & 3) * 20 + i];
         // 56-bit integer, then balanced base-256 digits: adding 128 to every digit and flipping the top bits back
         const long long f = __double2ll_rn(x * up);
         bits |= (unsigned long long)f;
@@ -286,22 +318,18 @@ __global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const dou
     if ((tid & 3) == 0 && bits) atomicOr(pl.bits + row, bits);
     const long plane_bytes = pl.plane_rows * pl.k_pad;
     int8_t *dst = pl.planes + ((long)(k0 / 128) * pl.plane_rows + row) * 128 + (k0 & 64) + kk;
-#pragma unroll 4
+#pragma unroll
     for (int d = 0; d < I8_MODULI; ++d, dst += plane_bytes) {
-        const int wl = (int)I8_TAB.digit_lo[d], wh = (int)I8_TAB.digit_hi[d];
-        const float p = I8_TAB.pf[d], inv = I8_TAB.invf[d];
+        const int wl = (int)I8_TAB.digit_lo[d], wh = (int)I8_TAB.digit_hi[d], lift = I8_TAB.lift[d];
+        const unsigned long long less_p = i8_twice(I8_TAB.less_p[d]), inv = i8_twice(I8_TAB.invf[d]), lifted = i8_twice(I8_TAB.lifted[d]);
         unsigned w[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             unsigned t[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                // x' mod p from its digits' residues, as their sum s added to the bits of 1.5 * 2^23 (raw = 1.5 * 2^23 + s, f = s); |s| <= 7 * 128 * 127 < 2^17, so s and the nearest
-                // multiple of p are found exactly in fp32 (s / p is off by 2^-13 at most, 1 / 2p from a tie) and |s - q p| <= p / 2
-                const float raw = __int_as_float(__dp4a((int)lo[4 * q + i], wl, __dp4a((int)hi[4 * q + i], wh, 0x4b400000))), f = raw - 12582912.0f;
-                const float k = fmaf(f, inv, 12582912.0f) - 12582912.0f;
-                t[i] = (unsigned)__float_as_int(fmaf(-k, p, raw));
-            }
+            for (int i = 0; i < 4; ++i) t[i] = (unsigned)__dp4a((int)lo[4 * q + i], wl, __dp4a((int)hi[4 * q + i], wh, lift));
+            i8_reduce_two(t[0], t[1], less_p, inv, lifted);
+            i8_reduce_two(t[2], t[3], less_p, inv, lifted);
             w[q] = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
         }
         *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);

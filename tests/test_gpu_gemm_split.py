@@ -233,3 +233,20 @@ def test_tiles_of_both_widths(g, columns, M, N, K):
             assert np.array_equal(product(g, x, y), x @ y)
     finally:
         g.gptq2d_internal_test_hook(9, 0)
+
+
+@pytest.mark.parametrize("M,K", [(32, 64), (33, 65), (70, 300)])
+def test_digits_at_the_ends_of_their_range(g, M, K):
+    # entries whose seven balanced base-256 digits are mostly -128, 127, 0 and +-1, where a residue is largest before it is reduced; the lowest
+    # digit 0 or -128, so 49 bits.  Against columns with a single one: sums of one term, multiples of 2^61 of the scaled product, so exact.
+    rng = np.random.default_rng(M + K)
+    digits = rng.choice([-128, -127, 127, 126, -1, 0, 1], size=(7, M, K))
+    digits[0] = rng.choice([0, -128], size=(M, K))
+    digits[6] = rng.choice([-126, 126, 0], size=(M, K))
+    digits[6, :, 0] = 126                                    # every row's scale is that of 56 bits
+    a = sum(digits[j].astype(np.int64) << (8 * j) for j in range(7)).astype(np.float64)
+    where = rng.integers(0, K, size=150)
+    b = np.zeros((K, 150))
+    b[where, np.arange(150)] = 1.0
+    assert np.array_equal(product(g, a, b), a[:, where])
+    assert np.array_equal(product(g, b.T.copy(), a.T.copy()), a[:, where].T)
