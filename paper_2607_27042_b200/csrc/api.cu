@@ -168,6 +168,8 @@ static int factor_pair(int m, int n, const double *A, long lda, const double *B,
     if (cudaEventRecord(hp->inputs_free, stream) != cudaSuccess ||
         cudaStreamWaitEvent(hp->copy, hp->inputs_free, 0) != cudaSuccess)
         return GPTQ2D_ERR_CUDA;
+    hp->look[0].beside = n;
+    hp->look[1].beside = m;
     int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, hp->look[0].spine ? &hp->look[0] : nullptr);
     int st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, hp->copy, hp->look[1].spine ? &hp->look[1] : nullptr);
     // join even if an enqueue failed, so that nothing of this call is left running behind the caller's stream

@@ -567,8 +567,8 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         return GPTQ2D_OK;
     };
     // the same update with the panels of block rows [K0, K1) at once (contraction over all their rows), on the int8 tensor
-    // cores: a rank-512 update of an 8192 x 8192 target runs at 63 TFLOP/s there, at 31.7 on the fp64 tensor path (rank 128:
-    // 29 against 24).  The panels are split once, by split_panels; both updates of an outer block read the same planes.
+    // cores, whose time at these ranks is in putting the sums together, whatever the rank: the higher, the cheaper.  The panels are
+    // split once, by split_panels; both updates of an outer block read the same planes.
     auto panel_planes = [&](int K0, int K1) -> I8Planes {
         const long k0 = (long)K0 * FB, k1 = (long)K1 * FB < k ? (long)K1 * FB : k;
         return i8_planes_at(i8_at, (int)k0, (int)(k1 - k0), 1);
@@ -593,14 +593,19 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         CK(e);
         return GPTQ2D_OK;
     };
-    constexpr int OUTER = 4;                 // block rows per outer block (512 rows)
-    // (orders below about 5 500 are a little faster with the one-level loop further down: 6.56 against 6.66 ms at 4096, two
-    // sides; from 6144 on the rank-512 updates win)
-    if (look && nblk >= 44) {
-        // Two-level right-looking factorisation.  The block rows are grouped four by four into outer blocks of 512
+    // Block rows per outer block.  More make the large updates cheaper and the steps inside a block, in fp64, dearer; 4 / 6 / 8 / 12
+    // measured, two sides of 8192: 19.75 / 18.94 / 19.09 / 19.37 ms, of 5000: 7.07 / 7.04 / 7.10 / 7.39, one of 8192: 11.8 / 11.8 / 11.9 / 12.3.
+    constexpr int OUTER = 6;
+    // Which loop.  With two levels less work is done, with one (below) less of it is in the chain of diagonal blocks; what the
+    // other side of the same call leaves idle decides between them.  Measured, one level against two, in ms: 4300 beside 4300 5.67 / 5.53, 4608
+    // beside 4608 6.32 / 5.88, 5000 beside 5000 7.88 / 7.04, beside 3750 6.27 / 6.00, beside 2500 5.65 / 5.68, 4400 beside 3300 4.88 / 5.04, 4608
+    // beside 64 4.31 / 4.52; from 44 block rows on two levels whatever is beside (6144 beside 64: the same).
+    const int beside = look ? std::min((look->beside + FB - 1) / FB, nblk) : 0;
+    if (look && (nblk >= 44 || (i8_room && 2 * nblk + beside >= 102))) {
+        // Two-level right-looking factorisation.  The block rows are grouped six by six into outer blocks of 768
         // rows.  Inside an outer block S the 128-row steps run as before (diag, panel, update of the outer block's
-        // own rows above the step), all on look->spine; the rows ABOVE the outer block receive the four panels in
-        // one update of rank 512: its first 512 rows (the next outer block, which the spine needs next) on the
+        // own rows above the step), all on look->spine; the rows ABOVE the outer block receive the six panels in
+        // one update of rank 768: its first 768 rows (the next outer block, which the spine needs next) on the
         // spine, the rest on `stream`, one outer block behind.  Event logic as in the one-level loop below, with
         // outer blocks in place of block rows: the large update of S+2 is the last one that touched the rows of S
         // before its own steps; the spine's update of the rows of S-1 and the large update of S+1 both write them.

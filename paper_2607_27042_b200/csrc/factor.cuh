@@ -10,6 +10,7 @@ namespace gptq2d {
 struct FactorLookahead {
     cudaStream_t spine;
     cudaEvent_t fork, join, panel, t2[2];
+    int beside;                              // order of the side that is factorised at the same time
 };
 
 // `planes`: with room for the residue planes of its large products (i8_gemm.cuh); without, all products are fp64 ones

@@ -158,3 +158,19 @@ def test_a_repeated_channel_is_a_zero_pivot(g, k, i, j):
         a = np.random.default_rng(seed).standard_normal((k, k))
         a[:, i] = a[:, j]
         assert g.gptq2d_factor_batched([dev(a)], [dev(np.eye(1))])[4].cpu().tolist() == [5, i, 0, 0]
+
+
+@pytest.mark.parametrize("m,n", [(4224, 4225), (4225, 4300), (5000, 3100), (4097, 5120)])
+def test_loops_with_one_and_two_levels_agree(g, m, n):
+    # both sides of the rule that chooses the loop by the orders of a call's two sides, last outer blocks of one to six block rows; against
+    # the calls with one basis, which take the loop with one level
+    torch.manual_seed(m)
+    A, B = (torch.randn(k, k, dtype=torch.float64, device="cuda") / (4 * k) ** 0.5 + torch.eye(k, dtype=torch.float64, device="cuda") for k in (m, n))
+    L, U, dL, dU, info = g.gptq2d_factor(A, B)
+    L1, _, dL1, _, i0 = g.gptq2d_factor(A, None, n=1)
+    _, U1, _, dU1, i1 = g.gptq2d_factor(None, B, m=1)
+    for i in (info, i0, i1):
+        g.check_info(i)
+    # two factorisations of a Gram of condition below 100 (singular values of the bases within 1/4 .. 2): k roundings of 2^-53 times that
+    for x, y, k in ((L, L1, m), (U, U1, n), (dL / dL1, torch.ones_like(dL), m), (dU / dU1, torch.ones_like(dU), n)):
+        assert float((x - y).abs().max()) <= k * 2.0 ** -53 * 100
