@@ -170,8 +170,14 @@ static int factor_pair(int m, int n, const double *A, long lda, const double *B,
         return GPTQ2D_ERR_CUDA;
     hp->look[0].beside = n;
     hp->look[1].beside = m;
-    int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, hp->look[0].spine ? &hp->look[0] : nullptr);
-    int st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, hp->copy, hp->look[1].spine ? &hp->look[1] : nullptr);
+    // The longer side first: it is the one that is waited for, and the host needs 0.1 ms for the launches of a side of order 500, 0.2 ms for one of
+    // 1100 (calls by themselves: 300 x 500 454 -> 397 us, 2048 x 2049 1850 -> 1640, 1100 x 4100 3965 -> 3780).
+    int st = GPTQ2D_OK, st2 = GPTQ2D_OK;
+    for (const int side : {n > m ? 1 : 0, n > m ? 0 : 1}) {
+        const FactorLookahead *look = hp->look[side].spine ? &hp->look[side] : nullptr;
+        if (side == 0) st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, look);
+        else st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, hp->copy, look);
+    }
     // join even if an enqueue failed, so that nothing of this call is left running behind the caller's stream
     if (cudaEventRecord(hp->copies_done, hp->copy) != cudaSuccess ||
         cudaStreamWaitEvent(stream, hp->copies_done, 0) != cudaSuccess)
