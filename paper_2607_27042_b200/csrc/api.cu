@@ -84,19 +84,24 @@ static HostPipe *host_pipe() {
         ok = ok && cudaEventCreateWithFlags(&hp.copies_done, cudaEventDisableTiming) == cudaSuccess;
         for (int sd = 0; ok && sd < 2; ++sd) {
             FactorLookahead &lk = hp.look[sd];
-            cudaEvent_t *ev[5] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1]};
+            cudaEvent_t *ev[6] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1], &lk.early_done};
             // highest priority: the one-CTA spine kernels must get an SM as soon as one is free, ahead of the
             // queued CTAs of the large updates
             int prio_lo = 0, prio_hi = 0;
             bool lok = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) == cudaSuccess &&
                        cudaStreamCreateWithPriority(&lk.spine, cudaStreamNonBlocking, prio_hi) == cudaSuccess;
-            for (int e = 0; lok && e < 5; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
+            for (int e = 0; lok && e < 6; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
             if (!lok) lk.spine = nullptr;        // the set-up then runs that side on one stream
         }
         hp.pool_ok = ok;
         for (int k = 0; hp.pool_ok && k < HostPipe::POOL; ++k)
             hp.pool_ok = cudaStreamCreateWithFlags(&hp.pool[k], cudaStreamNonBlocking) == cudaSuccess &&
                          cudaEventCreateWithFlags(&hp.pool_done[k], cudaEventDisableTiming) == cudaSuccess;
+        // (after all other streams)
+        for (int sd = 0; ok && sd < 2; ++sd) {
+            FactorLookahead &lk = hp.look[sd];
+            if (lk.spine && cudaStreamCreateWithFlags(&lk.early, cudaStreamNonBlocking) != cudaSuccess) lk.spine = nullptr;
+        }
         if (ok) { hp.write32 = reinterpret_cast<StreamWriteValue32Fn>(fn); hp.wait32 = reinterpret_cast<StreamWaitValue32Fn>(fnw); }
         (void)cudaGetLastError();
     }

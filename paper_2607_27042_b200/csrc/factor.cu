@@ -485,9 +485,9 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     const int nblk = (k + FB - 1) / FB;
     char *i8_at = static_cast<char *>(ws) + factor_side_workspace_bytes(k, false);
     const size_t i8_room = planes ? factor_i8_bytes(k) : 0;
-    // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream`, so one set of planes
-    // serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
-    auto product = [&](const GemmArgs &g, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
+    // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream` or on a stream that it is ordered with, so
+    // one set of planes serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
+    auto product = [&](const GemmArgs &g, cudaStream_t stream, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
         if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
             // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
@@ -516,7 +516,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         g.alpha = 1.0; g.beta = 0.0;
         g.A = M; g.lda = ldm; g.B = M; g.ldb = ldm;
         g.C = G; g.ldc = ld; g.batch = 1; g.lower_tiles_only = 1;
-        CK(product(g, true, true, true));      // a Cholesky basis has a dominant diagonal
+        CK(product(g, stream, true, true, true));      // a Cholesky basis has a dominant diagonal
     }
     const size_t diag_smem = CholBlock<128>::SMEM;
     CK(cudaFuncSetAttribute(factor_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem));
@@ -593,6 +593,56 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         CK(e);
         return GPTQ2D_OK;
     };
+    // X = P^{-1}: diagonal blocks are put in place by the factorisation; double the block size level by level.  A pair (s0, b), (s0 + b, b2) becomes one
+    // block: X21 = -X22 (P21 X11).  The last block of a level may be longer or shorter than b; where a level has an odd number
+    // of blocks, the last one joins the pair before it at once (carried up alone, the 4 rows left over at order 4100 met a
+    // block of 4096 columns: two products of one tile row and the longest contraction, 0.56 ms of 7.3).
+    auto join = [&](long s0, long b1, long b2, long cnt, long step, cudaStream_t s) -> int {     // cnt pairs, `step` rows apart
+        const long off11 = s0 * ld + s0, off21 = (s0 + b1) * ld + s0, off22 = (s0 + b1) * ld + (s0 + b1);
+        const long stride = step * (ld + 1);
+        GemmArgs g1{};   // T21 = P21 X11
+        g1.opA = OP_N; g1.opB = OP_N;
+        g1.M = (int)b2; g1.N = (int)b1; g1.K = (int)b1;
+        g1.alpha = 1.0; g1.beta = 0.0;
+        g1.A = G + off21; g1.lda = ld; g1.strideA = stride;
+        g1.B = X + off11; g1.ldb = ld; g1.strideB = stride;
+        g1.C = T + off21; g1.ldc = ld; g1.strideC = stride;
+        g1.batch = (int)cnt;
+        g1.b_lower = 1;  // X11 is lower triangular
+        // column j of P carries the scale of P[j][j], row j of X its inverse
+        I8Inner inner;
+        inner.p = p + s0; inner.stride = step;
+        CK(product(g1, s, false, false, true, inner));
+        GemmArgs g2{};   // X21 = -X22 T21
+        g2.opA = OP_N; g2.opB = OP_N;
+        g2.M = (int)b2; g2.N = (int)b1; g2.K = (int)b2;
+        g2.alpha = -1.0; g2.beta = 0.0;
+        g2.A = X + off22; g2.lda = ld; g2.strideA = stride;
+        g2.B = T + off21; g2.ldb = ld; g2.strideB = stride;
+        g2.C = X + off21; g2.ldc = ld; g2.strideC = stride;
+        g2.batch = (int)cnt;
+        g2.a_lower = 1;  // X22 is lower triangular
+        CK(product(g2, s, false, true, false));
+        return GPTQ2D_OK;
+    };
+    // the levels of the rows [r0, end) from blocks of b rows to blocks of `to` rows, nb blocks at first, the last one with whatever remains
+    auto levels = [&](long r0, long end, long nb, long b, long to, cudaStream_t s) -> int {
+        long last = end - r0 - (nb - 1) * b;
+        for (; nb > 1 && b < to; b *= 2) {
+            const bool odd = (nb & 1) != 0;
+            const long pairs = nb / 2;
+            // the second block of the last pair is the odd-sized one unless a single block follows
+            const long uniform = (odd || last == b) ? pairs : pairs - 1;
+            int st = GPTQ2D_OK;
+            if (uniform > 0) st = join(r0, b, b, uniform, 2 * b, s);
+            if (st == GPTQ2D_OK && uniform < pairs) st = join(r0 + (pairs - 1) * 2 * b, b, last, 1, 0, s);
+            if (st == GPTQ2D_OK && odd) st = join(r0 + (pairs - 1) * 2 * b, 2 * b, last, 1, 0, s);
+            if (st != GPTQ2D_OK) return st;
+            last = odd ? 2 * b + last : b + last;
+            nb = pairs;
+        }
+        return GPTQ2D_OK;
+    };
     // Block rows per outer block.  More make the large updates cheaper and the steps inside a block, in fp64, dearer; 4 / 6 / 8 / 12
     // measured, two sides of 8192: 19.75 / 18.94 / 19.09 / 19.37 ms, of 5000: 7.07 / 7.04 / 7.10 / 7.39, one of 8192: 11.8 / 11.8 / 11.9 / 12.3.
     constexpr int OUTER = 6;
@@ -601,7 +651,16 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     // beside 4608 6.32 / 5.88, 5000 beside 5000 7.88 / 7.04, beside 3750 6.27 / 6.00, beside 2500 5.65 / 5.68, 4400 beside 3300 4.88 / 5.04, 4608
     // beside 64 4.31 / 4.52; from 44 block rows on two levels whatever is beside (6144 beside 64: the same).
     const int beside = look ? std::min((look->beside + FB - 1) / FB, nblk) : 0;
-    if (look && (nblk >= 44 || (i8_room && 2 * nblk + beside >= 102))) {
+    const bool two_levels = look && (nblk >= 44 || (i8_room && 2 * nblk + beside >= 102));
+    // The inverse of the rows below the last doubling needs nothing of the rows above, which come last and leave most SMs idle: it is
+    // put together on a stream of its own beneath them: the joins up to 1024 rows took 0.5 of 3.77 ms at 1100 x 4100, now 3.46 in all; 600 x 1500
+    // 951 -> 906 us, 3000 x 3000 2.97 -> 2.90 ms.  (With two levels the planes that it takes are in use, and the SMs as well; below eight
+    // block rows there is one join to move.)
+    int nblk_top = nblk;                                        // blocks of the last level, two or three, of `top` rows
+    long top = FB;
+    for (; nblk_top > 3; nblk_top /= 2) top *= 2;
+    const bool halves = look && !two_levels && nblk >= 8;
+    if (two_levels) {
         // Two-level right-looking factorisation.  The block rows are grouped six by six into outer blocks of 768
         // rows.  Inside an outer block S the 128-row steps run as before (diag, panel, update of the outer block's
         // own rows above the step), all on look->spine; the rows ABOVE the outer block receive the six panels in
@@ -671,6 +730,10 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
                 if (K == 0) break;
                 if ((st = panel(K, sp)) != GPTQ2D_OK) return st;
                 CK(cudaEventRecord(look->panel, sp));
+                if (halves && K == top / FB) {
+                    CK(cudaStreamWaitEvent(look->early, look->panel, 0));
+                    if ((st = levels(top, k, nblk - K, FB, top, look->early)) != GPTQ2D_OK) return st;
+                }
                 if (K + 1 <= nblk - 1 && K + 1 >= 2) CK(cudaStreamWaitEvent(sp, look->t2[(K + 1) & 1], 0));
                 if ((st = trailing(K, (long)(K - 1) * FB, (long)K * FB, sp)) != GPTQ2D_OK) return st;
                 if (K >= 2) {
@@ -682,57 +745,17 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
             return GPTQ2D_OK;
         }();
         // join whatever happened above, so that nothing of this call runs on behind the caller's stream
-        const bool joined = cudaEventRecord(look->join, sp) == cudaSuccess &&
-                            cudaStreamWaitEvent(stream, look->join, 0) == cudaSuccess;
+        bool joined = cudaEventRecord(look->join, sp) == cudaSuccess &&
+                      cudaStreamWaitEvent(stream, look->join, 0) == cudaSuccess;
+        if (halves)
+            joined = cudaEventRecord(look->early_done, look->early) == cudaSuccess &&
+                     cudaStreamWaitEvent(stream, look->early_done, 0) == cudaSuccess && joined;
         if (st_spine != GPTQ2D_OK) return st_spine;
         if (!joined) return GPTQ2D_ERR_CUDA;
     }
-    // X = P^{-1}: diagonal blocks are in place; double the block size level by level.  A pair (s0, b), (s0 + b, b2) becomes one
-    // block: X21 = -X22 (P21 X11).  The last block of a level may be longer or shorter than b; where a level has an odd number
-    // of blocks, the last one joins the pair before it at once (carried up alone, the 4 rows left over at order 4100 met a
-    // block of 4096 columns: two products of one tile row and the longest contraction, 0.56 ms of 7.3).
-    auto join = [&](long s0, long b1, long b2, long cnt, long step) -> int {     // cnt pairs, `step` rows apart
-        const long off11 = s0 * ld + s0, off21 = (s0 + b1) * ld + s0, off22 = (s0 + b1) * ld + (s0 + b1);
-        const long stride = step * (ld + 1);
-        GemmArgs g1{};   // T21 = P21 X11
-        g1.opA = OP_N; g1.opB = OP_N;
-        g1.M = (int)b2; g1.N = (int)b1; g1.K = (int)b1;
-        g1.alpha = 1.0; g1.beta = 0.0;
-        g1.A = G + off21; g1.lda = ld; g1.strideA = stride;
-        g1.B = X + off11; g1.ldb = ld; g1.strideB = stride;
-        g1.C = T + off21; g1.ldc = ld; g1.strideC = stride;
-        g1.batch = (int)cnt;
-        g1.b_lower = 1;  // X11 is lower triangular
-        // column j of P carries the scale of P[j][j], row j of X its inverse
-        I8Inner inner;
-        inner.p = p + s0; inner.stride = step;
-        CK(product(g1, false, false, true, inner));
-        GemmArgs g2{};   // X21 = -X22 T21
-        g2.opA = OP_N; g2.opB = OP_N;
-        g2.M = (int)b2; g2.N = (int)b1; g2.K = (int)b2;
-        g2.alpha = -1.0; g2.beta = 0.0;
-        g2.A = X + off22; g2.lda = ld; g2.strideA = stride;
-        g2.B = T + off21; g2.ldb = ld; g2.strideB = stride;
-        g2.C = X + off21; g2.ldc = ld; g2.strideC = stride;
-        g2.batch = (int)cnt;
-        g2.a_lower = 1;  // X22 is lower triangular
-        CK(product(g2, false, true, false));
-        return GPTQ2D_OK;
-    };
-    long nb = nblk, last = k - (long)(nblk - 1) * FB;           // blocks of this level: nb - 1 of b rows and one of `last`
-    for (long b = FB; nb > 1; b *= 2) {
-        const bool odd = (nb & 1) != 0;
-        const long pairs = nb / 2;
-        // the second block of the last pair is the odd-sized one unless a single block follows
-        const long uniform = (odd || last == b) ? pairs : pairs - 1;
-        int st = GPTQ2D_OK;
-        if (uniform > 0) st = join(0, b, b, uniform, 2 * b);
-        if (st == GPTQ2D_OK && uniform < pairs) st = join((pairs - 1) * 2 * b, b, last, 1, 0);
-        if (st == GPTQ2D_OK && odd) st = join((pairs - 1) * 2 * b, 2 * b, last, 1, 0);
-        if (st != GPTQ2D_OK) return st;
-        last = odd ? 2 * b + last : b + last;
-        nb = pairs;
-    }
+    int st = halves ? levels(0, top, top / FB, FB, top, stream) : GPTQ2D_OK;
+    if (st == GPTQ2D_OK) st = halves ? levels(0, k, nblk_top, top, k, stream) : levels(0, k, nblk, FB, k, stream);
+    if (st != GPTQ2D_OK) return st;
     dim3 grid((k + 31) / 32, (k + 31) / 32);
     factor_finish_kernel<<<grid, 256, 0, stream>>>(X, ld, p, k, out, ldo, side, dinv);
     CK(cudaGetLastError());

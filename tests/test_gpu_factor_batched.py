@@ -174,3 +174,19 @@ def test_loops_with_one_and_two_levels_agree(g, m, n):
     # two factorisations of a Gram of condition below 100 (singular values of the bases within 1/4 .. 2): k roundings of 2^-53 times that
     for x, y, k in ((L, L1, m), (U, U1, n), (dL / dL1, torch.ones_like(dL), m), (dU / dU1, torch.ones_like(dU), n)):
         assert float((x - y).abs().max()) <= k * 2.0 ** -53 * 100
+
+
+@pytest.mark.parametrize("k", [897, 1024, 1025, 1500, 3000, 4100])
+def test_the_inverse_in_two_parts_is_bit_identical_to_the_one_in_one(g, k):
+    # eight block rows and more: the lower rows' inverse is put together beneath the factorisation of the upper ones; last levels of two blocks
+    # and of three, last blocks of one row, four and a whole one.  The same products as in the calls with one basis.
+    torch.manual_seed(k)
+    A, B = (torch.randn(j, j, dtype=torch.float64, device="cuda") / (4 * j) ** 0.5 + torch.eye(j, dtype=torch.float64, device="cuda") for j in (k, 200))
+    L1, _, dL1, _, i1 = g.gptq2d_factor(A, None, n=1)
+    _, U2, _, dU2, i2 = g.gptq2d_factor(None, A, m=1)
+    for _ in range(3):
+        L, _, dL, _, ia = g.gptq2d_factor(A, B)
+        _, U, _, dU, ib = g.gptq2d_factor(B, A)
+        for i in (i1, i2, ia, ib):
+            g.check_info(i)
+        assert torch.equal(L, L1) and torch.equal(dL, dL1) and torch.equal(U, U2) and torch.equal(dU, dU2)
