@@ -84,13 +84,13 @@ static HostPipe *host_pipe() {
         ok = ok && cudaEventCreateWithFlags(&hp.copies_done, cudaEventDisableTiming) == cudaSuccess;
         for (int sd = 0; ok && sd < 2; ++sd) {
             FactorLookahead &lk = hp.look[sd];
-            cudaEvent_t *ev[6] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1], &lk.early_done};
+            cudaEvent_t *ev[7] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1], &lk.left[0], &lk.left[1]};
             // highest priority: the one-CTA spine kernels must get an SM as soon as one is free, ahead of the
             // queued CTAs of the large updates
             int prio_lo = 0, prio_hi = 0;
             bool lok = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) == cudaSuccess &&
                        cudaStreamCreateWithPriority(&lk.spine, cudaStreamNonBlocking, prio_hi) == cudaSuccess;
-            for (int e = 0; lok && e < 6; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
+            for (int e = 0; lok && e < 7; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
             if (!lok) lk.spine = nullptr;        // the set-up then runs that side on one stream
         }
         hp.pool_ok = ok;
@@ -100,7 +100,8 @@ static HostPipe *host_pipe() {
         // (after all other streams)
         for (int sd = 0; ok && sd < 2; ++sd) {
             FactorLookahead &lk = hp.look[sd];
-            if (lk.spine && cudaStreamCreateWithFlags(&lk.early, cudaStreamNonBlocking) != cudaSuccess) lk.spine = nullptr;
+            for (cudaStream_t &e : lk.early)
+                if (lk.spine && cudaStreamCreateWithFlags(&e, cudaStreamNonBlocking) != cudaSuccess) lk.spine = nullptr;
         }
         if (ok) { hp.write32 = reinterpret_cast<StreamWriteValue32Fn>(fn); hp.wait32 = reinterpret_cast<StreamWaitValue32Fn>(fnw); }
         (void)cudaGetLastError();

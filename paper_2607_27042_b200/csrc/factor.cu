@@ -491,9 +491,9 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
         if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
             // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
-            // number of tiles)
+            // number of tiles); they also take the sums of a lower-triangular B in the better order
             const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
-            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && 2 * tiles <= device_sms();
+            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && (2 * tiles <= device_sms() || (g.b_lower && g.K <= 4 * FB));
             return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
         }
         const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);
@@ -594,41 +594,51 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         return GPTQ2D_OK;
     };
     // X = P^{-1}: diagonal blocks are put in place by the factorisation; double the block size level by level.  A pair (s0, b), (s0 + b, b2) becomes one
-    // block: X21 = -X22 (P21 X11).  The last block of a level may be longer or shorter than b; where a level has an odd number
+    // block: X21 = -(X22 P21) X11.  (In this order the first product waits for the lower rows only.  The error of the factors against 64 bits is 0.96 to
+    // 1.06 times that of X22 (P21 X11), 1.01 on average, over orders 260 to 4100 with plain and scaled channels.)  The last block of a level may be longer or shorter than b; where a level has an odd number
     // of blocks, the last one joins the pair before it at once (carried up alone, the 4 rows left over at order 4100 met a
     // block of 4096 columns: two products of one tile row and the longest contraction, 0.56 ms of 7.3).
-    auto join = [&](long s0, long b1, long b2, long cnt, long step, cudaStream_t s) -> int {     // cnt pairs, `step` rows apart
-        const long off11 = s0 * ld + s0, off21 = (s0 + b1) * ld + s0, off22 = (s0 + b1) * ld + (s0 + b1);
+    auto join_left = [&](long s0, long b1, long b2, long cnt, long step, cudaStream_t s) -> int {     // cnt pairs, `step` rows apart
+        const long off21 = (s0 + b1) * ld + s0, off22 = (s0 + b1) * ld + (s0 + b1);
         const long stride = step * (ld + 1);
-        GemmArgs g1{};   // T21 = P21 X11
-        g1.opA = OP_N; g1.opB = OP_N;
-        g1.M = (int)b2; g1.N = (int)b1; g1.K = (int)b1;
-        g1.alpha = 1.0; g1.beta = 0.0;
-        g1.A = G + off21; g1.lda = ld; g1.strideA = stride;
-        g1.B = X + off11; g1.ldb = ld; g1.strideB = stride;
-        g1.C = T + off21; g1.ldc = ld; g1.strideC = stride;
-        g1.batch = (int)cnt;
-        g1.b_lower = 1;  // X11 is lower triangular
-        // column j of P carries the scale of P[j][j], row j of X its inverse
-        I8Inner inner;
-        inner.p = p + s0; inner.stride = step;
-        CK(product(g1, s, false, false, true, inner));
-        GemmArgs g2{};   // X21 = -X22 T21
-        g2.opA = OP_N; g2.opB = OP_N;
-        g2.M = (int)b2; g2.N = (int)b1; g2.K = (int)b2;
-        g2.alpha = -1.0; g2.beta = 0.0;
-        g2.A = X + off22; g2.lda = ld; g2.strideA = stride;
-        g2.B = T + off21; g2.ldb = ld; g2.strideB = stride;
-        g2.C = X + off21; g2.ldc = ld; g2.strideC = stride;
-        g2.batch = (int)cnt;
-        g2.a_lower = 1;  // X22 is lower triangular
-        CK(product(g2, s, false, true, false));
+        GemmArgs g{};    // T21 = X22 P21
+        g.opA = OP_N; g.opB = OP_N;
+        g.M = (int)b2; g.N = (int)b1; g.K = (int)b2;
+        g.alpha = 1.0; g.beta = 0.0;
+        g.A = X + off22; g.lda = ld; g.strideA = stride;
+        g.B = G + off21; g.ldb = ld; g.strideB = stride;
+        g.C = T + off21; g.ldc = ld; g.strideC = stride;
+        g.batch = (int)cnt;
+        g.a_lower = 1;   // X22 is lower triangular
+        CK(product(g, s, false, true, false));
         return GPTQ2D_OK;
     };
-    // the levels of the rows [r0, end) from blocks of b rows to blocks of `to` rows, nb blocks at first, the last one with whatever remains
-    auto levels = [&](long r0, long end, long nb, long b, long to, cudaStream_t s) -> int {
+    auto join_right = [&](long s0, long b1, long b2, long cnt, long step, cudaStream_t s) -> int {
+        const long off11 = s0 * ld + s0, off21 = (s0 + b1) * ld + s0;
+        const long stride = step * (ld + 1);
+        GemmArgs g{};    // X21 = -T21 X11
+        g.opA = OP_N; g.opB = OP_N;
+        g.M = (int)b2; g.N = (int)b1; g.K = (int)b1;
+        g.alpha = -1.0; g.beta = 0.0;
+        g.A = T + off21; g.lda = ld; g.strideA = stride;
+        g.B = X + off11; g.ldb = ld; g.strideB = stride;
+        g.C = X + off21; g.ldc = ld; g.strideC = stride;
+        g.batch = (int)cnt;
+        g.b_lower = 1;   // X11 is lower triangular
+        // column j of P carries the scale of P[j][j], and so does that of T; row j of X its inverse
+        I8Inner inner;
+        inner.p = p + s0; inner.stride = step;
+        CK(product(g, s, false, false, true, inner));
+        return GPTQ2D_OK;
+    };
+    auto join = [&](long s0, long b1, long b2, long cnt, long step, cudaStream_t s) -> int {
+        const int st = join_left(s0, b1, b2, cnt, step, s);
+        return st != GPTQ2D_OK ? st : join_right(s0, b1, b2, cnt, step, s);
+    };
+    // the levels of the rows [r0, end) from blocks of b rows on, nb of them, the last one with whatever remains
+    auto levels = [&](long r0, long end, long nb, long b, cudaStream_t s) -> int {
         long last = end - r0 - (nb - 1) * b;
-        for (; nb > 1 && b < to; b *= 2) {
+        for (; nb > 1; b *= 2) {
             const bool odd = (nb & 1) != 0;
             const long pairs = nb / 2;
             // the second block of the last pair is the odd-sized one unless a single block follows
@@ -652,14 +662,19 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     // beside 64 4.31 / 4.52; from 44 block rows on two levels whatever is beside (6144 beside 64: the same).
     const int beside = look ? std::min((look->beside + FB - 1) / FB, nblk) : 0;
     const bool two_levels = look && (nblk >= 44 || (i8_room && 2 * nblk + beside >= 102));
-    // The inverse of the rows below the last doubling needs nothing of the rows above, which come last and leave most SMs idle: it is
-    // put together on a stream of its own beneath them: the joins up to 1024 rows took 0.5 of 3.77 ms at 1100 x 4100, now 3.46 in all; 600 x 1500
-    // 951 -> 906 us, 3000 x 3000 2.97 -> 2.90 ms.  (With two levels the planes that it takes are in use, and the SMs as well; below eight
-    // block rows there is one join to move.)
-    int nblk_top = nblk;                                        // blocks of the last level, two or three, of `top` rows
-    long top = FB;
-    for (; nblk_top > 3; nblk_top /= 2) top *= 2;
-    const bool halves = look && !two_levels && nblk >= 8;
+    // The inverse of the rows below the last doubling, and its product with the panels to the left of it, need nothing of the rows above, which come
+    // last and leave most SMs idle; so with the rows of the doubling before, and so on.  They are put together beneath the steps above, on two
+    // streams in turn, so that the levels of one part overlap the product of the one before; what is left for the end is one product a
+    // doubling.  All of it at the end, then the levels of the lowest part beneath, then every part with its product, then two streams: 1100 x 4100
+    // 3.77 / 3.46 / 3.41 / 3.23 ms, 2048 x 2049 1.62 / 1.60 / 1.47 / 1.46, 1000 x 3000 2.35 / 2.28 / 2.04 / 2.04, 600 x 1500 951 / 908 / 830 / 830 us.
+    // (With two levels the planes that these products take are in use, and the SMs as well; below eight block rows there is little to move.)
+    long top = 0;                                               // rows above the last doubling
+    const bool early = look && !two_levels && nblk >= 8;
+    if (early) {
+        int blocks = nblk;                                      // of the last level: two or three
+        for (top = FB; blocks > 3; blocks /= 2) top *= 2;
+        if (blocks == 3) top *= 2;
+    }
     if (two_levels) {
         // Two-level right-looking factorisation.  The block rows are grouped six by six into outer blocks of 768
         // rows.  Inside an outer block S the 128-row steps run as before (diag, panel, update of the outer block's
@@ -720,9 +735,11 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         // waits for the latter.  An event waited on takes its latest record at the time of the call, so two
         // alternating events tell the large updates of K+2 and K+1 apart.
         cudaStream_t sp = look->spine;
+        int parts = 0;                                          // of the inverse
         const int st_spine = [&]() -> int {
             CK(cudaEventRecord(look->fork, stream));
             CK(cudaStreamWaitEvent(sp, look->fork, 0));
+            long at = top, end = k;
             for (int K = nblk - 1; K >= 0; --K) {
                 if (K + 2 <= nblk - 1) CK(cudaStreamWaitEvent(sp, look->t2[(K + 2) & 1], 0));
                 int st = diag(K, sp);
@@ -730,9 +747,18 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
                 if (K == 0) break;
                 if ((st = panel(K, sp)) != GPTQ2D_OK) return st;
                 CK(cudaEventRecord(look->panel, sp));
-                if (halves && K == top / FB) {
-                    CK(cudaStreamWaitEvent(look->early, look->panel, 0));
-                    if ((st = levels(top, k, nblk - K, FB, top, look->early)) != GPTQ2D_OK) return st;
+                if (early && K == at / FB) {                    // rows [at, end) are final
+                    const int e = parts++ & 1;
+                    // what takes the planes goes one behind the other: the product with the panels, and the levels of 1024 rows and more
+                    const bool large = end - at >= 2048;
+                    CK(cudaStreamWaitEvent(look->early[e], look->panel, 0));
+                    if (parts > 1 && large) CK(cudaStreamWaitEvent(look->early[e], look->left[e ^ 1], 0));
+                    if ((st = levels(at, end, (end - at + FB - 1) / FB, FB, look->early[e])) != GPTQ2D_OK) return st;
+                    if (parts > 1 && !large) CK(cudaStreamWaitEvent(look->early[e], look->left[e ^ 1], 0));
+                    if ((st = join_left(0, at, end - at, 1, 0, look->early[e])) != GPTQ2D_OK) return st;
+                    CK(cudaEventRecord(look->left[e], look->early[e]));
+                    end = at;
+                    at /= 2;
                 }
                 if (K + 1 <= nblk - 1 && K + 1 >= 2) CK(cudaStreamWaitEvent(sp, look->t2[(K + 1) & 1], 0));
                 if ((st = trailing(K, (long)(K - 1) * FB, (long)K * FB, sp)) != GPTQ2D_OK) return st;
@@ -747,15 +773,21 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         // join whatever happened above, so that nothing of this call runs on behind the caller's stream
         bool joined = cudaEventRecord(look->join, sp) == cudaSuccess &&
                       cudaStreamWaitEvent(stream, look->join, 0) == cudaSuccess;
-        if (halves)
-            joined = cudaEventRecord(look->early_done, look->early) == cudaSuccess &&
-                     cudaStreamWaitEvent(stream, look->early_done, 0) == cudaSuccess && joined;
+        for (int e = 0; e < std::min(parts, 2); ++e)
+            joined = cudaEventRecord(look->left[e], look->early[e]) == cudaSuccess &&
+                     cudaStreamWaitEvent(stream, look->left[e], 0) == cudaSuccess && joined;
         if (st_spine != GPTQ2D_OK) return st_spine;
         if (!joined) return GPTQ2D_ERR_CUDA;
     }
-    int st = halves ? levels(0, top, top / FB, FB, top, stream) : GPTQ2D_OK;
-    if (st == GPTQ2D_OK) st = halves ? levels(0, k, nblk_top, top, k, stream) : levels(0, k, nblk, FB, k, stream);
-    if (st != GPTQ2D_OK) return st;
+    if (early) {
+        for (long b = FB; b <= top; b *= 2) {
+            const int st = join_right(0, b, (b == top ? k : 2 * b) - b, 1, 0, stream);
+            if (st != GPTQ2D_OK) return st;
+        }
+    } else {
+        const int st = levels(0, k, nblk, FB, stream);
+        if (st != GPTQ2D_OK) return st;
+    }
     dim3 grid((k + 31) / 32, (k + 31) / 32);
     factor_finish_kernel<<<grid, 256, 0, stream>>>(X, ld, p, k, out, ldo, side, dinv);
     CK(cudaGetLastError());

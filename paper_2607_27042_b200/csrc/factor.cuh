@@ -4,13 +4,13 @@
 
 namespace gptq2d {
 
-// Optional second and third stream and six events of the caller's.  With it the serial spine of the blocked
+// Optional further streams and events of the caller's.  With it the serial spine of the blocked
 // Cholesky (diagonal block, panel, and the update of the next block row) runs on `spine`, one block ahead
 // of the large trailing updates on the main stream.
 struct FactorLookahead {
     cudaStream_t spine;
-    cudaStream_t early;                      // the inverse of the lower rows, beneath the factorisation of the upper ones
-    cudaEvent_t fork, join, panel, t2[2], early_done;
+    cudaStream_t early[2];                   // the inverse of the lower rows, beneath the factorisation of the upper ones
+    cudaEvent_t fork, join, panel, t2[2], left[2];
     int beside;                              // order of the side that is factorised at the same time
 };
 
