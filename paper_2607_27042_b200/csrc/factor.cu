@@ -11,7 +11,7 @@
 //   panel GEMM   : P_K,0:K = W_KK^T G_K,0:K
 //   trailing GEMM: G_0:K,0:K -= P_K,0:K^T P_K,0:K           (lower tiles only)
 // then the triangular inverse X = P^{-1} by recursive doubling over diagonal blocks
-//   X21 = -X22 (P21 X11)      (strided-batched GEMMs, one batch entry per block pair)
+//   X21 = -(X22 P21) X11      (strided-batched GEMMs, one batch entry per block pair)
 // and a final column scaling (transposed on the way out for U).
 #include "common.cuh"
 #include "dmma_gemm.cuh"
@@ -493,7 +493,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
             // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
             // number of tiles); they also take the sums of a lower-triangular B in the better order
             const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
-            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && (2 * tiles <= device_sms() || (g.b_lower && g.K <= 4 * FB));
+            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && (2 * tiles <= device_sms() || g.b_lower);
             return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
         }
         const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);
