@@ -89,7 +89,7 @@ const char *gptq2d_status_string(int status);
  * dL (m) / dU (n), optional (NULL ok): 1/Lambda_L and 1/Lambda_U, so that
  * ||A (Z-X) B||_F^2 = sum_ij E_ij^2 dL_i dU_j for the local errors E.
  * A or B may be NULL, meaning the identity (L or U is then the identity).
- * From order 1024 on the Gram, the rank-512 updates and the larger products of the triangular inverse run on the int8 tensor cores,
+ * From order 1024 on the Gram, the rank-768 updates of large sides and the larger products of the triangular inverse run on the int8 tensor cores,
  * in fixed point 56 bits below the largest entry of a column of the basis or factor: errors relative to the norms of whole columns, below the
  * rounding of the factorisation itself.  A tile of the Gram or the inverse whose largest entries are below 1/512 of what its operand
  * rows could give is computed in fp64.
@@ -98,7 +98,7 @@ const char *gptq2d_status_string(int status);
  * Streams: everything is ordered after the work already on `stream`, and `stream` waits for all of it
  * before the call's outputs are used by later work on it.  With both bases given, part of the work runs
  * on streams of the library's own (per device, created on first use: the B side next to the A side, and
- * each side's chain of diagonal blocks ahead of its large updates); concurrent calls on one device are
+ * each side's chain of diagonal blocks ahead of its large updates and its inverse beneath them); concurrent calls on one device are
  * serialised while they enqueue.
  */
 size_t gptq2d_factor_workspace_bytes(int m, int n);

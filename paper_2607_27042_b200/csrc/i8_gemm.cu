@@ -21,7 +21,7 @@
 //
 // Bound, at K = 4096, by the loads of a stage (32 KB a CTA and 128 of k: 611 cycles against the 513 of the tensor pipe), then by power; at K = 512
 // by the reduction and by putting the entries together, some 45 thousand cycles of a tile each.  Measured, without the splitting, against
-// the 34 products of digits that stood here before: 8192^3 5.8 ms (189 TFLOP/s) against 12.5, 4096^3 0.86 against 1.38, 2048^3 0.126 against
+// the 34 products of digits that stood here before: 8192^3 5.7 ms (193 TFLOP/s) against 12.5, 4096^3 0.86 against 1.38, 2048^3 0.126 against
 // 0.208, rank-512 update of an 8192 x 8192 matrix 0.90 against 1.07.
 #include <cuda.h>
 #include "common.cuh"
