@@ -1071,19 +1071,6 @@ __global__ void __launch_bounds__(TILED_THREADS, 1) round_tiled_kernel(TiledKern
         // ================= B: the far part (every source tile of the contraction except the nearest)
         const TiledKernelParams &pk = VIEW(0);
         const int f_type = s_far[0], f_I = s_far[1], f_J = s_far[2], f_pos = s_far[3], f_nfar = s_far[4];
-        if (f_nfar == 0) {
-            // no sources: the cells start from zeros, or from what is there already
-            if (!((pk.preloaded >> f_type) & 1)) {
-                double *dst = tile_region();
-#pragma unroll 4
-                for (int k = tid; k < T * T / 2; k += TILED_THREADS)
-                    *reinterpret_cast<double2 *>(dst + CI((long)(k / (T / 2)) * pk.np + k % (T / 2) * 2, 127L * pk.np + T - 1, 200)) = double2{0.0, 0.0};
-            }
-            __syncthreads();
-            if (tid < TC) far_arrive(pk, f_I, f_J, tid);
-            if (tid == 0) s_has = 0;
-            continue;
-        }
         if (fresh) {
             if ((pk.preloaded >> f_type) & 1) load_acc(acc, tile_region(), pk.np, wm, wn, g, t);
             else acc.zero();
