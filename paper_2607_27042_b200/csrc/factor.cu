@@ -36,33 +36,34 @@ struct CholBlock {
     static __device__ __forceinline__ double inverse(const double *a, int i, int j) { return i > j ? a[j * LD + i] : a[NP * LD + i]; }
 };
 
-// 1 / sqrt(d) and 1 / d to the last bit or two.  NORMAL: by the approximations of the hardware (1e-6 off at most; zeros for subnormal numbers) and a
-// step of third order, then for the root a Newton step.  On a dependent chain 1 / d takes 41 cycles, 1 / sqrt(d) 73 (91 with rsqrt()).
-template <bool NORMAL>
-__device__ __forceinline__ double chol_rsqrt(double d) {
-    double r;
-    if (NORMAL) {
-        asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
-        const double e = fma(-(d * r), r, 1.0);
-        r = fma(r * e, fma(0.375, e, 0.5), r);
-    } else {
-        r = rsqrt(d);
-    }
-    return r * fma(-0.5 * d, r * r, 1.5);
-}
+// 1 / d.  NORMAL: by two steps of the Newton-Raphson iteration r <- r + r (1 - d r), each of which squares the relative error,
+// 1 - d r' = (1 - d r)^2, from the approximation that the hardware has an instruction for (good to 20 bits or so, zero for subnormal numbers):
+// half a unit in the last place, from 2^-960 to 2^900.  It is on the chain of the pivots, where the function takes longer (set-up 300 x 500
+// 402 against 425 us, 2048 x 2049 1560 against 1670, 128 pairs of order 96 81 against 84).
 template <bool NORMAL>
 __device__ __forceinline__ double chol_rcp(double d) {
     if (!NORMAL) return 1.0 / d;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(r) : "d"(d));
-    const double e = fma(-d, r, 1.0);
-    return fma(r, fma(e, e, e), r);
+    r = fma(r, fma(-d, r, 1.0), r);
+    return fma(r, fma(-d, r, 1.0), r);
+}
+// x / d from rc = 1 / d, corrected by its remainder (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990):
+// 1 where the two are the same
+__device__ __forceinline__ double chol_quotient(double x, double d, double rc) {
+    const double m = x * rc;
+    return fma(fma(-m, d, x), rc, m);
+}
+// 1 / sqrt(d): the function, then a Newton-Raphson step for r^-2 = d
+__device__ __forceinline__ double chol_rsqrt(double d) {
+    const double r = rsqrt(d);
+    return r * fma(-0.5 * d, r * r, 1.5);
 }
 
 // The 16 x 16 block at r, r of a, by one warp: elimination in [S_RR | I], last row first, column j of either in lanes j and 16 + j.  The block's lower
 // triangle becomes P_RR, above it comes W_RR = P_RR^{-1}, transposed, and V holds P_RR^{-T}.  Returns the largest index of a pivot that was not positive,
 // -1 if there is none.  NORMAL: no pivot is near an end of the range.
-// The chain is 57 cycles a pivot (inverse 41, multiply 8, multiply-add 8): pivots follow from each other as in an L D L^T factorisation, the roots
+// The chain is some 65 cycles a pivot (inverse, multiply, multiply-add): pivots follow from each other as in an L D L^T factorisation, the roots
 // are taken behind them, each in a lane of its own, and a row goes to all lanes through shared memory while its pivot is inverted; with the issue of some thirty fp64 operations a
 // pivot takes 130 cycles (by shuffles, with the root on the chain, 185; in a loop over two times eight rows 260, inlined into its caller 330).
 template <int NP, bool NORMAL>
@@ -94,14 +95,13 @@ __device__ __noinline__ int chol_block(int r) {
         // the next pivot, in every lane; a repeated channel (p = before = d) leaves zero, not a rounding error of either sign
         const bool same = p == d && before == d;
         const double pn = same ? 0.0 : p, next = fma(-(pn * rc), pn, same ? 0.0 : before);
-        double m = x[kk] * rc;
-        m = fma(fma(-m, d, x[kk]), rc, m);                      // x[kk] / d, rounded as a division is (1 where they are the same)
+        const double m = chol_quotient(x[kk], d, rc);
 #pragma unroll
         for (int i = kk - 1; i >= 0; --i) x[i] = fma(-((i & 1) ? y[i / 2].y : y[i / 2].x), m, x[i]);
         d = next;
     }
     // the roots, all at once
-    const double root = chol_rsqrt<NORMAL>(mine);
+    const double root = chol_rsqrt(mine);
     if (lane < 16) inv[j] = root;
     __syncwarp();
 #pragma unroll
@@ -422,6 +422,20 @@ __global__ void __launch_bounds__(256, NP == 64 ? 4 : (NP == 96 ? 2 : 1)) factor
     }
     if (q.dinv)
         for (int j = tid; j < k; j += blockDim.x) q.dinv[j] = a[j * LD + j] * a[j * LD + j];
+}
+
+// the functions above by themselves, for tests
+__global__ void chol_division_kernel(int n, const double *x, const double *d, double *rcp, double *quotient, double *root) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double r = chol_rcp<true>(d[i]);
+    rcp[i] = r;
+    quotient[i] = chol_quotient(x[i], d[i], r);
+    root[i] = chol_rsqrt(d[i]);
+}
+int launch_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, double *root, cudaStream_t stream) {
+    chol_division_kernel<<<(n + 255) / 256, 256, 0, stream>>>(n, x, d, rcp, quotient, root);
+    return cudaGetLastError() == cudaSuccess ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
 }
 
 int factor_small_class(int k) { return k <= 64 ? 0 : (k <= 96 ? 1 : 2); }
