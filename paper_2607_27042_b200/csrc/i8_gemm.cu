@@ -6,7 +6,8 @@
 // coprime numbers p_i <= 256 whose product P exceeds 2^125.3.  A residue of S is the residue of one int8 product of the residues
 // of a' and b', exact in int32: sixteen int8 products, where the signed base-256 digits that stood here before took 34
 // for the same 56 bits.  S / P is the fractional part of sum_i (S mod p_i) u_i / p_i with u_i = (P / p_i)^-1 mod p_i; it is summed in 80-bit fixed
-// point (the weights cut at 2^-80: S is off by 2^53 or so and at most 2^57, 2^-57 of the largest term, sixteen times less than what the 56 bits round off) and multiplied by P.  What the 56 bits round
+// point (the weights cut at 2^-80: S is off by 2^52 or so and at most 2^57, where rounding the operands to integers moves a sum by 2^54 sqrt(K / 6) if all
+// entries are as large as the largest) and multiplied by P with one rounding.  What the 56 bits round
 // off is of the order 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
 // entries: 4e-16 against 3e-15 of the fp64 tensor path).  Rows whose integers end in zero bits (integers, fp32 data) give an S that
 // ends in as many: it is rounded there, which makes such products exact.
@@ -598,17 +599,15 @@ __device__ __forceinline__ void i8_from_residues(double (&v)[4], const unsigned 
 #pragma unroll
             for (int g = 0; g < I8_MODULI / 4; ++g) d[b] = __dp4a(r[j][g], I8_TAB.weight[b][g], d[b]);
         }
-        // the sum modulo 2^80, as a signed number: hi 2^64 + mid 2^32 + lo
+        // the sum modulo 2^80, as a signed number: the last 16 bits of x2, 32 of x1, 32 of x0
         const unsigned long long x0 = (unsigned long long)(d[0] + (d[1] << 8)) + ((unsigned long long)(d[2] + (d[3] << 8)) << 16);
         const unsigned long long x1 = (unsigned long long)(d[4] + (d[5] << 8)) + ((unsigned long long)(d[6] + (d[7] << 8)) << 16) + (x0 >> 32);
         const unsigned x2 = d[8] + (d[9] << 8) + (unsigned)(x1 >> 32);
-        const int hi = (int)(x2 << 16) >> 16;
-        // (an unsigned number x as the low word of 2^52 + x)
+        // (the low word of 2^52 + x; the upper 48 bits, with 2^47 added, as those of 2^84 + 2^32 x: both exact, so that the product with P is rounded
+        // once, as a sum in fp64 would be)
         const double fl = __hiloint2double(0x43300000, (int)(unsigned)x0) - 4503599627370496.0;
-        const double fm = __hiloint2double(0x43300000, (int)(unsigned)x1) - 4503599627370496.0;
-        const double fh = __hiloint2double(0x43300000, hi ^ 0x80000000) - 4503601774854144.0;
-        const double s = fma(fh, 18446744073709551616.0, fma(fm, 4294967296.0, fl));
-        v[j] = fma(s, I8_TAB.product_hi, s * I8_TAB.product_lo);
+        const double up = __hiloint2double((int)(((x2 ^ 0x8000u) & 0xffffu) | 0x45300000u), (int)(unsigned)x1) - (0x1p84 + 0x1p79);
+        v[j] = fma(up, I8_TAB.product_hi, fma(up, I8_TAB.product_lo, fl * I8_TAB.product_hi));
     }
 }
 __device__ __forceinline__ void i8_load4(double (&v)[4], const double *src) {

@@ -250,3 +250,20 @@ def test_digits_at_the_ends_of_their_range(g, M, K):
     b[where, np.arange(150)] = 1.0
     assert np.array_equal(product(g, a, b), a[:, where])
     assert np.array_equal(product(g, b.T.copy(), a.T.copy()), a[:, where].T)
+
+
+@pytest.mark.parametrize("columns", [128, 256])
+def test_a_sum_is_rounded_once(g, columns):
+    # multiples of 2^-53 below 1/2 lose nothing as integers, so what is left is putting the sums together: one rounding, not two (1.41)
+    rng = np.random.default_rng(columns)
+    M, N, K = 300, 260, 700
+    a, b = rng.uniform(-0.5, 0.5, (M, K)), rng.uniform(-0.5, 0.5, (K, N))
+    want = a.astype(np.longdouble) @ b.astype(np.longdouble)
+    g.gptq2d_internal_test_hook(9, columns)
+    try:
+        got = product(g, a, b)
+    finally:
+        g.gptq2d_internal_test_hook(9, 0)
+    once = np.linalg.norm((want.astype(np.float64) - want).astype(np.float64))
+    # (the weights' 80 bits and 2^-64 sqrt(K) of the reference are a hundredth of it)
+    assert np.linalg.norm((got - want).astype(np.float64)) <= 1.05 * once
