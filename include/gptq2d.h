@@ -368,9 +368,9 @@ int gptq2d_internal_gemm_split(int transa, int transb, int M, int N, int K, doub
                                const double *A, long lda, const double *B, long ldb,
                                double beta, double *C, long ldc,
                                void *workspace, size_t workspace_bytes, int *info, void *stream);
-/* rcp[i] = 1 / d[i], quotient[i] = x[i] / d[i], root[i] = 1 / sqrt(d[i]) in the library's own arithmetic for the pivots of a diagonal block of the
+/* rcp[i] = 1 / d[i], quotient[i] = x[i] / d[i] in the library's own arithmetic for the pivots of a diagonal block of the
  * set-up (d from 2^-960 to 2^900).  Device arrays of n values.  Exposed for tests. */
-int gptq2d_internal_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, double *root, void *stream);
+int gptq2d_internal_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, void *stream);
 
 #ifdef __cplusplus
 }

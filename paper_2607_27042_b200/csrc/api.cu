@@ -613,11 +613,11 @@ int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alp
     return launch_gemm(g, static_cast<cudaStream_t>(stream_)) == cudaSuccess ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
 }
 
-int gptq2d_internal_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, double *root, void *stream_) {
-    if (n < 1 || !x || !d || !rcp || !quotient || !root) return GPTQ2D_ERR_INVALID_ARG;
-    if (!aligned(x, 8) || !aligned(d, 8) || !aligned(rcp, 8) || !aligned(quotient, 8) || !aligned(root, 8)) return GPTQ2D_ERR_INVALID_ARG;
+int gptq2d_internal_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, void *stream_) {
+    if (n < 1 || !x || !d || !rcp || !quotient) return GPTQ2D_ERR_INVALID_ARG;
+    if (!aligned(x, 8) || !aligned(d, 8) || !aligned(rcp, 8) || !aligned(quotient, 8)) return GPTQ2D_ERR_INVALID_ARG;
     const int st = check_device();
-    return st != GPTQ2D_OK ? st : launch_chol_division(n, x, d, rcp, quotient, root, static_cast<cudaStream_t>(stream_));
+    return st != GPTQ2D_OK ? st : launch_chol_division(n, x, d, rcp, quotient, static_cast<cudaStream_t>(stream_));
 }
 
 size_t gptq2d_internal_gemm_split_workspace_bytes(int M, int N, int K) {

@@ -54,11 +54,6 @@ __device__ __forceinline__ double chol_quotient(double x, double d, double rc) {
     const double m = x * rc;
     return fma(fma(-m, d, x), rc, m);
 }
-// 1 / sqrt(d): the function, then a Newton-Raphson step for r^-2 = d
-__device__ __forceinline__ double chol_rsqrt(double d) {
-    const double r = rsqrt(d);
-    return r * fma(-0.5 * d, r * r, 1.5);
-}
 
 // The 16 x 16 block at r, r of a, by one warp: elimination in [S_RR | I], last row first, column j of either in lanes j and 16 + j.  The block's lower
 // triangle becomes P_RR, above it comes W_RR = P_RR^{-1}, transposed, and V holds P_RR^{-T}.  Returns the largest index of a pivot that was not positive,
@@ -101,7 +96,7 @@ __device__ __noinline__ int chol_block(int r) {
         d = next;
     }
     // the roots, all at once
-    const double root = chol_rsqrt(mine);
+    const double root = rsqrt(mine);
     if (lane < 16) inv[j] = root;
     __syncwarp();
 #pragma unroll
@@ -425,16 +420,15 @@ __global__ void __launch_bounds__(256, NP == 64 ? 4 : (NP == 96 ? 2 : 1)) factor
 }
 
 // the functions above by themselves, for tests
-__global__ void chol_division_kernel(int n, const double *x, const double *d, double *rcp, double *quotient, double *root) {
+__global__ void chol_division_kernel(int n, const double *x, const double *d, double *rcp, double *quotient) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double r = chol_rcp<true>(d[i]);
     rcp[i] = r;
     quotient[i] = chol_quotient(x[i], d[i], r);
-    root[i] = chol_rsqrt(d[i]);
 }
-int launch_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, double *root, cudaStream_t stream) {
-    chol_division_kernel<<<(n + 255) / 256, 256, 0, stream>>>(n, x, d, rcp, quotient, root);
+int launch_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, cudaStream_t stream) {
+    chol_division_kernel<<<(n + 255) / 256, 256, 0, stream>>>(n, x, d, rcp, quotient);
     return cudaGetLastError() == cudaSuccess ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
 }
 

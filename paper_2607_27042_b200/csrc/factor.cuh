@@ -33,7 +33,7 @@ struct FactorSmallSide {
 int factor_small_class(int k);
 // dev_sides: device array of descriptors, those of class 0 first, then class 1, then class 2
 int launch_factor_small(const int (&counts)[3], const FactorSmallSide *dev_sides, int *info, cudaStream_t stream);
-// rcp = 1 / d, quotient = x / d, root = 1 / sqrt(d) as the elimination of a diagonal block computes them (tests)
-int launch_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, double *root, cudaStream_t stream);
+// rcp = 1 / d, quotient = x / d as the elimination of a diagonal block computes them (tests)
+int launch_chol_division(int n, const double *x, const double *d, double *rcp, double *quotient, cudaStream_t stream);
 
 }  // namespace gptq2d

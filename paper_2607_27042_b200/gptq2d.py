@@ -111,7 +111,7 @@ def _load():
     lib.gptq2d_internal_gemm_split.argtypes = [i32, i32, i32, i32, i32, c.c_double, vp, lng, vp, lng, c.c_double, vp, lng,
                                                vp, sz, vp, vp]
     lib.gptq2d_internal_chol_division.restype = i32
-    lib.gptq2d_internal_chol_division.argtypes = [i32, vp, vp, vp, vp, vp, vp]
+    lib.gptq2d_internal_chol_division.argtypes = [i32, vp, vp, vp, vp, vp]
     lib.gptq2d_internal_test_hook.restype = i32
     lib.gptq2d_internal_test_hook.argtypes = [i32, lng]
     lib.gptq2d_round_static_max_dim.restype = sz
@@ -464,8 +464,8 @@ def gptq2d_internal_gemm_split(A, B, C, transa=False, transb=False, alpha=1.0, b
 
 
 def gptq2d_internal_chol_division(x, d, stream=None):
-    """(1 / d, x / d, 1 / sqrt(d)) as the set-up computes them for the pivots of a diagonal block (1-D contiguous CUDA float64 tensors)."""
-    out = [torch.empty_like(d) for _ in range(3)]
+    """(1 / d, x / d) as the set-up computes them for the pivots of a diagonal block (1-D contiguous CUDA float64 tensors)."""
+    out = [torch.empty_like(d) for _ in range(2)]
     st = _lib.gptq2d_internal_chol_division(d.numel(), _ptr(x), _ptr(d), *[_ptr(t) for t in out], _stream_ptr(stream))
     if st != OK:
         raise Gptq2dError(st)

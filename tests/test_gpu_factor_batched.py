@@ -192,7 +192,7 @@ def test_the_inverse_in_two_parts_is_bit_identical_to_the_one_in_one(g, k):
         assert torch.equal(L, L1) and torch.equal(dL, dL1) and torch.equal(U, U2) and torch.equal(dU, dU2)
 
 
-def test_reciprocals_quotients_and_roots_of_the_pivots(g):
+def test_reciprocals_and_quotients_of_the_pivots(g):
     # d over the whole range in which the approximate inverse is taken, significands next to powers of two among them; x up to 2 d
     rng = np.random.default_rng(0)
     n = 200000
@@ -202,7 +202,7 @@ def test_reciprocals_quotients_and_roots_of_the_pivots(g):
     d = np.ldexp(significands, e)
     x = np.ldexp(rng.uniform(-2.0, 2.0, d.size), np.maximum(e + rng.integers(-40, 1, size=d.size), -960))
     x[::7] = d[::7]
-    rcp, quotient, root = (t.cpu().numpy() for t in g.gptq2d_internal_chol_division(dev(x), dev(d)))
+    rcp, quotient = (t.cpu().numpy() for t in g.gptq2d_internal_chol_division(dev(x), dev(d)))
     w = np.longdouble
     dw, u = d.astype(w), 2.0 ** -53
 
@@ -212,7 +212,5 @@ def test_reciprocals_quotients_and_roots_of_the_pivots(g):
     assert off(rcp, 1 / dw) <= 1.001 * u
     some = x != 0.0
     assert off(quotient[some], (x.astype(w) / dw)[some]) <= 1.001 * u and np.all(quotient[::7] == 1.0)
-    # three roundings: of r r, which counts half, of 1.5 - d r r / 2, which is next to one, and of the product
-    assert off(root, 1 / np.sqrt(dw)) <= 2.5 * u
-    # and the functions they stand for
-    assert np.max(np.abs(rcp * d - 1.0)) <= 2 * u and np.max(np.abs(quotient - x / d) - 2 * u * np.abs(x / d)) <= 0.0
+    # next to a division: a neighbour at most
+    assert np.max(np.abs(rcp * d - 1.0)) <= 2 * u and np.all(np.abs(quotient - x / d) <= 2 * u * np.abs(x / d))
