@@ -142,28 +142,9 @@ def workload(index, seed):
     return X, A, B, W.CONFIG_NAMES[index]
 
 
-def pieces_between_blocks(m, n):
-    """Launches of the int8 product in a sweep in blocks: the residue planes of a product, 16 bytes an operand entry, lie in 256 MB of their
-    own or in free rows of the workspace, where k is cut (round_tiled.cu)."""
-    up = lambda v: -(-v // 128) * 128
-    m0, n0 = (-(-m // 128) + 1) // 2 * 128, (-(-n // 128) + 1) // 2 * 128
-    m1, n1 = m - m0, n - n0
-    own = 16 * max((m0 + n0) * n0, (m0 + n0) * m0) <= 256 << 20
-    above, below = (256 << 20,) * 2 if own else (m0 * up(n) * 8, (up(m) - m0) * up(n) * 8)
-    total = 0
-    for rows, cols, k, room in ((m1, n0, m0, below), (m0, n1, n0, below), (m1, n1, m0, above), (m1, n1, n0, above)):
-        pieces = next(p for p in range(1, 17) if 16 * (up(rows) + up(cols)) * up(-(-k // p)) <= room)
-        total += -(-k // up(-(-k // pieces)))
-    return total
-
-
 def flops_between_blocks(g, m, n):
     """Flops of the products between the four blocks of a resident fp64 sweep, 0 if the library sweeps it whole."""
-    size = g.gptq2d_round_workspace_bytes(m, n)
-    g.gptq2d_internal_test_hook(7, 1 << 30)
-    whole = g.gptq2d_round_workspace_bytes(m, n)
-    g.gptq2d_internal_test_hook(7, 0)
-    if size == whole:
+    if not g.gptq2d_internal_round_products(m, n, g.gptq2d_round_workspace_bytes(m, n)):
         return 0.0
     m0, n0 = ((-(-k // 128) + 1) // 2 * 128 for k in (m, n))
     m1, n1 = m - m0, n - n0
@@ -292,7 +273,7 @@ def run_cuda(args):
     if flops_i8:
         # four blocks: three sweeps, descriptors, status; four products, a large one in pieces of k (each: scaling along k, two splitting
         # kernels an operand, the product)
-        kernel_name, launches = "round_tiled_kernel in 2x2 blocks + i8_gemm_kernel", 3 + 2 + pieces_between_blocks(m, n) * (1 + 2 * 2 + 1)
+        kernel_name, launches = "round_tiled_kernel in 2x2 blocks + i8_gemm_kernel", 3 + 2 + 6 * g.gptq2d_internal_round_products(m, n, g.gptq2d_round_workspace_bytes(m, n))
     traffic = None
     tp = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(tp):

@@ -351,6 +351,10 @@ int gptq2d_objective(int m, int n,
  */
 int gptq2d_internal_test_hook(int key, long value);
 
+/* Products on the int8 tensor cores that a resident GPTQ2D_FP64 sweep of an m x n matrix with a workspace of this size runs between its blocks
+ * (four, a large one in several pieces); 0: the matrix is swept whole.  Needs no GPU. */
+int gptq2d_internal_round_products(int m, int n, size_t workspace_bytes);
+
 /* The library's own fp64 product, exposed for tests and for measuring the fp64 tensor rate it reaches
  * (the denominator the sweep's roofline is quoted against): C = alpha op(A) op(B) + beta C, row-major,
  * op(A) M x K (stored K x M if transa), op(B) K x N (stored N x K if transb).  Device pointers, 8-byte

@@ -600,6 +600,10 @@ int gptq2d_internal_test_hook(int key, long value) {
     return GPTQ2D_ERR_INVALID_ARG;
 }
 
+int gptq2d_internal_round_products(int m, int n, size_t workspace_bytes) {
+    return m < 1 || n < 1 ? 0 : round_split_products(m, n, workspace_bytes);
+}
+
 int gptq2d_internal_gemm(int transa, int transb, int M, int N, int K, double alpha, const double *A, long lda,
                          const double *B, long ldb, double beta, double *C, long ldc, void *stream_) {
     if (M < 1 || N < 1 || K < 1 || !A || !B || !C) return GPTQ2D_ERR_INVALID_ARG;

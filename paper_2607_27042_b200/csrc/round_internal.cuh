@@ -61,6 +61,8 @@ size_t round_tiled_min_workspace_bytes(int m, int n);
 // device array inside the workspace: for each row of 128 x 128 tiles, how many of its tiles are swept
 unsigned *round_tiled_rowdone(void *ws, int m, int n);
 int launch_round_tiled(const TiledParams &p, void *ws, size_t ws_bytes, cudaStream_t stream);
+// products on the int8 tensor cores in a resident sweep with this workspace; 0: it is not run in blocks
+int round_split_products(int m, int n, size_t ws_bytes);
 // from which smaller order on resident matrices are swept in 2 x 2 blocks (tests; 0: the default)
 void round_split_set_min(long order);
 // most bits of a cell index in a batched launch; larger matrices are swept by themselves (tests; 0: the default)

@@ -1526,10 +1526,9 @@ __global__ void split_status_kernel(const int *a, const int *b, const int *c, in
 }
 
 // C (M x N, padded to whole tiles, row pitch ldc) = A B on the int8 tensor cores; A: M x K row-major, B: K x N row-major.  The residue planes
-// of kparts pieces of k lie at `at` in turn, what goes with them at `rows`.
-static int split_product(int M, int N, int K, int kparts, const double *A, long lda, const double *B, long ldb, double *C, long ldc, void *at,
+// of `step` k at a time lie at `at`, what goes with them at `rows`.
+static int split_product(int M, int N, int K, int step, const double *A, long lda, const double *B, long ldb, double *C, long ldc, void *at,
                          char *rows, int *info, cudaStream_t stream) {
-    const int step = ((K + kparts - 1) / kparts + T - 1) / T * T;
     for (int k0 = 0; k0 < K; k0 += step) {
         const int kk = std::min(step, K - k0);
         const I8Planes pa = i8_planes_at(at, M, kk, 1, rows);
@@ -1552,30 +1551,53 @@ static int split_product(int M, int N, int K, int kparts, const double *A, long 
     return GPTQ2D_OK;
 }
 
-// pieces of k for which the planes of an M x K and a K x N operand fit in `room` bytes; 0: none of up to sixteen
-static int split_kparts(int M, int N, int K, size_t room) {
-    for (int p = 1; p <= 16; ++p) {
+// The k that a product takes at a time: K cut into as few equal pieces (whole tiles) as let the planes of an M x step and a step x N operand fit in
+// `room` bytes.  0: no piece does.
+static int split_step(int M, int N, int K, size_t room) {
+    for (int p = 1;; ++p) {
         const int step = ((K + p - 1) / p + T - 1) / T * T;
-        if (step <= I8_MAX_K && i8_residue_bytes(M, step, 1) + i8_residue_bytes(N, step, 1) <= room) return p;
+        if (step <= I8_MAX_K && i8_residue_bytes(M, step, 1) + i8_residue_bytes(N, step, 1) <= room) return step;
+        if (step == T) return 0;
     }
-    return 0;
+}
+
+// How a matrix is swept in blocks with a workspace of this size; step[0] = 0: it is not.
+struct SplitPlan {
+    SplitLayout l;
+    int step[4];                         // k at a time of L10 E00, C00 U01, L10 E01 and C10 U01
+};
+static SplitPlan split_plan(int m, int n, size_t ws_bytes) {
+    SplitPlan p{};
+    p.l = split_layout(m, n);
+    if (p.l.m0 == 0 || ws_bytes < p.l.total) return p;
+    const TiledLayout t = tiled_layout(m, n);
+    const long np = (long)t.ntn * T;
+    const int m0 = p.l.m0, n0 = p.l.n0, m1 = m - m0, n1 = n - n0;
+    // room for residue planes: their own, or first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
+    const size_t room0 = p.l.planes_off ? SPLIT_OWN_PLANES : (size_t)(t.ntm * T - m0) * np * sizeof(double);
+    const size_t room1 = p.l.planes_off ? SPLIT_OWN_PLANES : (size_t)m0 * np * sizeof(double);
+    const int step[4] = {split_step(m1, n0, m0, room0), split_step(m0, n1, n0, room0), split_step(m1, n1, m0, room1), split_step(m1, n1, n0, room1)};
+    if (!step[0] || !step[1] || !step[2] || !step[3]) return p;
+    for (int k = 0; k < 4; ++k) p.step[k] = step[k];
+    return p;
+}
+int round_split_products(int m, int n, size_t ws_bytes) {
+    const SplitPlan p = split_plan(m, n, ws_bytes);
+    int count = 0;
+    for (int k = 0; k < 4 && p.step[0]; ++k) count += ((k & 1 ? p.l.n0 : p.l.m0) + p.step[k] - 1) / p.step[k];
+    return count;
 }
 
 // -1: this matrix is not swept in blocks
 static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, cudaStream_t stream) {
-    const SplitLayout sl = split_layout(in.m, in.n);
-    if (sl.m0 == 0 || in.panels_ready || ws_bytes < sl.total || !tensor_map_encoder()) return -1;
+    const SplitPlan plan = split_plan(in.m, in.n, ws_bytes);
+    const SplitLayout &sl = plan.l;
+    if (plan.step[0] == 0 || in.panels_ready || !tensor_map_encoder()) return -1;
     const TiledLayout l = tiled_layout(in.m, in.n);
     char *w = static_cast<char *>(ws);
     const long np = (long)l.ntn * T;
     double *E = reinterpret_cast<double *>(w + l.e_off), *C = reinterpret_cast<double *>(w + l.c_off);
     const int m0 = sl.m0, n0 = sl.n0, m1 = in.m - m0, n1 = in.n - n0;
-    // room for residue planes: their own, or first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
-    const size_t room0 = sl.planes_off ? SPLIT_OWN_PLANES : (size_t)(l.ntm * T - m0) * np * sizeof(double);
-    const size_t room1 = sl.planes_off ? SPLIT_OWN_PLANES : (size_t)m0 * np * sizeof(double);
-    const int k10 = split_kparts(m1, n0, m0, room0), k01 = split_kparts(m0, n1, n0, room0);
-    const int k11 = split_kparts(m1, n1, m0, room1), k11r = split_kparts(m1, n1, n0, room1);
-    if (!k10 || !k01 || !k11 || !k11r) return -1;
     char *rows = w + sl.rows_off;
 
     int dev = 0, sms = 0;
@@ -1627,8 +1649,8 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
     int st = sweep_one(block(0, 0, 0, 0));
     void *const own = sl.planes_off ? w + sl.planes_off : nullptr;
     void *at = own ? own : E + (long)m0 * np;
-    if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, k10, in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, rows, in.info, stream);
-    if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, k01, C, np, in.U + n0, in.ldu, E + n0, np, at, rows, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, plan.step[0], in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, rows, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, plan.step[1], C, np, in.U + n0, in.ldu, E + n0, np, at, rows, in.info, stream);
     if (st != GPTQ2D_OK) return st;
     {
         TiledKernelParams a = block(0, 1, 1, 2), b = block(1, 0, 1, 1), p{};
@@ -1652,8 +1674,8 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
             return GPTQ2D_ERR_CUDA;
     }
     at = own ? own : C;
-    st = split_product(m1, n1, m0, k11, in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, rows, in.info, stream);
-    if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, k11r, C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, rows, in.info, stream);
+    st = split_product(m1, n1, m0, plan.step[2], in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, rows, in.info, stream);
+    if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, plan.step[3], C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, rows, in.info, stream);
     if (st == GPTQ2D_OK) st = sweep_one(block(1, 1, 2, 3));
     if (st != GPTQ2D_OK) return st;
     if (in.info) {

@@ -40,7 +40,7 @@ EXPORTS = (
     "gptq2d_factor_batched_workspace_bytes", "gptq2d_factor_batched",
     "gptq2d_internal_test_hook", "gptq2d_internal_gemm",
     "gptq2d_internal_gemm_split_workspace_bytes", "gptq2d_internal_gemm_split",
-    "gptq2d_internal_chol_division",
+    "gptq2d_internal_chol_division", "gptq2d_internal_round_products",
 )
 FACTOR_SMALL_MAX = 128
 
@@ -110,6 +110,8 @@ def _load():
     lib.gptq2d_internal_gemm_split.restype = i32
     lib.gptq2d_internal_gemm_split.argtypes = [i32, i32, i32, i32, i32, c.c_double, vp, lng, vp, lng, c.c_double, vp, lng,
                                                vp, sz, vp, vp]
+    lib.gptq2d_internal_round_products.restype = i32
+    lib.gptq2d_internal_round_products.argtypes = [i32, i32, sz]
     lib.gptq2d_internal_chol_division.restype = i32
     lib.gptq2d_internal_chol_division.argtypes = [i32, vp, vp, vp, vp, vp]
     lib.gptq2d_internal_test_hook.restype = i32
@@ -425,6 +427,11 @@ def gptq2d_internal_test_hook(key, value):
     st = _lib.gptq2d_internal_test_hook(int(key), int(value))
     if st != OK:
         raise Gptq2dError(st)
+
+
+def gptq2d_internal_round_products(m, n, workspace_bytes):
+    """Products that a resident fp64 sweep runs between its blocks, 0 if it is run whole (see the header)."""
+    return int(_lib.gptq2d_internal_round_products(int(m), int(n), int(workspace_bytes)))
 
 
 def gptq2d_internal_gemm(A, B, C, transa=False, transb=False, alpha=1.0, beta=0.0, stream=None):

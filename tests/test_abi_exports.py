@@ -150,3 +150,22 @@ def test_blocks_begin_at_32_rows_and_columns_of_tiles():
         assert extra(m, n) > 0, (m, n)
     for m, n in ((3968, 3968), (3968, 3969), (3968, 65536), (65536, 3968)):
         assert extra(m, n) == 0, (m, n)
+
+
+def test_long_matrices_are_swept_in_blocks_whatever_k_has_to_be_cut_into():
+    """Whether a resident sweep runs in blocks, and in how many products: at least four, and as few more as their planes need."""
+    from paper_2607_27042_b200 import gptq2d as g
+
+    def products(m, n, less=0):
+        return g.gptq2d_internal_round_products(m, n, g.gptq2d_round_workspace_bytes(m, n) - less)
+
+    assert products(4096, 4096) == 4 and products(8192, 8192) == 8                 # 134 MB of planes; 537 MB in 268 MB of free rows
+    assert products(3968, 3968) == 0 and products(5632, 65537) == 0
+    # planes of (2048 + k / 2) x k / 2 entries, 16 bytes each, in free rows of 2048 x k values of 8 bytes: two pieces of 2048 rows and one for
+    # every 2048 k / (4096 + k) of the longer side
+    for n in (16384, 30000, 48000, 58000, 65536):
+        half = -(-n // 256) * 128
+        want = 2 * 2 + 2 * -(-16 * (2048 + half) * half // (2048 * 2 * half * 8))
+        for m, k in ((4000, n), (n, 4000)):
+            assert want <= products(m, k) <= want + 2, (m, k, products(m, k), want)
+    assert products(65409, 65409) >= 8
