@@ -1187,7 +1187,7 @@ void round_split_set_min(long order) { g_split_min.store(order > 0 ? order : SPL
 constexpr size_t SPLIT_OWN_PLANES = (size_t)256 << 20;
 struct SplitLayout {
     int m0, n0;                          // rows / columns of the first block (multiples of T); 0: not split
-    size_t hdr_off[3], flags_off[4], desc_off, table_off, zero_off, rows_off, planes_off, total;      // planes_off 0: no room of their own
+    size_t hdr_off[3], flags_off[4], desc_off, table_off, zero_off, rows_off, planes_off, total;      // planes_off = total: no room of their own
 };
 
 static size_t split_flag_bytes(int m, int n) {
@@ -1216,8 +1216,8 @@ static SplitLayout split_layout(int m, int n) {
     l.rows_off = off;
     off += i8_rows_bytes(l.m0, 1) + i8_rows_bytes(l.n0, 1) + i8_inner_bytes(std::min(std::max(l.m0, l.n0), I8_MAX_K));
     const size_t planes = std::max(i8_residue_bytes(l.m0, l.n0, 1) + i8_residue_bytes(l.n0, l.n0, 1), i8_residue_bytes(l.m0, l.m0, 1) + i8_residue_bytes(l.n0, l.m0, 1));
-    if (planes <= SPLIT_OWN_PLANES) { l.planes_off = off; off += planes; }
-    l.total = off;
+    l.planes_off = off;
+    l.total = off + (planes <= SPLIT_OWN_PLANES ? planes : 0);
     return l;
 }
 
@@ -1561,21 +1561,29 @@ static int split_step(int M, int N, int K, size_t room) {
     }
 }
 
-// How a matrix is swept in blocks with a workspace of this size; step[0] = 0: it is not.
+// How a matrix is swept in blocks with a workspace of this size; step[0] = 0: it is not.  What has no room behind the bookkeeping lies in the free rows:
+// the planes, and with a workspace that ends there what goes with them, too, which for square matrices means a piece of k more.  ms, whole / bookkeeping
+// alone / planes in free rows / room for all: 3969 x 3969 6.86 / 6.83 / 6.53 / 6.20, 4096 x 4096 6.14 / 6.41 / 6.07 / 5.76, 4608 x 4608 8.37 / 8.50 /
+// 8.07 / 7.57, 5000 x 6000 13.8 / 12.2 / 12.1 / 12.1 (planes above 256 MB), 8192 x 8192 39.3 / 30.6 / 29.8 / 29.8: with the bookkeeping alone from
+// 37 tiles on, five more than with more room.
 struct SplitPlan {
     SplitLayout l;
+    bool own_rows, own_planes;
     int step[4];                         // k at a time of L10 E00, C00 U01, L10 E01 and C10 U01
 };
 static SplitPlan split_plan(int m, int n, size_t ws_bytes) {
     SplitPlan p{};
     p.l = split_layout(m, n);
-    if (p.l.m0 == 0 || ws_bytes < p.l.total) return p;
+    if (p.l.m0 == 0 || ws_bytes < (std::min(m, n) < g_split_min.load() + 5 * T ? p.l.planes_off : p.l.rows_off)) return p;
+    p.own_rows = ws_bytes >= p.l.planes_off;
+    p.own_planes = p.l.planes_off < p.l.total && ws_bytes >= p.l.total;
     const TiledLayout t = tiled_layout(m, n);
     const long np = (long)t.ntn * T;
     const int m0 = p.l.m0, n0 = p.l.n0, m1 = m - m0, n1 = n - n0;
     // room for residue planes: their own, or first the rows of Ebuf below m0 (whole rows, not swept yet), then those of Cbuf above
-    const size_t room0 = p.l.planes_off ? SPLIT_OWN_PLANES : (size_t)(t.ntm * T - m0) * np * sizeof(double);
-    const size_t room1 = p.l.planes_off ? SPLIT_OWN_PLANES : (size_t)m0 * np * sizeof(double);
+    const size_t taken = p.own_rows ? 0 : p.l.planes_off - p.l.rows_off;
+    const auto room = [&](long rows) { return p.own_planes ? SPLIT_OWN_PLANES : std::max((size_t)rows * np * sizeof(double), taken) - taken; };
+    const size_t room0 = room((long)t.ntm * T - m0), room1 = room(m0);
     const int step[4] = {split_step(m1, n0, m0, room0), split_step(m0, n1, n0, room0), split_step(m1, n1, m0, room1), split_step(m1, n1, n0, room1)};
     if (!step[0] || !step[1] || !step[2] || !step[3]) return p;
     for (int k = 0; k < 4; ++k) p.step[k] = step[k];
@@ -1598,7 +1606,6 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
     const long np = (long)l.ntn * T;
     double *E = reinterpret_cast<double *>(w + l.e_off), *C = reinterpret_cast<double *>(w + l.c_off);
     const int m0 = sl.m0, n0 = sl.n0, m1 = in.m - m0, n1 = in.n - n0;
-    char *rows = w + sl.rows_off;
 
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GPTQ2D_ERR_CUDA;
@@ -1647,8 +1654,13 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
                    ? GPTQ2D_OK : GPTQ2D_ERR_CUDA;
     };
     int st = sweep_one(block(0, 0, 0, 0));
-    void *const own = sl.planes_off ? w + sl.planes_off : nullptr;
-    void *at = own ? own : E + (long)m0 * np;
+    char *rows = nullptr, *at = nullptr;
+    auto use = [&](double *free_rows) {                        // for the planes of the next products
+        char *f = reinterpret_cast<char *>(free_rows);
+        rows = plan.own_rows ? w + sl.rows_off : f;
+        at = plan.own_planes ? w + sl.planes_off : (plan.own_rows ? f : f + (sl.planes_off - sl.rows_off));
+    };
+    use(E + (long)m0 * np);
     if (st == GPTQ2D_OK) st = split_product(m1, n0, m0, plan.step[0], in.L + (long)m0 * in.ldl, in.ldl, E, np, C + (long)m0 * np, np, at, rows, in.info, stream);
     if (st == GPTQ2D_OK) st = split_product(m0, n1, n0, plan.step[1], C, np, in.U + n0, in.ldu, E + n0, np, at, rows, in.info, stream);
     if (st != GPTQ2D_OK) return st;
@@ -1673,7 +1685,7 @@ static int launch_round_split(const TiledParams &in, void *ws, size_t ws_bytes, 
         if (cudaLaunchCooperativeKernel(kernel, dim3(tiled_grid(sms, cells_of(a.m, a.n) + cells_of(b.m, b.n))), dim3(TILED_THREADS), args, TILED_SMEM, stream) != cudaSuccess)
             return GPTQ2D_ERR_CUDA;
     }
-    at = own ? own : C;
+    use(C);
     st = split_product(m1, n1, m0, plan.step[2], in.L + (long)m0 * in.ldl, in.ldl, E + n0, np, C + (long)m0 * np + n0, np, at, rows, in.info, stream);
     if (st == GPTQ2D_OK) st = split_product(m1, n1, n0, plan.step[3], C + (long)m0 * np, np, in.U + n0, in.ldu, E + (long)m0 * np + n0, np, at, rows, in.info, stream);
     if (st == GPTQ2D_OK) st = sweep_one(block(1, 1, 2, 3));

@@ -169,3 +169,24 @@ def test_long_matrices_are_swept_in_blocks_whatever_k_has_to_be_cut_into():
         for m, k in ((4000, n), (n, 4000)):
             assert want <= products(m, k) <= want + 2, (m, k, products(m, k), want)
     assert products(65409, 65409) >= 8
+
+
+def test_blocks_need_little_more_room_than_the_whole_sweep():
+    """The planes' own room only serves speed: with the bookkeeping alone they lie in rows of the workspace that are free at the time."""
+    from paper_2607_27042_b200 import gptq2d as g
+
+    for m, n in ((3969, 3969), (4096, 4096), (4609, 4700), (5003, 4100), (8192, 8192), (4000, 65536)):
+        g.gptq2d_internal_test_hook(7, 1 << 30)
+        whole = g.gptq2d_round_workspace_bytes(m, n)
+        g.gptq2d_internal_test_hook(7, 0)
+        full = g.gptq2d_round_workspace_bytes(m, n)
+        lo, hi = whole, full
+        while hi - lo > 1:
+            mid = (lo + hi) // 2
+            lo, hi = (lo, mid) if g.gptq2d_internal_round_products(m, n, mid) else (mid, hi)
+        # four counters a tile, two a cell of 32 x 32 a byte each, a table of far parts, three rings; below 37 tiles a scale, a top and the bits of
+        # half of the rows and columns
+        tiles = -(-m // 128) * -(-n // 128)
+        most = 60 * tiles + (1 << 17) + (16 * (m + n) if min(m, n) < 4609 else 0)
+        assert g.gptq2d_internal_round_products(m, n, whole) == 0 and hi - whole <= most, (m, n, hi - whole)
+        assert g.gptq2d_internal_round_products(m, n, hi) >= g.gptq2d_internal_round_products(m, n, full) >= 4

@@ -97,9 +97,15 @@ for m, n in [(545, 399), (399, 545), (512, 640)]:
     out = []
     for extra in (0, 1):
         E = padded(np.zeros((m, n)), 3)
-        for order in (1 << 30, 129):
+        for order, less in ((1 << 30, 0), (129, 0), (129, 1)):
             g.gptq2d_internal_test_hook(7, order)
-            Z, _, _, info = g.gptq2d_round(padded(X, extra), padded(L, m %% 2 + extra), padded(U, n %% 2 + extra), E=E)
+            size = g.gptq2d_round_workspace_bytes(m, n)
+            if less:                                     # no room for the planes between blocks: in free rows, in pieces
+                m0, n0 = ((-(-k // 128) + 1) // 2 * 128 for k in (m, n))
+                size -= 16 * (m0 + n0) * max(m0, n0)
+                assert (g.gptq2d_internal_round_products(m, n, size) > 4) == (m < n)      # (the rows below a tall block are too few)
+            ws = torch.full((size,), 0xff, dtype=torch.uint8, device="cuda")
+            Z, _, _, info = g.gptq2d_round(padded(X, extra), padded(L, m %% 2 + extra), padded(U, n %% 2 + extra), E=E, workspace=ws)
             g.check_info(info)
             out.append(Z.cpu())
     assert all(torch.equal(z, out[0]) for z in out)

@@ -27,6 +27,43 @@ def padded(a, extra):
     return buf[:, :c]
 
 
+def workspace(g, m, n, room):
+    """Room for everything, for all but the residue planes, or for the bookkeeping alone: what is missing lies in free rows."""
+    size = g.gptq2d_round_workspace_bytes(m, n)
+    m0, n0 = ((-(-k // 128) + 1) // 2 * 128 for k in (m, n))
+    if room != "all":
+        size -= 16 * (m0 + n0) * max(m0, n0)
+    if room == "none":                                   # scales, tops and bits of an operand's rows, scaling along k
+        up = lambda x: -(-x // 256) * 256
+        size -= sum(up(8 * k) + up(12 * k + k // 16) for k in (m0, n0)) + up(8 * max(m0, n0))
+    return torch.full((size,), 0xff, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("room", ["planes missing", "none"])
+@pytest.mark.parametrize("m,n,extra", [(780, 900, 1), (769, 1900, 3), (1500, 800, 1), (1027, 1290, 0)])
+def test_planes_in_free_rows(g, m, n, extra, room):
+    # k in two pieces and more; ragged last tiles, odd pitches, an outlier channel of integers.  The same sums as with room for the planes, in
+    # more pieces: a rounding of the result a piece.
+    X, A, B = W.gaussian_like(m, n, m + n)
+    L, U, _, _ = O.feedback_factors(A, B)
+    X[0] = np.round(X[0])
+    L[1:, 0] *= 1e6
+    dX, dL, dU = padded(X, extra), padded(L, extra), padded(U, extra)
+    out = []
+    for r in ("all", room):
+        ws = workspace(g, m, n, r)
+        out.append(g.gptq2d_round(dX, dL, dU, workspace=ws, want_E=True, want_margin=True) + (g.gptq2d_internal_round_products(m, n, ws.numel()),))
+        g.check_info(out[-1][3])
+    (Z0, E0, mm0, _, n0), (Z1, E1, mm1, _, n1) = out
+    assert n0 == 4 and n1 > 4, n1
+    assert torch.equal(Z0, Z1) and float((E0 - E1).abs().max()) < 1e-13 and abs(float(mm0[0]) - float(mm1[0])) < 1e-13
+    g.gptq2d_internal_test_hook(7, 0)
+    Z2, E2, _, info = g.gptq2d_round(dX, dL, dU, want_E=True)
+    g.check_info(info)
+    # sums of at most 2900 terms of order one in fp64
+    assert torch.equal(Z2, Z1) and float((E2 - E1).abs().max()) < 1e-12
+
+
 @pytest.mark.parametrize("m,n,extra", [(129, 130, 0), (256, 256, 0), (300, 330, 1), (200, 1000, 2), (1000, 140, 3), (770, 645, 0)])
 def test_blocks_equal_the_oracle_and_the_single_sweep(g, m, n, extra):
     def draw(seed):
@@ -84,8 +121,9 @@ def error(E, Z, X, L, U):
     return np.linalg.norm(np.linalg.solve(L, np.linalg.solve(U.T, R.T).T)) / np.linalg.norm(E)
 
 
+@pytest.mark.parametrize("room", ["all", "planes missing"])
 @pytest.mark.parametrize("kind", ["plain", "scaled", "heavy", "spectrum"])
-def test_blocks_lose_no_precision(g, kind):
+def test_blocks_lose_no_precision(g, kind, room):
     m, n = 640, 700
     rng = np.random.default_rng(21)
     sigma = {"plain": 0.0, "scaled": 1.0, "heavy": 1.5}
@@ -104,8 +142,9 @@ def test_blocks_lose_no_precision(g, kind):
     err = []
     for order in (1 << 30, 129):
         g.gptq2d_internal_test_hook(7, order)
-        Z, E, _, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0), want_E=True)
+        ws = workspace(g, m, n, room) if order == 129 else None
+        Z, E, _, info = g.gptq2d_round(padded(X, 0), padded(L, 0), padded(U, 0), workspace=ws, want_E=True)
         g.check_info(info)
         err.append(error(E.cpu().numpy(), Z.cpu().numpy(), X, L, U))
-    # the same sums, half of them rounded once instead of once a term
+    # the same sums, half of them rounded once (once a piece of k) instead of once a term
     assert err[1] <= 1.05 * err[0], err
