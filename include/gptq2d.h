@@ -16,7 +16,7 @@
  *     to rounding.  The set-up needs three square matrices of order k rounded up to 16, k rounded up to 32 values and 256
  *     bytes a side, the objective two m x n matrices (rows rounded up to 16) and a value per 128 x 128 tile; what the
  *     query returns on top holds the residue planes of large products (16 (k + 512) min(k + 512, 16384) bytes a side from
- *     order 1024 on), without which all products run on the fp64 tensor path.  A sweep needs two m x n matrices
+ *     order 1024 on); a product that the room behind the least does not suffice for runs on the fp64 tensor path.  A sweep needs two m x n matrices
  *     (both sizes rounded up to 128) and its bookkeeping; what lets a large one run in blocks, up to 258 MB, comes on top
  *     (less than 1 MB at order 8192, 136 MB at 4096); with less than 1 MB of that they run in blocks all the same, 2 to 7 % slower.
  *     The library itself holds 78 MB on every GPU where it is loaded, in which running products keep what does not fit on chip

@@ -157,18 +157,34 @@ size_t gptq2d_factor_workspace_bytes(int m, int n) {
     return factor_workspace_bytes(m, n, true);
 }
 
-// Both sides of one problem, arguments already checked, `info` already cleared.
+// Bytes for the residue planes of either side of a problem in a workspace of `bytes`
+struct FactorRooms {
+    size_t a, b;
+    FactorRooms(int m, int n, const double *A, const double *B, size_t bytes) {
+        const size_t extra = (bytes - factor_workspace_bytes(m, n, false)) / 256 * 256;
+        a = A ? factor_side_workspace_bytes(m, true) - factor_side_workspace_bytes(m, false) : 0;
+        b = B ? factor_side_workspace_bytes(n, true) - factor_side_workspace_bytes(n, false) : 0;
+        if (a + b > extra) {
+            a = (size_t)((double)extra / (double)(a + b) * (double)a) / 256 * 256;
+            b = std::min(b, extra - a);
+        }
+    }
+};
+
+// Both sides of one problem, arguments already checked, `info` already cleared.  What `bytes` leaves above the least is for residue planes, shared
+// between the sides in proportion to what either could use.
 static int factor_pair(int m, int n, const double *A, long lda, const double *B, long ldb, double *L, long ldl, double *U,
-                       long ldu, double *dL, double *dU, void *workspace, bool planes, int *info, cudaStream_t stream) {
+                       long ldu, double *dL, double *dU, void *workspace, size_t bytes, int *info, cudaStream_t stream) {
     // The two sides are independent.  Each has a serial spine (one small diagonal-block kernel per 128
     // rows, between the panel and trailing updates) that leaves most SMs idle, so the B side runs on a
     // second stream and its GEMMs fill the gaps of the A side and vice versa.
-    char *wsB = static_cast<char *>(workspace) + factor_side_workspace_bytes(m, planes);
+    const FactorRooms room(m, n, A, B, bytes);
+    char *wsB = static_cast<char *>(workspace) + factor_side_workspace_bytes(m, false) + room.a;
     HostPipe *hp = (A && B) ? host_pipe() : nullptr;
     if (!hp) {
-        int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, nullptr);
+        int st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, room.a, info, stream, nullptr);
         if (st != GPTQ2D_OK) return st;
-        return factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, stream, nullptr);
+        return factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, room.b, info, stream, nullptr);
     }
     std::unique_lock<std::mutex> lock(hp->enqueue);
     if (cudaEventRecord(hp->inputs_free, stream) != cudaSuccess ||
@@ -181,8 +197,8 @@ static int factor_pair(int m, int n, const double *A, long lda, const double *B,
     int st = GPTQ2D_OK, st2 = GPTQ2D_OK;
     for (const int side : {n > m ? 1 : 0, n > m ? 0 : 1}) {
         const FactorLookahead *look = hp->look[side].spine ? &hp->look[side] : nullptr;
-        if (side == 0) st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, planes, info, stream, look);
-        else st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, planes, info, hp->copy, look);
+        if (side == 0) st = factor_one_side(m, A, lda, 0, L, ldl, dL, workspace, room.a, info, stream, look);
+        else st2 = factor_one_side(n, B, ldb, 1, U, ldu, dU, wsB, room.b, info, hp->copy, look);
     }
     // join even if an enqueue failed, so that nothing of this call is left running behind the caller's stream
     if (cudaEventRecord(hp->copies_done, hp->copy) != cudaSuccess ||
@@ -203,8 +219,7 @@ int gptq2d_factor(int m, int n, const double *A, long lda, const double *B, long
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
-    return factor_pair(m, n, A, lda, B, ldb, L, ldl, U, ldu, dL, dU, workspace,
-                       workspace_bytes >= factor_workspace_bytes(m, n, true), info, stream);
+    return factor_pair(m, n, A, lda, B, ldb, L, ldl, U, ldu, dL, dU, workspace, workspace_bytes, info, stream);
 }
 
 static size_t factor_batched_table_bytes(int count) { return pad256((size_t)2 * count * sizeof(FactorSmallSide)); }
@@ -247,7 +262,6 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
     }
     if (!workspace || !aligned(workspace, 256) || workspace_bytes < factor_batched_bytes(count, pr, false))
         return GPTQ2D_ERR_WORKSPACE;
-    const bool planes = workspace_bytes >= factor_batched_bytes(count, pr, true);
     int st = check_device();
     if (st != GPTQ2D_OK) return st;
     if (info && cudaMemsetAsync(info, 0, 4 * sizeof(int), stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;
@@ -278,16 +292,18 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
     int nlarge = 0;
     for (int b = 0; b < count; ++b)
         if (factor_problem_is_large(pr[b])) {
-            slot_bytes = std::max(slot_bytes, factor_workspace_bytes(pr[b].m, pr[b].n, planes));
+            slot_bytes = std::max(slot_bytes, factor_workspace_bytes(pr[b].m, pr[b].n, true));
             ++nlarge;
         }
+    const int nslots = std::min(nlarge, (int)HostPipe::POOL);
+    if (nslots) slot_bytes = std::min(slot_bytes, (workspace_bytes - factor_batched_table_bytes(count)) / nslots / 256 * 256);
     HostPipe *hp = nlarge > 1 ? host_pipe() : nullptr;
     if (!hp || !hp->pool_ok) {
         // one problem (or no second stream): the two-stream route of gptq2d_factor, problem after problem
         for (int b = 0; b < count; ++b) {
             const gptq2d_factor_problem_t &q = pr[b];
             if (!factor_problem_is_large(q)) continue;
-            st = factor_pair(q.m, q.n, q.A, q.lda, q.B, q.ldb, q.L, q.ldl, q.U, q.ldu, q.dL, q.dU, wl, planes, info, stream);
+            st = factor_pair(q.m, q.n, q.A, q.lda, q.B, q.ldb, q.L, q.ldl, q.U, q.ldu, q.dL, q.dU, wl, slot_bytes, info, stream);
             if (st != GPTQ2D_OK) return st;
         }
         return GPTQ2D_OK;
@@ -295,7 +311,6 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
     // Several problems: each is a chain of many small launches, so independent problems go to different
     // streams (round robin; a stream and its workspace slot are shared by every POOL-th problem, in order).
     std::unique_lock<std::mutex> lock(hp->enqueue);
-    const int nslots = std::min(nlarge, (int)HostPipe::POOL);
     if (cudaEventRecord(hp->inputs_free, stream) != cudaSuccess) return GPTQ2D_ERR_CUDA;      // nothing enqueued yet
     int idx = 0, first_err = GPTQ2D_OK;
     for (int k = 0; k < nslots && first_err == GPTQ2D_OK; ++k)
@@ -305,8 +320,9 @@ int gptq2d_factor_batched(int count, const gptq2d_factor_problem_t *pr, void *wo
         if (!factor_problem_is_large(q)) continue;
         const int k = idx++ % nslots;
         char *wk = wl + (size_t)k * slot_bytes;
-        int s1 = factor_one_side(q.m, q.A, q.lda, 0, q.L, q.ldl, q.dL, wk, planes, info, hp->pool[k], nullptr);
-        int s2 = factor_one_side(q.n, q.B, q.ldb, 1, q.U, q.ldu, q.dU, wk + factor_side_workspace_bytes(q.m, planes), planes, info,
+        const FactorRooms room(q.m, q.n, q.A, q.B, slot_bytes);
+        int s1 = factor_one_side(q.m, q.A, q.lda, 0, q.L, q.ldl, q.dL, wk, room.a, info, hp->pool[k], nullptr);
+        int s2 = factor_one_side(q.n, q.B, q.ldb, 1, q.U, q.ldu, q.dU, wk + factor_side_workspace_bytes(q.m, false) + room.a, room.b, info,
                                  hp->pool[k], nullptr);
         if (first_err == GPTQ2D_OK) first_err = s1 != GPTQ2D_OK ? s1 : s2;
     }

@@ -476,7 +476,7 @@ size_t factor_workspace_bytes(int m, int n, bool planes) {
     } while (0)
 
 // side 0: S = M^T M -> out = F (unit lower).  side 1: S = M M^T -> out = F^T (unit upper).
-int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws, bool planes,
+int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws, size_t i8_room,
                     int *info, cudaStream_t stream, const FactorLookahead *look) {
     if (!M) {
         long tot = (long)k * k;
@@ -492,7 +492,6 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     double *p = T + mat;
     const int nblk = (k + FB - 1) / FB;
     char *i8_at = static_cast<char *>(ws) + factor_side_workspace_bytes(k, false);
-    const size_t i8_room = planes ? factor_i8_bytes(k) : 0;
     // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream` or on a stream that it is ordered with, so
     // one set of planes serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
     auto product = [&](const GemmArgs &g, cudaStream_t stream, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
@@ -581,8 +580,12 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         const long k0 = (long)K0 * FB, k1 = (long)K1 * FB < k ? (long)K1 * FB : k;
         return i8_planes_at(i8_at, (int)k0, (int)(k1 - k0), 1);
     };
+    // Block rows per outer block.  More make the large updates cheaper and the steps inside a block, in fp64, dearer; 4 / 6 / 8 / 12
+    // measured, two sides of 8192: 19.75 / 18.94 / 19.09 / 19.37 ms, of 5000: 7.07 / 7.04 / 7.10 / 7.39, one of 8192: 11.8 / 11.8 / 11.9 / 12.3.
+    constexpr int OUTER = 6;
+    const bool panels_fit = i8_room >= i8_planes_bytes(k, OUTER * FB, 1);
     auto split_panels = [&](int K0, int K1, cudaStream_t s) -> int {
-        if (i8_room) CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));
+        if (panels_fit) CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));
         return GPTQ2D_OK;
     };
     auto trailing_multi = [&](int K0, int K1, long r0, long r1, cudaStream_t s) -> int {
@@ -597,7 +600,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         t.C = G + r0 * ld; t.ldc = ld; t.batch = 1; t.lower_tiles_only = r0 == 0 ? 1 : 0;
         const I8Planes pl = panel_planes(K0, K1);
         cudaError_t e = cudaSuccess;
-        if (!i8_room || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
+        if (!panels_fit || !launch_gemm_i8(t, pl.part((int)r0, t.M), pl.part(0, t.N), info, s, &e)) e = launch_gemm(t, s);
         CK(e);
         return GPTQ2D_OK;
     };
@@ -661,15 +664,12 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         }
         return GPTQ2D_OK;
     };
-    // Block rows per outer block.  More make the large updates cheaper and the steps inside a block, in fp64, dearer; 4 / 6 / 8 / 12
-    // measured, two sides of 8192: 19.75 / 18.94 / 19.09 / 19.37 ms, of 5000: 7.07 / 7.04 / 7.10 / 7.39, one of 8192: 11.8 / 11.8 / 11.9 / 12.3.
-    constexpr int OUTER = 6;
     // Which loop.  With two levels less work is done, with one (below) less of it is in the chain of diagonal blocks; what the
     // other side of the same call leaves idle decides between them.  Measured, one level against two, in ms: 4300 beside 4300 5.67 / 5.53, 4608
     // beside 4608 6.32 / 5.88, 5000 beside 5000 7.88 / 7.04, beside 3750 6.27 / 6.00, beside 2500 5.65 / 5.68, 4400 beside 3300 4.88 / 5.04, 4608
     // beside 64 4.31 / 4.52; from 44 block rows on two levels whatever is beside (6144 beside 64: the same).
     const int beside = look ? std::min((look->beside + FB - 1) / FB, nblk) : 0;
-    const bool two_levels = look && (nblk >= 44 || (i8_room && 2 * nblk + beside >= 102));
+    const bool two_levels = look && (nblk >= 44 || (panels_fit && 2 * nblk + beside >= 102));
     // The inverse of the rows below the last doubling, and its product with the panels to the left of it, need nothing of the rows above, which come
     // last and leave most SMs idle; so with the rows of the doubling before, and so on.  They are put together beneath the steps above, on two
     // streams in turn, so that the levels of one part overlap the product of the one before; what is left for the end is one product a

@@ -17,8 +17,9 @@ struct FactorLookahead {
 // `planes`: with room for the residue planes of its large products (i8_gemm.cuh); without, all products are fp64 ones
 size_t factor_workspace_bytes(int m, int n, bool planes);
 size_t factor_side_workspace_bytes(int k, bool planes);
-// side 0: S = M^T M -> out = F (unit lower).  side 1: S = M M^T -> out = F^T (unit upper).
-int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws, bool planes,
+// side 0: S = M^T M -> out = F (unit lower).  side 1: S = M M^T -> out = F^T (unit upper).  i8_room: bytes behind the side's workspace without
+// planes that may hold them; every product that they suffice for is an int8 one
+int factor_one_side(int k, const double *M, long ldm, int side, double *out, long ldo, double *dinv, void *ws, size_t i8_room,
                     int *info, cudaStream_t stream, const FactorLookahead *look);
 
 // One side of a small problem for factor_small_kernel (order k <= FACTOR_SMALL_MAX).

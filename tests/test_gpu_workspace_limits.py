@@ -55,6 +55,26 @@ def test_set_up(g):
     refused(g, lambda w: g.gptq2d_factor_reverse(dA, dB, workspace=w), own + least - 256)
 
 
+def test_set_up_with_room_for_some_planes(g):
+    # each side's updates of rank 768 need a tenth of the room for all products, its largest joins all of it
+    m, n = 4700, 4610
+    A, B = (torch.randn(k, k, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(k)) / (4 * k) ** 0.5 +
+            torch.eye(k, dtype=torch.float64, device="cuda") for k in (m, n))
+    least, most = side(m) + side(n), g.gptq2d_factor_workspace_bytes(m, n)
+    out = []
+    for share in (0.0, 0.2, 0.45, 1.0):
+        got = g.gptq2d_factor(A, B, workspace=ws(least + int(share * (most - least))))
+        g.check_info(got[4])
+        out.append(got)
+    for got in out[1:]:
+        for x, y in zip(got[:4], out[0][:4]):
+            # two fp64 factorisations of Grams of condition below 100
+            assert float((x - y).abs().max()) <= 1e-12 * float(y.abs().max())
+    # every share takes products that the one before had no room for
+    for x, y in zip(out, out[1:]):
+        assert not torch.equal(x[0], y[0]) and not torch.equal(x[1], y[1])
+
+
 def test_set_up_batched(g):
     shapes = [(1100, 40), (1030, 1024), (60, 70)]
     cases = [W.gaussian_like(m, n, 6 + i, samples=2 * max(m, n)) for i, (m, n) in enumerate(shapes)]
