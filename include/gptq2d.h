@@ -346,6 +346,8 @@ int gptq2d_objective(int m, int n,
  *   key 7: smaller order from which on resident fp64 sweeps run in 2 x 2 blocks (0: the default).  Workspace queries follow it.
  *   key 8: most bits of a cell index in a batched sweep (0: what the number of matrices leaves); matrices with more cells of 32 x 32
  *          are swept in launches of their own.  Tests.
+ *   key 10: multiplications from which on the products of set-up and objective run on the int8 tensor cores (0: by their shape).  Workspace queries of
+ *          the objective follow it.  Tests.
  *   key 9: columns of a tile of the products on the int8 tensor cores, 128 or 256 (0: by their size).  Tests.
  * Returns GPTQ2D_OK, or GPTQ2D_ERR_INVALID_ARG for an unknown key.
  */

@@ -84,13 +84,13 @@ static HostPipe *host_pipe() {
         ok = ok && cudaEventCreateWithFlags(&hp.copies_done, cudaEventDisableTiming) == cudaSuccess;
         for (int sd = 0; ok && sd < 2; ++sd) {
             FactorLookahead &lk = hp.look[sd];
-            cudaEvent_t *ev[7] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1], &lk.left[0], &lk.left[1]};
+            cudaEvent_t *ev[8] = {&lk.fork, &lk.join, &lk.panel, &lk.t2[0], &lk.t2[1], &lk.left[0], &lk.left[1], &lk.planes};
             // highest priority: the one-CTA spine kernels must get an SM as soon as one is free, ahead of the
             // queued CTAs of the large updates
             int prio_lo = 0, prio_hi = 0;
             bool lok = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) == cudaSuccess &&
                        cudaStreamCreateWithPriority(&lk.spine, cudaStreamNonBlocking, prio_hi) == cudaSuccess;
-            for (int e = 0; lok && e < 7; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
+            for (int e = 0; lok && e < 8; ++e) lok = cudaEventCreateWithFlags(ev[e], cudaEventDisableTiming) == cudaSuccess;
             if (!lok) lk.spine = nullptr;        // the set-up then runs that side on one stream
         }
         hp.pool_ok = ok;
@@ -602,6 +602,7 @@ int gptq2d_internal_test_hook(int key, long value) {
     if (key == 6) { round_tiled_f32_set_tma_mode((int)value); return GPTQ2D_OK; }
     if (key == 7) { round_split_set_min(value); return GPTQ2D_OK; }
     if (key == 9) { i8_set_tile((int)value); return GPTQ2D_OK; }
+    if (key == 10) { i8_set_least((double)value); return GPTQ2D_OK; }
     if (key == 8) { round_batched_set_cell_bits(value); return GPTQ2D_OK; }
 #ifdef GPTQ2D_CHECKED
     if (key == 5) {          // value: device int[5]; [0..3] receive the status words, [4] the redirected index

@@ -492,8 +492,10 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     double *p = T + mat;
     const int nblk = (k + FB - 1) / FB;
     char *i8_at = static_cast<char *>(ws) + factor_side_workspace_bytes(k, false);
-    // A large product on the int8 tensor cores; everything that uses it is enqueued on `stream` or on a stream that it is ordered with, so
-    // one set of planes serves all.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
+    // A large product on the int8 tensor cores.  One set of planes serves all: a product on another stream than the one that used them last waits
+    // for that one.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
+    bool planes_used = false;
+    cudaStream_t planes_on = stream;
     auto product = [&](const GemmArgs &g, cudaStream_t stream, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
         if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
@@ -507,10 +509,14 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         const I8Planes pb = same ? pa : i8_planes_at(i8_at + bytesA, g.N, g.K, g.batch);
         I8Inner undo = inner;
         undo.inverse = !inner.inverse;
-        cudaError_t e = i8_split(pa, g.A, g.lda, g.strideA, g.opA == OP_N, stream, undo, diag_a);
+        cudaError_t e = planes_used && planes_on != stream ? cudaStreamWaitEvent(stream, look->planes, 0) : cudaSuccess;
+        if (e == cudaSuccess) e = i8_split(pa, g.A, g.lda, g.strideA, g.opA == OP_N, stream, undo, diag_a);
         if (e == cudaSuccess && !same) e = i8_split(pb, g.B, g.ldb, g.strideB, g.opB == OP_T, stream, inner, diag_b);
         if (e != cudaSuccess) return e;
-        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b, I8_LEAST_SETUP)) return launch_gemm(g, stream);
+        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b, I8_LEAST_SETUP)) e = launch_gemm(g, stream);
+        planes_used = true;
+        planes_on = stream;
+        if (e == cudaSuccess && look) e = cudaEventRecord(look->planes, stream);
         return e;
     };
 
@@ -757,14 +763,9 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
                 CK(cudaEventRecord(look->panel, sp));
                 if (early && K == at / FB) {                    // rows [at, end) are final
                     const int e = parts++ & 1;
-                    // what takes the planes goes one behind the other: the product with the panels, and the levels of 1024 rows and more
-                    const bool large = end - at >= 2048;
                     CK(cudaStreamWaitEvent(look->early[e], look->panel, 0));
-                    if (parts > 1 && large) CK(cudaStreamWaitEvent(look->early[e], look->left[e ^ 1], 0));
                     if ((st = levels(at, end, (end - at + FB - 1) / FB, FB, look->early[e])) != GPTQ2D_OK) return st;
-                    if (parts > 1 && !large) CK(cudaStreamWaitEvent(look->early[e], look->left[e ^ 1], 0));
                     if ((st = join_left(0, at, end - at, 1, 0, look->early[e])) != GPTQ2D_OK) return st;
-                    CK(cudaEventRecord(look->left[e], look->early[e]));
                     end = at;
                     at /= 2;
                 }

@@ -11,6 +11,7 @@ struct FactorLookahead {
     cudaStream_t spine;
     cudaStream_t early[2];                   // the inverse of the lower rows, beneath the factorisation of the upper ones
     cudaEvent_t fork, join, panel, t2[2], left[2];
+    cudaEvent_t planes;                      // behind the last product that used the residue planes
     int beside;                              // order of the side that is factorised at the same time
 };
 

@@ -1097,8 +1097,14 @@ i8_gemm_kernel(const __grid_constant__ I8Params p, const __grid_constant__ CUten
     }
 }
 
+static std::atomic<double> g_i8_least{0.0};                    // tests: every product of so many multiplications
+void i8_set_least(double multiplications) { g_i8_least.store(multiplications > 0.0 ? multiplications : 0.0); }
+
 bool gemm_i8_pays(long M, long N, long K, long batch) {
-    if (K > I8_MAX_K || K < 256) return false;
+    if (K > I8_MAX_K) return false;
+    const double least = g_i8_least.load();
+    if (least > 0.0) return (double)M * N * K * batch >= least;
+    if (K < 256) return false;
     // fewer tiles leave SMs idle, and the launches of the splitting are not repaid below some 10^9 products (1024^3: 0.106 ms with the splitting
     // against 0.148)
     const long tiles = ((M + 127) / 128) * ((N + 127) / 128) * batch;

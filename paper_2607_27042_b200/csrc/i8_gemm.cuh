@@ -82,6 +82,7 @@ bool gemm_i8_pays(long M, long N, long K, long batch);
 bool launch_gemm_i8(const GemmArgs &g, const I8Planes &A, const I8Planes &B, int *info, cudaStream_t stream, cudaError_t *err,
                     bool diag_a = false, bool diag_b = false, double least = 0.0);
 
+void i8_set_least(double multiplications);      // tests: products from that many multiplications on pay; 0: by the rule
 void i8_set_tile(int columns);          // tests: tiles of 128 or 256 columns; 0: by the rule
 
 }  // namespace gptq2d

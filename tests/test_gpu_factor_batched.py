@@ -192,6 +192,29 @@ def test_the_inverse_in_two_parts_is_bit_identical_to_the_one_in_one(g, k):
         assert torch.equal(L, L1) and torch.equal(dL, dL1) and torch.equal(U, U2) and torch.equal(dU, dU2)
 
 
+@pytest.mark.parametrize("k", [1100, 1990, 2300, 4090])
+def test_the_planes_serve_one_stream_at_a_time(g, k):
+    # with every product on the int8 tensor cores both streams of the inverse's parts use the planes all the time: bit for bit the call with one
+    # basis, which has one stream
+    torch.manual_seed(k)
+    A, B = (torch.randn(j, j, dtype=torch.float64, device="cuda") / (4 * j) ** 0.5 + torch.eye(j, dtype=torch.float64, device="cuda") for j in (k, 1030))
+    plain = g.gptq2d_factor(A, None, n=1)
+    g.gptq2d_internal_test_hook(10, 1)
+    try:
+        L1, _, dL1, _, i1 = g.gptq2d_factor(A, None, n=1)
+        _, U2, _, dU2, i2 = g.gptq2d_factor(None, A, m=1)
+        for _ in range(5):
+            L, _, dL, _, ia = g.gptq2d_factor(A, B)
+            _, U, _, dU, ib = g.gptq2d_factor(B, A)
+            for i in (i1, i2, ia, ib):
+                g.check_info(i)
+            assert torch.equal(L, L1) and torch.equal(dL, dL1) and torch.equal(U, U2) and torch.equal(dU, dU2)
+    finally:
+        g.gptq2d_internal_test_hook(10, 0)
+    # and with most of them on the fp64 tensor path: a Gram of condition below 100, k roundings of 2^-53 times that
+    assert not torch.equal(plain[0], L1) and float((plain[0] - L1).abs().max()) <= k * 2.0 ** -53 * 100
+
+
 def test_reciprocals_and_quotients_of_the_pivots(g):
     # d over the whole range in which the approximate inverse is taken, significands next to powers of two among them; x up to 2 d
     rng = np.random.default_rng(0)
