@@ -589,6 +589,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     // Block rows per outer block.  More make the large updates cheaper and the steps inside a block, in fp64, dearer; 4 / 6 / 8 / 12
     // measured, two sides of 8192: 19.75 / 18.94 / 19.09 / 19.37 ms, of 5000: 7.07 / 7.04 / 7.10 / 7.39, one of 8192: 11.8 / 11.8 / 11.9 / 12.3.
     constexpr int OUTER = 6;
+    static_assert(OUTER * FB % I8_PAIR_ROWS == 0, "views of the panels' planes begin at outer blocks");
     const bool panels_fit = i8_room >= i8_planes_bytes(k, OUTER * FB, 1);
     auto split_panels = [&](int K0, int K1, cudaStream_t s) -> int {
         if (panels_fit) CK(i8_split(panel_planes(K0, K1), G + (long)K0 * FB * ld, ld, 0, false, s));

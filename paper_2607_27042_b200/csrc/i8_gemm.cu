@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(128, 8) i8_split_kernel(I8Planes pl, const dou
     __shared__ double tile[32][PITCH], factor[80];
     const int k0 = blockIdx.x * 64, r0 = blockIdx.y * 32, b = blockIdx.z, tid = threadIdx.x;
     {
-        const int blocks = (int)(pl.rows_pad / 128), all = (pl.K + I8_KCHUNK - 1) / I8_KCHUNK, pair = r0 / 256 * 2;
+        const int blocks = (int)(pl.rows_pad / 128), all = (pl.K + I8_KCHUNK - 1) / I8_KCHUNK, pair = r0 / I8_PAIR_ROWS * 2;
         int lo, hi;
         i8_chunks(pl.range + (long)b * blocks * 2, pair, 2, blocks, all, lo, hi);
         const int per = 128 / I8_KCHUNK;

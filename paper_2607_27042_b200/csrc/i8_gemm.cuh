@@ -11,6 +11,7 @@
 namespace gptq2d {
 
 constexpr int I8_MODULI = 16;
+constexpr int I8_PAIR_ROWS = 256;       // rows of op(A) that a pair of CTAs takes
 constexpr int I8_KCHUNK = 64;           // granularity along k at which rows of zeros are noticed
 constexpr double I8_LEAST_SETUP = 0x1p-9;
 constexpr int I8_MAX_K = 16384;         // sums up to K 2^110 are determined by their residues
@@ -28,7 +29,8 @@ struct I8Planes {
     int rows, K, batch;
     long rows_pad, k_pad;
     long plane_rows;                    // rows from one plane to the next
-    // the planes of rows [r0, r0 + count) of a single matrix; r0 a multiple of 128
+    // the planes of rows [r0, r0 + count) of a single matrix; r0 a multiple of I8_PAIR_ROWS: stages in which such a group of rows has no entry are not
+    // written (i8_split), and the product finds them by the groups of the view
     I8Planes part(int r0, int count) const {
         I8Planes v = *this;
         v.planes += (long)r0 * 128; v.scale += r0; v.bits += r0; v.maxbits += r0; v.range += r0 / 128 * 2;
