@@ -92,7 +92,8 @@ const char *gptq2d_status_string(int status);
  * From order 1024 on the Gram, the rank-768 updates of large sides and the larger products of the triangular inverse run on the int8 tensor cores,
  * in fixed point 56 bits below the largest entry of a column of the basis or factor: errors relative to the norms of whole columns, below the
  * rounding of the factorisation itself.  A tile of the Gram or the inverse whose largest entries are below 1/512 of what its operand
- * rows could give is computed in fp64.
+ * rows could give is computed in fp64.  How a side's updates are grouped may depend on the order of the other basis of the call (sides from 4353 rows on):
+ * the last bits of L may then change with n, and those of U with m.
  * Device error: GPTQ2D_ERR_NOT_SPD when a Gram is numerically not positive definite
  * (A or B singular); L and U are then undefined.
  * Streams: everything is ordered after the work already on `stream`, and `stream` waits for all of it

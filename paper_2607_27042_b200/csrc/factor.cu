@@ -671,12 +671,14 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         }
         return GPTQ2D_OK;
     };
-    // Which loop.  With two levels less work is done, with one (below) less of it is in the chain of diagonal blocks; what the
-    // other side of the same call leaves idle decides between them.  Measured, one level against two, in ms: 4300 beside 4300 5.67 / 5.53, 4608
-    // beside 4608 6.32 / 5.88, 5000 beside 5000 7.88 / 7.04, beside 3750 6.27 / 6.00, beside 2500 5.65 / 5.68, 4400 beside 3300 4.88 / 5.04, 4608
-    // beside 64 4.31 / 4.52; from 44 block rows on two levels whatever is beside (6144 beside 64: the same).
+    // Which loop.  With two levels less work is done, with one (below) less of it is in the chain of diagonal blocks and the inverse runs beneath; what
+    // the other side of the same call leaves idle decides between them.  Measured, one level against two, in ms (block rows, those beside):
+    // 4300 beside 4300 (34, 34) 5.45 / 5.54, 4480 beside 4480 (35, 35) 5.85 / 5.86, 4500 beside 4500 (36, 36) 6.05 / 5.96, 5000 beside 5000 7.78 / 7.03;
+    // 4736 beside 4000 (37, 32) 5.54 / 5.78, 4500 beside 4200 (36, 33) 5.50 / 5.59, 5000 beside 3300 (40, 26) 5.53 / 5.58, beside 3750 (40, 30) 6.03 / 5.84, 5500
+    // beside 2500 (43, 20) 6.11 / 6.33, beside 3400 (43, 27) 6.64 / 6.60; beside 64 rows 5632 (44) 5.91 / 6.10, 5800 (46) 6.49 / 6.49, 5900 (47)
+    // 6.84 / 6.73, 6144 (48) 7.08 / 6.92, 8192 14.3 / 11.7.
     const int beside = look ? std::min((look->beside + FB - 1) / FB, nblk) : 0;
-    const bool two_levels = look && (nblk >= 44 || (panels_fit && 2 * nblk + beside >= 102));
+    const bool two_levels = look && (nblk >= 46 || (panels_fit && nblk + beside >= 70));
     // The inverse of the rows below the last doubling, and its product with the panels to the left of it, need nothing of the rows above, which come
     // last and leave most SMs idle; so with the rows of the doubling before, and so on.  They are put together beneath the steps above, on two
     // streams in turn, so that the levels of one part overlap the product of the one before; what is left for the end is one product a

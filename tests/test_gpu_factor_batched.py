@@ -160,20 +160,24 @@ def test_a_repeated_channel_is_a_zero_pivot(g, k, i, j):
         assert g.gptq2d_factor_batched([dev(a)], [dev(np.eye(1))])[4].cpu().tolist() == [5, i, 0, 0]
 
 
-@pytest.mark.parametrize("m,n", [(4224, 4225), (4225, 4300), (5000, 3100), (4097, 5120)])
-def test_loops_with_one_and_two_levels_agree(g, m, n):
+@pytest.mark.parametrize("scaled", [False, True])
+@pytest.mark.parametrize("m,n", [(4352, 4353), (4480, 4481), (5000, 3750), (4097, 5120), (40, 5889), (5760, 100)])
+def test_loops_with_one_and_two_levels_agree(g, m, n, scaled):
     # both sides of the rule that chooses the loop by the orders of a call's two sides, last outer blocks of one to six block rows; against
     # the calls with one basis, which take the loop with one level
     torch.manual_seed(m)
     A, B = (torch.randn(k, k, dtype=torch.float64, device="cuda") / (4 * k) ** 0.5 + torch.eye(k, dtype=torch.float64, device="cuda") for k in (m, n))
+    # channels of log-normal scales: column j of A, row j of B; entry (i, j) of L then is s_j / s_i times as large, (i, j) of U s_i / s_j
+    a, b = (torch.exp(torch.randn(k, dtype=torch.float64, device="cuda")) if scaled else torch.ones(k, dtype=torch.float64, device="cuda") for k in (m, n))
+    A, B = A * a, B * b[:, None]
     L, U, dL, dU, info = g.gptq2d_factor(A, B)
     L1, _, dL1, _, i0 = g.gptq2d_factor(A, None, n=1)
     _, U1, _, dU1, i1 = g.gptq2d_factor(None, B, m=1)
     for i in (info, i0, i1):
         g.check_info(i)
-    # two factorisations of a Gram of condition below 100 (singular values of the bases within 1/4 .. 2): k roundings of 2^-53 times that
-    for x, y, k in ((L, L1, m), (U, U1, n), (dL / dL1, torch.ones_like(dL), m), (dU / dU1, torch.ones_like(dU), n)):
-        assert float((x - y).abs().max()) <= k * 2.0 ** -53 * 100
+    # the same sums in pieces of 128 and 768 k: ten times what is measured, 1.1e-16 for entries of 0.1 and less and 1.8e-15 for squared pivots
+    assert float(((L - L1) * a[:, None] / a).abs().max()) <= 1e-15 and float(((U - U1) * b / b[:, None]).abs().max()) <= 1e-15
+    assert float((dL / dL1 - 1).abs().max()) <= 1.8e-14 and float((dU / dU1 - 1).abs().max()) <= 1.8e-14
 
 
 @pytest.mark.parametrize("k", [897, 1024, 1025, 1500, 3000, 4100])
