@@ -159,14 +159,47 @@ def test_extreme_magnitudes(g, ea, eb):
     assert np.abs(want).max() < 2.0 ** 1023 and np.all(np.abs(product(g, a, b) - want) <= bound)
 
 
-def test_the_largest_digit_sums_fit_int32(g):
-    # all digits at an end of their range and of one sign, K at its limit: seven pairs of 128 * 128 * 16384 in one sum
+def test_constant_entries_with_all_digits_at_an_end_of_their_range(g):
+    # K at its limit; every residue is the same along k, so that its sums are K times a square
     K = 16384
     low = sum(256.0 ** -d for d in range(2, 8))
     for x, y in ((126 / 256 + 127 * low, 126 / 256 + 127 * low), (-126 / 256 - 128 * low, 126 / 256 + 127 * low),
                  (-126 / 256 - 128 * low, -126 / 256 - 128 * low)):
         got = product(g, np.full((130, K), x), np.full((K, 5), y))
         assert np.max(np.abs(got - K * x * y)) <= 2.0 ** -50 * abs(K * x * y)
+
+
+@pytest.mark.parametrize("columns", [128, 256])
+@pytest.mark.parametrize("K", [1024, 1025, 16384])
+def test_the_largest_sums_of_residues(g, K, columns):
+    # For every modulus p, entries that are (p - 1) / 2 or its negative modulo p: sums of K ((p - 1) / 2)^2 of either sign, the largest that are reduced
+    # (by one formula up to K = 1024 and another one above).  A residue that is wrong puts S off by a multiple of P / p, 2^117 and more.
+    p = [256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193]
+    rng = np.random.default_rng(K)
+
+    def operand():
+        # integers from 2^54 to 2^55 that are multiples of four (53 bits), a row for either sign of every modulus; all of one binary order, so that
+        # scaling along k and rows' scales leave them as they are
+        rows = []
+        for q in p:
+            for r in ((q - 1) // 2, -((q - 1) // 2)) if q % 2 else (124, -128):
+                if q % 2:
+                    y = rng.integers(2 ** 52, int(1.94 * 2 ** 52), size=K)
+                    x = 4 * (y + (r * pow(4, -1, q) - y) % q)
+                else:
+                    x = rng.integers(2 ** 46, int(1.94 * 2 ** 46), size=K) * 256 + r
+                assert np.all((x - r) % q == 0) and np.all(x % 4 == 0)
+                rows.append(x.astype(np.float64))
+        return np.array(rows)
+    a, b = operand(), operand().T.copy()
+    want = a.astype(np.longdouble) @ b.astype(np.longdouble)
+    g.gptq2d_internal_test_hook(9, columns)
+    try:
+        got = product(g, a, b)
+    finally:
+        g.gptq2d_internal_test_hook(9, 0)
+    # K terms of 2^108 and more, each sum rounded once
+    assert np.max(np.abs(got / want - 1)) <= 2.0 ** -52
 
 
 @pytest.mark.parametrize("k", [1100, 2200])
