@@ -8,8 +8,8 @@
 // for the same 56 bits.  S / P is the fractional part of sum_i (S mod p_i) u_i / p_i with u_i = (P / p_i)^-1 mod p_i; it is summed in 80-bit fixed
 // point (the weights cut at 2^-80: S is off by 2^52 or so and at most 2^57, where rounding the operands to integers moves a sum by 2^54 sqrt(K / 6) if all
 // entries are as large as the largest) and multiplied by P with one rounding.  What the 56 bits round
-// off is of the order 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, normal
-// entries: 4e-16 against 3e-15 of the fp64 tensor path).  Rows whose integers end in zero bits (integers, fp32 data) give an S that
+// off is of the order 2^-57 * sqrt(K) * max|a| * typical|b|, below what a chain of K fp64 additions accumulates (measured at 8192^3, 2-norm
+// of the error over that of the result: normal entries 9.5e-17, uniform ones 4.7e-17, one rounding, against 3.0e-15 of the fp64 tensor path).  Rows whose integers end in zero bits (integers, fp32 data) give an S that
 // ends in as many: it is rounded there, which makes such products exact.
 // An entry far below the largest of its row keeps fewer than its 53 bits, which matters where the largest one meets
 // a zero: a scaling along k (i8_inner_tops) or a look at the result (end of the kernel) takes care of that.
@@ -1105,8 +1105,9 @@ bool gemm_i8_pays(long M, long N, long K, long batch) {
     const double least = g_i8_least.load();
     if (least > 0.0) return (double)M * N * K * batch >= least;
     if (K < 256) return false;
-    // fewer tiles leave SMs idle, and the launches of the splitting are not repaid below some 10^9 products (1024^3: 0.106 ms with the splitting
-    // against 0.148)
+    // Fewer tiles leave SMs idle, and the launches of the splitting are not repaid below some 10^9 products.  us, DMMA / with the splitting, operands in
+    // HBM: 512^3 102 / 113, 640^3 119 / 123, 768^3 136 / 125, 896^3 152 / 133, 1024^3 172 / 139; 1024 x 1024 x 512 101 / 113, 1536 x 1536 x 512 102 / 115, 2048 x
+    // 2048 x 256 105 / 133, x 384 141 / 135, 512 x 4096 x 512 95 / 112.  Set-ups of 1100 to 4100 rows take the same time with the line at 25 to 100 tiles.
     const long tiles = ((M + 127) / 128) * ((N + 127) / 128) * batch;
     return tiles >= 64 && (double)M * N * K * batch >= 0.9e9;
 }

@@ -1176,14 +1176,16 @@ static TiledLayout tiled_layout(int m, int n) {
 // ---- large matrices in 2 x 2 blocks (launch_round_split below): its own bookkeeping, behind the E and C buffers.  One header and ring
 // for each of the three launches and flags for each of the four blocks (cleared per call), then two descriptors and a table
 // of far parts for the launch that sweeps two blocks at once (written per call, on the device).
-// From 32 rows and columns of tiles on (ms, whole / in blocks, E asked for: 3584 x 3584 4.56 / 4.90, 3712 x 3712 4.88 / 5.13, 3840 x 3840 5.35 / 5.42,
-// 3968 x 3968 5.65 / 5.80, 4064 x 4064 6.23 / 6.11, 4000 x 4100 6.39 / 6.15, 4096 x 4096 6.20 / 6.09; 4608 x 4608 8.36 / 7.85, 5120 x 5120 10.98 / 9.87).
-// Odd pitches (3841 x 3841 6.38 / 6.21) and long matrices (3328 x 8192 12.9 / 11.7) gain earlier; those stay with the line of square ones.
+// From 32 rows and columns of tiles on, where square matrices gained with products of digits, and keep gaining with those of residues (ms, whole / in
+// blocks, E asked for: 3584 x 3584 4.53 / 4.59, 3712 x 3712 4.80 / 4.79, 3840 x 3840 5.33 / 5.09, 3968 x 3968 5.59 / 5.46, 4064 x 4064 6.22 / 5.76, 4000 x 4100
+// 6.35 / 5.80, 4096 x 4096 6.15 / 5.75; 4608 x 4608 8.38 / 7.58, 5120 x 5120 11.0 / 9.53).  The crossing has come down to 29 tiles since, odd pitches (3841 x
+// 3841 6.31 / 5.85) and long matrices (3328 x 8192 12.8 / 12.1, 3000 x 6000 7.57 / 6.75, 2500 x 16384 31.5 / 27.5; 2048 x 8192 the same) gain earlier; below the
+// line the last bits of E are those of the whole sweep.
 constexpr int SPLIT_MIN = 31 * T + 1;
 static std::atomic<long> g_split_min{SPLIT_MIN};
 void round_split_set_min(long order) { g_split_min.store(order > 0 ? order : SPLIT_MIN); }
 // Residue planes of a product up to this size get room of their own; those of larger ones lie in rows of the E and C buffers that are free at the time,
-// where k has to be cut (4096 x 4096, 134 MB: 5.80 ms, with two pieces of k 6.13; 8192 x 8192, 537 MB: 29.2 and 30.1).
+// where k has to be cut (4096 x 4096, 134 MB: 5.75 ms, with two pieces of k 6.06; 8192 x 8192, 537 MB: 29.2 and 30.1).
 constexpr size_t SPLIT_OWN_PLANES = (size_t)256 << 20;
 struct SplitLayout {
     int m0, n0;                          // rows / columns of the first block (multiples of T); 0: not split
@@ -1486,11 +1488,12 @@ int launch_round_tiled_batched(int count, const TiledParams *pr, double *min_mar
 // where the far parts of the sweep run at 35.  Three sweeps (the middle one takes two blocks in one launch) replace one; each has
 // its own ramp, which is why small matrices are not cut.
 // Nothing but the workspace is used: where a product's residue planes have no room of their own they lie in rows of Ebuf whose blocks have not been
-// swept yet, or in rows of Cbuf that nobody reads any more; they do not fit there at once, so k is cut (square matrices: in two).
-// ms, whole / in blocks: 4096 x 4096 6.20 / 6.09, 5632 x 5632 14.2 / 12.6, 6144 x 6144 17.9 / 15.2, 4096 x 8192 16.4 / 14.5, 5120 x 8192
-// 21.4 / 18.3; with tasks of 64 x 64 before cells 8192 x 8192 38.0 / 31.9 and 4096 x 4096 6.6 / 8.0.
+// swept yet, or in rows of Cbuf that nobody reads any more; they do not fit there at once, so k is cut (square matrices: in two; 4000 x 65536: the
+// longer side in eighteen).
+// ms, whole / in blocks: 4096 x 4096 6.15 / 5.75, 5632 x 5632 14.2 / 11.6, 6144 x 6144 17.9 / 14.6, 4096 x 8192 16.3 / 14.3, 5120 x 8192
+// 21.4 / 18.0, 8192 x 8192 39.4 / 29.8, 4000 x 16000 46.7 / 38.0, 4000 x 30000 143 / 108, 4000 x 58000 499 / 370.
 // The error of E against an 80-bit residual does not grow: at 3969 x 3969, 4096 x 4096, 4100 x 5003 and 5631 x 5631, with Gaussian, log-normal
-// (sigma 1 and 1.5) and condition 1e6 Grams, it is 0.77 to 0.92 times that of the whole sweep in the 2-norm.
+// (sigma 1, 1.5 and 3) and condition 1e6 Grams, it is 0.77 to 0.96 times that of the whole sweep in the 2-norm.
 
 // descriptors and claim order of a launch that sweeps two matrices (what the host builds for batched launches)
 __global__ void __launch_bounds__(256) split_pair_kernel(TiledKernelParams a, TiledKernelParams b, TiledKernelParams *desc, unsigned *table) {

@@ -1,5 +1,5 @@
 """Resident sweeps in 2 x 2 blocks (the route of large matrices) at small sizes: blocks of one tile and of several, ragged last tiles, odd
-leading dimensions, products whose digit planes fit only piece by piece."""
+leading dimensions, products whose residue planes fit only piece by piece."""
 import numpy as np
 import pytest
 import torch

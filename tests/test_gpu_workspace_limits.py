@@ -1,4 +1,4 @@
-"""Workspaces without room for what only makes a call faster (the digit planes of large products, the bookkeeping of a sweep in
+"""Workspaces without room for what only makes a call faster (the residue planes of large products, the bookkeeping of a sweep in
 blocks): accepted, with the same results; a byte less is refused."""
 import numpy as np
 import pytest
