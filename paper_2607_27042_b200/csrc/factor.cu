@@ -492,21 +492,22 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
     double *p = T + mat;
     const int nblk = (k + FB - 1) / FB;
     char *i8_at = static_cast<char *>(ws) + factor_side_workspace_bytes(k, false);
+    auto in_fp64 = [](const GemmArgs &g, cudaStream_t stream) -> cudaError_t {
+        // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
+        // number of tiles).  They also take the sums of a lower-triangular B in the better order, for which every such product without planes goes to
+        // them: set-ups without any, 128 x 128 / narrow, ms and error of L with scaled channels: 2300 beside 64 1.79 / 1.74, 1.28e-15 / 1.09e-15; 3000
+        // beside 3000 4.06 / 4.12, 1.49e-15 / 1.15e-15; 5000 15.1 / 15.3, 1.83e-15 / 1.41e-15; 8192 56.6 / 58.5, 2.47e-15 / 1.73e-15.
+        const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
+        const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && (2 * tiles <= device_sms() || g.b_lower);
+        return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
+    };
     // A large product on the int8 tensor cores.  One set of planes serves all: a product on another stream than the one that used them last waits
     // for that one.  B = op(A)^T (a Gram, a rank-k update) needs one operand's planes only.
     bool planes_used = false;
     cudaStream_t planes_on = stream;
     auto product = [&](const GemmArgs &g, cudaStream_t stream, bool same, bool diag_a = false, bool diag_b = false, const I8Inner &inner = I8Inner()) -> cudaError_t {
         const size_t bytesA = i8_planes_bytes(g.M, g.K, g.batch), bytesB = same ? 0 : i8_planes_bytes(g.N, g.K, g.batch);
-        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) {
-            // tiles for half of the SMs at most: narrower ones finish sooner (a 128 x 128 tile takes 18 us per 128 k whatever the
-            // number of tiles).  They also take the sums of a lower-triangular B in the better order, for which every such product without planes goes to
-            // them: set-ups without any, 128 x 128 / narrow, ms and error of L with scaled channels: 2300 beside 64 1.79 / 1.74, 1.28e-15 / 1.09e-15; 3000
-            // beside 3000 4.06 / 4.12, 1.49e-15 / 1.15e-15; 5000 15.1 / 15.3, 1.83e-15 / 1.41e-15; 8192 56.6 / 58.5, 2.47e-15 / 1.73e-15.
-            const long tiles = ((g.M + 127L) / 128) * ((g.N + 127L) / 128) * g.batch;
-            const bool narrow = g.opA == OP_N && g.opB == OP_N && g.beta == 0.0 && !g.lower_tiles_only && (2 * tiles <= device_sms() || g.b_lower);
-            return narrow ? launch_gemm_narrow(g, stream) : launch_gemm(g, stream);
-        }
+        if (!gemm_i8_pays(g.M, g.N, g.K, g.batch) || bytesA + bytesB > i8_room) return in_fp64(g, stream);
         const I8Planes pa = i8_planes_at(i8_at, g.M, g.K, g.batch);
         const I8Planes pb = same ? pa : i8_planes_at(i8_at + bytesA, g.N, g.K, g.batch);
         I8Inner undo = inner;
@@ -515,7 +516,7 @@ int factor_one_side(int k, const double *M, long ldm, int side, double *out, lon
         if (e == cudaSuccess) e = i8_split(pa, g.A, g.lda, g.strideA, g.opA == OP_N, stream, undo, diag_a);
         if (e == cudaSuccess && !same) e = i8_split(pb, g.B, g.ldb, g.strideB, g.opB == OP_T, stream, inner, diag_b);
         if (e != cudaSuccess) return e;
-        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b, I8_LEAST_SETUP)) e = launch_gemm(g, stream);
+        if (!launch_gemm_i8(g, pa, pb, info, stream, &e, diag_a, diag_b, I8_LEAST_SETUP)) e = in_fp64(g, stream);
         planes_used = true;
         planes_on = stream;
         if (e == cudaSuccess && look) e = cudaEventRecord(look->planes, stream);

@@ -30,15 +30,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) gemm_kernel(GemmArgs p) {
     B.mn_valid = min(BN, p.N - n0);
     B.aligned16 = ((((uintptr_t)B.ptr) & 15) == 0) && ((p.ldb & 1) == 0);
 
-    // k-range of this tile (whole range unless an operand is triangular); both ends are multiples of 128
-    const int k_lo = p.b_lower ? min(p.K, n0) : 0;
-    const int k_hi = p.a_lower ? min(p.K, m0 + BM) : p.K;
-    A.ptr += A_KCONTIG ? (long)k_lo : (long)k_lo * p.lda;
-    B.ptr += B_KCONTIG ? (long)k_lo : (long)k_lo * p.ldb;
+    // contraction of this tile: all of k unless A is triangular
+    const int K = p.a_lower ? min(p.K, m0 + BM) : p.K;
 
     Acc acc;
     acc.zero();
-    if (k_hi > k_lo) gemm_tile<A_KCONTIG, B_KCONTIG, GEMM_NSTAGE>(acc, smem, A, B, k_hi - k_lo);
+    if (K > 0) gemm_tile<A_KCONTIG, B_KCONTIG, GEMM_NSTAGE>(acc, smem, A, B, K);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int wm = warp >> 2, wn = warp & 3, g = lane >> 2, t = lane & 3;
@@ -164,13 +161,12 @@ gemm_tma_kernel(GemmArgs p, const __grid_constant__ CUtensorMap mapA, const __gr
     tma_ring_init<GEMM_TMA_NSTAGE, GEMM_THREADS / 32>(ring, bars, stages, tid);
     __syncthreads();
 
-    const int k_lo = p.b_lower ? min(p.K, n0) : 0;
-    const int k_hi = p.a_lower ? min(p.K, m0 + BM) : p.K;
+    const int K = p.a_lower ? min(p.K, m0 + BM) : p.K;
     Acc acc;
     acc.zero();
-    if (k_hi > k_lo) {
-        TmaOperand A{&mapA, m0, k_lo, bz}, B{&mapB, n0, k_lo, bz};
-        const int nk = (k_hi - k_lo + TMA_BK - 1) / TMA_BK;
+    if (K > 0) {
+        TmaOperand A{&mapA, m0, 0, bz}, B{&mapB, n0, 0, bz};
+        const int nk = (K + TMA_BK - 1) / TMA_BK;
         if (!gemm_tma_mainloop<A_KCONTIG, B_KCONTIG, GEMM_TMA_NSTAGE, SLAB_SYNC ? 1 : -1>(acc, ring, A, B, nk, warp, lane, abort))
             return;
     }
