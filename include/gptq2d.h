@@ -18,7 +18,7 @@
  *     query returns on top holds the residue planes of large products (16 (k + 512) min(k + 512, 16384) bytes a side from
  *     order 1024 on); a product that the room behind the least does not suffice for runs on the fp64 tensor path.  A sweep needs two m x n matrices
  *     (both sizes rounded up to 128) and its bookkeeping; what lets a large one run in blocks, up to 258 MB, comes on top
- *     (less than 1 MB at order 8192, 136 MB at 4096); with less than 1 MB of that they run in blocks all the same, 2 to 7 % slower.
+ *     (less than 1 MB at order 8192, 136 MB at 4096); with about 1 MB of that they run in blocks all the same, 2 to 9 % slower.
  *     The library itself holds 78 MB on every GPU where it is loaded, in which running products keep what does not fit on chip
  *     (i8_gemm.cu); calls on any number of streams share it.
  *   - `stream` is a cudaStream_t passed as void* (NULL = default stream).  Calls
